@@ -117,7 +117,10 @@ void prof_reset() {
   for (int c = 0; c < PROF_NCLASS; ++c) { g_prof.launches[c] = 0; g_prof.ms[c] = 0.0; }
 }
 
-constexpr int kElasticThreads = 256;
+// 128 threads: the float64 local step of a mesh of a few hundred tets then has
+// one warp per SM sub-partition (its float64 pipe serves one warp about every
+// 66 cycles), and large meshes lose nothing
+constexpr int kElasticThreads = 128;
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -165,7 +168,121 @@ __global__ void k_actuation(int T, const double* __restrict__ fiber,
   }
 }
 
-template <int PREC>
+// a = axial(skew(R^T M)) of the matrices given by their columns' products:
+// the right-hand side of the rotation correction below
+__device__ __forceinline__ void skew_rtm(const double R[3][3], const double M[3][3], float a[3]) {
+  const double d0 = R[0][2] * M[0][1] + R[1][2] * M[1][1] + R[2][2] * M[2][1] -
+                    R[0][1] * M[0][2] - R[1][1] * M[1][2] - R[2][1] * M[2][2];
+  const double d1 = R[0][0] * M[0][2] + R[1][0] * M[1][2] + R[2][0] * M[2][2] -
+                    R[0][2] * M[0][0] - R[1][2] * M[1][0] - R[2][2] * M[2][0];
+  const double d2 = R[0][1] * M[0][0] + R[1][1] * M[1][0] + R[2][1] * M[2][0] -
+                    R[0][0] * M[0][1] - R[1][0] * M[1][1] - R[2][0] * M[2][1];
+  a[0] = 0.5f * (float)d0;
+  a[1] = 0.5f * (float)d1;
+  a[2] = 0.5f * (float)d2;
+}
+
+// Rotation factor of M in float64 from a float32 rotation and two
+// corrections.  Each correction re-orthonormalises R (D = (I - R^T R) / 2) and
+// rotates it by w, the solution of ((tr S) I - S) w = 2 axial(skew(R^T M)),
+// S = sym(R^T M): the first-order condition for R^T M to be symmetric.  The
+// residuals R^T R - I and skew(R^T M) are formed to float64 accuracy; the
+// corrections themselves are tiny (1e-7, then 1e-14), so they are computed and
+// applied in float32, which leaves about 1e-7 of each: 1e-14 after the
+// first, rounding of R after the second.  About 130 float64 operations where
+// a float64 Jacobi SVD takes about 2,200, and GB300 issues a warp-wide
+// float64 operation only every 66 cycles per SM sub-partition.  M with
+// det <= 0, nearly singular, or where (tr S) I - S is, keeps the Jacobi SVD.
+__device__ __forceinline__ bool polar_refined_f64(const double M[3][3], double R[3][3]) {
+  float Mf[3][3], R0[3][3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) Mf[i][j] = (float)M[i][j];
+  if (!polar_rotation_newton(Mf, R0)) return false;
+  // S = R0^T M and the inverse of (tr S) I - S (adjugate) in float32
+  float S[3][3];
+  matmul_tn(R0, Mf, S);
+  const float s01 = 0.5f * (S[0][1] + S[1][0]), s02 = 0.5f * (S[0][2] + S[2][0]);
+  const float s12 = 0.5f * (S[1][2] + S[2][1]);
+  const float A00 = S[1][1] + S[2][2], A11 = S[0][0] + S[2][2], A22 = S[0][0] + S[1][1];
+  const float c00 = A11 * A22 - s12 * s12, c01 = s02 * s12 + s01 * A22, c02 = s01 * s12 + s02 * A11;
+  const float c11 = A00 * A22 - s02 * s02, c12 = s01 * s02 + s12 * A00, c22 = A00 * A11 - s01 * s01;
+  const float det = A00 * c00 - s01 * c01 - s02 * c02;
+  const float tr = S[0][0] + S[1][1] + S[2][2];
+  if (!(det > 1e-3f * tr * tr * tr)) return false;
+  const float id = 2.f / det;
+  auto turn = [&](const float a[3], float w[3]) {
+    w[0] = id * (c00 * a[0] + c01 * a[1] + c02 * a[2]);
+    w[1] = id * (c01 * a[0] + c11 * a[1] + c12 * a[2]);
+    w[2] = id * (c02 * a[0] + c12 * a[1] + c22 * a[2]);
+  };
+  // first correction: D from exact float32 products, the skew part from R0
+  // in float64 plus the part of R0 D in float32
+  float D[3][3], Rc[3][3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = i; j < 3; ++j) {
+      const df g = df_dot3_ff(R0[0][i], R0[0][j], R0[1][i], R0[1][j], R0[2][i], R0[2][j]);
+      D[i][j] = D[j][i] = 0.5f * ((i == j ? 1.f - g.hi : -g.hi) - g.lo);
+    }
+  matmul(R0, D, Rc);
+  double Rd[3][3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) Rd[i][j] = (double)R0[i][j];
+  float a[3], w[3];
+  skew_rtm(Rd, M, a);
+  {
+    float C[3][3];
+    matmul_tn(Rc, Mf, C);
+    a[0] += 0.5f * (C[2][1] - C[1][2]);
+    a[1] += 0.5f * (C[0][2] - C[2][0]);
+    a[2] += 0.5f * (C[1][0] - C[0][1]);
+  }
+  turn(a, w);
+  if (!(w[0] * w[0] + w[1] * w[1] + w[2] * w[2] < 1e-9f)) return false;
+  {   // R1 = R0 + R0 D + R0 [w] (the products of the corrections are left to the second)
+    const float W[3][3] = {{0.f, -w[2], w[1]}, {w[2], 0.f, -w[0]}, {-w[1], w[0], 0.f}};
+    float T[3][3];
+    matmul(R0, W, T);
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) Rd[i][j] += (double)(Rc[i][j] + T[i][j]);
+  }
+  // second correction: both residuals in float64; skew(D S) is what the
+  // re-orthonormalisation adds to the skew part
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = i; j < 3; ++j) {
+      const double g = Rd[0][i] * Rd[0][j] + Rd[1][i] * Rd[1][j] + Rd[2][i] * Rd[2][j];
+      D[i][j] = D[j][i] = 0.5f * (float)((i == j ? 1.0 : 0.0) - g);
+    }
+  skew_rtm(Rd, M, a);
+  {
+    float C[3][3];
+    matmul(D, S, C);
+    a[0] += 0.5f * (C[2][1] - C[1][2]);
+    a[1] += 0.5f * (C[0][2] - C[2][0]);
+    a[2] += 0.5f * (C[1][0] - C[0][1]);
+  }
+  turn(a, w);
+  const float W[3][3] = {{D[0][0], D[0][1] - w[2], D[0][2] + w[1]},
+                         {D[1][0] + w[2], D[1][1], D[1][2] - w[0]},
+                         {D[2][0] - w[1], D[2][1] + w[0], D[2][2]}};
+  float T[3][3];
+  matmul(R0, W, T);
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) R[i][j] = Rd[i][j] + (double)T[i][j];
+  return true;
+}
+
 __global__ void __launch_bounds__(kElasticThreads)
 k_elastic(int T, const int4* __restrict__ tets, const double* __restrict__ dminv,
           const double* __restrict__ w, const double* __restrict__ act,
@@ -201,22 +318,7 @@ k_elastic(int T, const int4* __restrict__ tets, const double* __restrict__ dminv
     A[2][2] = act[5 * (size_t)T + t];
     double M[3][3], R[3][3];
     matmul(F, A, M);
-    if (PREC == 0) {
-      polar_rotation<double, 10>(M, R);
-    } else {
-      float Mf[3][3], Rf[3][3];
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) Mf[i][j] = (float)M[i][j];
-      polar_rotation<float, 6>(Mf, Rf);
-      double R0[3][3];
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) R0[i][j] = (double)Rf[i][j];
-      polar_refine(M, R0, R);
-    }
+    if (!polar_refined_f64(M, R)) polar_rotation<double, 10>(M, R);
     double P[3][3];
     matmul(R, A, P);
     const double wt = w[t];
@@ -261,7 +363,7 @@ k_elastic(int T, const int4* __restrict__ tets, const double* __restrict__ dminv
 //   F = Ds Dm^-1 = I + Du Dm^-1,  Du = [u1 - u0, u2 - u0, u3 - u0],
 // which keeps F - I (the strain) to double-float accuracy relative to itself.
 // Then M = F A, a float32 rotation R0 of M (Jacobi SVD) refined to float64
-// accuracy as in polar_refine but with the small terms in float32:
+// accuracy by one correction step with the small terms in float32:
 // R1 = R0 + R0 D with D = (I - R0^T R0) / 2 (about 1e-7), the skew part of
 // S = R1^T M kept in double-float, w = ((tr S) I - S)^-1 2 a in float32, and
 // R = R1 exp([w]) = R0 + C with C = R0 D + R0 (E - I) + R0 D (E - I) (all
@@ -350,7 +452,7 @@ __device__ __forceinline__ void elastic_df_body(int T, const int4* __restrict__ 
       for (int i = 0; i < 3; ++i)
 #pragma unroll
         for (int j = 0; j < 3; ++j) Mf[i][j] = M[i][j].hi;
-      polar_rotation<float, 6>(Mf, R0);
+      if (!polar_rotation_newton(Mf, R0)) polar_rotation<float, 6>(Mf, R0);
     }
     // D = (I - R0^T R0) / 2 from exact float products summed in double-float
     float Dm[3][3];
@@ -364,22 +466,27 @@ __device__ __forceinline__ void elastic_df_body(int T, const int4* __restrict__ 
       }
     float R1c[3][3];
     matmul(R0, Dm, R1c);
-    // S = R1^T M = R0^T M (double-float) + R1c^T M (float)
+    // S = R1^T M = R0^T M (double-float) + R1c^T M (float); the diagonal only
+    // enters (tr S) I - S, so float32 serves
     df S[3][3];
+    float Sd[3];
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
+    for (int i = 0; i < 3; ++i) {
+      Sd[i] = R0[0][i] * M[0][i].hi + R0[1][i] * M[1][i].hi + R0[2][i] * M[2][i].hi;
 #pragma unroll
       for (int j = 0; j < 3; ++j) {
+        if (i == j) continue;
         df acc = df_dot3_f(M[0][j], R0[0][i], M[1][j], R0[1][i], M[2][j], R0[2][i]);
         const float c = R1c[0][i] * M[0][j].hi + R1c[1][i] * M[1][j].hi + R1c[2][i] * M[2][j].hi;
         // c is a correction of relative size ~1e-7: it joins the low part
         S[i][j] = df_fast_two_sum(acc.hi, __fadd_rn(acc.lo, c));
       }
+    }
     float wv0 = 0.f, wv1 = 0.f, wv2 = 0.f;
     {
       const df d0 = df_sub(S[2][1], S[1][2]), d1 = df_sub(S[0][2], S[2][0]), d2 = df_sub(S[1][0], S[0][1]);
       const float a0 = 0.5f * (d0.hi + d0.lo), a1 = 0.5f * (d1.hi + d1.lo), a2 = 0.5f * (d2.hi + d2.lo);
-      const float s00 = S[0][0].hi, s11 = S[1][1].hi, s22 = S[2][2].hi;
+      const float s00 = Sd[0], s11 = Sd[1], s22 = Sd[2];
       const float s01 = 0.5f * (S[0][1].hi + S[1][0].hi);
       const float s02 = 0.5f * (S[0][2].hi + S[2][0].hi);
       const float s12 = 0.5f * (S[1][2].hi + S[2][1].hi);
@@ -659,31 +766,24 @@ void launch_actuation(cudaStream_t s, int T, const double* fiber, const double* 
 
 int elastic_blocks(int T) { return (T + kElasticThreads - 1) / kElasticThreads; }
 
-bool elastic_uses_df(const DevMesh& m, int precision) {
-  return precision != 0 && m.dminv_df && m.act_df && m.w_df && m.udf;
-}
-
 void launch_elastic(cudaStream_t s, const DevMesh& m, const double* x, double* tetf,
                     double* proj, double* partials, int precision) {
   const int nb = elastic_blocks(m.T);
   ProfScope ps(PROF_ELASTIC, s);
   if (precision == 0) {
-    k_elastic<0><<<nb, kElasticThreads, 0, s>>>(m.T, m.tets, m.dminv, m.w, m.act, x, tetf, proj, partials);
+    k_elastic<<<nb, kElasticThreads, 0, s>>>(m.T, m.tets, m.dminv, m.w, m.act, x, tetf, proj, partials);
     count_launch();
-  } else if (elastic_uses_df(m, precision)) {
+  } else {
     k_disp_df<<<(3 * m.n + 255) / 256, 256, 0, s>>>(3 * m.n, x, m.rest, m.udf);
     k_elastic_df<<<nb, kElasticThreads, 0, s>>>(m.T, m.tets, m.dminv_df, m.w_df, m.act_df, m.udf,
                                                reinterpret_cast<float2*>(tetf), proj, partials);
     count_launch(2);
-  } else {
-    k_elastic<1><<<nb, kElasticThreads, 0, s>>>(m.T, m.tets, m.dminv, m.w, m.act, x, tetf, proj, partials);
-    count_launch();
   }
 }
 
 void launch_gather_forces(cudaStream_t s, const DevMesh& m, const double* tetf, double* g,
                           int precision) {
-  if (elastic_uses_df(m, precision))
+  if (precision != 0)
     k_gather_forces_df<<<(m.n + 255) / 256, 256, 0, s>>>(m.n, m.T, m.vinc_ptr, m.vinc_slot,
                                                          reinterpret_cast<const float2*>(tetf),
                                                          m.pinned, g);
