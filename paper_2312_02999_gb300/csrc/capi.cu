@@ -305,7 +305,8 @@ int graph_slot(const DevMesh& m, int first, int count, const void* key, int key2
 // ---------------------------------------------------------------------------
 // one evaluation at positions xb: local step (energy + per-tet forces into
 // tetf), proxy positions sb and the constraint set with barrier energy.
-// Leaves E in scal[2], B in scal[0], |C| in counters[0].
+// Leaves E in scal[2], B in scal[0], |C| in counters[0].  With tetf NULL the
+// local step is left out (a caller that only wants the contacts).
 // ---------------------------------------------------------------------------
 int evaluate(const Exec& ex, const MeshState& ms, const DevMesh& m, const double* xb, double* sb,
              double* tetf, double* proj, int prec, double kappa) {
@@ -314,16 +315,18 @@ int evaluate(const Exec& ex, const MeshState& ms, const DevMesh& m, const double
   CK(cudaMemsetAsync(m.counters + 5, 0, sizeof(int), s));       // touching pair
   CK(cudaMemsetAsync(m.counters + 8, 0, sizeof(int), s));       // near-pair list
   CK(cudaMemsetAsync(m.scal, 0, sizeof(double) * 1, s));
-  launch_elastic(s, m, xb, tetf, proj, m.partials, prec);
-  launch_sum_partials(s, m.partials, elastic_blocks(m.T), m.scal + 2);
+  if (tetf) {
+    launch_elastic(s, m, xb, tetf, proj, m.partials, prec);
+    launch_sum_partials(s, m.partials, elastic_blocks(m.T), m.scal + 2);
+  }
   launch_proxy(s, m, xb, sb);
   launch_detect(s, m, sb, ms.p.dhat, kappa);
   CK(cudaGetLastError());
   return FSIM_OK;
 }
 
-// Gradient g-hat (elastic from tetf + barrier over the pairs in m.pairs at
-// sb) into gout, the contact-affected set, B-check and ||g||^2.
+// Gradient g-hat (elastic from tetf, zero if NULL, + barrier over the pairs in
+// m.pairs at sb) into gout, the contact-affected set, B-check and ||g||^2.
 // Requires counters[0] (|C|) already on the host in npairs.
 // bprec is the precision of the pairs' PSD eigen-solves (prec unless the
 // frame switched its contact Hessian to float64).
@@ -331,7 +334,8 @@ int gradient_and_hessian(const Exec& ex, const MeshState& ms, DevMesh& m, const 
                          const double* tetf, double* gout, int64_t npairs, int prec, int* nc_out,
                          double* gn2_out, double kappa, int bprec = -1) {
   cudaStream_t s = ex.stream;
-  launch_gather_forces(s, m, tetf, gout, prec);
+  if (tetf) launch_gather_forces(s, m, tetf, gout, prec);
+  else CK(cudaMemsetAsync(gout, 0, sizeof(double) * 3 * (size_t)m.n, s));
   CK(cudaMemsetAsync(m.x2mark, 0, sizeof(int) * std::max(m.n2, 1), s));
   launch_barrier_pairs(s, m, npairs, sb, ms.p.dhat, kappa, bprec < 0 ? prec : bprec);
   if (m.n2 > 0) launch_mark_scan(s, m);
@@ -1063,7 +1067,7 @@ fsim_status fsim_read_contacts(fsim_ctx_t ctx, int mesh_id, int32_t* keys, int64
   cudaSetDevice(ctx->device);
   DevMesh& m = ms->d;
   const Exec ex = ctx_exec(ctx, *ms);
-  TRY(evaluate(ex, *ms, m, m.x, m.st, m.tetf_t, nullptr, 0, ms->kappa));
+  TRY(evaluate(ex, *ms, m, m.x, m.st, nullptr, nullptr, 0, ms->kappa));
   TRY(sync_read(ex, m));
   if (ctx->h_counters[2]) return FSIM_ECONTACT_OVERFLOW;
   return copy_keys(ctx, *ms, ctx->h_counters[0], keys, cap, count);
@@ -1120,7 +1124,7 @@ fsim_status fsim_eval_contacts(fsim_ctx_t ctx, int mesh_id, const double* x, int
   DevMesh& m = ms->d;
   TRY(stage_x(ctx, *ms, x));
   const Exec ex = ctx_exec(ctx, *ms);
-  TRY(evaluate(ex, *ms, m, m.xt, m.st, m.tetf_t, nullptr, 0, ms->kappa));
+  TRY(evaluate(ex, *ms, m, m.xt, m.st, nullptr, nullptr, 0, ms->kappa));
   TRY(sync_read(ex, m));
   if (ctx->h_counters[2]) return FSIM_ECONTACT_OVERFLOW;
   if (barrier_energy_out) *barrier_energy_out = ctx->h_scal[0];
@@ -1137,15 +1141,14 @@ fsim_status fsim_eval_barrier(fsim_ctx_t ctx, int mesh_id, const double* x, doub
   cudaStream_t s = ctx->stream;
   TRY(stage_x(ctx, *ms, x));
   const Exec ex = ctx_exec(ctx, *ms);
-  TRY(evaluate(ex, *ms, m, m.xt, m.st, m.tetf_t, nullptr, 0, ms->kappa));
+  TRY(evaluate(ex, *ms, m, m.xt, m.st, nullptr, nullptr, 0, ms->kappa));
   TRY(sync_read(ex, m));
   if (ctx->h_counters[2]) return FSIM_ECONTACT_OVERFLOW;
   const int64_t np = ctx->h_counters[0];
-  // barrier gradient only: zero elastic forces by gathering a zero tetf
-  CK(cudaMemsetAsync(m.tetf_t, 0, sizeof(double) * 12 * (size_t)m.T, s));
+  // barrier gradient only: no elastic forces
   int nc = 0;
   double gn2 = 0.0;
-  TRY(gradient_and_hessian(ex, *ms, m, m.st, m.tetf_t, ms->gtmp, np, 0, &nc, &gn2, ms->kappa));
+  TRY(gradient_and_hessian(ex, *ms, m, m.st, nullptr, ms->gtmp, np, 0, &nc, &gn2, ms->kappa));
   if (n_c) *n_c = nc;
   if (grad_out)
     CK(cudaMemcpy(grad_out, ms->gtmp, sizeof(double) * 3 * (size_t)m.n, cudaMemcpyDeviceToHost));
