@@ -236,13 +236,14 @@ __device__ __forceinline__ void to_rel_f(const double X[4][3], float Y[4][3]) {
     for (int d = 0; d < 3; ++d) Y[k][d] = (float)(X[k][d] - X[0][d]);
 }
 
-// IPC barrier and its first two derivatives (reading of Eq. 3's b).
-__device__ __forceinline__ void barrier3(double d, double dhat, double& b, double& b1, double& b2) {
+// First two derivatives of the IPC barrier (reading of Eq. 3's b).
+__device__ __forceinline__ void barrier_derivatives(double d, double inv_d, double dhat, double& b1,
+                                                    double& b2) {
   const double u = d - dhat;
-  const double L = log(d / dhat);
-  b = -u * u * L;
-  b1 = -2.0 * u * L - u * u / d;
-  b2 = -2.0 * L - 4.0 * u / d + u * u / (d * d);
+  const double L2 = 2.0 * log(d / dhat);
+  const double q = u * inv_d;
+  b1 = -u * (L2 + q);
+  b2 = fma(q, q, -fma(4.0, q, L2));
 }
 
 __device__ __forceinline__ double barrier_value(double d, double dhat) {
@@ -265,93 +266,142 @@ struct PairReduced {
   double A[5][5];      // reduced Hessian (n x n used)
 };
 
+// The cost is float64 instructions (one per warp every 66 cycles per SM
+// sub-partition, and a division is about 16 of them), so the divisions are
+// reciprocals shared by their numerators, products feeding sums are fused,
+// and only the upper triangle is formed.  With F' = F / 2 (F as at the top of
+// this file) the reduced Hessian is
+//   K2 v^ v^T + K1 (|c|^2 (I - v^ v^T) - F' (E^T E)^-1 F'^T),
+//   K1 = kappa b' / d, K2 = kappa b'' |c|^2:
+// the two parts that nearly cancel near a face or an edge interior are
+// subtracted before the factor 1 / d.
+__device__ __forceinline__ double dot4(const double* a, const double* b) {
+  return fma(a[3], b[3], fma(a[2], b[2], fma(a[1], b[1], a[0] * b[0])));
+}
+
 __device__ void pair_reduced(int type, const double X[4][3], double dhat, double kappa,
                              PairReduced& r) {
   PairGeom g;
   pair_geometry(type, X, g);
   const double d = sqrt(g.d2);
-  double b, b1, b2;
-  barrier3(d, dhat, b, b1, b2);
+  const double inv_d = 1.0 / d;
+  double b1, b2;
+  barrier_derivatives(d, inv_d, dhat, b1, b2);
   const int k = g.k, n = 3 + k;
   r.n = n; r.k = k; r.d = d; r.gfac = kappa * b1;
-  // orthonormal (c^, q_1 .. q_k) in R^4
-  const double cn = sqrt(g.c[0] * g.c[0] + g.c[1] * g.c[1] + g.c[2] * g.c[2] + g.c[3] * g.c[3]);
-  for (int i = 0; i < 4; ++i) { r.c[i] = g.c[i]; r.ch[i] = g.c[i] / cn; }
-  double qc[2][2] = {{0, 0}, {0, 0}};   // q_m . c'_k
-  double chc[2] = {0, 0};                // c^ . c'_k
-  for (int m = 0; m < k; ++m) {
+  // orthonormal (c^, q_1 .. q_k) in R^4 by Gram-Schmidt; the coefficients
+  // c^ . c'_k and q_m . c'_k of c'_k come out of it (q_2 . c'_1 = 0)
+  const double cn2 = dot4(g.c, g.c);
+  const double cn = sqrt(cn2), icn = 1.0 / cn;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    r.c[i] = g.c[i];
+    r.ch[i] = g.c[i] * icn;
+    r.q[0][i] = 0.0;
+    r.q[1][i] = 0.0;
+  }
+  double chc[2] = {0.0, 0.0}, q00 = 0.0, q01 = 0.0, q11 = 0.0;
+  double E[2][3] = {{0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}};
+#pragma unroll
+  for (int kk = 0; kk < 2; ++kk) {
+    if (kk >= k) continue;
+    chc[kk] = dot4(r.ch, g.cp[kk]);
     double w[4];
-    for (int i = 0; i < 4; ++i) w[i] = g.cp[m][i];
-    double a = 0;
-    for (int i = 0; i < 4; ++i) a += r.ch[i] * w[i];
-    for (int i = 0; i < 4; ++i) w[i] -= a * r.ch[i];
-    for (int l = 0; l < m; ++l) {
-      double bq = 0;
-      for (int i = 0; i < 4; ++i) bq += r.q[l][i] * w[i];
-      for (int i = 0; i < 4; ++i) w[i] -= bq * r.q[l][i];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) w[i] = fma(-chc[kk], r.ch[i], g.cp[kk][i]);
+    if (kk == 1) {
+      q01 = dot4(r.q[0], w);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) w[i] = fma(-q01, r.q[0][i], w[i]);
     }
-    const double wn = sqrt(w[0] * w[0] + w[1] * w[1] + w[2] * w[2] + w[3] * w[3]);
-    for (int i = 0; i < 4; ++i) r.q[m][i] = w[i] / wn;
-  }
-  for (int m = k; m < 2; ++m)
-    for (int i = 0; i < 4; ++i) r.q[m][i] = 0.0;
-  for (int kk = 0; kk < k; ++kk) {
-    double t = 0;
-    for (int i = 0; i < 4; ++i) t += r.ch[i] * g.cp[kk][i];
-    chc[kk] = t;
-    for (int m = 0; m < k; ++m) {
-      double u = 0;
-      for (int i = 0; i < 4; ++i) u += r.q[m][i] * g.cp[kk][i];
-      qc[m][kk] = u;
-    }
-  }
-  double E[2][3];
-  for (int kk = 0; kk < k; ++kk)
+    const double w2 = dot4(w, w), iw = rsqrt(w2);
+    if (kk == 0) q00 = w2 * iw;
+    else q11 = w2 * iw;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) r.q[kk][i] = w[i] * iw;
+#pragma unroll
     for (int dd = 0; dd < 3; ++dd)
-      E[kk][dd] = g.cp[kk][0] * X[0][dd] + g.cp[kk][1] * X[1][dd] + g.cp[kk][2] * X[2][dd] +
-                  g.cp[kk][3] * X[3][dd];
-  // reduced hess d^2: diag(2|c|^2 I3, 0) - F (2 E^T E)^-1 F^T
-  double Hd2[5][5];
-  for (int i = 0; i < 5; ++i)
-    for (int j = 0; j < 5; ++j) Hd2[i][j] = 0.0;
-  for (int a = 0; a < 3; ++a) Hd2[a][a] = 2.0 * cn * cn;
-  if (k > 0) {
-    double Fr[5][2];
-    for (int kk = 0; kk < k; ++kk) {
-      for (int a = 0; a < 3; ++a) Fr[a][kk] = 2.0 * (chc[kk] * g.v[a] + cn * E[kk][a]);
-      for (int m = 0; m < k; ++m) Fr[3 + m][kk] = 2.0 * qc[m][kk] * d;
-    }
-    double G[2][2], Gi[2][2];
-    for (int a = 0; a < k; ++a)
-      for (int bb = 0; bb < k; ++bb) G[a][bb] = 2.0 * dot3(E[a], E[bb]);
-    if (k == 1) {
-      Gi[0][0] = 1.0 / G[0][0];
-    } else {
-      const double det = G[0][0] * G[1][1] - G[0][1] * G[1][0];
-      Gi[0][0] = G[1][1] / det; Gi[1][1] = G[0][0] / det;
-      Gi[0][1] = -G[0][1] / det; Gi[1][0] = -G[1][0] / det;
-    }
-    for (int i = 0; i < n; ++i)
-      for (int j = 0; j < n; ++j) {
-        double t = 0.0;
-        for (int a = 0; a < k; ++a)
-          for (int bb = 0; bb < k; ++bb) t += Fr[i][a] * Gi[a][bb] * Fr[j][bb];
-        Hd2[i][j] -= t;
-      }
+      E[kk][dd] = fma(g.cp[kk][3], X[3][dd],
+                      fma(g.cp[kk][2], X[2][dd], fma(g.cp[kk][1], X[1][dd], g.cp[kk][0] * X[0][dd])));
   }
-  // grad d = (|c| v^, 0); hess d = hess d^2/(2d) - (|c|^2 v^ v^T (+) 0)/d
-  for (int a = 0; a < 3; ++a) r.vh[a] = g.v[a] / d;
-  const double gr[5] = {cn * r.vh[0], cn * r.vh[1], cn * r.vh[2], 0.0, 0.0};
-  for (int i = 0; i < 5; ++i)
-    for (int j = 0; j < 5; ++j) {
-      if (i < n && j < n) {
-        const double hdd = Hd2[i][j] / (2.0 * d) -
-                           (i < 3 && j < 3 ? cn * cn * r.vh[i] * r.vh[j] / d : 0.0);
-        r.A[i][j] = kappa * (b2 * gr[i] * gr[j] + b1 * hdd);
-      } else {
-        r.A[i][j] = 0.0;
-      }
+  // F' and (E^T E)^-1 F'^T
+  double F[5][2], T[5][2];
+#pragma unroll
+  for (int kk = 0; kk < 2; ++kk) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) F[a][kk] = kk < k ? fma(chc[kk], g.v[a], cn * E[kk][a]) : 0.0;
+  }
+  F[3][0] = q00 * d; F[3][1] = q01 * d;
+  F[4][0] = 0.0;     F[4][1] = q11 * d;
+  double G00 = 0.0, G01 = 0.0, G11 = 0.0;      // (E^T E)^-1
+  if (k > 0) {
+    const double e00 = dot3(E[0], E[0]);
+    if (k == 1) {
+      G00 = 1.0 / e00;
+    } else {
+      const double e01 = dot3(E[0], E[1]), e11 = dot3(E[1], E[1]);
+      const double id = 1.0 / fma(e00, e11, -(e01 * e01));
+      G00 = e11 * id; G01 = -e01 * id; G11 = e00 * id;
     }
+  }
+#pragma unroll
+  for (int i = 0; i < 5; ++i) {
+    T[i][0] = fma(G00, F[i][0], G01 * F[i][1]);
+    T[i][1] = fma(G01, F[i][0], G11 * F[i][1]);
+  }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) r.vh[a] = g.v[a] * inv_d;
+  const double K1 = r.gfac * inv_d, K2 = kappa * b2 * cn2;
+#pragma unroll
+  for (int i = 0; i < 5; ++i)
+#pragma unroll
+    for (int j = i; j < 5; ++j) {
+      double h = 0.0;
+      if (i < n && j < n) {
+        h = -fma(F[i][0], T[j][0], F[i][1] * T[j][1]);
+        if (j < 3) {
+          const double vv = r.vh[i] * r.vh[j];
+          h = fma(cn2, (i == j ? 1.0 : 0.0) - vv, h);
+          h = fma(K1, h, K2 * vv);
+        } else {
+          h *= K1;
+        }
+      }
+      r.A[i][j] = h;
+      r.A[j][i] = h;
+    }
+}
+
+// Plane rotation (c, s, t = s / c) of a cyclic Jacobi step that annihilates
+// apq.  float32: the textbook formulas.  float64: t to float32 accuracy only
+// (about 1e-7 of apq stays, which the next sweep removes; the diagonal is
+// updated by the full products), c by one third-order step from the float32
+// reciprocal square root, so c^2 + s^2 = 1 to rounding: about 14 float64
+// instructions instead of about 90 for the divisions and square roots.
+__device__ __forceinline__ void jacobi_rotation(float app, float aqq, float apq, float& c, float& s,
+                                                float& t) {
+  const float th = (aqq - app) / (2.f * apq);
+  t = (th >= 0.f ? 1.f : -1.f) / (fabsf(th) + sqrtf(th * th + 1.f));
+  c = 1.f / sqrtf(t * t + 1.f);
+  s = t * c;
+}
+__device__ __forceinline__ void jacobi_rotation(double app, double aqq, double apq, double& c,
+                                                double& s, double& t) {
+  // a difference and an entry outside the float32 range are scaled alike
+  double dif = aqq - app, two = 2.0 * apq;
+  const double big = fmax(fabs(dif), fabs(two));
+  if (!(big < 1e30 && big > 1e-20)) {
+    dif /= big;
+    two /= big;
+  }
+  const float th = (float)dif / (float)two;
+  const float tf = (th >= 0.f ? 1.f : -1.f) / (fabsf(th) + sqrtf(fmaf(th, th, 1.f)));
+  t = (double)tf;
+  const double u = fma(t, t, 1.0);
+  const double r0 = (double)rsqrtf((float)u);
+  const double e = fma(-u * r0, r0, 1.0);
+  c = fma(r0 * e, fma(0.375, e, 0.5), r0);
+  s = t * c;
 }
 
 // ---------------------------------------------------------------------------

@@ -236,9 +236,11 @@ __device__ __forceinline__ void k_barrier_pairs_warp_body(const int* __restrict_
                 int* __restrict__ x2mark) {
   __shared__ ET As[kPairWarps][5][5];
   __shared__ ET Qs[kPairWarps][5][5];
+  __shared__ double Qd[kPairWarps][5][5], Ld[kPairWarps][5];
   __shared__ double Hp[kPairWarps][5][5];
   __shared__ double hv[kPairWarps][4][3];
   __shared__ double sq[kPairWarps][4][4];
+  __shared__ double cs[kPairWarps][4], chs[kPairWarps][4], qs[kPairWarps][2][4], vs[kPairWarps][3];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int64_t np = *count;
   np = np < cap ? np : cap;
@@ -250,14 +252,32 @@ __device__ __forceinline__ void k_barrier_pairs_warp_body(const int* __restrict_
     load_pair(type, i, j, tris, edges, V);
     double X[4][3];
     gather_X(s, V, X);
-    PairReduced r;
-    pair_reduced(type, X, dhat, kappa, r);
-    const int n = r.n;
-    if (lane < 25) {
-      const int a = lane / 5, b = lane % 5;
-      As[w][a][b] = (ET)r.A[a][b];
-      Qs[w][a][b] = a == b ? ET(1) : ET(0);
+    int n, k;
+    double gfac;
+    {   // every lane forms the pair's reduced Hessian; lane 0 stores it for the
+        // lane-parallel parts, which index it by lane
+      PairReduced r;
+      pair_reduced(type, X, dhat, kappa, r);
+      n = r.n; k = r.k; gfac = r.gfac;
+      if (lane == 0) {
+#pragma unroll
+        for (int a = 0; a < 5; ++a)
+#pragma unroll
+          for (int b = a; b < 5; ++b) {
+            const ET v = (ET)r.A[a][b];
+            As[w][a][b] = v;
+            As[w][b][a] = v;
+          }
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+          cs[w][a] = r.c[a]; chs[w][a] = r.ch[a];
+          qs[w][0][a] = r.q[0][a]; qs[w][1][a] = r.q[1][a];
+        }
+#pragma unroll
+        for (int a = 0; a < 3; ++a) vs[w][a] = r.vh[a];
+      }
     }
+    if (lane < 25) Qs[w][lane / 5][lane % 5] = lane / 5 == lane % 5 ? ET(1) : ET(0);
     __syncwarp();
     const ET tiny = sizeof(ET) == 8 ? ET(1e-300) : ET(1e-30);
     const ET tol = sizeof(ET) == 8 ? ET(1e-30) : ET(1e-13);
@@ -273,27 +293,38 @@ __device__ __forceinline__ void k_barrier_pairs_warp_body(const int* __restrict_
           const ET apq = As[w][pp][qq];
           if (!(fabs(apq) > tiny)) continue;
           const ET app = As[w][pp][pp], aqq = As[w][qq][qq];
-          const ET th = (aqq - app) / (ET(2) * apq);
-          const ET t = (th >= ET(0) ? ET(1) : ET(-1)) / (fabs(th) + sqrt(th * th + ET(1)));
-          const ET c = ET(1) / sqrt(t * t + ET(1)), sn = t * c;
+          ET c, sn, t;
+          jacobi_rotation(app, aqq, apq, c, sn, t);
+          // lanes 0..4: rows of A (columns pp, qq), lanes 8..12: rows of Q,
+          // lanes 16..18: the 2 x 2 block itself
           ET x0 = 0, x1 = 0;
           const bool rowl = lane < n && lane != pp && lane != qq;
           const bool qlan = lane >= 8 && lane < 8 + n;
           if (rowl) { x0 = As[w][lane][pp]; x1 = As[w][lane][qq]; }
           if (qlan) { x0 = Qs[w][lane - 8][pp]; x1 = Qs[w][lane - 8][qq]; }
+          const ET np_ = c * x0 - sn * x1, nq = sn * x0 + c * x1;
+          ET blk = 0;
+          if (sizeof(ET) == 8) {
+            const ET cc = c * c, ss = sn * sn, sc = c * sn;
+            const ET k0 = lane == 16 ? cc : lane == 17 ? ss : sc;
+            const ET k1 = lane == 16 ? -2 * sc : lane == 17 ? 2 * sc : cc - ss;
+            const ET k2 = lane == 16 ? ss : lane == 17 ? cc : -sc;
+            blk = k0 * app + k1 * apq + k2 * aqq;
+          } else {
+            blk = lane == 16 ? app - t * apq : lane == 17 ? aqq + t * apq : ET(0);
+          }
           __syncwarp();
           if (rowl) {
-            const ET np_ = c * x0 - sn * x1, nq = sn * x0 + c * x1;
             As[w][lane][pp] = np_; As[w][pp][lane] = np_;
             As[w][lane][qq] = nq; As[w][qq][lane] = nq;
           }
           if (qlan) {
-            Qs[w][lane - 8][pp] = c * x0 - sn * x1;
-            Qs[w][lane - 8][qq] = sn * x0 + c * x1;
+            Qs[w][lane - 8][pp] = np_;
+            Qs[w][lane - 8][qq] = nq;
           }
-          if (lane == 16) As[w][pp][pp] = app - t * apq;
-          if (lane == 17) As[w][qq][qq] = aqq + t * apq;
-          if (lane == 18) { As[w][pp][qq] = ET(0); As[w][qq][pp] = ET(0); }
+          if (lane == 16) As[w][pp][pp] = blk;
+          if (lane == 17) As[w][qq][qq] = blk;
+          if (lane == 18) { As[w][pp][qq] = blk; As[w][qq][pp] = blk; }
           __syncwarp();
         }
     }
@@ -304,35 +335,39 @@ __device__ __forceinline__ void k_barrier_pairs_warp_body(const int* __restrict_
     const ET floor_ = sizeof(ET) == 8 ? ET(0) : ET(1e-6) * lmax;
     if (lane < 25) {
       const int a = lane / 5, b = lane % 5;
+      Qd[w][a][b] = a < n && b < n ? (double)Qs[w][a][b] : 0.0;
+    } else if (lane < 30) {
+      const int l = lane - 25;
+      const ET lam = l < n ? As[w][l][l] : ET(0);
+      Ld[w][l] = lam > floor_ ? (double)lam : 0.0;
+    }
+    __syncwarp();
+    if (lane < 25) {
+      const int a = lane / 5, b = lane % 5;
       double acc = 0.0;
-      if (a < n && b < n)
-        for (int l = 0; l < n; ++l) {
-          const ET lam = As[w][l][l];
-          if (lam > floor_) acc += (double)Qs[w][a][l] * (double)lam * (double)Qs[w][b][l];
-        }
+#pragma unroll
+      for (int l = 0; l < 5; ++l) acc = fma(Qd[w][a][l] * Ld[w][l], Qd[w][b][l], acc);
       Hp[w][a][b] = acc;
     }
     __syncwarp();
-    const int k = r.k;
     if (lane < 12) {                  // hv[i][a] = sum_m q_m[i] Hp[a][3+m]
       const int ii = lane / 3, a = lane % 3;
-      double acc = 0.0;
-      for (int m = 0; m < k; ++m) acc += r.q[m][ii] * Hp[w][a][3 + m];
-      hv[w][ii][a] = acc;
+      hv[w][ii][a] = fma(qs[w][1][ii], Hp[w][a][4], qs[w][0][ii] * Hp[w][a][3]);
     } else if (lane < 28) {           // sq[i][j] = sum q_m[i] q_l[j] Hp[3+m][3+l]
       const int ii = (lane - 12) / 4, jj = (lane - 12) % 4;
-      double acc = 0.0;
-      for (int m = 0; m < k; ++m)
-        for (int l = 0; l < k; ++l) acc += r.q[m][ii] * r.q[l][jj] * Hp[w][3 + m][3 + l];
-      sq[w][ii][jj] = acc;
+      const double t0 = fma(Hp[w][3][4], qs[w][1][jj], Hp[w][3][3] * qs[w][0][jj]);
+      const double t1 = fma(Hp[w][4][4], qs[w][1][jj], Hp[w][4][3] * qs[w][0][jj]);
+      sq[w][ii][jj] = fma(qs[w][1][ii], t1, qs[w][0][ii] * t0);
     }
     __syncwarp();
-    if (lane < 12) pgrad[p * 12 + lane] = r.gfac * r.c[lane / 3] * r.vh[lane % 3];
+    if (lane < 12) pgrad[p * 12 + lane] = gfac * cs[w][lane / 3] * vs[w][lane % 3];
+    // block (i, j) entry (a, b), factored as in the lane-per-pair form
     for (int e = lane; e < 144; e += 32) {
       const int ab = e / 9, rc = e % 9;
       const int ii = ab / 4, jj = ab % 4, a = rc / 3, b = rc % 3;
-      phess[p * 144 + e] = r.ch[ii] * r.ch[jj] * Hp[w][a][b] + r.ch[ii] * hv[w][jj][a] * r.vh[b] +
-                           r.ch[jj] * r.vh[a] * hv[w][ii][b] + sq[w][ii][jj] * r.vh[a] * r.vh[b];
+      const double t1 = fma(hv[w][jj][a], vs[w][b], chs[w][jj] * Hp[w][a][b]);
+      const double t2 = fma(sq[w][ii][jj], vs[w][b], chs[w][jj] * hv[w][ii][b]);
+      phess[p * 144 + e] = fma(chs[w][ii], t1, vs[w][a] * t2);
     }
     if (lane < 4)
       for (int64_t e = Wptr[V[lane]]; e < Wptr[V[lane] + 1]; ++e) {
@@ -402,9 +437,8 @@ __device__ __forceinline__ void barrier_pair_lane(int64_t p, const unsigned long
         const ET apq = A[pp][qq];
         if (!(fabs(apq) > tiny)) continue;
         const ET app = A[pp][pp], aqq = A[qq][qq];
-        const ET th = (aqq - app) / (ET(2) * apq);
-        const ET t = (th >= ET(0) ? ET(1) : ET(-1)) / (fabs(th) + sqrt(th * th + ET(1)));
-        const ET c = ET(1) / sqrt(t * t + ET(1)), sn = t * c;
+        ET c, sn, t;
+        jacobi_rotation(app, aqq, apq, c, sn, t);
 #pragma unroll
         for (int l = 0; l < 5; ++l) {
           if (l == pp || l == qq || l >= n) continue;
@@ -420,9 +454,16 @@ __device__ __forceinline__ void barrier_pair_lane(int64_t p, const unsigned long
           Q[l][pp] = c * x0 - sn * x1;
           Q[l][qq] = sn * x0 + c * x1;
         }
-        A[pp][pp] = app - t * apq;
-        A[qq][qq] = aqq + t * apq;
-        A[pp][qq] = ET(0); A[qq][pp] = ET(0);
+        if (sizeof(ET) == 8) {     // t is not exact: the full products
+          const ET cc = c * c, ss = sn * sn, sc = c * sn;
+          A[pp][pp] = cc * app - 2 * sc * apq + ss * aqq;
+          A[qq][qq] = ss * app + 2 * sc * apq + cc * aqq;
+          A[pp][qq] = A[qq][pp] = sc * (app - aqq) + (cc - ss) * apq;
+        } else {
+          A[pp][pp] = app - t * apq;
+          A[qq][qq] = aqq + t * apq;
+          A[pp][qq] = ET(0); A[qq][pp] = ET(0);
+        }
       }
   }
   // projection: keep eigenvalues above a relative floor (zero in float64;
@@ -432,48 +473,45 @@ __device__ __forceinline__ void barrier_pair_lane(int64_t p, const unsigned long
   for (int a = 0; a < 5; ++a)
     if (a < n) lmax = fmax(lmax, A[a][a]);
   const ET floor_ = sizeof(ET) == 8 ? ET(0) : ET(1e-6) * lmax;
-  double Hp[5][5];
+  double Qd[5][5], Ld[5], Hp[5][5];
 #pragma unroll
-  for (int a = 0; a < 5; ++a)
+  for (int l = 0; l < 5; ++l) {
+    Ld[l] = l < n && A[l][l] > floor_ ? (double)A[l][l] : 0.0;
 #pragma unroll
-    for (int b = 0; b < 5; ++b) {
+    for (int a = 0; a < 5; ++a) Qd[a][l] = a < n && l < n ? (double)Q[a][l] : 0.0;
+  }
+#pragma unroll
+  for (int a = 0; a < 5; ++a) {
+    double ql[5];
+#pragma unroll
+    for (int l = 0; l < 5; ++l) ql[l] = Qd[a][l] * Ld[l];
+#pragma unroll
+    for (int b = a; b < 5; ++b) {
       double acc = 0.0;
-      if (a < n && b < n)
 #pragma unroll
-        for (int l = 0; l < 5; ++l) {
-          if (l >= n) continue;
-          const ET lam = A[l][l];
-          if (lam > floor_) acc += (double)Q[a][l] * (double)lam * (double)Q[b][l];
-        }
+      for (int l = 0; l < 5; ++l) acc = fma(ql[l], Qd[b][l], acc);
       Hp[a][b] = acc;
+      Hp[b][a] = acc;
     }
-  const int k = r.k;
+  }
   double hv[4][3], sq[4][4];        // hv[i][a] = sum_m q_m[i] Hp[a][3+m]
 #pragma unroll
   for (int ii = 0; ii < 4; ++ii) {
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      double acc = 0.0;
+    for (int a = 0; a < 3; ++a) hv[ii][a] = fma(r.q[1][ii], Hp[a][4], r.q[0][ii] * Hp[a][3]);
+    // sq[i][j] = sum q_m[i] q_l[j] Hp[3+m][3+l] (symmetric)
+    const double t0 = fma(r.q[1][ii], Hp[4][3], r.q[0][ii] * Hp[3][3]);
+    const double t1 = fma(r.q[1][ii], Hp[4][4], r.q[0][ii] * Hp[3][4]);
 #pragma unroll
-      for (int m = 0; m < 2; ++m)
-        if (m < k) acc += r.q[m][ii] * Hp[a][3 + m];
-      hv[ii][a] = acc;
-    }
-#pragma unroll
-    for (int jj = 0; jj < 4; ++jj) {  // sq[i][j] = sum q_m[i] q_l[j] Hp[3+m][3+l]
-      double acc = 0.0;
-#pragma unroll
-      for (int m = 0; m < 2; ++m)
-#pragma unroll
-        for (int l = 0; l < 2; ++l)
-          if (m < k && l < k) acc += r.q[m][ii] * r.q[l][jj] * Hp[3 + m][3 + l];
-      sq[ii][jj] = acc;
+    for (int jj = ii; jj < 4; ++jj) {
+      sq[ii][jj] = fma(t1, r.q[1][jj], t0 * r.q[0][jj]);
+      sq[jj][ii] = sq[ii][jj];
     }
   }
 #pragma unroll
   for (int e = 0; e < 12; ++e) pgrad[p * 12 + e] = r.gfac * r.c[e / 3] * r.vh[e % 3];
-  // block (i, j) entry (a, b) of the lift, factored so that a lane's float64
-  // operations fall from about 1,440 to about 540:
+  // block (i, j) entry (a, b) of the lift, factored and fused: about 460
+  // float64 operations per lane
   //   ch_i (ch_j Hp[a][b] + hv[j][a] vh[b]) + vh[a] (ch_j hv[i][b] + sq[i][j] vh[b])
   double T1[4][3][3];
 #pragma unroll
@@ -481,20 +519,20 @@ __device__ __forceinline__ void barrier_pair_lane(int64_t p, const unsigned long
 #pragma unroll
     for (int a = 0; a < 3; ++a)
 #pragma unroll
-      for (int b = 0; b < 3; ++b) T1[jj][a][b] = r.ch[jj] * Hp[a][b] + hv[jj][a] * r.vh[b];
+      for (int b = 0; b < 3; ++b) T1[jj][a][b] = fma(hv[jj][a], r.vh[b], r.ch[jj] * Hp[a][b]);
 #pragma unroll
   for (int ii = 0; ii < 4; ++ii)
 #pragma unroll
     for (int jj = 0; jj < 4; ++jj) {
       double T2[3];
 #pragma unroll
-      for (int b = 0; b < 3; ++b) T2[b] = r.ch[jj] * hv[ii][b] + sq[ii][jj] * r.vh[b];
+      for (int b = 0; b < 3; ++b) T2[b] = fma(sq[ii][jj], r.vh[b], r.ch[jj] * hv[ii][b]);
 #pragma unroll
       for (int a = 0; a < 3; ++a)
 #pragma unroll
         for (int b = 0; b < 3; ++b)
           phess[p * 144 + (ii * 4 + jj) * 9 + a * 3 + b] =
-              r.ch[ii] * T1[jj][a][b] + r.vh[a] * T2[b];
+              fma(r.ch[ii], T1[jj][a][b], r.vh[a] * T2[b]);
     }
 #pragma unroll
   for (int a = 0; a < 4; ++a)
