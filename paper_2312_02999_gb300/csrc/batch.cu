@@ -86,8 +86,8 @@ namespace fsim {
 
 class Batch {
  public:
-  Batch(fsim_ctx_t ctx, MeshState& ms, int cap, cudaStream_t stream)
-      : ctx_(ctx), ms_(ms), cap_(cap), s_(stream) {}
+  Batch(fsim_ctx_t ctx, MeshState& ms, int cap, cudaStream_t stream, int coop_ctas)
+      : ctx_(ctx), ms_(ms), cap_(cap), coop_ctas_(coop_ctas), s_(stream) {}
   ~Batch() { release(); }
 
   int init() {
@@ -197,7 +197,7 @@ class Batch {
     ex.stream = s_;
     ex.h_counters = ctx_->h_counters;
     ex.h_scal = ctx_->h_scal;
-    ex.coop_ctas = ctx_->num_sms;
+    ex.coop_ctas = coop_ctas_;
     ex.alone = false;
     ex.allocs = const_cast<std::vector<void*>*>(&allocs_);
     ex.bytes = nullptr;
@@ -433,7 +433,7 @@ class Batch {
       BTRY(gradient(one));
     }
     BCK(cudaMemsetAsync(m.counters + 6, 0, sizeof(int) * 2, s_));
-    BCK(global_step(s_, m, m.g, m.dx, FSIM_FP64, m.counters + 6, ctx_->num_sms, false, false,
+    BCK(global_step(s_, m, m.g, m.dx, FSIM_FP64, m.counters + 6, coop_ctas_, false, false,
                     frames_[f].nc));
     launch_proxy(s_, m, m.dx, m.ds);
     launch_ccd_reset(s_, m);
@@ -498,6 +498,7 @@ class Batch {
     bs.cols_dev = cols_dev_;
     bs.x1s_dev = x1s_dev_;
     bs.num_sms = ctx_->num_sms;
+    bs.coop_ctas = coop_ctas_;
     bs.use_tc = ms_.p.sigma_product_simt == 0;
     if (any_b) {
       BCK(global_step_b(bs));
@@ -590,7 +591,7 @@ class Batch {
 
   fsim_ctx_t ctx_;
   MeshState& ms_;
-  int cap_ = 1, nr_ = 32;
+  int cap_ = 1, nr_ = 32, coop_ctas_ = 1;
   cudaStream_t s_ = nullptr, s2_ = nullptr;
   cudaEvent_t ev_[4] = {nullptr, nullptr, nullptr, nullptr};
   std::vector<Frame> frames_;
@@ -624,8 +625,9 @@ class Batch {
   size_t bytes_ = 0;
 };
 
-Batch* batch_create(fsim_ctx_t ctx, MeshState& ms, int cap, cudaStream_t stream, int* status) {
-  auto* b = new (std::nothrow) Batch(ctx, ms, cap, stream);
+Batch* batch_create(fsim_ctx_t ctx, MeshState& ms, int cap, cudaStream_t stream, int coop_ctas,
+                    int* status) {
+  auto* b = new (std::nothrow) Batch(ctx, ms, cap, stream, coop_ctas);
   if (!b) { *status = FSIM_ENOMEM; return nullptr; }
   *status = b->init();
   if (*status != FSIM_OK) { delete b; return nullptr; }
@@ -660,7 +662,7 @@ extern "C" fsim_status fsim_solve_batch(fsim_ctx_t ctx, int32_t n_req, const fsi
   if (ms->p.solver != FSIM_SOLVER_WOODBURY) return FSIM_EINVAL;
   if (cudaSetDevice(ctx->device) != cudaSuccess) return FSIM_ECUDA;
   int rc = FSIM_OK;
-  Batch* b = batch_create(ctx, *ms, std::min<int>(max_frames, n_req), ctx->stream, &rc);
+  Batch* b = batch_create(ctx, *ms, std::min<int>(max_frames, n_req), ctx->stream, ctx->num_sms, &rc);
   if (!b) return rc;
   int next = 0, first_err = FSIM_OK;
   const BatchPull pull = [&](BatchReq* out) {

@@ -26,7 +26,10 @@ using BatchDone = std::function<void(void* user, int status, const fsim_frame_st
 // A batch of up to cap frames of mesh ms running on `stream` (NULL on error,
 // with the status in *status: FSIM_EINVAL when the mesh cannot be batched,
 // FSIM_ENOMEM, FSIM_ECUDA).
-Batch* batch_create(fsim_ctx_t ctx, MeshState& ms, int cap, cudaStream_t stream, int* status);
+// coop_ctas: CTAs its cooperative launches may use (all batches that run at
+// once together at most one per SM).
+Batch* batch_create(fsim_ctx_t ctx, MeshState& ms, int cap, cudaStream_t stream, int coop_ctas,
+                    int* status);
 void batch_destroy(Batch* b);
 // Device bytes the batch holds.
 size_t batch_bytes(const Batch* b);

@@ -136,6 +136,8 @@ int ensure_reduced(const Exec& ex, DevMesh& m, int nc) {
   const int64_t n3 = 3 * (int64_t)cap;
   TRY(dalloc(*ex.allocs, &m.Bc, (size_t)(n3 * n3), ex.bytes));
   TRY(dalloc(*ex.allocs, &m.bocc, (size_t)(2 * (int64_t)cap * cap + cap + 32), ex.bytes));
+  // the barrier counters after the lists start at zero (and are left at zero)
+  CK(cudaMemsetAsync(m.bocc + 2 * (int64_t)cap * cap + cap, 0, sizeof(int) * 32, ex.stream));
   m.red_cap = reduced_workspace_elems(cap);
   TRY(dalloc(*ex.allocs, &m.red, (size_t)m.red_cap, ex.bytes));
   TRY(dalloc(*ex.allocs, &m.redf, (size_t)m.red_cap, ex.bytes));
@@ -443,7 +445,10 @@ int solve_frame_impl(const Exec& ex, const MeshState& ms, DevMesh& m, const doub
     } else {
       // one graph per precision and reduced-system path (n_c decides the path)
       const bool schur = p.solver == FSIM_SOLVER_SCHUR;
-      const int gkey = 8 * gprec + (schur ? 4 : reduced_path(nc, gprec, m.one_cta_max));
+      // (5: float64 without contact, whose launches differ from path 0's)
+      const int gkey = 8 * gprec + (schur ? 4 : gprec == FSIM_FP64 && nc == 0
+                                                    ? 5
+                                                    : reduced_path(nc, gprec, m.one_cta_max));
       TRY(with_graph(ex, m, graph_slot(m, 0, 6, m.g, gkey), m.g, gkey, m.red_gen, [&]() -> int {
         CK(cudaMemsetAsync(m.counters + 6, 0, sizeof(int) * 2, s));
         CK(global_step(s, m, m.g, m.dx, gprec, m.counters + 6, ex.coop_ctas, ex.alone, schur, nc));

@@ -128,11 +128,11 @@ int pcg_global_step(cudaStream_t s, const DevMesh& m, const double* g, double* d
   double* q = m.cg_q;
   double* red = m.cg_red;   // 2 doubles on the device
   // the preconditioner M^-1 r = H^-1 r is the global step without contact:
-  // the reduced-system kernels read n_c = 0 from counters[3]
+  // n_c = 0 (counters[3] too)
   auto precond = [&](const double* rin, double* zout) -> int {
     k_neg<<<nb, 256, 0, s>>>(n3, rin, m.cg_tmp);
     count_launch();
-    if (global_step(s, m, m.cg_tmp, zout, 0, info_dev, num_sms, true) != cudaSuccess) return -1;
+    if (global_step(s, m, m.cg_tmp, zout, 0, info_dev, num_sms, true, false, 0) != cudaSuccess) return -1;
     return 0;
   };
   auto dots = [&](const double* a, const double* b, const double* c, const double* d) -> int {

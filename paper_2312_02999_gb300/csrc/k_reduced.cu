@@ -1,23 +1,21 @@
-// Reduced contact system of Sec. 3.2.  The cooperative kernel k_reduced
-// (float64, or n_c above the cluster path) runs the phases below in one
-// launch; the float32 paths for small n_c (k_small_s/x/n/v, the 4-CTA
-// cluster k_clus_v) run the same phases as separate kernels, the first ones
-// on a side stream.
+// Reduced contact system of Sec. 3.2.
 //
 // Eq. 10-11: Sigma-hat^-1 y2 = u - Sigma^-1 Q^T v with u = Sigma^-1 y2 and,
 // in the push-through form (B-check is PSD and usually singular, so it is
 // never inverted), v = (I + B S)^-1 B u_c, S = Sigma^-1[c, c] (x) I_3.  With
 // S = L L^T (L = L_s (x) I_3) this is v = L^-T (I + L^T B L)^-1 L^T B u_c and
 // I + L^T B L is SPD with eigenvalues >= 1, so both factorisations are plain
-// Cholesky.  Phases, separated by grid-wide barriers:
-//   1 gather S = Sigma^-1[c,c], the block-row lists of B, y = B u_c
-//   2 S = L_s L_s^T                         (right-looking, 32-wide panels)
+// Cholesky.  Steps:
+//   1 gather S = Sigma^-1[c,c], the block-row lists of B
+//   2 S = L_s L_s^T
 //   3 X = B (L_s (x) I_3)
-//   4 N = I + (L_s (x) I_3)^T X, and the extra row t0 = (L_s (x) I_3)^T y
-//   5 N = L_N L_N^T; the extra row becomes l = L_N^-1 t0
-//   6 v = (L_s (x) I_3)^-T L_N^-T l           (one CTA)
-//   7 float32 factors only: refinement, rho = y - v - B (S v) in float64,
-//     v += L^-T N^-1 L^T rho.  The error of v reaches the global residual as
+//   4 N = I + (L_s (x) I_3)^T X
+//   5 N = L_N L_N^T
+//   6 y = B u_c, v = (L_s (x) I_3)^-T N^-1 (L_s (x) I_3)^T y
+//   7 refinement, rho = y - v - B (S v) in float64, v += L^-T N^-1 L^T rho:
+//     one step with float64 factors (it takes back what solving with explicit
+//     inverse factors loses against substitution); float32 factors refine to
+//     a stopping test.  The error of v reaches the global residual as
 //     Q^T rho itself, so the stopping test compares |rho| with |y2| (the
 //     Schur right-hand side), not with |y| = |B u_c|, which carries the
 //     barrier stiffness and can be many orders larger.  At most
@@ -26,14 +24,17 @@
 //     factor gains only 4-10x per step, and 4 steps left |rho| near
 //     1e-3 |y2|; the stopping rule ends well-conditioned solves after 1-2.
 //   8 z2 = u - (Sigma^-1[:, c] (x) I_3) v
-// Pivots use a float32 reciprocal square root refined by two float64 Newton
-// steps (float64-accurate, a far shorter dependent chain than sqrt and a
-// division on GB300's float64 pipe).
+// Steps 1-5 need only B-check and Sigma^-1, so they run on a side stream while
+// the forward solve makes u.  Two forms: the grid form (float64, and float32
+// with n_c > 128), and for float32 n_c <= 128 the one-CTA and cluster kernels
+// k_small_s/x/n/v and k_clus_v.
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <type_traits>
+#include <vector>
 
 #include "kernels.h"
 
@@ -79,17 +80,30 @@ struct RedArgs {
   int one_cta_max;      // largest n_c of the one-CTA path (float32 factors); the
                         // 4-CTA cluster takes n_c up to kClusNc above it
   FT* spk;              // one-CTA path: L_s packed, diagonal blocks inverted
+  unsigned* bar;        // grid form: two counters of each of its two kernels
 };
 
 // Offsets of the workspace for a given n_c (every kernel of the reduced solve
-// derives them from the n_c it reads on the device).
+// derives them from the n_c it reads on the device).  red_tail: the float64
+// vectors and the block lists, where both forms have them; red_layout: those
+// and the matrices of the one-CTA and cluster forms.
+template <typename FT>
+__device__ __forceinline__ void red_tail(RedArgs<FT>& a, int nc) {
+  const int n3 = 3 * nc;
+  a.nc = nc;
+  a.y = a.dtail_end - 4 * (size_t)n3 - 8;
+  a.v = a.y + n3; a.rho = a.v + n3; a.w = a.rho + n3; a.nrm = a.w + n3;
+  a.S64 = a.y - (size_t)nc * nc;
+  a.list = a.ibase;
+  a.cnt = a.list + (size_t)nc * nc;
+}
 template <typename FT>
 __device__ __forceinline__ void red_layout(RedArgs<FT>& a, int nc) {
   const int n3 = 3 * nc;
+  red_tail(a, nc);
   // every segment starts on a 16-byte boundary (vector loads)
   constexpr size_t q = 16 / sizeof(FT);
   auto al = [](size_t x) { return (x + q - 1) / q * q; };
-  a.nc = nc;
   a.S = a.base;
   a.X = a.S + al((size_t)nc * nc);
   a.N = a.X + al((size_t)n3 * n3);
@@ -97,190 +111,6 @@ __device__ __forceinline__ void red_layout(RedArgs<FT>& a, int nc) {
   a.dinv_n = a.dinv_s + al(nc);
   a.fv = a.dinv_n + al(n3);
   a.spk = a.fv + al(2 * (size_t)n3);
-  a.y = a.dtail_end - 4 * (size_t)n3 - 8;
-  a.v = a.y + n3; a.rho = a.v + n3; a.w = a.rho + n3; a.nrm = a.w + n3;
-  a.S64 = a.y - (size_t)nc * nc;
-  a.list = a.ibase;
-  a.cnt = a.list + (size_t)nc * nc;
-}
-
-__device__ __forceinline__ double rsqrt_refined(double d) {
-  if (!(d > 1e-30 && d < 1e30)) return 1.0 / sqrt(d);
-  double r = (double)rsqrtf((float)d);
-  r = r * (1.5 - 0.5 * d * r * r);
-  r = r * (1.5 - 0.5 * d * r * r);
-  return r;
-}
-__device__ __forceinline__ float rsqrt_refined(float d) { return rsqrtf(d); }
-
-template <typename FT>
-struct Smem {
-  FT D[32][33];
-  FT Pi[32][33];
-  FT Pj[32][33];
-  FT dv[32];
-};
-
-// CTA-level factorisation of the kb x kb diagonal block at (k0, k0).
-template <typename FT>
-__device__ void factor_diag(FT* A, int k0, int kb, int ld, FT* dinv, int* info, Smem<FT>& sm) {
-  const int tid = threadIdx.x;
-  for (int e = tid; e < kb * kb; e += kRT) {
-    const int i = e / kb, j = e % kb;
-    sm.D[i][j] = (j <= i) ? A[(size_t)(k0 + i) * ld + k0 + j] : FT(0);
-  }
-  __syncthreads();
-  for (int j = 0; j < kb; ++j) {
-    if (tid == 0) {
-      FT d = sm.D[j][j];
-      if (!(d > FT(0))) { atomicOr(info, 1); d = FT(1); }
-      const FT r = rsqrt_refined(d);
-      sm.D[j][j] = d * r;
-      sm.dv[j] = r;
-    }
-    __syncthreads();
-    for (int i = j + 1 + tid; i < kb; i += kRT) sm.D[i][j] *= sm.dv[j];
-    __syncthreads();
-    const int m = kb - j - 1;
-    for (int e = tid; e < m * m; e += kRT) {
-      const int i = j + 1 + e / m, c = j + 1 + e % m;
-      if (c <= i) sm.D[i][c] -= sm.D[i][j] * sm.D[c][j];
-    }
-    __syncthreads();
-  }
-  for (int e = tid; e < kb * kb; e += kRT) {
-    const int i = e / kb, j = e % kb;
-    A[(size_t)(k0 + i) * ld + k0 + j] = (j <= i) ? sm.D[i][j] : FT(0);
-  }
-  for (int j = tid; j < kb; j += kRT) dinv[k0 + j] = sm.dv[j];
-  __syncthreads();
-}
-
-// Right-looking blocked Cholesky of the leading N x N block of an
-// (N + extra) x N row-major matrix (extra rows get A L^-T), by all CTAs.
-template <typename FT>
-__device__ void coop_chol(cg::grid_group& grid, FT* A, int N, int extra, int ld, FT* dinv,
-                          int* info, Smem<FT>& sm) {
-  const int M = N + extra;
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  if (blockIdx.x == 0 && N > 0) factor_diag(A, 0, min(32, N), ld, dinv, info, sm);
-  grid.sync();
-  for (int k0 = 0; k0 < N; k0 += 32) {
-    const int kb = min(32, N - k0);
-    const int k1 = k0 + kb;
-    for (int e = tid; e < kb * kb; e += kRT) {
-      const int i = e / kb, j = e % kb;
-      sm.D[i][j] = A[(size_t)(k0 + i) * ld + k0 + j];
-    }
-    for (int j = tid; j < kb; j += kRT) sm.dv[j] = dinv[k0 + j];
-    __syncthreads();
-    // panel: rows [k1, M) := A L_kk^-T, one warp per row (forward substitution)
-    for (int r = blockIdx.x * (kRT / 32) + wid; r < M - k1; r += gridDim.x * (kRT / 32)) {
-      FT* arow = A + (size_t)(k1 + r) * ld + k0;
-      FT xv = (lane < kb) ? arow[lane] : FT(0);
-      for (int j = 0; j < kb; ++j) {
-        const FT xj = __shfl_sync(0xffffffffu, xv, j) * sm.dv[j];
-        if (lane == j) xv = xj;
-        if (lane > j && lane < kb) xv -= xj * sm.D[lane][j];
-      }
-      if (lane < kb) arow[lane] = xv;
-    }
-    grid.sync();
-    if (k1 < N) {
-      const int nrb = (M - k1 + 31) / 32, ncb = (N - k1 + 31) / 32;
-      int ntiles = 0;
-      for (int rb = 0; rb < nrb; ++rb) ntiles += min(rb + 1, ncb);
-      for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        int rb = 0, rem = tile;
-        while (rem >= min(rb + 1, ncb)) { rem -= min(rb + 1, ncb); ++rb; }
-        const int cb = rem;
-        const int r0 = k1 + rb * 32, c0 = k1 + cb * 32;
-        const int rn = min(32, M - r0), cn = min(32, N - c0);
-        for (int e = tid; e < 32 * kb; e += kRT) {
-          const int i = e / kb, l = e % kb;
-          sm.Pi[i][l] = (i < rn) ? A[(size_t)(r0 + i) * ld + k0 + l] : FT(0);
-          sm.Pj[i][l] = (i < cn) ? A[(size_t)(c0 + i) * ld + k0 + l] : FT(0);
-        }
-        __syncthreads();
-        for (int e = tid; e < 32 * 32; e += kRT) {
-          const int i = e >> 5, j = e & 31;
-          if (i < rn && j < cn && (r0 + i >= c0 + j || r0 + i >= N)) {
-            FT acc = 0;
-            for (int l = 0; l < kb; ++l) acc += sm.Pi[i][l] * sm.Pj[j][l];
-            A[(size_t)(r0 + i) * ld + c0 + j] -= acc;
-          }
-        }
-        __syncthreads();
-        if (tile == 0) factor_diag(A, k1, min(32, N - k1), ld, dinv, info, sm);   // look-ahead
-      }
-    }
-    grid.sync();
-  }
-}
-
-// One CTA: solve L x = b (lower) or L^T x = b in place for n unknowns and
-// nrhs right-hand sides (b[i * nrhs + r]); dinv holds 1 / L[j][j].
-template <typename FT, bool TRANS>
-__device__ void cta_trsv(const FT* L, const FT* dinv, int n, int ld, FT* b, int nrhs, Smem<FT>& sm) {
-  const int tid = threadIdx.x;
-  const int nblk = (n + 31) / 32;
-  for (int bi = 0; bi < nblk; ++bi) {
-    const int blk = TRANS ? nblk - 1 - bi : bi;
-    const int i0 = blk * 32, nb = min(32, n - i0);
-    // stage the diagonal block and 1/diag in shared memory: the sequential
-    // substitution below then never waits on global memory
-    for (int e = tid; e < nb * nb; e += kRT) {
-      const int i = e / nb, j = e % nb;
-      sm.D[i][j] = (j <= i) ? L[(size_t)(i0 + i) * ld + i0 + j] : FT(0);
-    }
-    for (int j = tid; j < nb; j += kRT) sm.dv[j] = dinv[i0 + j];
-    __syncthreads();
-    if (tid < 32) {
-      for (int r = 0; r < nrhs; ++r) {
-        FT xv = (tid < nb) ? b[(size_t)(i0 + tid) * nrhs + r] : FT(0);
-        for (int s = 0; s < nb; ++s) {
-          const int j = TRANS ? nb - 1 - s : s;
-          const FT xj = __shfl_sync(0xffffffffu, xv, j) * sm.dv[j];
-          if (tid == j) xv = xj;
-          if (TRANS) {
-            if (tid < j) xv -= sm.D[j][tid] * xj;
-          } else {
-            if (tid > j && tid < nb) xv -= sm.D[tid][j] * xj;
-          }
-        }
-        if (tid < nb) { b[(size_t)(i0 + tid) * nrhs + r] = xv; sm.Pi[tid][r] = xv; }
-      }
-    }
-    __syncthreads();
-    if (TRANS) {   // rows above: b[i] -= sum_j L[i0+j][i] x[j]
-      for (int e = tid; e < i0 * nrhs; e += kRT) {
-        const int i = e / nrhs, r = e % nrhs;
-        FT acc = 0;
-        for (int j = 0; j < nb; ++j) acc += L[(size_t)(i0 + j) * ld + i] * sm.Pi[j][r];
-        b[(size_t)i * nrhs + r] -= acc;
-      }
-    } else {       // rows below: b[i] -= sum_j L[i][i0+j] x[j]
-      const int below = n - (i0 + nb);
-      for (int e = tid; e < below * nrhs; e += kRT) {
-        const int i = i0 + nb + e / nrhs, r = e % nrhs;
-        FT acc = 0;
-        for (int j = 0; j < nb; ++j) acc += L[(size_t)i * ld + i0 + j] * sm.Pi[j][r];
-        b[(size_t)i * nrhs + r] -= acc;
-      }
-    }
-    __syncthreads();
-  }
-}
-
-// q = (L_s (x) I_3)^T p for vectors laid out q[(i, a)] = q[3 i + a] (one CTA)
-template <typename FT, typename VT>
-__device__ void cta_lt_apply(const FT* L, int nc, const VT* p, FT* q) {
-  for (int e = threadIdx.x; e < 3 * nc; e += kRT) {
-    const int i = e / 3, a = e % 3;
-    double acc = 0.0;
-    for (int j = i; j < nc; ++j) acc += (double)L[(size_t)j * nc + i] * (double)p[3 * j + a];
-    q[e] = (FT)acc;
-  }
 }
 
 // z2 = u - (Sigma^-1[:, c] (x) I_3) v, one warp per row (warp w of nw): the
@@ -345,7 +175,7 @@ __device__ __forceinline__ void k_z2_update_body(RedArgs<float> a, bool rows) {
       a.z2[e] = a.u[e];
     return;
   }
-  if (nc > a.small_lim) return;         // the cooperative kernel owns larger n_c
+  if (nc > a.small_lim) return;         // the grid form updates its own z2
   red_layout(a, nc);
   const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
   if (rows) z2_update_rows(a, nc, w, nw);
@@ -355,164 +185,826 @@ __global__ void __launch_bounds__(256) k_z2_update(RedArgs<float> a) {
   k_z2_update_body(a, false);
 }
 
+// ---------------------------------------------------------------------------
+// Grid form: n_c of any size, float64 or float32 factors, the matrices in
+// global memory (L2) and G CTAs per system.
+//
+// k_grid_prepare does steps 1-5.  The time of a blocked Cholesky this small
+// (32 ceil(n / 32), n = 3 n_c of a few hundred) is its chain of panels, so each
+// panel is two phases with a barrier after each, and its serial part, the
+// 32 x 32 diagonal factor, is made by CTA 0 while the other CTAs update the
+// trailing tiles (look-ahead).  The identity is carried along below the
+// matrix: its rows become U = L^-T, so every later solve is two products with
+// U, which spread over the grid, in place of a chain of 2 n / 32 dependent
+// blocks.  The matrices are padded to whole blocks by the identity.
+// k_grid_solve does steps 6-8 once u is known.
+//
+// Measured (one system, all SMs): float64 n_c = 93: 311 us of preparation, of
+// which the forward solve covers about 200, and 48 us of solve, where one
+// launch after the forward solve took 723 us (a diagonal factor with three
+// barriers per column, one-CTA solves); float32 n_c = 242: 426 + 105 us from
+// 1,676.  A batch's systems run side by side, each on a share of the CTAs,
+// where they ran one after the other (60k face, 8 frames, two of them with
+// n_c > 128: 1,760 -> 375 us per iteration).
+// ---------------------------------------------------------------------------
+constexpr int kBk = 32;                     // block edge
+constexpr int kSpinLimit = 1 << 21;         // polls of a barrier before it gives up (about a second)
+
+// systems of a launch: grid = G n CTAs, CTA b works on system b / G
+struct GridFrames {
+  static constexpr int kMax = 64;
+  int n, G;
+  unsigned char id[kMax];
+};
+
 template <typename FT>
-__global__ void __launch_bounds__(kRT) k_reduced(RedArgs<FT> a) {
-  cg::grid_group grid = cg::this_grid();
-  __shared__ Smem<FT> sm;
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const int gtid = blockIdx.x * kRT + tid, gsz = gridDim.x * kRT;
-  const int gwarp = blockIdx.x * (kRT / 32) + wid, nwarps = gridDim.x * (kRT / 32);
-  // n_c is read on the device, so the launch (and a captured graph) does not
-  // depend on it; every thread reads the same value
-  const int nc = *a.nc_dev, n3 = 3 * nc;
-  if (nc == 0) {          // no contact: Sigma-hat = Sigma, z2 = u
-    for (int e = gtid; e < 3 * a.n2; e += gsz) a.z2[e] = a.u[e];
-    return;
-  }
-  red_layout(a, nc);
-  if (nc > a.small_lim) {   // otherwise phases 1-7 ran in the one-CTA path
-    // 1. S, block lists, y = B u_c
-    if (gtid == 0) a.nrm[2] = 0.0;
-    for (int e = gtid; e < nc * nc; e += gsz) {
-      const int i = e / nc, j = e % nc;
-      a.S[e] = (FT)a.Sinv[(size_t)a.clist[i] * a.n2 + a.clist[j]];
-    }
-    for (int i = gwarp; i < nc; i += nwarps) {
-      int base = 0;
-      for (int j0 = 0; j0 < nc; j0 += 32) {
-        const int j = j0 + lane;
-        const bool f = j < nc && a.bocc[(size_t)i * nc + j] != 0;
-        const unsigned msk = __ballot_sync(0xffffffffu, f);
-        if (f) a.list[(size_t)i * nc + base + __popc(msk & ((1u << lane) - 1u))] = j;
-        base += __popc(msk);
-      }
-      if (lane == 0) a.cnt[i] = base;
-    }
-    grid.sync();
-    for (int row = gtid; row < n3; row += gsz) {
-      const int i = row / 3;
-      const double* brow = a.Bc + (size_t)row * n3;
-      double acc = 0.0;
-      for (int e = 0; e < a.cnt[i]; ++e) {
-        const int j = a.list[(size_t)i * nc + e];
-        const double* uj = a.u + 3 * (size_t)a.clist[j];
-        acc += brow[3 * j] * uj[0] + brow[3 * j + 1] * uj[1] + brow[3 * j + 2] * uj[2];
-      }
-      a.y[row] = acc;
-    }
-    if (a.refine > 0) {
-      double q = 0.0;
-      for (int e = gtid; e < 3 * a.n2; e += gsz) q += (double)a.y2[e] * (double)a.y2[e];
-      for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
-      if (lane == 0 && q != 0.0) atomicAdd(&a.nrm[2], q);
-    }
-    // 2. L_s
-    coop_chol<FT>(grid, a.S, nc, 0, nc, a.dinv_s, a.info, sm);
-    // 3. X[(i,a),(k,b)] = sum_{j in row i, j >= k} B[(i,a),(j,b)] L_s[j][k]
-    for (int64_t e = gtid; e < (int64_t)n3 * n3; e += gsz) {
-      const int row = (int)(e / n3), colx = (int)(e % n3);
-      const int i = row / 3, k = colx / 3, b = colx % 3;
-      const double* brow = a.Bc + (size_t)row * n3;
-      double acc = 0.0;
-      for (int q = 0; q < a.cnt[i]; ++q) {
-        const int j = a.list[(size_t)i * nc + q];
-        if (j >= k) acc += brow[3 * j + b] * (double)a.S[(size_t)j * nc + k];
-      }
-      a.X[e] = (FT)acc;
-    }
-    grid.sync();
-    // 4. N = I + (L_s (x) I)^T X (lower part suffices) and t0
-    for (int64_t e = gtid; e < (int64_t)(n3 + 1) * n3; e += gsz) {
-      const int row = (int)(e / n3), col = (int)(e % n3);
-      double acc;
-      if (row < n3) {
-        if (col > row) continue;
-        const int i = row / 3, ax = row % 3;
-        acc = (row == col) ? 1.0 : 0.0;
-        for (int j = i; j < nc; ++j)
-          acc += (double)a.S[(size_t)j * nc + i] * (double)a.X[(size_t)(3 * j + ax) * n3 + col];
-      } else {
-        const int i = col / 3, ax = col % 3;
-        acc = 0.0;
-        for (int j = i; j < nc; ++j) acc += (double)a.S[(size_t)j * nc + i] * a.y[3 * j + ax];
-      }
-      a.N[e] = (FT)acc;
-    }
-    grid.sync();
-    // 5. L_N (the extra row becomes l = L_N^-1 t0)
-    coop_chol<FT>(grid, a.N, n3, 1, n3, a.dinv_n, a.info, sm);
-    // 6. v = (L_s (x) I)^-T L_N^-T l
-    FT* t = a.fv;
-    if (blockIdx.x == 0) {
-      for (int e = tid; e < n3; e += kRT) t[e] = a.N[(size_t)n3 * n3 + e];
-      __syncthreads();
-      cta_trsv<FT, true>(a.N, a.dinv_n, n3, n3, t, 1, sm);
-      cta_trsv<FT, true>(a.S, a.dinv_s, nc, nc, t, 3, sm);
-      for (int e = tid; e < n3; e += kRT) a.v[e] = (double)t[e];
-    }
-    grid.sync();
-    // 7. refinement with float64 residuals (float32 factors), until
-    //    |rho| <= 1e-7 |y2|, until a step fails to halve |rho|, or after
-    //    a.refine steps
-    double prev = -1.0;
-    for (int it = 0; it < a.refine; ++it) {
-      if (gtid == 0) a.nrm[0] = 0.0;
-      grid.sync();
-      // w = S v with S = Sigma^-1[c, c] (x) I_3 in float64
-      for (int e = gtid; e < n3; e += gsz) {
-        const int i = e / 3, ax = e % 3;
-        const double* srow = a.Sinv + (size_t)a.clist[i] * a.n2;
-        double acc = 0.0;
-        for (int j = 0; j < nc; ++j) acc += srow[a.clist[j]] * a.v[3 * j + ax];
-        a.w[e] = acc;
-      }
-      grid.sync();
-      for (int row = gtid; row < n3; row += gsz) {
-        const int i = row / 3;
-        const double* brow = a.Bc + (size_t)row * n3;
-        double acc = 0.0;
-        for (int e = 0; e < a.cnt[i]; ++e) {
-          const int j = a.list[(size_t)i * nc + e];
-          acc += brow[3 * j] * a.w[3 * j] + brow[3 * j + 1] * a.w[3 * j + 1] +
-                 brow[3 * j + 2] * a.w[3 * j + 2];
+struct GridLay {
+  int nc, n3, nbs, nbn, lds, ldn;
+  FT *S, *Us, *N, *U, *dg, *t, *l;
+};
+template <typename FT>
+__host__ __device__ __forceinline__ GridLay<FT> grid_layout(FT* base, int nc) {
+  GridLay<FT> g;
+  g.nc = nc;
+  g.n3 = 3 * nc;
+  g.nbs = (nc + kBk - 1) / kBk;
+  g.nbn = (g.n3 + kBk - 1) / kBk;
+  g.lds = g.nbs * kBk;
+  g.ldn = g.nbn * kBk;
+  g.S = base;                                   // L_s
+  g.Us = g.S + (size_t)g.lds * g.lds;           // L_s^-T
+  g.N = g.Us + (size_t)g.lds * g.lds;           // L_N
+  g.U = g.N + (size_t)g.ldn * g.ldn;            // X, then L_N^-T
+  g.dg = g.U + (size_t)g.ldn * g.ldn;           // two diagonal factors (by parity) + 1 / diag
+  g.t = g.dg + 2 * (kBk * kBk + kBk);           // vectors of ldn
+  g.l = g.t + g.ldn;
+  return g;
+}
+int64_t grid_front_elems(int nc) {
+  const GridLay<float> g = grid_layout<float>(nullptr, nc);
+  return (int64_t)2 * g.lds * g.lds + 2 * (int64_t)g.ldn * g.ldn + 2 * (kBk * kBk + kBk) +
+         2 * (int64_t)g.ldn + 16;
+}
+
+// Barrier of a system's CTAs: a counter that only grows within the launch
+// (the last CTA to leave resets it).  All CTAs are resident (cooperative
+// launch).  A wait that runs out sets the info flag, and the CTA waits no more.
+struct GroupBar {
+  unsigned* word;       // [0] arrivals, [1] departures
+  unsigned target;
+  int G;
+  int* info;
+  bool dead;
+};
+__device__ __forceinline__ void group_sync(GroupBar& b) {
+  __syncthreads();
+  if (b.G > 1) {
+    if (threadIdx.x == 0) {
+      b.target += b.G;
+      __threadfence();
+      atomicAdd(b.word, 1u);
+      int polls = 0;
+      while (!b.dead) {
+        unsigned v;
+        asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(v) : "l"(b.word) : "memory");
+        if ((int)(v - b.target) >= 0) break;
+        if (++polls > kSpinLimit) {
+          atomicOr(b.info, 4);
+          b.dead = true;
         }
-        const double rr = a.y[row] - a.v[row] - acc;
-        a.rho[row] = rr;
-        atomicAdd(&a.nrm[0], rr * rr);
       }
-      grid.sync();
-      {   // the same values for every thread of the grid: a uniform decision
-        const double r2 = __ldcg(a.nrm), ys = __ldcg(a.nrm + 2);
-        if (!(r2 > 1e-14 * ys)) break;
-        if (prev >= 0.0 && !(r2 < 0.25 * prev)) break;
-        prev = r2;
-      }
-      if (blockIdx.x == 0) {
-        cta_lt_apply<FT, double>(a.S, nc, a.rho, t);
-        __syncthreads();
-        cta_trsv<FT, false>(a.N, a.dinv_n, n3, n3, t, 1, sm);
-        cta_trsv<FT, true>(a.N, a.dinv_n, n3, n3, t, 1, sm);
-        cta_trsv<FT, true>(a.S, a.dinv_s, nc, nc, t, 3, sm);
-        for (int e = tid; e < n3; e += kRT) a.v[e] += (double)t[e];
-      }
-      grid.sync();
+      __threadfence();
     }
+    __syncthreads();
+  }
+}
+__device__ __forceinline__ void group_leave(GroupBar& b) {
+  __syncthreads();
+  if (threadIdx.x == 0 && b.G > 1) {
+    __threadfence();
+    if (atomicAdd(b.word + 1, 1u) == (unsigned)b.G - 1u) {
+      b.word[0] = 0;
+      b.word[1] = 0;
+      __threadfence();
+    }
+  }
+}
+
+// cross-CTA data is read past L1
+template <typename T>
+__device__ __forceinline__ T ldg2(const T* p) { return __ldcg(p); }
+
+// x 2^-e and the significand of x (x = m 2^e, 1 <= m < 2), x positive and normal
+__device__ __forceinline__ int exponent_of(float x) {
+  return ((__float_as_int(x) >> 23) & 255) - 127;
+}
+__device__ __forceinline__ float significand(float x) {
+  return __int_as_float((__float_as_int(x) & 0x007fffff) | 0x3f800000);
+}
+__device__ __forceinline__ float scale_down(float x, int e) {
+  return x * __int_as_float((127 - max(-126, min(126, e))) << 23);
+}
+__device__ __forceinline__ int exponent_of(double x) {
+  return ((__double2hiint(x) >> 20) & 2047) - 1023;
+}
+__device__ __forceinline__ double significand(double x) {
+  return __hiloint2double((__double2hiint(x) & 0x000fffff) | 0x3ff00000, __double2loint(x));
+}
+__device__ __forceinline__ double scale_down(double x, int e) {   // integer work only
+  const int h = __double2hiint(x), ne = ((h >> 20) & 2047) - e;
+  return ne > 0 && ne < 2047 && ((h >> 20) & 2047) != 0
+             ? __hiloint2double(h - (int)((unsigned)e << 20), __double2loint(x))
+             : 0.0;
+}
+__device__ __forceinline__ float rsqrt_ft(float v) {
+  float r = rsqrtf(v);
+  return r * (1.5f - 0.5f * v * r * r);
+}
+__device__ __forceinline__ double rsqrt_ft(double v) { return rsqrt(v); }
+
+template <typename FT>
+struct GridSmem {
+  union {
+    struct {                       // diagonal block (CTA 0)
+      FT P[kBk][kBk + 1];
+      FT col[kBk][kBk + 1];        // col[j][r]: column j before its scaling
+      FT rs[kBk], dv[kBk];
+    } d;
+    struct {                       // panel: the diagonal factor, L[r][q] at [q][r]
+      FT Lt[kBk][kBk];
+      FT dv[kBk];
+    } p;
+    float tile[4][2][kBk][kBk + 4];        // float32 trailing tiles, four at a time
+    struct {                       // float64 trailing sub-tiles; tiles of step 4
+      FT a[16][kBk + 1];
+      FT b[16][kBk + 1];
+    } q;
+    struct {
+      FT X[48][kBk];
+      FT L[16][12];
+    } n;
+    struct {
+      FT b[64][9];
+      int j[64];
+    } x;
+    FT part[8][kBk];
+    double red[kRT / 32];
+  };
+};
+
+// element e of the lower triangle of a 32 x 32 block, columns from the last to
+// the first: the elements of the columns > j are then the first ones, so that
+// the work left after column j fills whole warps
+__device__ __forceinline__ void tri_element(int e, int& r, int& c) {
+  int m = (int)((sqrtf(8.f * e + 1.f) - 1.f) * 0.5f);      // column 31 - m holds m + 1 elements
+  while ((m + 1) * (m + 2) / 2 <= e) ++m;
+  while (m * (m + 1) / 2 > e) --m;
+  c = kBk - 1 - m;
+  r = c + e - m * (m + 1) / 2;
+}
+
+// CTA 0: D = A(k, k) - P P^T (P the block row's panel of the step before; none
+// when kp < 0), its Cholesky factor into A, and the factor transposed with
+// 1 / diag into dg.
+//
+// The elimination is free of divisions: with pivot p = ph 2^e (1 <= ph < 2),
+//   D[r][c] <- D[r][c] ph - D[r][j] (D[c][j] 2^-e),
+// which is the Schur complement times ph, so that after column j every entry
+// carries the product of the ph so far (at most 2^31).  A column then costs two
+// dependent operations and a barrier; the reciprocal (float32: hardware
+// approximation; float64: half a dozen dependent float64 operations of about
+// 66 cycles) is off the chain, and the square roots of all columns are taken
+// at once at the end.  Every thread owns two elements of the triangle (16
+// threads a third one, in column 0, which no step changes).
+template <typename FT>
+__device__ void grid_diag(FT* A, int k, int ld, int kp, FT* dg, int* info, GridSmem<FT>& sm) {
+  const int tid = threadIdx.x;
+  const size_t o = (size_t)kBk * k * ld + kBk * k;
+  __syncthreads();
+  if (kp >= 0)
+    for (int e = tid; e < kBk * kBk; e += kRT)
+      sm.d.P[e >> 5][e & 31] = ldg2(A + (size_t)(kBk * k + (e >> 5)) * ld + kBk * kp + (e & 31));
+  __syncthreads();
+  FT v[3];
+  int er[3], ec[3];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const int e = tid + q * kRT;
+    er[q] = 0;
+    ec[q] = -1;
+    if (e >= kBk * (kBk + 1) / 2) continue;
+    tri_element(e, er[q], ec[q]);
+    FT x = ldg2(A + o + (size_t)er[q] * ld + ec[q]);
+    if (kp >= 0) {
+      FT a0 = 0, a1 = 0;
+#pragma unroll 8
+      for (int l = 0; l < kBk; l += 2) {
+        a0 += sm.d.P[er[q]][l] * sm.d.P[ec[q]][l];
+        a1 += sm.d.P[er[q]][l + 1] * sm.d.P[ec[q]][l + 1];
+      }
+      x -= a0 + a1;
+    }
+    v[q] = x;
+    if (ec[q] == 0) sm.d.col[0][er[q]] = x;
+  }
+  for (int j = 0; j + 1 < kBk; ++j) {
+    __syncthreads();
+    if (ec[0] <= j && ec[1] <= j) continue;          // (elements 0 and 1 exist for every thread)
+    FT p = sm.d.col[j][j];
+    if (!(p > FT(0))) p = FT(1);                     // reported below
+    const int e = exponent_of(p);
+    const FT ph = significand(p);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      if (ec[q] <= j) continue;
+      const FT w = scale_down(sm.d.col[j][ec[q]], e);
+      v[q] = v[q] * ph - sm.d.col[j][er[q]] * w;
+      if (ec[q] == j + 1) sm.d.col[j + 1][er[q]] = v[q];
+    }
+  }
+  __syncthreads();
+  if (tid < kBk) {
+    // pi = product of the significands before column tid; the true pivot is
+    // col[j][j] / pi, so L[r][j] = col[j][r] / sqrt(col[j][j] pi)
+    FT p = sm.d.col[tid][tid];
+    const bool bad = !(p > FT(0));
+    if (bad) { atomicOr(info, 1); p = FT(1); }
+    FT pi = significand(p);
+#pragma unroll
+    for (int s = 1; s < 32; s <<= 1) {
+      const FT x = __shfl_up_sync(0xffffffffu, pi, s);
+      if (tid >= s) pi *= x;
+    }
+    pi = __shfl_up_sync(0xffffffffu, pi, 1);
+    if (tid == 0) pi = FT(1);
+    const FT rs = rsqrt_ft(p * pi);
+    sm.d.rs[tid] = rs;
+    sm.d.dv[tid] = pi * rs;
+    dg[kBk * kBk + tid] = pi * rs;
+    if (bad) sm.d.col[tid][tid] = FT(1);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    if (ec[q] < 0) continue;
+    const FT x = sm.d.col[ec[q]][er[q]] * sm.d.rs[ec[q]];
+    A[o + (size_t)er[q] * ld + ec[q]] = x;
+    dg[ec[q] * kBk + er[q]] = x;
+  }
+}
+
+// Panel k: every row below the diagonal block and every identity row so far,
+// x L_kk^T = a.  A row is one thread with its 32 values in registers (float32),
+// or one warp (float64: 32 x 2 dependent warp instructions per row where a
+// thread per row would need 528 per warp), four rows per CTA at a time so that
+// each SM sub-partition has one.
+__device__ void grid_panel(float* A, float* U, int k, int nb, int ld, const float* dg, int rank, int G,
+                           GridSmem<float>& sm) {
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  if (rank >= nb) return;
+  for (int e = tid; e < kBk * kBk / 4; e += kRT)
+    reinterpret_cast<float4*>(&sm.p.Lt[0][0])[e] = ldg2(reinterpret_cast<const float4*>(dg) + e);
+  if (tid < kBk) sm.p.dv[tid] = ldg2(dg + kBk * kBk + tid);
+  __syncthreads();
+  for (int b = rank + wid * G; b < nb; b += (kRT / 32) * G) {
+    float* row = (b > k ? A : U) + (size_t)(kBk * b + lane) * ld + kBk * k;
+    float x[kBk];
+    if (b == k) {
+#pragma unroll
+      for (int l = 0; l < kBk; ++l) x[l] = l == lane ? 1.f : 0.f;
+    } else {
+#pragma unroll
+      for (int l = 0; l < kBk / 4; ++l) {
+        const float4 f = ldg2(reinterpret_cast<const float4*>(row) + l);
+        x[4 * l] = f.x; x[4 * l + 1] = f.y; x[4 * l + 2] = f.z; x[4 * l + 3] = f.w;
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < kBk; ++q) {
+      x[q] *= sm.p.dv[q];
+#pragma unroll
+      for (int l = q + 1; l < kBk; ++l) x[l] -= x[q] * sm.p.Lt[q][l];
+    }
+#pragma unroll
+    for (int l = 0; l < kBk / 4; ++l)
+      reinterpret_cast<float4*>(row)[l] = make_float4(x[4 * l], x[4 * l + 1], x[4 * l + 2], x[4 * l + 3]);
+  }
+}
+__device__ void grid_panel(double* A, double* U, int k, int nb, int ld, const double* dg, int rank,
+                           int G, GridSmem<double>& sm) {
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  if (rank >= nb * (kBk / 4)) return;
+  for (int e = tid; e < kBk * kBk; e += kRT) (&sm.p.Lt[0][0])[e] = ldg2(dg + e);
+  if (tid < kBk) sm.p.dv[tid] = ldg2(dg + kBk * kBk + tid);
+  __syncthreads();
+  for (int g = rank + (wid >> 2) * G; g < nb * (kBk / 4); g += 2 * G) {
+    const int r = 4 * g + (wid & 3), b = r >> 5;
+    double* row = (b > k ? A : U) + (size_t)r * ld + kBk * k;
+    double x = b == k ? ((r & 31) == lane ? 1.0 : 0.0) : ldg2(row + lane);
+#pragma unroll 4
+    for (int q = 0; q < kBk; ++q) {
+      const double xq = __shfl_sync(0xffffffffu, x, q) * sm.p.dv[q];
+      if (lane == q) x = xq;
+      if (lane > q) x -= xq * sm.p.Lt[q][lane];
+    }
+    row[lane] = x;
+  }
+}
+
+// Trailing update of step k, without the diagonal block of step k + 1 (CTA 0's):
+// A(i, j) -= P_i P_j^T for k < j <= i, and the identity rows
+// U(i, j) -= P_i P_j^T for i <= k < j (U(k, j) starts at zero).
+__device__ void grid_trail(float* A, float* U, int k, int nb, int ld, int slot, int nslots,
+                           GridSmem<float>& sm) {
+  // four 32 x 32 tiles per CTA, 64 threads each, 4 x 4 values per thread: rows
+  // ti + 8 p, columns tj + 8 q, so that the float4 reads of a quarter warp fall
+  // in different banks
+  const int m = nb - k - 1, tri = m * (m + 1) / 2, total = tri + (k + 1) * m;
+  const int qd = threadIdx.x >> 6, tq = threadIdx.x & 63, ti = tq >> 3, tj = tq & 7;
+  float(*Pi)[kBk + 4] = sm.tile[qd][0];
+  float(*Pj)[kBk + 4] = sm.tile[qd][1];
+  for (int t = slot + qd * nslots; t < total; t += 4 * nslots) {
+    if (t == 0) continue;                  // the diagonal block
+    int i, j;
+    if (t < tri) {
+      int I = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
+      while ((I + 1) * (I + 2) / 2 <= t) ++I;
+      while (I * (I + 1) / 2 > t) --I;
+      i = k + 1 + I;
+      j = k + 1 + t - I * (I + 1) / 2;
+    } else {
+      i = (t - tri) / m;
+      j = k + 1 + (t - tri) % m;
+    }
+    const float* src_i = (i > k ? A : U) + (size_t)kBk * i * ld + kBk * k;
+    const float* src_j = A + (size_t)kBk * j * ld + kBk * k;
+    float* dst = (i > k ? A : U) + (size_t)kBk * i * ld + kBk * j;
+    const bool first = i == k;
+    float4 a[4], b[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int e = tq + 64 * u;
+      a[u] = ldg2(reinterpret_cast<const float4*>(src_i + (size_t)(e >> 3) * ld) + (e & 7));
+      b[u] = ldg2(reinterpret_cast<const float4*>(src_j + (size_t)(e >> 3) * ld) + (e & 7));
+    }
+    float acc[4][4];
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        acc[p][q] = first ? 0.f : ldg2(dst + (size_t)(ti + 8 * p) * ld + tj + 8 * q);
+    asm volatile("bar.sync %0, 64;" ::"r"(qd + 1) : "memory");   // the tile before is read
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int e = tq + 64 * u;
+      *reinterpret_cast<float4*>(&Pi[e >> 3][4 * (e & 7)]) = a[u];
+      *reinterpret_cast<float4*>(&Pj[e >> 3][4 * (e & 7)]) = b[u];
+    }
+    asm volatile("bar.sync %0, 64;" ::"r"(qd + 1) : "memory");
+#pragma unroll 2
+    for (int l = 0; l < kBk; l += 4) {
+      float4 x[4], y[4];
+#pragma unroll
+      for (int p = 0; p < 4; ++p) x[p] = *reinterpret_cast<const float4*>(&Pi[ti + 8 * p][l]);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) y[q] = *reinterpret_cast<const float4*>(&Pj[tj + 8 * q][l]);
+#pragma unroll
+      for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          acc[p][q] -= x[p].x * y[q].x + x[p].y * y[q].y + x[p].z * y[q].z + x[p].w * y[q].w;
+    }
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) dst[(size_t)(ti + 8 * p) * ld + tj + 8 * q] = acc[p][q];
+  }
+}
+__device__ void grid_trail(double* A, double* U, int k, int nb, int ld, int slot, int nslots,
+                           GridSmem<double>& sm) {
+  // 16 x 16 sub-tiles, one value per thread: a 32 x 32 tile would hold an SM's
+  // float64 pipes for 8 us
+  const int m = nb - k - 1, m2 = 2 * m, tri = m2 * (m2 + 1) / 2, total = tri + 2 * (k + 1) * m2;
+  const int r = threadIdx.x >> 4, c = threadIdx.x & 15;
+  // sub-tiles 0..2 are the diagonal block
+  for (int t = 3 + slot; t < total; t += nslots) {
+    int i, j;                              // sub-tile rows and columns, in units of 16
+    bool low;
+    if (t < tri) {
+      int I = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
+      while ((I + 1) * (I + 2) / 2 <= t) ++I;
+      while (I * (I + 1) / 2 > t) --I;
+      i = 2 * (k + 1) + I;
+      j = 2 * (k + 1) + t - I * (I + 1) / 2;
+      low = true;
+    } else {
+      i = (t - tri) / m2;
+      j = 2 * (k + 1) + (t - tri) % m2;
+      low = false;
+    }
+    const double* src_i = (low ? A : U) + (size_t)16 * i * ld + kBk * k;
+    const double* src_j = A + (size_t)16 * j * ld + kBk * k;
+    double* dst = (low ? A : U) + (size_t)(16 * i + r) * ld + 16 * j + c;
+    const double a0 = ldg2(src_i + (size_t)r * ld + c), a1 = ldg2(src_i + (size_t)r * ld + c + 16);
+    const double b0 = ldg2(src_j + (size_t)r * ld + c), b1 = ldg2(src_j + (size_t)r * ld + c + 16);
+    double acc = !low && (i >> 1) == k ? 0.0 : ldg2(dst);
+    __syncthreads();
+    sm.q.a[r][c] = a0; sm.q.a[r][c + 16] = a1;
+    sm.q.b[r][c] = b0; sm.q.b[r][c + 16] = b1;
+    __syncthreads();
+#pragma unroll 8
+    for (int l = 0; l < kBk; ++l) acc -= sm.q.a[r][l] * sm.q.b[c][l];
+    *dst = acc;
+  }
+}
+
+// A = L L^T (nb x nb blocks, lower; L in place) and U = L^-T (upper)
+template <typename FT>
+__device__ void grid_chol(FT* A, FT* U, int nb, int ld, FT* dg, GroupBar& bar, int rank,
+                          GridSmem<FT>& sm) {
+  constexpr int kDg = kBk * kBk + kBk;
+  if (rank == 0) grid_diag<FT>(A, 0, ld, -1, dg, bar.info, sm);
+  group_sync(bar);
+  for (int k = 0; k < nb; ++k) {
+    grid_panel(A, U, k, nb, ld, dg + (k & 1) * kDg, rank, bar.G, sm);
+    group_sync(bar);
+    if (k + 1 < nb) {
+      if (rank == 0) {
+        grid_diag<FT>(A, k + 1, ld, k, dg + ((k + 1) & 1) * kDg, bar.info, sm);
+        __syncthreads();
+      }
+      if (bar.G == 1) grid_trail(A, U, k, nb, ld, 0, 1, sm);
+      else if (rank > 0) grid_trail(A, U, k, nb, ld, rank - 1, bar.G - 1, sm);
+      group_sync(bar);
+    }
+  }
+}
+
+// CTAs of the launch that a system of this size uses: with more, the barriers
+// cost more than the extra CTAs give (float32: four tiles at a time per CTA)
+template <typename FT>
+__device__ __forceinline__ int grid_ctas(int nbn, int G) {
+  const int want = std::is_same<FT, double>::value ? 2 * nbn * nbn : 8 + nbn * nbn / 8;
+  return want < G ? want : G;
+}
+
+template <typename FT>
+__device__ void grid_prepare(RedArgs<FT> a, int rank, int G, GridSmem<FT>& sm) {
+  const int nc = *a.nc_dev;
+  if (nc == 0 || nc <= a.small_lim) return;
+  const GridLay<FT> g = grid_layout(a.base, nc);
+  red_tail(a, nc);
+  G = grid_ctas<FT>(g.nbn, G);
+  if (rank >= G) return;
+  GroupBar bar{a.bar, 0u, G, a.info, false};
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, n3 = g.n3;
+  const int gwarp = rank * (kRT / 32) + wid, nwarps = G * (kRT / 32);
+  // 1. S (lower, padded by the identity) and the block-row lists
+  for (int i = gwarp; i < g.lds; i += nwarps) {
+    const double* srow = i < nc ? a.Sinv + (size_t)a.clist[i] * a.n2 : nullptr;
+    for (int j = lane; j <= i; j += 32)
+      g.S[(size_t)i * g.lds + j] = i < nc ? (FT)srow[a.clist[j]] : (i == j ? FT(1) : FT(0));
+    if (i >= nc) continue;
+    int base = 0;
+    for (int j0 = 0; j0 < nc; j0 += 32) {
+      const int j = j0 + lane;
+      const bool f = j < nc && a.bocc[(size_t)i * nc + j] != 0;
+      const unsigned msk = __ballot_sync(0xffffffffu, f);
+      if (f) a.list[(size_t)i * nc + base + __popc(msk & ((1u << lane) - 1u))] = j;
+      base += __popc(msk);
+    }
+    if (lane == 0) a.cnt[i] = base;
+  }
+  group_sync(bar);
+  // 2. L_s, U_s
+  grid_chol<FT>(g.S, g.Us, g.nbs, g.lds, g.dg, bar, rank, sm);
+  // 3. X[(i,a),(k,b)] = sum_{j in row i, j >= k} B[(i,a),(j,b)] L_s[j][k]: a CTA
+  // takes block row i and 256 columns k, the row's blocks of B staged (64 at a
+  // time) in the factor's type; a thread keeps the nine values of one k
+  for (int it = rank; it < nc * ((nc + kRT - 1) / kRT); it += G) {
+    const int i = it % nc, k = (it / nc) * kRT + tid, ci = ldg2(a.cnt + i);
+    FT acc[3][3];
+#pragma unroll
+    for (int p = 0; p < 3; ++p)
+#pragma unroll
+      for (int q = 0; q < 3; ++q) acc[p][q] = FT(0);
+    for (int e0 = 0; e0 < ci; e0 += 64) {
+      const int en = min(64, ci - e0);
+      __syncthreads();
+      for (int e = tid; e < 9 * en; e += kRT) {
+        const int u = e / 9, pq = e % 9, j = ldg2(a.list + (size_t)i * nc + e0 + u);
+        sm.x.b[u][pq] = (FT)a.Bc[(size_t)(3 * i + pq / 3) * n3 + 3 * j + pq % 3];
+        if (pq == 0) sm.x.j[u] = j;
+      }
+      __syncthreads();
+      if (k < nc) {
+#pragma unroll 4
+        for (int u = 0; u < en; ++u) {
+          const int j = sm.x.j[u];
+          if (j < k) continue;
+          const FT L = ldg2(g.S + (size_t)j * g.lds + k);
+#pragma unroll
+          for (int p = 0; p < 3; ++p)
+#pragma unroll
+            for (int q = 0; q < 3; ++q) acc[p][q] += sm.x.b[u][3 * p + q] * L;
+        }
+      }
+    }
+    if (k < nc)
+#pragma unroll
+      for (int p = 0; p < 3; ++p)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) g.U[(size_t)(3 * i + p) * g.ldn + 3 * k + q] = acc[p][q];
+  }
+  group_sync(bar);
+  // 4. N = I + (L_s (x) I)^T X, lower triangle, by tiles of 32 x 32 (float32) or
+  // 16 x 16 (float64): N[(i, ax)][col] sums L_s[j][i] X[(j, ax)][col] over
+  // j >= i, 16 values of j staged at a time.  float32: each stage's sum joins
+  // a two-term total (two-sum), so the long sums round like one addition
+  {
+    constexpr bool f32 = std::is_same<FT, float>::value;
+    constexpr int TS = f32 ? 32 : 16, kV = TS * TS / kRT;
+    const int nt = g.ldn / TS;
+    const int c = tid % TS, r0 = tid / TS;
+    for (int t = rank; t < nt * (nt + 1) / 2; t += G) {
+      int ti = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
+      while ((ti + 1) * (ti + 2) / 2 <= t) ++ti;
+      while (ti * (ti + 1) / 2 > t) --ti;
+      const int tj = t - ti * (ti + 1) / 2, R0 = TS * ti, C0 = TS * tj, i0 = R0 / 3;
+      FT hi[kV], lo[kV];
+#pragma unroll
+      for (int q = 0; q < kV; ++q) {
+        hi[q] = R0 + r0 + q * (kRT / TS) == C0 + c ? FT(1) : FT(0);
+        lo[q] = FT(0);
+      }
+      for (int j0 = i0; j0 < nc; j0 += 16) {
+        __syncthreads();
+        for (int e = tid; e < 48 * TS; e += kRT) {
+          const int xr = 3 * j0 + e / TS, xc = C0 + e % TS;
+          sm.n.X[e / TS][e % TS] = xr < n3 && xc < n3 ? ldg2(g.U + (size_t)xr * g.ldn + xc) : FT(0);
+        }
+        for (int e = tid; e < 16 * 12; e += kRT) {
+          const int j = j0 + e / 12, i = i0 + e % 12;
+          sm.n.L[e / 12][e % 12] = j < nc && i < nc && j >= i ? ldg2(g.S + (size_t)j * g.lds + i) : FT(0);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < kV; ++q) {
+          const int row = R0 + r0 + q * (kRT / TS), iv = row / 3 - i0, ax = row % 3;
+          FT s = f32 ? FT(0) : hi[q];
+#pragma unroll
+          for (int jj = 0; jj < 16; ++jj) s += sm.n.L[jj][iv] * sm.n.X[3 * jj + ax][c];
+          if (f32) {
+            const FT h = hi[q] + s, bb = h - hi[q];
+            lo[q] += (hi[q] - (h - bb)) + (s - bb);
+            hi[q] = h;
+          } else {
+            hi[q] = s;
+          }
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < kV; ++q)
+        g.N[(size_t)(R0 + r0 + q * (kRT / TS)) * g.ldn + C0 + c] = hi[q] + lo[q];
+    }
+  }
+  group_sync(bar);
+  // 5. L_N, U_N (over X)
+  grid_chol<FT>(g.N, g.U, g.nbn, g.ldn, g.dg, bar, rank, sm);
+  group_leave(bar);
+}
+
+// out = (L_s (x) I_3)^T p (padded with zeros), one warp per entry
+template <typename FT>
+__device__ __forceinline__ void grid_lt(const GridLay<FT>& g, const double* p, FT* out, int gwarp,
+                                        int nwarps) {
+  const int lane = threadIdx.x & 31;
+  for (int e = gwarp; e < g.ldn; e += nwarps) {
+    const int i = e / 3, ax = e % 3;
+    double acc = 0.0;
+    if (e < g.n3)
+      for (int j = i + lane; j < g.nc; j += 32)
+        acc += (double)g.S[(size_t)j * g.lds + i] * ldg2(p + 3 * j + ax);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) out[e] = (FT)acc;
+  }
+}
+// out = U^T x: a CTA per block column, its 8 warps share the rows (lane = column)
+template <typename FT>
+__device__ __forceinline__ void grid_ut(const GridLay<FT>& g, const FT* x, FT* out, int rank, int G,
+                                        GridSmem<FT>& sm) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int b = rank; b < g.nbn; b += G) {
+    const int j = kBk * b + lane;
+    FT acc = 0;
+#pragma unroll 8
+    for (int i = wid; i < kBk * (b + 1); i += kRT / 32)
+      acc += (i <= j ? g.U[(size_t)i * g.ldn + j] : FT(0)) * ldg2(x + i);
+    __syncthreads();
+    sm.part[wid][lane] = acc;
+    __syncthreads();
+    if (wid == 0) {
+      FT s = 0;
+#pragma unroll
+      for (int w = 0; w < kRT / 32; ++w) s += sm.part[w][lane];
+      out[j] = s;
+    }
+  }
+}
+// out = U x, one warp per row
+template <typename FT>
+__device__ __forceinline__ void grid_u(const GridLay<FT>& g, const FT* x, FT* out, int gwarp,
+                                       int nwarps) {
+  const int lane = threadIdx.x & 31;
+  for (int i = gwarp; i < g.ldn; i += nwarps) {
+    FT acc = 0;
+#pragma unroll 4
+    for (int j = (i & ~31) + lane; j < g.ldn; j += 32)
+      acc += (j >= i ? g.U[(size_t)i * g.ldn + j] : FT(0)) * ldg2(x + j);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) out[i] = acc;
+  }
+}
+
+template <typename FT>
+__device__ void grid_solve(RedArgs<FT> a, int rank, int Gall, GridSmem<FT>& sm) {
+  const int nc = *a.nc_dev;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  if (nc == 0 || nc <= a.small_lim) return;
+  const GridLay<FT> g = grid_layout(a.base, nc);
+  red_tail(a, nc);
+  const int G = Gall, n3 = g.n3;     // the z2 update has a row per x2 vertex: all CTAs
+  GroupBar bar{a.bar + 2, 0u, G, a.info, false};
+  const int gtid = rank * kRT + tid, gsz = G * kRT;
+  const int gwarp = rank * (kRT / 32) + wid, nwarps = G * (kRT / 32);
+  // 6. y = B u_c (a warp per block row: its lanes share the row's blocks), |y2|^2
+  if (gtid == 0) { a.nrm[0] = 0.0; a.nrm[1] = 0.0; a.nrm[2] = 0.0; }
+  for (int i = gwarp; i < nc; i += nwarps) {
+    const double* b0 = a.Bc + (size_t)(3 * i) * n3;
+    const int ci = a.cnt[i];
+    double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+    for (int e = lane; e < ci; e += 32) {
+      const int j = a.list[(size_t)i * nc + e];
+      const double* uj = a.u + 3 * (size_t)a.clist[j];
+      const double u0 = uj[0], u1 = uj[1], u2 = uj[2];
+      const double* bp = b0 + 3 * j;
+      s0 += bp[0] * u0 + bp[1] * u1 + bp[2] * u2;
+      s1 += bp[n3] * u0 + bp[n3 + 1] * u1 + bp[n3 + 2] * u2;
+      s2 += bp[2 * n3] * u0 + bp[2 * n3 + 1] * u1 + bp[2 * n3 + 2] * u2;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+      s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+      s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+    }
+    if (lane == 0) { a.y[3 * i] = s0; a.y[3 * i + 1] = s1; a.y[3 * i + 2] = s2; }
+  }
+  group_sync(bar);
+  if (!std::is_same<FT, double>::value) {
+    double q = 0.0;
+    for (int e = gtid; e < 3 * a.n2; e += gsz) q += (double)a.y2[e] * (double)a.y2[e];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+    if (lane == 0 && q != 0.0) atomicAdd(&a.nrm[2], q);
+  }
+  // v (+)= (U_s (x) I) U U^T (L_s (x) I)^T p
+  auto apply = [&](const double* p, bool add) {
+    grid_lt(g, p, g.t, gwarp, nwarps);
+    group_sync(bar);
+    grid_ut(g, g.t, g.l, rank, G, sm);
+    group_sync(bar);
+    grid_u(g, g.l, g.t, gwarp, nwarps);
+    group_sync(bar);
+    for (int i = gwarp; i < nc; i += nwarps) {
+      FT s0 = 0, s1 = 0, s2 = 0;
+#pragma unroll 4
+      for (int j = i + lane; j < nc; j += 32) {
+        const FT u = g.Us[(size_t)i * g.lds + j];
+        s0 += u * ldg2(g.t + 3 * j);
+        s1 += u * ldg2(g.t + 3 * j + 1);
+        s2 += u * ldg2(g.t + 3 * j + 2);
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+      }
+      if (lane < 3) {
+        const double d = (double)(lane == 0 ? s0 : lane == 1 ? s1 : s2);
+        a.v[3 * i + lane] = (add ? ldg2(a.v + 3 * i + lane) : 0.0) + d;
+      }
+    }
+    group_sync(bar);
+  };
+  apply(a.y, false);
+  // 7. refinement with float64 residuals: a.refine steps with float64 factors;
+  //    with float32 factors until |rho| <= 1e-7 |y2|, until a step fails to
+  //    halve |rho|, or after a.refine steps.  |rho|^2 alternates between two
+  //    accumulators
+  constexpr bool f64 = std::is_same<FT, double>::value;
+  double prev = -1.0;
+  for (int it = 0; it < a.refine; ++it) {
+    // w = S v with S = Sigma^-1[c, c] (x) I_3 in float64, a warp per row
+    for (int i = gwarp; i < nc; i += nwarps) {
+      const double* srow = a.Sinv + (size_t)a.clist[i] * a.n2;
+      double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+      for (int j = lane; j < nc; j += 32) {
+        const double sv = srow[a.clist[j]];
+        s0 += sv * ldg2(a.v + 3 * j);
+        s1 += sv * ldg2(a.v + 3 * j + 1);
+        s2 += sv * ldg2(a.v + 3 * j + 2);
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+      }
+      if (lane < 3) a.w[3 * i + lane] = lane == 0 ? s0 : lane == 1 ? s1 : s2;
+    }
+    group_sync(bar);
+    if (gtid == 0) a.nrm[(it + 1) & 1] = 0.0;
+    double r2 = 0.0;
+    for (int i = gwarp; i < nc; i += nwarps) {
+      const double* b0 = a.Bc + (size_t)(3 * i) * n3;
+      const int ci = a.cnt[i];
+      double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+      for (int e = lane; e < ci; e += 32) {
+        const int j = a.list[(size_t)i * nc + e];
+        const double w0 = ldg2(a.w + 3 * j), w1 = ldg2(a.w + 3 * j + 1), w2 = ldg2(a.w + 3 * j + 2);
+        const double* bp = b0 + 3 * j;
+        s0 += bp[0] * w0 + bp[1] * w1 + bp[2] * w2;
+        s1 += bp[n3] * w0 + bp[n3 + 1] * w1 + bp[n3 + 2] * w2;
+        s2 += bp[2 * n3] * w0 + bp[2 * n3 + 1] * w1 + bp[2 * n3 + 2] * w2;
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+      }
+      if (lane < 3) {
+        const int row = 3 * i + lane;
+        const double rr = ldg2(a.y + row) - ldg2(a.v + row) - (lane == 0 ? s0 : lane == 1 ? s1 : s2);
+        a.rho[row] = rr;
+        r2 += rr * rr;
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) r2 += __shfl_xor_sync(0xffffffffu, r2, o);
+    if (!f64) {
+      __syncthreads();
+      if (lane == 0) sm.red[wid] = r2;
+      __syncthreads();
+      if (tid == 0) {
+        double s = 0.0;
+        for (int w = 0; w < kRT / 32; ++w) s += sm.red[w];
+        if (s != 0.0) atomicAdd(&a.nrm[it & 1], s);
+      }
+    }
+    group_sync(bar);
+    if (!f64) {
+      // the same values for every thread of the system: a uniform decision
+      const double tot = ldg2(a.nrm + (it & 1)), ys = ldg2(a.nrm + 2);
+      if (!(tot > 1e-14 * ys)) break;
+      if (prev >= 0.0 && !(tot < 0.25 * prev)) break;
+      prev = tot;
+    }
+    apply(a.rho, true);
   }
   // 8. z2 = u - (Sigma^-1[:, c] (x) I_3) v
   z2_update(a, nc, gwarp, nwarps);
+  group_leave(bar);
+}
+
+// A: per-system arguments on the device (batches), else `one`
+template <typename FT>
+__global__ void __launch_bounds__(kRT) k_grid_prepare(RedArgs<FT> one, const RedArgs<FT>* A,
+                                                      GridFrames fr) {
+  __shared__ __align__(16) GridSmem<FT> sm;
+  grid_prepare<FT>(A ? A[fr.id[blockIdx.x / fr.G]] : one, blockIdx.x % fr.G, fr.G, sm);
+}
+template <typename FT>
+__global__ void __launch_bounds__(kRT) k_grid_solve(RedArgs<FT> one, const RedArgs<FT>* A,
+                                                    GridFrames fr) {
+  __shared__ __align__(16) GridSmem<FT> sm;
+  grid_solve<FT>(A ? A[fr.id[blockIdx.x / fr.G]] : one, blockIdx.x % fr.G, fr.G, sm);
 }
 
 // ---------------------------------------------------------------------------
 // One-CTA path for small n_c (float32 factors): the two factorisations and
 // all triangular solves run inside one CTA with the matrix in shared memory,
 // so no grid-wide barrier is needed; only the data-parallel products run
-// over the grid.  Launch sequence (all read n_c on the device and return
-// when 0 < n_c <= kSmallNc does not hold):
+// over the grid.  Launch sequence (all read n_c on the device):
 //   k_small_s   (1 CTA)  S = Sigma^-1[c,c], L_s, block lists of B
 //   k_small_x   (grid)   y = B u_c (float64), |y2|^2, X = B (L_s (x) I_3)
 //   k_small_n   (grid)   N = I + (L_s (x) I_3)^T X  (lower part)
 //   k_small_v   (1 CTA)  L_N, v = L^-T N^-1 L^T y and its float64 refinement
-// then the cooperative kernel runs only its z2 update.
+//   k_z2_update (grid)   z2
 // ---------------------------------------------------------------------------
 constexpr int kSmallNc = 96;               // 3 n_c <= 288 fits in one CTA's shared memory
 constexpr int kSmallN3 = 3 * kSmallNc;
@@ -1530,6 +2022,7 @@ RedArgs<FT> make_args(const DevMesh& m, const double* u, const FT* y2, double* z
   a.info = info;
   a.small_lim = std::is_same<FT, float>::value ? kClusNc : 0;
   a.one_cta_max = std::max(0, std::min(m.one_cta_max, kSmallNc));
+  a.bar = reinterpret_cast<unsigned*>(m.bocc + 2 * (size_t)m.nc_cap * m.nc_cap + m.nc_cap);
   return a;
 }
 
@@ -1552,86 +2045,78 @@ cudaError_t launch_clus_v(cudaStream_t s, const RedArgs<float>& a) {
   return e;
 }
 
+// The two kernels of the grid form for one frame: cooperative launches, since
+// their CTAs wait on one another (all of them are resident together).
 template <typename FT>
-cudaError_t launch_reduced_t(cudaStream_t s, const DevMesh& m, const double* u, const FT* y2,
-                             double* z2, int* info, int num_sms, int refine, int nc_host,
-                             bool prepared) {
-  RedArgs<FT> a = make_args<FT>(m, u, y2, z2, info, refine);
-  if constexpr (std::is_same<FT, float>::value) {
-    // one-CTA path for 0 < n_c <= kSmallNc, 4-CTA cluster for n_c <= kClusNc
-    // (every kernel reads n_c on the device and exits when it is not its
-    // range).  With n_c known on the host (nc_host >= 0) only the kernels of
-    // its path are launched and the z2 update runs as a plain launch, so
-    // n_c <= kClusNc needs no cooperative launch (whose grid must find all of
-    // its SMs free at once when other solves share the GPU).
-    ProfScope ps(PROF_CHOL, s);
-    const int zgrid = std::max(1, std::min(2 * std::max(1, num_sms), (m.n2 + 7) / 8));
-    if (nc_host == 0) {
-      k_z2_update<<<zgrid, 256, 0, s>>>(a);
-      count_launch();
-      return cudaGetLastError();
-    }
-    const bool known = nc_host > 0 && nc_host <= kClusNc;
-    const bool want_small = !known || nc_host <= a.one_cta_max;
-    const bool want_clus = !known || nc_host > a.one_cta_max;
-    if (prepared) {       // S, L_s, lists, X and N came from reduced_prepare
-      if (cudaStreamWaitEvent(s, m.ev_join, 0) != cudaSuccess) return cudaGetLastError();
-      k_small_x<1><<<2 * std::max(1, num_sms), 256, 0, s>>>(a);
-      count_launch();
-    } else {
-      k_small_s<<<1, kST, kSmallSmemS, s>>>(a);
-      k_small_x<3><<<2 * std::max(1, num_sms), 256, 0, s>>>(a);
-      k_small_n<<<kNTiles, 256, 0, s>>>(a);
-      count_launch(3);
-    }
-    if (want_small) {
+cudaError_t launch_grid(cudaStream_t s, RedArgs<FT> a, int ctas, bool prepare) {
+  GridFrames fr{};
+  fr.n = 1;
+  fr.G = std::max(1, ctas);
+  const RedArgs<FT>* none = nullptr;
+  void* args[] = {&a, &none, &fr};
+  ProfScope ps(PROF_CHOL, s);
+  const void* k = prepare ? (const void*)k_grid_prepare<FT> : (const void*)k_grid_solve<FT>;
+  const cudaError_t e = cudaLaunchCooperativeKernel(k, dim3(fr.G), dim3(kRT), args, 0, s);
+  count_launch();
+  return e;
+}
+
+// float32 factors, n_c <= kClusNc: the one-CTA path up to one_cta_max, the
+// 4-CTA cluster above it.  The z2 update is a plain launch, so no cooperative
+// launch is needed (whose grid must find all of its SMs free at once when
+// other solves share the GPU).
+cudaError_t launch_small(cudaStream_t s, const DevMesh& m, const RedArgs<float>& a, int num_sms,
+                         int nc) {
+  ProfScope ps(PROF_CHOL, s);
+  const int zgrid = std::max(1, std::min(2 * std::max(1, num_sms), (m.n2 + 7) / 8));
+  if (nc > 0) {
+    k_small_x<1><<<2 * std::max(1, num_sms), 256, 0, s>>>(a);
+    count_launch();
+    if (nc <= a.one_cta_max) {
       k_small_v<<<1, kST, kSmallSmemV, s>>>(a);
       count_launch();
-    }
-    if (want_clus) {
+    } else {
       const cudaError_t e = launch_clus_v(s, a);
       if (e != cudaSuccess) return e;
     }
-    if (known) {
-      k_z2_update<<<zgrid, 256, 0, s>>>(a);
-      count_launch();
-      return cudaGetLastError();
-    }
   }
-  void* args[] = {&a};
-  const int grid = std::max(1, num_sms);
-  ProfScope ps(PROF_CHOL, s);
-  const cudaError_t e = cudaLaunchCooperativeKernel((void*)k_reduced<FT>, dim3(grid), dim3(kRT), args, 0, s);
+  k_z2_update<<<zgrid, 256, 0, s>>>(a);
   count_launch();
-  return e;
+  return cudaGetLastError();
 }
 
 }  // namespace
 
 int64_t reduced_workspace_elems(int nc) {
   const int64_t n3 = 3 * (int64_t)nc;
-  // S, X, N (+1 row), 1/diag of both factors, two FT vectors, packed L_s, and
-  // (at the tail of the float64 buffer) four float64 vectors
-  return (int64_t)nc * nc + n3 * n3 + (n3 + 1) * n3 + nc + n3 + 2 * n3 +
-         (prow(nc) + 1024 * ((int64_t)nc + 31) / 32 + 16) + 4 * n3 + (int64_t)nc * nc + 128;
+  // one-CTA / cluster forms: S, X, N (+1 row), 1/diag of both factors, two FT
+  // vectors, packed L_s
+  const int64_t small = (int64_t)nc * nc + n3 * n3 + (n3 + 1) * n3 + nc + n3 + 2 * n3 +
+                        (prow(nc) + 1024 * ((int64_t)nc + 31) / 32 + 16) + 64;
+  // at the tail of the float64 buffer four float64 vectors, three norms and S64
+  return std::max(small, grid_front_elems(nc)) + 4 * n3 + (int64_t)nc * nc + 64;
 }
 
 // Most float64 refinement steps of a float32 reduced factor (see step 7).
 constexpr int kMixedRefineSteps = 12;
 
 int reduced_path(int nc_host, int precision, int one_cta_max) {
-  if (precision == 0 || nc_host < 0 || nc_host > kClusNc) return 0;   // cooperative kernel
+  if (precision == 0 || nc_host > kClusNc) return 0;   // grid form
   if (nc_host == 0) return 1;
   return nc_host <= std::min(one_cta_max, kSmallNc) ? 2 : 3;
 }
 
 cudaError_t reduced_solve(cudaStream_t s, const DevMesh& m, const double* u, const void* y2,
-                          double* z2, int* info, int num_sms, int precision, int nc_host,
-                          bool prepared) {
+                          double* z2, int* info, int num_sms, int precision, int nc_host) {
+  if (nc_host <= 0)       // z2 = u
+    return launch_small(s, m, make_args<float>(m, u, nullptr, z2, info, 0), num_sms, 0);
+  // S .. L_N come from the side stream (reduced_prepare)
+  if (cudaStreamWaitEvent(s, m.ev_join, 0) != cudaSuccess) return cudaGetLastError();
   if (precision == 0)
-    return launch_reduced_t<double>(s, m, u, (const double*)y2, z2, info, num_sms, 0, nc_host, false);
-  return launch_reduced_t<float>(s, m, u, (const float*)y2, z2, info, num_sms, kMixedRefineSteps,
-                                 nc_host, prepared);
+    return launch_grid(s, make_args<double>(m, u, (const double*)y2, z2, info, 1), num_sms, false);
+  const RedArgs<float> a = make_args<float>(m, u, (const float*)y2, z2, info, kMixedRefineSteps);
+  if (nc_host > kClusNc) return launch_grid(s, a, num_sms, false);
+  return launch_small(s, m, a, num_sms, nc_host);
 }
 
 namespace {
@@ -1649,28 +2134,29 @@ __global__ void __launch_bounds__(32 * kPhiSplit) k_phi_apply(RedArgs<float> a, 
   __shared__ int cs[kClusNc];
   __shared__ float part[kPhiSplit][3][32];
   const int nc = *a.nc_dev;
-  const bool have = nc > 0 && nc <= a.small_lim;
-  if (have) {
-    red_layout(a, nc);
-    for (int k = threadIdx.x; k < nc; k += blockDim.x) {
-      const bool okc = FSIM_CHECK_IDX(a.clist[k], a.n2, CHECK_CLIST);
-      cs[k] = okc ? a.clist[k] : 0;
-      vs[3 * k] = okc ? (float)a.v[3 * k] : 0.f;
-      vs[3 * k + 1] = okc ? (float)a.v[3 * k + 1] : 0.f;
-      vs[3 * k + 2] = okc ? (float)a.v[3 * k + 2] : 0.f;
-    }
-  }
-  __syncthreads();
+  if (nc > 0) red_tail(a, nc);
   const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
   const int p = blockIdx.x * 32 + lane;
   float c0 = 0.f, c1 = 0.f, c2 = 0.f;
-  if (have && p < n1) {
+  for (int k0 = 0; k0 < nc; k0 += kClusNc) {       // n_c in chunks of the staging size
+    const int kn = min(kClusNc, nc - k0);
+    __syncthreads();
+    for (int k = threadIdx.x; k < kn; k += blockDim.x) {
+      const bool okc = FSIM_CHECK_IDX(a.clist[k0 + k], a.n2, CHECK_CLIST);
+      cs[k] = okc ? a.clist[k0 + k] : 0;
+      vs[3 * k] = okc ? (float)a.v[3 * (k0 + k)] : 0.f;
+      vs[3 * k + 1] = okc ? (float)a.v[3 * (k0 + k) + 1] : 0.f;
+      vs[3 * k + 2] = okc ? (float)a.v[3 * (k0 + k) + 2] : 0.f;
+    }
+    __syncthreads();
+    if (p < n1) {
 #pragma unroll 4
-    for (int k = wq; k < nc; k += kPhiSplit) {
-      const float f = phi_t[(size_t)cs[k] * n1 + p];
-      c0 += f * vs[3 * k];
-      c1 += f * vs[3 * k + 1];
-      c2 += f * vs[3 * k + 2];
+      for (int k = wq; k < kn; k += kPhiSplit) {
+        const float f = phi_t[(size_t)cs[k] * n1 + p];
+        c0 += f * vs[3 * k];
+        c1 += f * vs[3 * k + 1];
+        c2 += f * vs[3 * k + 2];
+      }
     }
   }
   part[wq][0][lane] = c0;
@@ -1730,7 +2216,7 @@ __global__ void __launch_bounds__(32 * kPhiSplit) k_phi_apply_b(const RedArgs<fl
   const int nc = *a.nc_dev;
   const int col = cols[blockIdx.y];
   double* x1 = x1s[blockIdx.y];
-  if (nc > 0) red_layout(a, nc);
+  if (nc > 0) red_tail(a, nc);
   const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
   const int p = blockIdx.x * 32 + lane;
   float c0 = 0.f, c1 = 0.f, c2 = 0.f;
@@ -1778,18 +2264,48 @@ void reduced_args_fill(void* dst, const DevMesh& m, int active) {
   std::memcpy(dst, &a, sizeof(a));
 }
 
-cudaError_t reduced_prepare_b(cudaStream_t s2, const void* args_dev, int nb, int num_sms) {
+namespace {
+// Frames of a batch whose n_c takes the grid form, as few launches as fit:
+// every frame gets an equal share of the ctas (at least kGridMinCtas).
+constexpr int kGridMinCtas = 8;
+cudaError_t launch_grid_b(cudaStream_t s, const RedArgs<float>* A, const RedArgs<float>* H, int nb,
+                          const int* nc_host, int ctas, bool prepare) {
+  std::vector<int> todo;
+  for (int f = 0; f < nb; ++f)
+    if (H[f].active && nc_host[f] > kClusNc) todo.push_back(f);
+  const int per = std::max(1, std::min<int>(GridFrames::kMax, ctas / kGridMinCtas));
+  for (size_t i = 0; i < todo.size(); i += per) {
+    GridFrames fr{};
+    fr.n = (int)std::min<size_t>(per, todo.size() - i);
+    fr.G = std::max(1, ctas / fr.n);
+    for (int q = 0; q < fr.n; ++q) fr.id[q] = (unsigned char)todo[i + q];
+    RedArgs<float> unused{};
+    void* args[] = {&unused, &A, &fr};
+    const void* k = prepare ? (const void*)k_grid_prepare<float> : (const void*)k_grid_solve<float>;
+    const cudaError_t e =
+        cudaLaunchCooperativeKernel(k, dim3(fr.G * fr.n), dim3(kRT), args, 0, s);
+    count_launch();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+}  // namespace
+
+cudaError_t reduced_prepare_b(cudaStream_t s2, const void* args_dev, const void* args_host, int nb,
+                              const int* nc_host, int coop_ctas) {
   const auto* A = static_cast<const RedArgs<float>*>(args_dev);
   ProfScope ps(PROF_CHOL, s2);
   k_small_s_b<<<dim3(1, nb), kST, kSmallSmemS, s2>>>(A);
   k_small_x_b<2><<<dim3((3 * kClusNc + kXRows - 1) / kXRows, nb), 256, 0, s2>>>(A);
   k_small_n_b<<<dim3(kNTiles, nb), 256, 0, s2>>>(A);
   count_launch(3);
-  return cudaGetLastError();
+  const cudaError_t e =
+      launch_grid_b(s2, A, static_cast<const RedArgs<float>*>(args_host), nb, nc_host, coop_ctas, true);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t reduced_solve_b(cudaStream_t s, const void* args_dev, const void* args_host, int nb,
-                            const int* nc_host, int num_sms) {
+                            const int* nc_host, int num_sms, int coop_ctas) {
   const auto* A = static_cast<const RedArgs<float>*>(args_dev);
   const auto* H = static_cast<const RedArgs<float>*>(args_host);
   bool any_small = false, any_clus = false;
@@ -1822,17 +2338,9 @@ cudaError_t reduced_solve_b(cudaStream_t s, const void* args_dev, const void* ar
     count_launch();
     if (e != cudaSuccess) return e;
   }
-  // n_c beyond the cluster path: the cooperative kernel, one frame at a time
-  for (int f = 0; f < nb; ++f) {
-    if (!H[f].active || nc_host[f] <= kClusNc) continue;
-    RedArgs<float> a = H[f];
-    void* args[] = {&a};
-    const cudaError_t e = cudaLaunchCooperativeKernel((void*)k_reduced<float>,
-                                                      dim3(std::max(1, num_sms)), dim3(kRT), args,
-                                                      0, s);
-    count_launch();
-    if (e != cudaSuccess) return e;
-  }
+  // n_c beyond the cluster path: the grid form, all such frames side by side
+  const cudaError_t eg = launch_grid_b(s, A, H, nb, nc_host, coop_ctas, false);
+  if (eg != cudaSuccess) return eg;
   // float64 row products, one row per lane: 256 rows per CTA of 8 warps,
   // enough CTAs to cover the rows of every frame (at least 2 per frame, also
   // for the n_c = 0 copy)
@@ -1859,25 +2367,31 @@ cudaError_t phi_apply(cudaStream_t s, const DevMesh& m, const double* u, const v
   return cudaGetLastError();
 }
 
-bool reduced_prepare(cudaStream_t s, const DevMesh& m, const double* u, const void* y2, double* z2,
-                     int* info, int num_sms, int nc_host) {
-  if (nc_host <= 0 || nc_host > kClusNc || !m.aux_stream || !m.ev_fork || !m.ev_join) return false;
-  const RedArgs<float> a = make_args<float>(m, u, (const float*)y2, z2, info, kMixedRefineSteps);
+cudaError_t reduced_prepare(cudaStream_t s, const DevMesh& m, const double* u, const void* y2,
+                            double* z2, int* info, int num_sms, int precision, int nc_host) {
+  if (nc_host <= 0) return cudaSuccess;
   cudaStream_t s2 = m.aux_stream;
-  if (cudaEventRecord(m.ev_fork, s) != cudaSuccess || cudaStreamWaitEvent(s2, m.ev_fork, 0) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  {
-    ProfScope ps(PROF_CHOL, s2);
-    k_small_s<<<1, kST, kSmallSmemS, s2>>>(a);
-    k_small_x<2><<<2 * std::max(1, num_sms), 256, 0, s2>>>(a);
-    k_small_n<<<kNTiles, 256, 0, s2>>>(a);
-    count_launch(3);
+  if (cudaEventRecord(m.ev_fork, s) != cudaSuccess || cudaStreamWaitEvent(s2, m.ev_fork, 0) != cudaSuccess)
+    return cudaGetLastError();
+  cudaError_t e = cudaSuccess;
+  if (precision == 0) {
+    e = launch_grid(s2, make_args<double>(m, u, (const double*)y2, z2, info, 1), num_sms, true);
+  } else {
+    const RedArgs<float> a = make_args<float>(m, u, (const float*)y2, z2, info, kMixedRefineSteps);
+    if (nc_host > kClusNc) {
+      e = launch_grid(s2, a, num_sms, true);
+    } else {
+      ProfScope ps(PROF_CHOL, s2);
+      k_small_s<<<1, kST, kSmallSmemS, s2>>>(a);
+      k_small_x<2><<<2 * std::max(1, num_sms), 256, 0, s2>>>(a);
+      k_small_n<<<kNTiles, 256, 0, s2>>>(a);
+      count_launch(3);
+      e = cudaGetLastError();
+    }
   }
   // the join is recorded even if a launch failed, so the fork always closes
-  cudaEventRecord(m.ev_join, s2);
-  return true;
+  const cudaError_t ej = cudaEventRecord(m.ev_join, s2);
+  return e != cudaSuccess ? e : ej;
 }
 
 }  // namespace fsim

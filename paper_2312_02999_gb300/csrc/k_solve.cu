@@ -600,11 +600,13 @@ cudaError_t global_step_t(cudaStream_t s, const DevMesh& m, const double* g, dou
   const T* Z = f64 ? (const T*)m.Z : (const T*)m.Zf;
   k_gather_rhs<T><<<nblk(nf, 256), 256, 0, s>>>(nf, m.perm, g, b);
   count_launch();
-  // the reduced system's factorisation needs only B-check and Sigma^-1: in
-  // mixed precision it starts on the side stream and overlaps the forward solve
-  const bool prepared = !f64 && !dense_schur && n2 > 0 &&
-                        reduced_prepare(s, m, m.u, b + 3 * (size_t)n1, r + 3 * (size_t)n1, info,
-                                        num_sms, nc_host);
+  // the reduced system's factorisation needs only B-check and Sigma^-1: it
+  // starts on the side stream and overlaps the forward solve
+  if (!dense_schur && n2 > 0) {
+    const cudaError_t e = reduced_prepare(s, m, m.u, b + 3 * (size_t)n1, r + 3 * (size_t)n1, info,
+                                          num_sms, f64 ? 0 : 1, nc_host);
+    if (e != cudaSuccess) return e;
+  }
   if (n1 > 0) trisolve_fwd<T>(s, m, Z, b, y, wide);
   if (n2 > 0) {
     T* y2 = b + 3 * (size_t)n1;
@@ -613,7 +615,7 @@ cudaError_t global_step_t(cudaStream_t s, const DevMesh& m, const double* g, dou
     // With Phi available the x1 block is split: x1 = L1^-T (y1 - L21^T u)
     // (contact-free, on the side stream while the reduced system is solved)
     // + Phi[:, c] v after it, instead of a backward pass after z2.
-    const bool phi = prepared && m.Phi_t && m.bx && n1 > 0;
+    const bool phi = !f64 && !dense_schur && nc_host > 0 && m.Phi_t && m.bx && n1 > 0;
     if (phi) {
       {
         ProfScope psg(PROF_GEMV, s);
@@ -630,7 +632,7 @@ cudaError_t global_step_t(cudaStream_t s, const DevMesh& m, const double* g, dou
       if (cudaEventRecord(m.ev_join2, s2) != cudaSuccess) return cudaGetLastError();
       {
         ProfScope psr(PROF_REDUCED, s);
-        const cudaError_t e = reduced_solve(s, m, u, y2, z2, info, num_sms, 1, nc_host, true);
+        const cudaError_t e = reduced_solve(s, m, u, y2, z2, info, num_sms, 1, nc_host);
         if (e != cudaSuccess) return e;
       }
       if (cudaStreamWaitEvent(s, m.ev_join2, 0) != cudaSuccess) return cudaGetLastError();
@@ -662,8 +664,7 @@ cudaError_t global_step_t(cudaStream_t s, const DevMesh& m, const double* g, dou
       // float64 factors, or float32 factors refined with float64 residuals.
       // n_c is read on the device (z2 = u when it is 0).
       ProfScope psr(PROF_REDUCED, s);
-      const cudaError_t e = reduced_solve(s, m, u, y2, z2, info, num_sms, f64 ? 0 : 1, nc_host,
-                                          prepared);
+      const cudaError_t e = reduced_solve(s, m, u, y2, z2, info, num_sms, f64 ? 0 : 1, nc_host);
       if (e != cudaSuccess) return e;
     }
     if (!f64) {
@@ -695,7 +696,7 @@ cudaError_t global_step_b(const BatchStep& bs) {
   // on the side stream, overlapping the forward solve
   if (cudaEventRecord(bs.ev[0], s) != cudaSuccess || cudaStreamWaitEvent(s2, bs.ev[0], 0) != cudaSuccess)
     return cudaGetLastError();
-  cudaError_t e = reduced_prepare_b(s2, bs.args_dev, nb, bs.num_sms);
+  cudaError_t e = reduced_prepare_b(s2, bs.args_dev, bs.args_host, nb, bs.nc_host, bs.coop_ctas);
   if (e != cudaSuccess) return e;
   if (cudaEventRecord(bs.ev[1], s2) != cudaSuccess) return cudaGetLastError();
   for (int l = 0; l < m.n_levels && n1 > 0; ++l) {
@@ -747,7 +748,7 @@ cudaError_t global_step_b(const BatchStep& bs) {
   if (cudaStreamWaitEvent(s, bs.ev[1], 0) != cudaSuccess) return cudaGetLastError();
   {
     ProfScope ps(PROF_REDUCED, s);
-    e = reduced_solve_b(s, bs.args_dev, bs.args_host, nb, bs.nc_host, bs.num_sms);
+    e = reduced_solve_b(s, bs.args_dev, bs.args_host, nb, bs.nc_host, bs.num_sms, bs.coop_ctas);
     if (e != cudaSuccess) return e;
   }
   if (cudaStreamWaitEvent(s, bs.ev[3], 0) != cudaSuccess) return cudaGetLastError();

@@ -207,11 +207,9 @@ void launch_ccd_reset(cudaStream_t s, const DevMesh& m);
 // per workspace and can be captured in a CUDA graph).  num_sms is the CTA
 // count of the cooperative reduced-system launch; alone = no other solve
 // shares the GPU (selects wider triangular-solve work items).
-// nc_host: n_c as read back by the host (selects the reduced-system path
-// and skips the launches of the others), or -1 when the host does not know it.
+// nc_host: n_c as read back by the host (selects the reduced-system path).
 cudaError_t global_step(cudaStream_t s, const DevMesh& m, const double* g, double* dx, int precision,
-                        int* info_dev, int num_sms, bool alone, bool dense_schur = false,
-                        int nc_host = -1);
+                        int* info_dev, int num_sms, bool alone, bool dense_schur, int nc_host);
 // Reduced-system path a global step takes for this n_c and precision (graph key).
 int reduced_path(int nc_host, int precision, int one_cta_max);
 // Schur-only variant of the x2 block (k_schur.cu): z2 = Sigma-hat^-1 y2 with
@@ -230,15 +228,14 @@ int pcg_global_step(cudaStream_t s, const DevMesh& m, const double* g, double* d
 // precision 0: float64 factors, 1: float32 factors + float64 refinement.
 // y2 (double for precision 0, float for 1) is the Schur right-hand side with
 // u = Sigma^-1 y2; it scales the refinement's stopping test.
+// Needs reduced_prepare before it.
 cudaError_t reduced_solve(cudaStream_t s, const DevMesh& m, const double* u, const void* y2,
-                          double* z2, int* info, int num_sms, int precision, int nc_host = -1,
-                          bool prepared = false);
-// Mixed precision, 0 < nc_host <= 128: forks the workspace's side stream off
-// s and launches there the kernels that need only B-check and Sigma^-1 (S,
-// L_s, block lists, X, N); reduced_solve(..., prepared = true) joins it.
-// Returns false (nothing launched) when that split does not apply.
-bool reduced_prepare(cudaStream_t s, const DevMesh& m, const double* u, const void* y2, double* z2,
-                     int* info, int num_sms, int nc_host);
+                          double* z2, int* info, int num_sms, int precision, int nc_host);
+// n_c > 0: forks the workspace's side stream off s and launches there the part
+// that needs only B-check and Sigma^-1 (S, L_s, block lists, X, N; in the grid
+// form L_N too); reduced_solve joins it.
+cudaError_t reduced_prepare(cudaStream_t s, const DevMesh& m, const double* u, const void* y2,
+                            double* z2, int* info, int num_sms, int precision, int nc_host);
 // x1 = bx1 + Phi[:, c] v (float64 out, solver order, 3 per position) after a
 // prepared reduced solve (k_reduced.cu); reads n_c on the device.
 cudaError_t phi_apply(cudaStream_t s, const DevMesh& m, const double* u, const void* y2, double* z2,
@@ -301,6 +298,7 @@ struct BatchStep {
   const int* cols_dev = nullptr;            // 3 col per frame (device)
   double* const* x1s_dev = nullptr;         // r of each frame (device array of pointers)
   int num_sms = 1;
+  int coop_ctas = 1;                        // CTAs of a cooperative launch of this batch
   bool use_tc = true;                       // Sigma^-1 product on the tensor cores
 };
 cudaError_t global_step_b(const BatchStep& bs);
@@ -319,9 +317,10 @@ cudaError_t launch_sinv_tc(cudaStream_t s, const DevMesh& m, const float* Y, int
                            int num_sms, int* err);
 size_t reduced_args_bytes();
 void reduced_args_fill(void* dst, const DevMesh& m, int active);
-cudaError_t reduced_prepare_b(cudaStream_t s2, const void* args_dev, int nb, int num_sms);
+cudaError_t reduced_prepare_b(cudaStream_t s2, const void* args_dev, const void* args_host, int nb,
+                              const int* nc_host, int coop_ctas);
 cudaError_t reduced_solve_b(cudaStream_t s, const void* args_dev, const void* args_host, int nb,
-                            const int* nc_host, int num_sms);
+                            const int* nc_host, int num_sms, int coop_ctas);
 cudaError_t phi_apply_b(cudaStream_t s, const void* args_dev, const int* cols_dev, int nb, int n1,
                         const float* phi_t, const float* bxm, int nr, double* const* x1s_dev);
 

@@ -329,7 +329,7 @@ void batch_worker_main(fsim_server_s* sv, int wi) {
       if (rc == FSIM_OK) {
         sv->used += (size_t)cap * per;          // reserved while the batch is built
         lk.unlock();
-        b = batch_create(sv->ctx, ms, cap, w.stream, &rc);
+        b = batch_create(sv->ctx, ms, cap, w.stream, sv->coop_ctas, &rc);
         lk.lock();
         sv->used -= std::min(sv->used, (size_t)cap * per);
         if (b) {
