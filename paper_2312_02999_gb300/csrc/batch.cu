@@ -95,6 +95,7 @@ class Batch {
     nr_ = ((3 * cap_ + 31) / 32) * 32;
     if (!batch_supported(m0, nr_)) return FSIM_EINVAL;
     BCK(cudaStreamCreateWithFlags(&s2_, cudaStreamNonBlocking));
+    BCK(cudaStreamCreateWithFlags(&s3_, cudaStreamNonBlocking));
     for (auto& e : ev_) BCK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     frames_.assign(cap_, Frame{});
     tab_.assign(cap_, DevMesh{});
@@ -207,6 +208,7 @@ class Batch {
   void release() {
     if (s_) cudaStreamSynchronize(s_);
     if (s2_) cudaStreamSynchronize(s2_);
+    if (s3_) cudaStreamSynchronize(s3_);
     if (ev_done_) cudaEventDestroy(ev_done_);
     for (auto& e : ev_tab_)
       if (e) cudaEventDestroy(e);
@@ -215,6 +217,7 @@ class Batch {
     for (auto& e : ev_)
       if (e) cudaEventDestroy(e);
     if (s2_) cudaStreamDestroy(s2_);
+    if (s3_) cudaStreamDestroy(s3_);
     if (h_tab_) cudaFreeHost(h_tab_);
     if (h_counters_) cudaFreeHost(h_counters_);
     if (h_scal_) cudaFreeHost(h_scal_);
@@ -227,8 +230,9 @@ class Batch {
       if (m.ev_fork2) cudaEventDestroy(m.ev_fork2);
       if (m.ev_join2) cudaEventDestroy(m.ev_join2);
       if (m.aux_stream) cudaStreamDestroy(m.aux_stream);
+      if (m.aux_stream2) cudaStreamDestroy(m.aux_stream2);
       m.ev_fork = m.ev_join = m.ev_fork2 = m.ev_join2 = nullptr;
-      m.aux_stream = nullptr;
+      m.aux_stream = m.aux_stream2 = nullptr;
     }
   }
 
@@ -486,6 +490,7 @@ class Batch {
     BatchStep bs;
     bs.s = s_;
     bs.s2 = s2_;
+    bs.s3 = s3_;
     for (int k = 0; k < 4; ++k) bs.ev[k] = ev_[k];
     bs.tab = tab_dev_;
     bs.m0 = &tab_[0];
@@ -592,7 +597,7 @@ class Batch {
   fsim_ctx_t ctx_;
   MeshState& ms_;
   int cap_ = 1, nr_ = 32, coop_ctas_ = 1;
-  cudaStream_t s_ = nullptr, s2_ = nullptr;
+  cudaStream_t s_ = nullptr, s2_ = nullptr, s3_ = nullptr;
   cudaEvent_t ev_[4] = {nullptr, nullptr, nullptr, nullptr};
   std::vector<Frame> frames_;
   std::vector<DevMesh> tab_;

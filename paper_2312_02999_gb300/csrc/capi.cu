@@ -154,9 +154,10 @@ int alloc_workspace(const MeshState& ms, DevMesh& m, std::vector<void*>& al, siz
   // use its side stream
   for (auto& g : m.graphs) g = DevMesh::Graph{};
   m.red_gen = 0;
-  m.aux_stream = nullptr;
+  m.aux_stream = m.aux_stream2 = nullptr;
   m.ev_fork = m.ev_join = m.ev_fork2 = m.ev_join2 = nullptr;
   if (cudaStreamCreateWithFlags(&m.aux_stream, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaStreamCreateWithFlags(&m.aux_stream2, cudaStreamNonBlocking) != cudaSuccess ||
       cudaEventCreateWithFlags(&m.ev_fork, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&m.ev_join, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&m.ev_fork2, cudaEventDisableTiming) != cudaSuccess ||
@@ -234,8 +235,9 @@ void destroy_graphs(DevMesh& m) {
   if (m.ev_fork2) cudaEventDestroy(m.ev_fork2);
   if (m.ev_join2) cudaEventDestroy(m.ev_join2);
   if (m.aux_stream) cudaStreamDestroy(m.aux_stream);
+  if (m.aux_stream2) cudaStreamDestroy(m.aux_stream2);
   m.ev_fork = m.ev_join = m.ev_fork2 = m.ev_join2 = nullptr;
-  m.aux_stream = nullptr;
+  m.aux_stream = m.aux_stream2 = nullptr;
 }
 
 // Run a fixed launch sequence through a CUDA graph captured on first use

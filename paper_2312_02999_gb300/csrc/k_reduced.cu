@@ -46,6 +46,13 @@ namespace {
 
 constexpr int kRT = 256;   // threads per CTA
 
+// Padded packed lower storage: row i holds columns 0..i, padded to a
+// multiple of 4 floats, so 32-column segments of a row are 16-byte aligned.
+__host__ __device__ constexpr int prow(int i) {
+  const int q = i >> 2;
+  return 8 * q * (q + 1) + (i - 4 * q) * 4 * (q + 1);
+}
+
 template <typename FT>
 struct RedArgs {
   int nc, n2, refine;
@@ -63,23 +70,22 @@ struct RedArgs {
   const FT* y2;         // n2 * 3: right-hand side of the Schur system (u = Sigma^-1 y2)
   double* z2;           // n2 * 3 (out)
   FT* S;                // nc x nc  -> L_s
-  FT* X;                // n3 x n3
-  FT* N;                // (n3 + 1) x n3 -> L_N and l
-  FT* dinv_s;           // nc: 1 / L_s[j][j]
-  FT* dinv_n;           // n3
+  FT* X;                // n3 x n3, then L_N^-1
+  FT* N;                // packed lower N -> L_N, diagonal blocks inverted
+  FT* Vs;               // small forms: nc x nc L_s^-1
   FT* fv;               // 2 * n3 scratch in FT
   double* y;            // n3: B u_c
   double* v;            // n3
   double* rho;          // n3
   double* w;            // n3
-  double* nrm;          // 3: |rho|^2 of a refinement step, unused, |y2|^2
-  double* S64;          // one-CTA path: Sigma^-1[c, c] in float64 (n_c x n_c)
+  double* nrm;          // 3: |rho|^2 of a refinement step (two slots), |y2|^2
+  double* S64;          // small forms: Sigma^-1[c, c] in float64 (n_c x n_c)
   int* info;
-  int small_lim;        // n_c handled by the one-CTA path (0: none)
+  int small_lim;        // n_c handled by the small forms (0: none)
   int active;           // lock-step batches: the frame takes part in the launch
   int one_cta_max;      // largest n_c of the one-CTA path (float32 factors); the
                         // 4-CTA cluster takes n_c up to kClusNc above it
-  FT* spk;              // one-CTA path: L_s packed, diagonal blocks inverted
+  FT* spk;              // small forms: L_s packed, its diagonal blocks inverted
   unsigned* bar;        // grid form: two counters of each of its two kernels
 };
 
@@ -107,9 +113,8 @@ __device__ __forceinline__ void red_layout(RedArgs<FT>& a, int nc) {
   a.S = a.base;
   a.X = a.S + al((size_t)nc * nc);
   a.N = a.X + al((size_t)n3 * n3);
-  a.dinv_s = a.N + al((size_t)(n3 + 1) * n3);
-  a.dinv_n = a.dinv_s + al(nc);
-  a.fv = a.dinv_n + al(n3);
+  a.Vs = a.N + al(prow(n3));
+  a.fv = a.Vs + al((size_t)nc * nc);
   a.spk = a.fv + al(2 * (size_t)n3);
 }
 
@@ -996,15 +1001,22 @@ __global__ void __launch_bounds__(kRT) k_grid_solve(RedArgs<FT> one, const RedAr
 }
 
 // ---------------------------------------------------------------------------
-// One-CTA path for small n_c (float32 factors): the two factorisations and
-// all triangular solves run inside one CTA with the matrix in shared memory,
-// so no grid-wide barrier is needed; only the data-parallel products run
-// over the grid.  Launch sequence (all read n_c on the device):
-//   k_small_s   (1 CTA)  S = Sigma^-1[c,c], L_s, block lists of B
-//   k_small_x   (grid)   y = B u_c (float64), |y2|^2, X = B (L_s (x) I_3)
-//   k_small_n   (grid)   N = I + (L_s (x) I_3)^T X  (lower part)
-//   k_small_v   (1 CTA)  L_N, v = L^-T N^-1 L^T y and its float64 refinement
-//   k_z2_update (grid)   z2
+// Small forms (float32 factors, 0 < n_c <= kClusNc).  Every kernel reads n_c on
+// the device.  On the side stream, while the forward solve makes u:
+//   k_small_s     (1 CTA)  S = Sigma^-1[c,c], L_s, block lists of B
+//   k_small_x     (grid)   X = B (L_s (x) I_3)
+//   k_small_n     (grid)   N = I + (L_s (x) I_3)^T X  (lower part, packed)
+//   k_small_v     (1 CTA, n_c <= kSmallNc) or k_clus_v (4-CTA cluster): L_N, the
+//                          whole matrix in shared memory, so no grid-wide barrier
+//   k_small_u     (CTA per block column)  V = L_N^-1, V_s = L_s^-1
+// and after it
+//   k_small_solve (8-CTA cluster)  y = B u_c, v and its float64 refinement
+//   k_z2_update   (grid)   z2
+// With explicit inverses a solve is four products that spread over the cluster;
+// substitution would be a chain of 2 n / 32 + n_c / 32 dependent blocks, each a
+// cluster barrier or two CTA barriers.  n_c = 93, one frame: 16 + 240 us stood
+// between u and v; now 67 us do, with the factor and the inverses (104 + 45 us)
+// beside the forward solve.
 // ---------------------------------------------------------------------------
 constexpr int kSmallNc = 96;               // 3 n_c <= 288 fits in one CTA's shared memory
 constexpr int kSmallN3 = 3 * kSmallNc;
@@ -1014,12 +1026,6 @@ constexpr int kCl = 4;                     // CTAs per cluster
 constexpr int kST = 512;                   // threads of the one-CTA kernels
 constexpr int kSW = kST / 32;
 
-// Padded packed lower storage: row i holds columns 0..i, padded to a
-// multiple of 4 floats, so 32-column segments of a row are 16-byte aligned.
-__host__ __device__ constexpr int prow(int i) {
-  const int q = i >> 2;
-  return 8 * q * (q + 1) + (i - 4 * q) * 4 * (q + 1);
-}
 constexpr int kPtLd = kSmallN3;            // panel scratch: 32 x kPtLd floats
 
 // Outer-product elimination of the unscaled 32 x 32 diagonal block Ds: after
@@ -1177,82 +1183,6 @@ __device__ void cta_chol_packed(float* A, int n, float* Pt, int* info, bool inv_
   }
 }
 
-// Solve L x = t (TRANS = false) or L^T x = t (TRANS = true) in place for a
-// packed factor, with nr interleaved right-hand sides t[i * nr + r].  The
-// inverted diagonal blocks come from DI (32 x 32 row-major per block) or,
-// when DI is null, from the diagonal blocks of A itself (cta_chol_packed
-// with inv_diag).  The 32-term dot products are unrolled so that their
-// shared-memory loads overlap.
-template <bool TRANS>
-__device__ void cta_trsv_packed(const float* A, const float* DI, int n, float* t, int nr) {
-  __shared__ float xb[32 * 3];
-  __shared__ int rp[32];
-  const int tid = threadIdx.x;
-  const int nblk = (n + 31) / 32;
-  for (int bi = 0; bi < nblk; ++bi) {
-    const int blk = TRANS ? nblk - 1 - bi : bi;
-    const int k0 = blk * 32, kb = min(32, n - k0), k1 = k0 + kb;
-    if (tid < 32) rp[tid] = prow(k0 + tid);
-    // x_k = Linv_kk t_k (or Linv_kk^T t_k): one thread per (row, rhs)
-    if (tid < kb * nr) {
-      const int i = tid / nr, r = tid % nr;
-      float acc = 0.f;
-#pragma unroll
-      for (int l = 0; l < 32; ++l) {
-        if (l < kb && (TRANS ? l >= i : l <= i)) {
-          const int rr = TRANS ? l : i, cc = TRANS ? i : l;
-          const float d = DI ? DI[(size_t)blk * 1024 + rr * 32 + cc] : A[prow(k0 + rr) + k0 + cc];
-          acc += d * t[(k0 + l) * nr + r];
-        }
-      }
-      xb[i * nr + r] = acc;
-    }
-    __syncthreads();
-    if (tid < kb * nr) t[k0 * nr + tid] = xb[tid];
-    if (TRANS) {      // rows above: t[j] -= sum_l L[k0 + l][j] x_l
-      for (int e = tid; e < k0 * nr; e += kST) {
-        const int j = e / nr, r = e % nr;
-        float acc = 0.f;
-#pragma unroll
-        for (int l = 0; l < 32; ++l)
-          if (l < kb) acc += A[rp[l] + j] * xb[l * nr + r];
-        t[e] -= acc;
-      }
-    } else {          // rows below: t[i] -= sum_l L[i][k0 + l] x_l (kb = 32 here)
-      for (int e = tid; e < (n - k1) * nr; e += kST) {
-        const int i = k1 + e / nr, r = e % nr;
-        const float4* arow = reinterpret_cast<const float4*>(A + prow(i) + k0);
-        float acc = 0.f;
-#pragma unroll
-        for (int l4 = 0; l4 < 8; ++l4) {
-          const float4 v = arow[l4];
-          acc += v.x * xb[(4 * l4) * nr + r] + v.y * xb[(4 * l4 + 1) * nr + r] +
-                 v.z * xb[(4 * l4 + 2) * nr + r] + v.w * xb[(4 * l4 + 3) * nr + r];
-        }
-        t[k1 * nr + e] -= acc;
-      }
-    }
-    __syncthreads();
-  }
-}
-
-__device__ __forceinline__ double block_sum_d(double v, double* red) {
-  // red holds kSW + 1 doubles; warp 0 adds the warp sums (float64 adds are
-  // slow on GB300: one shuffle tree, not a loop in every thread)
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  __syncthreads();
-  if (lane == 0) red[wid] = v;
-  __syncthreads();
-  if (wid == 0) {
-    double t = lane < kSW ? red[lane] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    if (lane == 0) red[kSW] = t;
-  }
-  __syncthreads();
-  return red[kSW];
-}
-
 // k_small_s: S = Sigma^-1[c, c], its factor (plain, row-major into a.S for
 // the products; packed with inverted diagonal blocks into a.spk for the
 // solves) and the block-row lists of B.
@@ -1306,71 +1236,43 @@ __global__ void __launch_bounds__(kST) k_small_s(RedArgs<float> a) {
   k_small_s_body(a);
 }
 
-// k_small_x (grid): y = B u_c in float64, |y2|^2 (PARTS & 1: these need the
-// right-hand side), X = B (L_s (x) I_3) (PARTS & 2: needs only B and L_s).
+// k_small_x (grid): X = B (L_s (x) I_3) by blocks of kXRows rows: the block's
+// rows of B-check are converted to float32 once into shared memory (a float64
+// conversion costs a float64-pipe issue on GB300), then every thread forms
+// entries of the block from them
 constexpr int kXRows = 4;                  // rows of X per staged block
-template <int PARTS>
 __device__ __forceinline__ void k_small_x_body(RedArgs<float> a) {
   const int nc = *a.nc_dev;
   if (nc == 0 || nc > a.small_lim) return;
   red_layout(a, nc);
   const int n3 = 3 * nc;
-  const int gtid = blockIdx.x * blockDim.x + threadIdx.x, gsz = gridDim.x * blockDim.x;
-  const int lane = threadIdx.x & 31;
-  if (PARTS & 1)
-  for (int row = gtid; row < n3; row += gsz) {
-    const int i = row / 3;
-    const double* brow = a.Bc + (size_t)row * n3;
-    double acc = 0.0;
-    const int ci = a.cnt[i];
-#pragma unroll 4
-    for (int e = 0; e < ci; ++e) {
-      const int j = a.list[(size_t)i * nc + e];
-      const double* uj = a.u + 3 * (size_t)a.clist[j];
-      acc += brow[3 * j] * uj[0] + brow[3 * j + 1] * uj[1] + brow[3 * j + 2] * uj[2];
+  __shared__ float bs[kXRows][3 * kClusNc];
+  const int nblk = (n3 + kXRows - 1) / kXRows;
+  for (int rb = blockIdx.x; rb < nblk; rb += gridDim.x) {
+    const int r0 = rb * kXRows;
+    __syncthreads();
+    for (int e = threadIdx.x; e < kXRows * n3; e += blockDim.x) {
+      const int rr = e / n3, c = e - rr * n3, row = r0 + rr;
+      bs[rr][c] = row < n3 ? (float)a.Bc[(size_t)row * n3 + c] : 0.f;
     }
-    a.y[row] = acc;
-  }
-  if (PARTS & 1) {
-    double q = 0.0;
-    for (int e = gtid; e < 3 * a.n2; e += gsz) q += (double)a.y2[e] * (double)a.y2[e];
-    for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
-    if (lane == 0 && q != 0.0) atomicAdd(&a.nrm[2], q);
-  }
-  if (PARTS & 2) {
-    // X by blocks of kXRows rows: the block's rows of B-check are converted
-    // to float32 once into shared memory (a float64 conversion costs a
-    // float64-pipe issue on GB300), then every thread forms entries of the
-    // block from them
-    __shared__ float bs[kXRows][3 * kClusNc];
-    const int nblk = (n3 + kXRows - 1) / kXRows;
-    for (int rb = blockIdx.x; rb < nblk; rb += gridDim.x) {
-      const int r0 = rb * kXRows;
-      __syncthreads();
-      for (int e = threadIdx.x; e < kXRows * n3; e += blockDim.x) {
-        const int rr = e / n3, c = e - rr * n3, row = r0 + rr;
-        bs[rr][c] = row < n3 ? (float)a.Bc[(size_t)row * n3 + c] : 0.f;
-      }
-      __syncthreads();
-      for (int e = threadIdx.x; e < kXRows * n3; e += blockDim.x) {
-        const int rr = e / n3, colx = e - rr * n3, row = r0 + rr;
-        if (row >= n3) continue;
-        const int i = row / 3, k = colx / 3, b = colx % 3;
-        float acc = 0.f;
-        const int ci = a.cnt[i];
+    __syncthreads();
+    for (int e = threadIdx.x; e < kXRows * n3; e += blockDim.x) {
+      const int rr = e / n3, colx = e - rr * n3, row = r0 + rr;
+      if (row >= n3) continue;
+      const int i = row / 3, k = colx / 3, b = colx % 3;
+      float acc = 0.f;
+      const int ci = a.cnt[i];
 #pragma unroll 4
-        for (int q = 0; q < ci; ++q) {
-          const int j = a.list[(size_t)i * nc + q];
-          if (j >= k) acc += bs[rr][3 * j + b] * a.S[(size_t)j * nc + k];
-        }
-        a.X[(size_t)row * n3 + colx] = acc;
+      for (int q = 0; q < ci; ++q) {
+        const int j = a.list[(size_t)i * nc + q];
+        if (j >= k) acc += bs[rr][3 * j + b] * a.S[(size_t)j * nc + k];
       }
+      a.X[(size_t)row * n3 + colx] = acc;
     }
   }
 }
-template <int PARTS>
 __global__ void __launch_bounds__(256) k_small_x(RedArgs<float> a) {
-  k_small_x_body<PARTS>(a);
+  k_small_x_body(a);
 }
 
 // k_small_n (grid): N = I + (L_s (x) I_3)^T X, lower part, packed.
@@ -1428,21 +1330,6 @@ __device__ __forceinline__ void k_small_n_body(RedArgs<float> a, int tile) {
 }
 __global__ void __launch_bounds__(256) k_small_n(RedArgs<float> a) {
   k_small_n_body(a, blockIdx.x);
-}
-
-// q = (L_s (x) I_3)^T p (float; L_s packed plain, in shared memory)
-// (one warp per entry)
-__device__ void cta_lt_apply_f(const float* Lp, int nc, const double* p, float* q) {
-  const int lane = threadIdx.x & 31;
-  for (int e = threadIdx.x >> 5; e < 3 * nc; e += kSW) {
-    const int i = e / 3, ax = e % 3;
-    float acc = 0.f;
-#pragma unroll 4
-    for (int j = i + lane; j < nc; j += 32) acc += Lp[prow(j) + i] * (float)p[3 * j + ax];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) q[e] = acc;
-  }
 }
 
 // Float64 refinement products.  GB300 issues a warp-wide float64 FMA about
@@ -1529,12 +1416,10 @@ __device__ double refine_rho(const RedArgs<float>& a, int nc, int t, int nt) {
   return r2;
 }
 
-// k_small_v (1 CTA): L_N in shared memory, v = (L_s (x) I)^-T N^-1 (L_s (x) I)^T y
-// and the float64-residual refinement of v (same stopping rule as the
-// cooperative kernel).
+// k_small_v (1 CTA): L_N in shared memory, back to the packed N with inverted
+// diagonal blocks
 __device__ __forceinline__ void k_small_v_body(RedArgs<float> a) {
   extern __shared__ float smem_f[];
-  __shared__ double red[kSW + 1];
   const int nc = *a.nc_dev;
   if (nc == 0 || nc > a.one_cta_max) return;
   red_layout(a, nc);
@@ -1542,69 +1427,304 @@ __device__ __forceinline__ void k_small_v_body(RedArgs<float> a) {
   const int tid = threadIdx.x;
   float* A = smem_f;                      // prow(kSmallN3) floats
   float* Pt = A + prow(kSmallN3);         // 32 x kPtLd
-  float* t = Pt + 32 * kPtLd;             // n3
-  {   // packed N (padding included: prow(n3) is a multiple of 4)
-    const float4* src = reinterpret_cast<const float4*>(a.N);
-    float4* dst = reinterpret_cast<float4*>(A);
+  // packed N (padding included: prow(n3) is a multiple of 4)
+  float4* gN = reinterpret_cast<float4*>(a.N);
+  float4* sN = reinterpret_cast<float4*>(A);
 #pragma unroll 4
-    for (int e = tid; e < prow(n3) / 4; e += kST) dst[e] = src[e];
-  }
+  for (int e = tid; e < prow(n3) / 4; e += kST) sN[e] = gN[e];
   __syncthreads();
   cta_chol_packed(A, n3, Pt, a.info, true, nullptr, 0, nullptr);
-  // L_s (packed plain + inverted diagonal blocks) into the panel scratch
-  float* Ls = Pt;
-  const float* LsDI = Pt + prow(nc);
-  {
-    const float4* src = reinterpret_cast<const float4*>(a.spk);
-    float4* dst = reinterpret_cast<float4*>(Ls);
-    const int n4 = (prow(nc) + 1024 * ((nc + 31) / 32)) / 4;
 #pragma unroll 4
-    for (int e = tid; e < n4; e += kST) dst[e] = src[e];
-  }
-  __syncthreads();
-  cta_lt_apply_f(Ls, nc, a.y, t);
-  __syncthreads();
-  cta_trsv_packed<false>(A, nullptr, n3, t, 1);
-  cta_trsv_packed<true>(A, nullptr, n3, t, 1);
-  cta_trsv_packed<true>(Ls, LsDI, nc, t, 3);
-  for (int e = tid; e < n3; e += kST) a.v[e] = (double)t[e];
-  __syncthreads();
-  double prev = -1.0;
-  for (int it = 0; it < a.refine; ++it) {
-    // w = S v with S = Sigma^-1[c, c] (x) I_3 in float64 (S gathered by k_small_s)
-    refine_sv(a, nc, tid, kST);
-    __syncthreads();
-    double r2 = refine_rho(a, nc, tid, kST);
-    r2 = block_sum_d(r2, red);
-    const double ys = __ldcg(a.nrm + 2);
-    if (!(r2 > 1e-14 * ys)) break;
-    if (prev >= 0.0 && !(r2 < 0.25 * prev)) break;
-    prev = r2;
-    cta_lt_apply_f(Ls, nc, a.rho, t);
-    __syncthreads();
-    cta_trsv_packed<false>(A, nullptr, n3, t, 1);
-    cta_trsv_packed<true>(A, nullptr, n3, t, 1);
-    cta_trsv_packed<true>(Ls, LsDI, nc, t, 3);
-    for (int e = tid; e < n3; e += kST) a.v[e] += (double)t[e];
-    __syncthreads();
-  }
+  for (int e = tid; e < prow(n3) / 4; e += kST) gN[e] = sN[e];
 }
 __global__ void __launch_bounds__(kST) k_small_v(RedArgs<float> a) {
   k_small_v_body(a);
 }
 
+// k_small_u: a CTA per block column j of V = L^-1 (the first kUN CTAs V of L_N,
+// the others V_s of L_s): V_jj = L_jj^-1, then down the column
+//   V_ij = -L_ii^-1 sum_{k = j .. i-1} L_ik V_kj.
+// The column's blocks stay in shared memory, transposed, so that both operands
+// of the products are read along l; four groups of 64 threads take every
+// fourth k (4 x 4 values per thread: rows ti + 8 p, columns tj + 8 q) and their
+// partial sums are added before the product with the inverted diagonal block.
+constexpr int kUN = kClusN3 / 32, kUCtas = kUN + kClusNc / 32;
+constexpr int kULd = 36;
+constexpr size_t kSmallSmemU = sizeof(float) * (size_t)(kUN + 4 + 1) * 32 * kULd;
+__device__ __forceinline__ void k_small_u_body(RedArgs<float> a, int cta) {
+  extern __shared__ __align__(16) float smem_f[];
+  const int nc = *a.nc_dev;
+  if (nc == 0 || nc > a.small_lim) return;
+  red_layout(a, nc);
+  const bool is_n = cta < kUN;
+  const int n = is_n ? 3 * nc : nc, j = is_n ? cta : cta - kUN, nb = (n + 31) / 32;
+  if (j >= nb) return;
+  const float* P = is_n ? a.N : a.spk;                  // packed factor
+  const float* DI = is_n ? nullptr : a.spk + prow(nc);  // inverted diagonal blocks, else in P
+  float* V = is_n ? a.X : a.Vs;
+  const int tid = threadIdx.x, gr = tid >> 6, tq = tid & 63, ti = tq >> 3, tj = tq & 7;
+  float(*VT)[kULd] = reinterpret_cast<float(*)[kULd]>(smem_f);            // [32 block + column][row]
+  float(*Lk)[kULd] = VT + kUN * 32 + gr * 32;                              // this group's L_ik
+  float(*part)[kULd] = VT + kUN * 32;                                      // 4 x 32 rows
+  float(*Di)[kULd] = VT + (kUN + 4) * 32;
+  auto load_diag = [&](int i) {          // L_ii^-1, zero above the diagonal and past n
+    for (int e = tid; e < 32 * 32; e += kRT) {
+      const int r = e >> 5, c = e & 31;
+      float v = 0.f;
+      if (c <= r && 32 * i + r < n) v = DI ? DI[1024 * i + e] : P[prow(32 * i + r) + 32 * i + c];
+      Di[r][c] = v;
+    }
+  };
+  auto store = [&](int i, int r, int c, float v) {
+    VT[32 * i + c][r] = v;
+    if (32 * i + r < n && 32 * j + c < n) V[(size_t)(32 * i + r) * n + 32 * j + c] = v;
+  };
+  load_diag(j);
+  __syncthreads();
+  for (int e = tid; e < 32 * 32; e += kRT) store(j, e >> 5, e & 31, Di[e >> 5][e & 31]);
+  for (int i = j + 1; i < nb; ++i) {
+    __syncthreads();
+    load_diag(i);
+    float acc[4][4];
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[p][q] = 0.f;
+    for (int k = j + gr; k < i; k += 4) {
+      float4 f[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int e = tq + 64 * u, r = 32 * i + (e >> 3);
+        f[u] = r < n ? *(reinterpret_cast<const float4*>(P + prow(r) + 32 * k) + (e & 7))
+                     : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+      asm volatile("bar.sync %0, 64;" ::"r"(gr + 1) : "memory");   // the tile before is read
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int e = tq + 64 * u;
+        *reinterpret_cast<float4*>(&Lk[e >> 3][4 * (e & 7)]) = f[u];
+      }
+      asm volatile("bar.sync %0, 64;" ::"r"(gr + 1) : "memory");
+#pragma unroll 2
+      for (int l = 0; l < 32; l += 4) {
+        float4 x[4], y[4];
+#pragma unroll
+        for (int p = 0; p < 4; ++p) x[p] = *reinterpret_cast<const float4*>(&Lk[ti + 8 * p][l]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          y[q] = *reinterpret_cast<const float4*>(&VT[32 * k + tj + 8 * q][l]);
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            acc[p][q] += x[p].x * y[q].x + x[p].y * y[q].y + x[p].z * y[q].z + x[p].w * y[q].w;
+      }
+    }
+    __syncthreads();                     // all tiles are read: part overlays them
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) part[32 * gr + tj + 8 * q][ti + 8 * p] = acc[p][q];   // [column][row]
+    __syncthreads();
+    // column c, rows r0 .. r0 + 3 of -L_ii^-1 (sum of the parts)
+    const int c = tid >> 3, r0 = 4 * (tid & 7);
+    float o[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+    for (int l = 0; l < 32; ++l) {
+      const float s = part[c][l] + part[32 + c][l] + part[64 + c][l] + part[96 + c][l];
+#pragma unroll
+      for (int p = 0; p < 4; ++p) o[p] -= Di[r0 + p][l] * s;
+    }
+#pragma unroll
+    for (int p = 0; p < 4; ++p) store(i, r0 + p, c, o[p]);
+  }
+}
+__global__ void __launch_bounds__(kRT) k_small_u(RedArgs<float> a) {
+  k_small_u_body(a, blockIdx.x);
+}
+
+// k_small_solve: y = B u_c, v = (V_s (x) I)^T V^T V (L_s (x) I)^T y and its
+// float64-residual refinement (same stopping rule as the grid form), on a
+// cluster of kSolveCl CTAs: the vectors live in global memory and a cluster
+// barrier separates the products.  Warps and threads are numbered interleaved
+// over the CTAs, so that every SM gets its share of the float64 work.
+constexpr int kSolveCl = 8;
+constexpr int kSolveW = kRT / 32;           // warps per CTA
+__device__ __forceinline__ void k_small_solve_body(RedArgs<float> a) {
+  namespace cgx = cooperative_groups;
+  cgx::cluster_group cl = cgx::this_cluster();
+  __shared__ float part[3][kSolveW][32];
+  __shared__ double wred[kSolveW];
+  __shared__ double nrm_parts[2][kSolveCl];
+  const int nc = *a.nc_dev;
+  if (nc == 0 || nc > a.small_lim) return;          // uniform over the cluster
+  red_layout(a, nc);
+  const int n3 = 3 * nc, rank = (int)cl.block_rank();
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int gw = wid * kSolveCl + rank, nw = kSolveW * kSolveCl;
+  const int gt = 32 * gw + lane, nt = 32 * nw;
+  float* t = a.fv;
+  float* l = a.fv + n3;
+  const float* V = a.X;
+  // sum over the cluster in slot `slot` (one barrier; the same value everywhere)
+  auto cluster_sum = [&](double v, int slot) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    __syncthreads();
+    if (lane == 0) wred[wid] = v;
+    __syncthreads();
+    if (tid < kSolveCl) {
+      double s = 0.0;
+      for (int w = 0; w < kSolveW; ++w) s += wred[w];
+      cl.map_shared_rank(&nrm_parts[slot][0], tid)[rank] = s;
+    }
+    cl.sync();
+    double s = 0.0;
+    for (int q = 0; q < kSolveCl; ++q) s += nrm_parts[slot][q];
+    return s;
+  };
+  auto apply = [&](const double* p, bool add) {
+    // t = (L_s (x) I)^T p, one warp per entry
+    for (int e = gw; e < n3; e += nw) {
+      const int i = e / 3, ax = e % 3;
+      float acc = 0.f;
+#pragma unroll 4
+      for (int j = i + lane; j < nc; j += 32) acc += a.S[(size_t)j * nc + i] * (float)p[3 * j + ax];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if (lane == 0) t[e] = acc;
+    }
+    cl.sync();
+    // l = V t, one warp per two rows (their loads in flight together)
+    for (int i = gw; i < n3; i += 2 * nw) {
+      const int i1 = i + nw;
+      float a0 = 0.f, a1 = 0.f;
+#pragma unroll 4
+      for (int j = lane; j < n3; j += 32) {
+        const float tv = t[j];
+        if (j <= i) a0 += V[(size_t)i * n3 + j] * tv;
+        if (j <= i1 && i1 < n3) a1 += V[(size_t)i1 * n3 + j] * tv;
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        a0 += __shfl_xor_sync(0xffffffffu, a0, o);
+        a1 += __shfl_xor_sync(0xffffffffu, a1, o);
+      }
+      if (lane == 0) {
+        l[i] = a0;
+        if (i1 < n3) l[i1] = a1;
+      }
+    }
+    cl.sync();
+    // t = V^T l: block column b on CTA b, its warps share the rows (lane = column)
+    for (int b = rank; 32 * b < n3; b += kSolveCl) {
+      const int j = 32 * b + lane;
+      float acc = 0.f;
+      if (j < n3)
+#pragma unroll 8
+        for (int i = 32 * b + wid; i < n3; i += kSolveW) acc += V[(size_t)i * n3 + j] * l[i];
+      __syncthreads();
+      part[0][wid][lane] = acc;
+      __syncthreads();
+      if (wid == 0 && j < n3) {
+        float s = 0.f;
+#pragma unroll
+        for (int w = 0; w < kSolveW; ++w) s += part[0][w][lane];
+        t[j] = s;
+      }
+    }
+    cl.sync();
+    // v (+)= (V_s (x) I)^T t
+    for (int b = rank; 32 * b < nc; b += kSolveCl) {
+      const int i = 32 * b + lane;
+      float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+      if (i < nc)
+#pragma unroll 4
+        for (int j = 32 * b + wid; j < nc; j += kSolveW) {
+          const float vs = a.Vs[(size_t)j * nc + i];
+          s0 += vs * t[3 * j];
+          s1 += vs * t[3 * j + 1];
+          s2 += vs * t[3 * j + 2];
+        }
+      __syncthreads();
+      part[0][wid][lane] = s0;
+      part[1][wid][lane] = s1;
+      part[2][wid][lane] = s2;
+      __syncthreads();
+      if (wid < 3 && i < nc) {
+        float s = 0.f;
+#pragma unroll
+        for (int w = 0; w < kSolveW; ++w) s += part[wid][w][lane];
+        a.v[3 * i + wid] = (add ? a.v[3 * i + wid] : 0.0) + (double)s;
+      }
+    }
+    cl.sync();
+  };
+  // y = B u_c over the block lists (kRP lanes per block row), |y2|^2
+  for (int base = 0; base < kRP * nc; base += nt) {
+    const int item = base + gt;
+    const bool ok = item < kRP * nc;
+    const int i = ok ? item / kRP : 0, q = item % kRP;
+    double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+    if (ok) {
+      const double* b0 = a.Bc + (size_t)(3 * i) * n3;
+      const double* b1 = b0 + n3;
+      const double* b2 = b1 + n3;
+      const int ci = a.cnt[i];
+      for (int e = q; e < ci; e += kRP) {
+        const int j = a.list[(size_t)i * nc + e];
+        if (!FSIM_CHECK_IDX(a.clist[j], a.n2, CHECK_CLIST)) continue;
+        const double* uj = a.u + 3 * (size_t)a.clist[j];
+        const double u0 = uj[0], u1 = uj[1], u2 = uj[2];
+        const int j3 = 3 * j;
+        s0 += b0[j3] * u0 + b0[j3 + 1] * u1 + b0[j3 + 2] * u2;
+        s1 += b1[j3] * u0 + b1[j3 + 1] * u1 + b1[j3 + 2] * u2;
+        s2 += b2[j3] * u0 + b2[j3 + 1] * u1 + b2[j3 + 2] * u2;
+      }
+    }
+#pragma unroll
+    for (int o = kRP / 2; o > 0; o >>= 1) {
+      s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+      s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+      s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+    }
+    if (ok && q == 0) {
+      a.y[3 * i] = s0;
+      a.y[3 * i + 1] = s1;
+      a.y[3 * i + 2] = s2;
+    }
+  }
+  double ys = 0.0;
+  for (int e = gt; e < 3 * a.n2; e += nt) ys += (double)a.y2[e] * (double)a.y2[e];
+  ys = cluster_sum(ys, 0);
+  apply(a.y, false);
+  double prev = -1.0;
+  for (int it = 0; it < a.refine; ++it) {
+    refine_sv(a, nc, gt, nt);
+    cl.sync();
+    // two slots in turn: a CTA may still read the one of the step before
+    const double r2 = cluster_sum(refine_rho(a, nc, gt, nt), (it + 1) & 1);
+    if (!(r2 > 1e-14 * ys)) break;
+    if (prev >= 0.0 && !(r2 < 0.25 * prev)) break;
+    prev = r2;
+    apply(a.rho, true);
+  }
+  cl.sync();       // no CTA leaves while its shared memory may still be written
+}
+__global__ void __launch_bounds__(kRT) k_small_solve(RedArgs<float> a) {
+  k_small_solve_body(a);
+}
+
 // ---------------------------------------------------------------------------
-// k_clus_v: the same solve for kSmallNc < n_c <= kClusNc on a cluster of kCl
-// CTAs.  32-row blocks of the packed N are spread block-cyclically over the
-// CTAs' shared memory.  Per panel the owner factors its diagonal block and the
-// others copy it through distributed shared memory; each CTA solves its own
+// k_clus_v: the same factorisation for kSmallNc < n_c <= kClusNc on a cluster
+// of kCl CTAs.  32-row blocks of the packed N are spread block-cyclically over
+// the CTAs' shared memory.  Per panel the owner factors its diagonal block and
+// the others copy it through distributed shared memory; each CTA solves its own
 // rows of the panel and stores them into the panel copy of every CTA
 // (distributed shared-memory stores, visible after the cluster barrier that
 // follows), then updates only its own rows.  The diagonal blocks are
-// inverted after the factorisation, one warp per block.  The triangular
-// solves pass 32-value blocks through distributed shared memory with one
-// cluster barrier per block, and the float64 residuals of the refinement are
-// split over the CTAs.
+// inverted after the factorisation, one warp per block, and the rows go back to
+// global memory.
 // ---------------------------------------------------------------------------
 constexpr int kClusRowsMax = 32 * ((kClusN3 / 32 + kCl - 1) / kCl);   // own rows per CTA
 // largest packed storage of the rows one CTA owns (padded row lengths)
@@ -1621,8 +1741,7 @@ constexpr int clus_aloc() {
 constexpr int kClusALoc = clus_aloc();
 static_assert(kClusALoc % 4 == 0, "panel scratch must stay 16-byte aligned");
 constexpr size_t kClusSmem =
-    sizeof(float) * ((size_t)kClusALoc + 32 * (size_t)kClusN3 + (size_t)prow(kClusNc) +
-                     1024 * (kClusNc / 32) + 2 * (size_t)kClusN3);
+    sizeof(float) * ((size_t)kClusALoc + 32 * (size_t)kClusN3);
 
 // (__maxnreg__ rather than __launch_bounds__: with the latter ptxas settles
 // on 64 registers and spills; 512 threads x 128 registers fill one SM)
@@ -1634,12 +1753,7 @@ __device__ __forceinline__ void k_clus_v_body(RedArgs<float> a) {
   __shared__ float dv[32];
   __shared__ float dvown[kClusRowsMax];            // 1 / L_ii of own rows
   __shared__ float Dinv[kClusRowsMax / 32][32][33];  // own diagonal blocks, inverted at the end
-  __shared__ float xb[2][32];
-  __shared__ float part[2][kCl][32];
-  __shared__ double nrm_parts[kCl];
-  __shared__ float wsum[kSW][32];
   __shared__ int loff[kClusRowsMax];
-  __shared__ double red[kSW + 1];
   const int nc = *a.nc_dev;
   if (nc <= a.one_cta_max || nc > kClusNc) return;  // uniform over the cluster
   red_layout(a, nc);
@@ -1648,10 +1762,6 @@ __device__ __forceinline__ void k_clus_v_body(RedArgs<float> a) {
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   float* A = smem_f;                               // own rows, packed
   float* Pt = A + kClusALoc;                       // 32 x kClusN3, panel by global row - k1
-  float* Ls = Pt + 32 * kClusN3;                   // L_s packed plain, then inverted blocks
-  float* LsDI = Ls + prow(nc);
-  float* t = Ls + prow(kClusNc) + 1024 * (kClusNc / 32);   // n3: rhs / solution (own rows valid)
-  float* xg = t + kClusN3;                         // n3: gathered solution (rank 0)
   // own rows: block b is owned by b % kCl; local row lb * 32 + (r % 32)
   auto lrow = [&](int r) { return ((r >> 5) / kCl) * 32 + (r & 31); };
   if (tid < kClusRowsMax) {
@@ -1664,7 +1774,7 @@ __device__ __forceinline__ void k_clus_v_body(RedArgs<float> a) {
   }
   __syncthreads();
   auto Ael = [&](int r, int c) -> float& { return A[loff[lrow(r)] + c]; };
-  // load own rows of the packed N and L_s.  A packed row r is a 16-byte
+  // load own rows of the packed N.  A packed row r is a 16-byte
   // aligned run of 4 (r / 4 + 1) floats in both layouts (padding included,
   // never read), so rows move as float4: warp w takes own rows w, w + 16, ..
   // two rows and all their loads in flight at once (a row has <= 96 float4)
@@ -1691,13 +1801,6 @@ __device__ __forceinline__ void k_clus_v_body(RedArgs<float> a) {
       for (int u = 0; u < 3; ++u)
         if (lane + 32 * u < len4[h]) dst[lane + 32 * u] = v[h][u];
     }
-  }
-  {
-    const float4* src = reinterpret_cast<const float4*>(a.spk);
-    float4* dst = reinterpret_cast<float4*>(Ls);
-    const int n4 = (prow(nc) + 1024 * ((nc + 31) / 32)) / 4;
-#pragma unroll 4
-    for (int e = tid; e < n4; e += kST) dst[e] = src[e];
   }
   __syncthreads();
 
@@ -1859,154 +1962,23 @@ __device__ __forceinline__ void k_clus_v_body(RedArgs<float> a) {
         if (i < kb && i >= lane) A[loff[lb + i] + k0 + lane] = x[i];
     }
   }
-  cl.sync();
-
-  // ---- distributed solves with L_N (own rows of t hold the values) ---------
-  auto solve_n = [&]() {
-    // forward: L x = t
-    for (int k = 0; k < nblk; ++k) {
-      const int k0 = 32 * k, kb = min(32, n3 - k0), owner = k % kCl, buf = k & 1;
-      if (rank == owner) {
-        {   // x_k = L_kk^-1 t_k: 16 threads per row, two terms each, shuffle sum
-          const int rw = tid >> 4, pp = tid & 15;
-          float acc = 0.f;
-          if (rw < kb) {
-            const float* drow = &Ael(k0 + rw, k0);
-            if (pp <= rw) acc += drow[pp] * t[k0 + pp];
-            if (pp + 16 <= rw) acc += drow[pp + 16] * t[k0 + pp + 16];
-          }
-#pragma unroll
-          for (int o = 8; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-          if (pp == 0 && rw < kb) xb[buf][rw] = acc;
-        }
-        __syncthreads();
-        if (tid < kb) {
-          t[k0 + tid] = xb[buf][tid];
-          for (int q = 0; q < kCl; ++q)
-            if (q != rank) cl.map_shared_rank(&xb[buf][0], q)[tid] = xb[buf][tid];
-        }
-      }
-      cl.sync();
-      for (int idx = tid; idx < kClusRowsMax; idx += kST) {
-        const int b = ((idx >> 5) * kCl) + rank;
-        const int r = 32 * b + (idx & 31);
-        if (b > k && r < n3) {
-          const float* row = &Ael(r, k0);
-          float acc = 0.f;
-#pragma unroll
-          for (int l = 0; l < 32; ++l) acc += row[l] * xb[buf][l];
-          t[r] -= acc;
-        }
-      }
-      __syncthreads();
-    }
-    // backward: L^T x = t
-    for (int k = nblk - 1; k >= 0; --k) {
-      const int k0 = 32 * k, kb = min(32, n3 - k0), owner = k % kCl, buf = k & 1;
-      // partial sums over own rows below block k for its columns: warp w
-      // takes own rows w, w + 16, ...; lane = column
-      {
-        float acc = 0.f;
-        if (lane < kb)
-          for (int idx = wid; idx < kClusRowsMax; idx += kSW) {
-            const int b = ((idx >> 5) * kCl) + rank;
-            const int r = 32 * b + (idx & 31);
-            if (b > k && r < n3) acc += Ael(r, k0 + lane) * t[r];
-          }
-        wsum[wid][lane] = acc;
-        __syncthreads();
-        if (tid < 32) {
-          float tot = 0.f;
-          for (int w = 0; w < kSW; ++w) tot += wsum[w][tid];
-          cl.map_shared_rank(&part[buf][0][0], owner)[rank * 32 + tid] = tot;
-        }
-      }
-      cl.sync();
-      if (rank == owner) {
-        if (tid < kb) {
-          float s = t[k0 + tid];
-          for (int q = 0; q < kCl; ++q) s -= part[buf][q][tid];
-          xb[buf][tid] = s;
-        }
-        __syncthreads();
-        {   // x_k = L_kk^-T s_k: 16 threads per column, two terms each
-          const int col = tid >> 4, pp = tid & 15;
-          float acc = 0.f;
-          if (col < kb) {
-            if (pp >= col && pp < kb) acc += Ael(k0 + pp, k0 + col) * xb[buf][pp];
-            if (pp + 16 >= col && pp + 16 < kb)
-              acc += Ael(k0 + pp + 16, k0 + col) * xb[buf][pp + 16];
-          }
-#pragma unroll
-          for (int o = 8; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-          if (pp == 0 && col < kb) t[k0 + col] = acc;
-        }
-        __syncthreads();
-      }
-    }
-    cl.sync();
-  };
-  // (L_s (x) I)^-T on the gathered solution (rank 0), result into a.v / added to it
-  auto finish = [&](bool add) {
-    if (rank == 0) {
-      // every row from the CTA that owns it, all remote loads in flight at once
-      for (int r = tid; r < n3; r += kST) {
-        const int q = (r >> 5) % kCl;
-        xg[r] = (q == 0) ? t[r] : cl.map_shared_rank(t, q)[r];
-      }
-      __syncthreads();
-      cta_trsv_packed<true>(Ls, LsDI, nc, xg, 3);
-      for (int e = tid; e < n3; e += kST) a.v[e] = (add ? a.v[e] : 0.0) + (double)xg[e];
-    }
-    cl.sync();
-  };
-  // t = (L_s (x) I_3)^T p on own rows
-  auto lt_own = [&](const double* p) {     // one warp per own row
-    for (int idx = wid; idx < kClusRowsMax; idx += kSW) {
-      const int r = 32 * (((idx >> 5) * kCl) + rank) + (idx & 31);
-      if (r >= n3) continue;
-      const int i = r / 3, ax = r % 3;
-      float acc = 0.f;
-#pragma unroll 4
-      for (int j = i + lane; j < nc; j += 32) acc += Ls[prow(j) + i] * (float)p[3 * j + ax];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-      if (lane == 0) t[r] = acc;
-    }
-    __syncthreads();
-  };
-  lt_own(a.y);
-  solve_n();
-  finish(false);
-
-  // ---- float64 refinement, rows split over the cluster ----------------------
-  double prev = -1.0;
-  // refinement threads numbered warp-interleaved over the cluster's CTAs
-  const int gt = (wid * kCl + rank) * 32 + lane;
-  for (int it = 0; it < a.refine; ++it) {
-    refine_sv(a, nc, gt, kCl * kST);
-    cl.sync();
-    double r2 = refine_rho(a, nc, gt, kCl * kST);
-    r2 = block_sum_d(r2, red);
-    if (tid < kCl) cl.map_shared_rank(&nrm_parts[0], tid)[rank] = r2;
-    cl.sync();
-    double tot = 0.0;
-    for (int q = 0; q < kCl; ++q) tot += nrm_parts[q];     // same order everywhere
-    const double ys = __ldcg(a.nrm + 2);
-    if (!(tot > 1e-14 * ys)) break;
-    if (prev >= 0.0 && !(tot < 0.25 * prev)) break;
-    prev = tot;
-    lt_own(a.rho);
-    solve_n();
-    finish(true);
+  __syncthreads();
+  // own rows back to the packed N
+  for (int lr = wid; lr < kClusRowsMax; lr += kSW) {
+    const int r = 32 * (((lr >> 5) * kCl) + rank) + (lr & 31);
+    if (r >= n3) continue;
+    const float4* src = reinterpret_cast<const float4*>(A + loff[lr]);
+    float4* dst = reinterpret_cast<float4*>(a.N + prow(r));
+    for (int u = lane; u < (r >> 2) + 1; u += 32) dst[u] = src[u];
   }
+  cl.sync();       // no CTA leaves while its shared memory may still be read
 }
 __global__ void __maxnreg__(128) k_clus_v(RedArgs<float> a) {
   k_clus_v_body(a);
 }
 
 constexpr size_t kSmallSmemS = sizeof(float) * ((size_t)prow(kClusNc) + 32 * kPtLd);
-constexpr size_t kSmallSmemV = sizeof(float) * ((size_t)prow(kSmallN3) + 32 * kPtLd + kSmallN3);
+constexpr size_t kSmallSmemV = sizeof(float) * ((size_t)prow(kSmallN3) + 32 * kPtLd);
 
 template <typename FT>
 RedArgs<FT> make_args(const DevMesh& m, const double* u, const FT* y2, double* z2, int* info,
@@ -2061,24 +2033,52 @@ cudaError_t launch_grid(cudaStream_t s, RedArgs<FT> a, int ctas, bool prepare) {
   return e;
 }
 
-// float32 factors, n_c <= kClusNc: the one-CTA path up to one_cta_max, the
-// 4-CTA cluster above it.  The z2 update is a plain launch, so no cooperative
-// launch is needed (whose grid must find all of its SMs free at once when
+// Launch k_small_solve(_b): one cluster of kSolveCl CTAs per system.
+template <typename K, typename A>
+cudaError_t launch_solve_clusters(cudaStream_t s, K kernel, int nsys, const A& arg) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kSolveCl, nsys);
+  cfg.blockDim = dim3(kRT);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = kSolveCl;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, arg);
+  count_launch();
+  return e;
+}
+
+// float32 factors, n_c <= kClusNc, on the side stream: one-CTA factor up to
+// one_cta_max, the 4-CTA cluster above it, then the inverses of both factors.
+// No cooperative launch (whose grid must find all of its SMs free at once when
 // other solves share the GPU).
+cudaError_t launch_small_prepare(cudaStream_t s2, const RedArgs<float>& a, int num_sms, int nc) {
+  ProfScope ps(PROF_CHOL, s2);
+  k_small_s<<<1, kST, kSmallSmemS, s2>>>(a);
+  k_small_x<<<2 * std::max(1, num_sms), 256, 0, s2>>>(a);
+  k_small_n<<<kNTiles, 256, 0, s2>>>(a);
+  if (nc <= a.one_cta_max) {
+    k_small_v<<<1, kST, kSmallSmemV, s2>>>(a);
+  } else {
+    const cudaError_t e = launch_clus_v(s2, a);
+    if (e != cudaSuccess) return e;
+  }
+  k_small_u<<<kUCtas, kRT, kSmallSmemU, s2>>>(a);
+  count_launch(nc <= a.one_cta_max ? 5 : 4);
+  return cudaGetLastError();
+}
+// the solve, and the z2 update as a plain launch
 cudaError_t launch_small(cudaStream_t s, const DevMesh& m, const RedArgs<float>& a, int num_sms,
                          int nc) {
   ProfScope ps(PROF_CHOL, s);
   const int zgrid = std::max(1, std::min(2 * std::max(1, num_sms), (m.n2 + 7) / 8));
   if (nc > 0) {
-    k_small_x<1><<<2 * std::max(1, num_sms), 256, 0, s>>>(a);
-    count_launch();
-    if (nc <= a.one_cta_max) {
-      k_small_v<<<1, kST, kSmallSmemV, s>>>(a);
-      count_launch();
-    } else {
-      const cudaError_t e = launch_clus_v(s, a);
-      if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = launch_solve_clusters(s, k_small_solve, 1, a);
+    if (e != cudaSuccess) return e;
   }
   k_z2_update<<<zgrid, 256, 0, s>>>(a);
   count_launch();
@@ -2089,10 +2089,10 @@ cudaError_t launch_small(cudaStream_t s, const DevMesh& m, const RedArgs<float>&
 
 int64_t reduced_workspace_elems(int nc) {
   const int64_t n3 = 3 * (int64_t)nc;
-  // one-CTA / cluster forms: S, X, N (+1 row), 1/diag of both factors, two FT
-  // vectors, packed L_s
-  const int64_t small = (int64_t)nc * nc + n3 * n3 + (n3 + 1) * n3 + nc + n3 + 2 * n3 +
-                        (prow(nc) + 1024 * ((int64_t)nc + 31) / 32 + 16) + 64;
+  // small forms: S, X, packed N, L_s^-1, two FT vectors, packed L_s with its
+  // inverted diagonal blocks (each rounded up to 16 bytes)
+  const int64_t small = 2 * (int64_t)nc * nc + n3 * n3 + n3 * (n3 + 4) / 2 + 8 + 2 * n3 +
+                        (int64_t)nc * (nc + 4) / 2 + 8 + 1024 * (((int64_t)nc + 31) / 32) + 64;
   // at the tail of the float64 buffer four float64 vectors, three norms and S64
   return std::max(small, grid_front_elems(nc)) + 4 * n3 + (int64_t)nc * nc + 64;
 }
@@ -2172,10 +2172,17 @@ __global__ void __launch_bounds__(32 * kPhiSplit) k_phi_apply(RedArgs<float> a, 
 }
 
 // ---- lock-step batches: blockIdx.y = frame, RedArgs per frame on the device
-template <int PARTS>
 __global__ void __launch_bounds__(256) k_small_x_b(const RedArgs<float>* __restrict__ A) {
   const RedArgs<float> a = A[blockIdx.y];
-  if (a.active) k_small_x_body<PARTS>(a);
+  if (a.active) k_small_x_body(a);
+}
+__global__ void __launch_bounds__(kRT) k_small_u_b(const RedArgs<float>* __restrict__ A) {
+  const RedArgs<float> a = A[blockIdx.y];
+  if (a.active) k_small_u_body(a, blockIdx.x);
+}
+__global__ void __launch_bounds__(kRT) k_small_solve_b(const RedArgs<float>* __restrict__ A) {
+  const RedArgs<float> a = A[blockIdx.y];
+  if (a.active) k_small_solve_body(a);       // uniform over a cluster
 }
 __global__ void __launch_bounds__(kST) k_small_s_b(const RedArgs<float>* __restrict__ A) {
   const RedArgs<float> a = A[blockIdx.y];
@@ -2294,19 +2301,6 @@ cudaError_t launch_grid_b(cudaStream_t s, const RedArgs<float>* A, const RedArgs
 cudaError_t reduced_prepare_b(cudaStream_t s2, const void* args_dev, const void* args_host, int nb,
                               const int* nc_host, int coop_ctas) {
   const auto* A = static_cast<const RedArgs<float>*>(args_dev);
-  ProfScope ps(PROF_CHOL, s2);
-  k_small_s_b<<<dim3(1, nb), kST, kSmallSmemS, s2>>>(A);
-  k_small_x_b<2><<<dim3((3 * kClusNc + kXRows - 1) / kXRows, nb), 256, 0, s2>>>(A);
-  k_small_n_b<<<dim3(kNTiles, nb), 256, 0, s2>>>(A);
-  count_launch(3);
-  const cudaError_t e =
-      launch_grid_b(s2, A, static_cast<const RedArgs<float>*>(args_host), nb, nc_host, coop_ctas, true);
-  return e != cudaSuccess ? e : cudaGetLastError();
-}
-
-cudaError_t reduced_solve_b(cudaStream_t s, const void* args_dev, const void* args_host, int nb,
-                            const int* nc_host, int num_sms, int coop_ctas) {
-  const auto* A = static_cast<const RedArgs<float>*>(args_dev);
   const auto* H = static_cast<const RedArgs<float>*>(args_host);
   bool any_small = false, any_clus = false;
   for (int f = 0; f < nb; ++f) {
@@ -2314,31 +2308,53 @@ cudaError_t reduced_solve_b(cudaStream_t s, const void* args_dev, const void* ar
     any_small |= nc_host[f] > 0 && nc_host[f] <= H[f].one_cta_max;
     any_clus |= nc_host[f] > H[f].one_cta_max && nc_host[f] <= kClusNc;
   }
-  ProfScope ps(PROF_CHOL, s);
-  k_small_x_b<1><<<dim3(std::max(1, 2 * num_sms / nb), nb), 256, 0, s>>>(A);
-  count_launch();
-  if (any_small) {
-    k_small_v_b<<<dim3(1, nb), kST, kSmallSmemV, s>>>(A);
+  ProfScope ps(PROF_CHOL, s2);
+  cudaError_t e = cudaSuccess;
+  if (any_small || any_clus) {
+    k_small_s_b<<<dim3(1, nb), kST, kSmallSmemS, s2>>>(A);
+    k_small_x_b<<<dim3((3 * kClusNc + kXRows - 1) / kXRows, nb), 256, 0, s2>>>(A);
+    k_small_n_b<<<dim3(kNTiles, nb), 256, 0, s2>>>(A);
+    count_launch(3);
+    if (any_small) {
+      k_small_v_b<<<dim3(1, nb), kST, kSmallSmemV, s2>>>(A);
+      count_launch();
+    }
+    if (any_clus) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(kCl, nb);
+      cfg.blockDim = dim3(kST);
+      cfg.dynamicSmemBytes = kClusSmem;
+      cfg.stream = s2;
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = kCl;
+      at[0].val.clusterDim.y = 1;
+      at[0].val.clusterDim.z = 1;
+      cfg.attrs = at;
+      cfg.numAttrs = 1;
+      e = cudaLaunchKernelEx(&cfg, k_clus_v_b, A);
+      count_launch();
+      if (e != cudaSuccess) return e;
+    }
+    k_small_u_b<<<dim3(kUCtas, nb), kRT, kSmallSmemU, s2>>>(A);
     count_launch();
-  }
-  if (any_clus) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(kCl, nb);
-    cfg.blockDim = dim3(kST);
-    cfg.dynamicSmemBytes = kClusSmem;
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = kCl;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_clus_v_b, A);
-    count_launch();
-    if (e != cudaSuccess) return e;
   }
   // n_c beyond the cluster path: the grid form, all such frames side by side
+  e = launch_grid_b(s2, A, H, nb, nc_host, coop_ctas, true);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+cudaError_t reduced_solve_b(cudaStream_t s, const void* args_dev, const void* args_host, int nb,
+                            const int* nc_host, int coop_ctas) {
+  const auto* A = static_cast<const RedArgs<float>*>(args_dev);
+  const auto* H = static_cast<const RedArgs<float>*>(args_host);
+  bool any = false;
+  for (int f = 0; f < nb; ++f) any |= H[f].active && nc_host[f] > 0 && nc_host[f] <= kClusNc;
+  ProfScope ps(PROF_CHOL, s);
+  if (any) {
+    const cudaError_t e = launch_solve_clusters(s, k_small_solve_b, nb, A);
+    if (e != cudaSuccess) return e;
+  }
   const cudaError_t eg = launch_grid_b(s, A, H, nb, nc_host, coop_ctas, false);
   if (eg != cudaSuccess) return eg;
   // float64 row products, one row per lane: 256 rows per CTA of 8 warps,
@@ -2378,16 +2394,8 @@ cudaError_t reduced_prepare(cudaStream_t s, const DevMesh& m, const double* u, c
     e = launch_grid(s2, make_args<double>(m, u, (const double*)y2, z2, info, 1), num_sms, true);
   } else {
     const RedArgs<float> a = make_args<float>(m, u, (const float*)y2, z2, info, kMixedRefineSteps);
-    if (nc_host > kClusNc) {
-      e = launch_grid(s2, a, num_sms, true);
-    } else {
-      ProfScope ps(PROF_CHOL, s2);
-      k_small_s<<<1, kST, kSmallSmemS, s2>>>(a);
-      k_small_x<2><<<2 * std::max(1, num_sms), 256, 0, s2>>>(a);
-      k_small_n<<<kNTiles, 256, 0, s2>>>(a);
-      count_launch(3);
-      e = cudaGetLastError();
-    }
+    e = nc_host > kClusNc ? launch_grid(s2, a, num_sms, true)
+                          : launch_small_prepare(s2, a, num_sms, nc_host);
   }
   // the join is recorded even if a launch failed, so the fork always closes
   const cudaError_t ej = cudaEventRecord(m.ev_join, s2);
@@ -2404,6 +2412,8 @@ void set_reduced_smem_limits() {
   cudaFuncSetAttribute(k_small_s_b, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallSmemS);
   cudaFuncSetAttribute(k_small_v_b, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallSmemV);
   cudaFuncSetAttribute(k_clus_v_b, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClusSmem);
+  cudaFuncSetAttribute(k_small_u, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallSmemU);
+  cudaFuncSetAttribute(k_small_u_b, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallSmemU);
 }
 FSIM_CHECK_READER(check_word_reduced)
 

@@ -623,7 +623,7 @@ cudaError_t global_step_t(cudaStream_t s, const DevMesh& m, const double* g, dou
         k_convert<float, double><<<nblk(3 * (int64_t)n2, 256), 256, 0, s>>>(3 * n2, m.uf, u);
         count_launch(2);
       }
-      cudaStream_t s2 = m.aux_stream;
+      cudaStream_t s2 = m.aux_stream2;
       if (cudaEventRecord(m.ev_fork2, s) != cudaSuccess || cudaStreamWaitEvent(s2, m.ev_fork2, 0) != cudaSuccess)
         return cudaGetLastError();
       k_convert<float, float><<<nblk(3 * (int64_t)n2, 256), 256, 0, s2>>>(3 * n2, m.uf, m.bx + 3 * (size_t)n1);
@@ -687,14 +687,15 @@ cudaError_t global_step_t(cudaStream_t s, const DevMesh& m, const double* g, dou
 
 cudaError_t global_step_b(const BatchStep& bs) {
   const DevMesh& m = *bs.m0;
-  cudaStream_t s = bs.s, s2 = bs.s2;
+  cudaStream_t s = bs.s, s2 = bs.s2, s3 = bs.s3;
   const int nb = bs.nb, nr = bs.nr, n1 = m.n1, n2 = m.n2, nf = m.nf;
   const int chunks = nr / kMrCols;
   k_gather_rhs_mr<<<dim3((nf + 255) / 256, nb), 256, 0, s>>>(bs.tab, bs.rb, nr);
   count_launch();
   // S, L_s, block lists, X, N of every frame need only B-check and Sigma^-1:
   // on the side stream, overlapping the forward solve
-  if (cudaEventRecord(bs.ev[0], s) != cudaSuccess || cudaStreamWaitEvent(s2, bs.ev[0], 0) != cudaSuccess)
+  if (cudaEventRecord(bs.ev[0], s) != cudaSuccess || cudaStreamWaitEvent(s2, bs.ev[0], 0) != cudaSuccess ||
+      cudaStreamWaitEvent(s3, bs.ev[0], 0) != cudaSuccess)
     return cudaGetLastError();
   cudaError_t e = reduced_prepare_b(s2, bs.args_dev, bs.args_host, nb, bs.nc_host, bs.coop_ctas);
   if (e != cudaSuccess) return e;
@@ -729,26 +730,26 @@ cudaError_t global_step_b(const BatchStep& bs) {
     if (e != cudaSuccess) return e;
   }
   // the contact-free backward solve x1 = L1^-T (y1 - L21^T u) on the side
-  // stream while the reduced systems are solved
+  // stream s3 while the reduced systems are factored (s2) and solved (s)
   // x1 rows of the backward solution accumulate atomically: zeroed first
-  if (n1 > 0 && cudaMemsetAsync(bs.bx, 0, sizeof(float) * (size_t)n1 * nr, s2) != cudaSuccess)
+  if (n1 > 0 && cudaMemsetAsync(bs.bx, 0, sizeof(float) * (size_t)n1 * nr, s3) != cudaSuccess)
     return cudaGetLastError();
-  if (cudaEventRecord(bs.ev[2], s) != cudaSuccess || cudaStreamWaitEvent(s2, bs.ev[2], 0) != cudaSuccess)
+  if (cudaEventRecord(bs.ev[2], s) != cudaSuccess || cudaStreamWaitEvent(s3, bs.ev[2], 0) != cudaSuccess)
     return cudaGetLastError();
   for (int l = m.n_levels - 1; l >= 0 && n1 > 0; --l) {
     const int a = m.h_bwd32_ptr[l], z = m.h_bwd32_ptr[l + 1];
     if (z <= a) continue;
-    ProfScope ps(PROF_TRSV_BWD, s2);
-    k_bwd_mr<<<dim3(z - a, chunks), 256, 0, s2>>>(m.bwd_items32 + a, m.sn_c0, m.sn_ns, m.sn_nr1,
+    ProfScope ps(PROF_TRSV_BWD, s3);
+    k_bwd_mr<<<dim3(z - a, chunks), 256, 0, s3>>>(m.bwd_items32 + a, m.sn_c0, m.sn_ns, m.sn_nr1,
                                                   m.sn_roff, m.sn_zoff, m.sn_rows, m.Zf, bs.yb,
                                                   bs.bx, nr, nf);
     count_launch();
   }
-  if (cudaEventRecord(bs.ev[3], s2) != cudaSuccess) return cudaGetLastError();
+  if (cudaEventRecord(bs.ev[3], s3) != cudaSuccess) return cudaGetLastError();
   if (cudaStreamWaitEvent(s, bs.ev[1], 0) != cudaSuccess) return cudaGetLastError();
   {
     ProfScope ps(PROF_REDUCED, s);
-    e = reduced_solve_b(s, bs.args_dev, bs.args_host, nb, bs.nc_host, bs.num_sms, bs.coop_ctas);
+    e = reduced_solve_b(s, bs.args_dev, bs.args_host, nb, bs.nc_host, bs.coop_ctas);
     if (e != cudaSuccess) return e;
   }
   if (cudaStreamWaitEvent(s, bs.ev[3], 0) != cudaSuccess) return cudaGetLastError();

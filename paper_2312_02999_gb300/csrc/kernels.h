@@ -136,6 +136,9 @@ struct DevMesh {
   // reduced system that does not need the right-hand side runs there while
   // the forward solve runs on the solve's own stream
   cudaStream_t aux_stream = nullptr;
+  // second side stream: the contact-free backward solve, beside the end of the
+  // reduced system's factorisation (aux_stream) and its solve
+  cudaStream_t aux_stream2 = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   cudaEvent_t ev_fork2 = nullptr, ev_join2 = nullptr;
   // Phi = K11^-1 K12 Sigma^-1 (n1 x n2, float, stored transposed: row j of
@@ -283,7 +286,7 @@ void launch_axpy_b(cudaStream_t s, const DevMesh* tab, int nb, const DevMesh& m0
 // systems of all frames in batched launches (k_reduced.cu), then
 // x1 = bx1 + Phi[:, c] v and dx per frame.
 struct BatchStep {
-  cudaStream_t s = nullptr, s2 = nullptr;   // main and side stream
+  cudaStream_t s = nullptr, s2 = nullptr, s3 = nullptr;   // main and side stream
   cudaEvent_t ev[4] = {};                   // fork / join events
   const DevMesh* tab = nullptr;             // device table (nb frames)
   const DevMesh* m0 = nullptr;              // host copy of one frame (mesh constants)
@@ -320,7 +323,7 @@ void reduced_args_fill(void* dst, const DevMesh& m, int active);
 cudaError_t reduced_prepare_b(cudaStream_t s2, const void* args_dev, const void* args_host, int nb,
                               const int* nc_host, int coop_ctas);
 cudaError_t reduced_solve_b(cudaStream_t s, const void* args_dev, const void* args_host, int nb,
-                            const int* nc_host, int num_sms, int coop_ctas);
+                            const int* nc_host, int coop_ctas);
 cudaError_t phi_apply_b(cudaStream_t s, const void* args_dev, const int* cols_dev, int nb, int n1,
                         const float* phi_t, const float* bxm, int nr, double* const* x1s_dev);
 
