@@ -347,7 +347,6 @@ class Batch {
   int evaluate(const std::vector<char>& want, int at) {
     BTRY(upload_table(want));
     const DevMesh& m0 = tab_[0];
-    launch_eval_reset_b(s_, tab_dev_, cap_);
     if (at) launch_axpy_b(s_, tab_dev_, cap_, m0);
     launch_local_b(s_, tab_dev_, cap_, m0, at);
     launch_proxy_b(s_, tab_dev_, cap_, m0, at);
@@ -379,7 +378,7 @@ class Batch {
       if (nc > cap_now) {          // buffers grew: assemble B-check again (one frame)
         BCK(cudaMemsetAsync(m.Bc, 0, sizeof(double) * 9 * (size_t)nc * nc, s_));
         BCK(cudaMemsetAsync(m.bocc, 0, sizeof(int) * (size_t)nc * nc, s_));
-        launch_barrier_scatter(s_, m, fr.npairs, m.nc_cap, 2, m.g);
+        launch_barrier_scatter(s_, m, m.nc_cap, 2, m.g);
       }
       fr.nc = nc;
       fr.gn = std::sqrt(scl(f)[3]);
@@ -439,8 +438,7 @@ class Batch {
     BCK(cudaMemsetAsync(m.counters + 6, 0, sizeof(int) * 2, s_));
     BCK(global_step(s_, m, m.g, m.dx, FSIM_FP64, m.counters + 6, coop_ctas_, false, false,
                     frames_[f].nc));
-    launch_proxy(s_, m, m.dx, m.ds);
-    launch_ccd_reset(s_, m);
+    launch_proxy(s_, m, m.dx, m.ds, RESET_CCD);
     launch_ccd(s_, m, m.s, m.ds, p.dhat, p.ccd_s, p.accd_max_iters);
     BCK(cudaGetLastError());
     return FSIM_OK;

@@ -98,10 +98,10 @@ Exec ctx_exec(fsim_ctx_t ctx, MeshState& ms) {
   return ex;
 }
 
+// The scalars and the counters lie one after the other on the device and in the
+// pinned words (kStatusBytes): one copy reads both back.
 int sync_read(const Exec& ex, const DevMesh& m) {
-  CK(cudaMemcpyAsync(ex.h_counters, m.counters, sizeof(int) * kCounters, cudaMemcpyDeviceToHost,
-                     ex.stream));
-  CK(cudaMemcpyAsync(ex.h_scal, m.scal, sizeof(double) * kScal, cudaMemcpyDeviceToHost, ex.stream));
+  CK(cudaMemcpyAsync(ex.h_scal, m.scal, kStatusBytes, cudaMemcpyDeviceToHost, ex.stream));
   CK(cudaStreamSynchronize(ex.stream));
   return FSIM_OK;
 }
@@ -183,9 +183,13 @@ int alloc_workspace(const MeshState& ms, DevMesh& m, std::vector<void*>& al, siz
   TRY(dalloc(al, &m.pkey, 12 * np, bytes));
   TRY(dalloc(al, &m.sf, 3 * Ns, bytes));
   TRY(dalloc(al, &m.dsf, 3 * Ns, bytes));
-  TRY(dalloc(al, &m.counters, kCounters, bytes));
-  CK(cudaMemset(m.counters, 0, sizeof(int) * kCounters));   // skin list starts invalid
-  TRY(dalloc(al, &m.scal, kScal, bytes));
+  {   // scalars, then counters (read back by one copy)
+    char* status = nullptr;
+    TRY(dalloc(al, &status, kStatusBytes, bytes));
+    CK(cudaMemset(status, 0, kStatusBytes));                 // skin list starts invalid
+    m.scal = reinterpret_cast<double*>(status);
+    m.counters = reinterpret_cast<int*>(status + sizeof(double) * kScal);
+  }
   TRY(dalloc(al, &m.partials, (size_t)m.n_partials, bytes));
   TRY(dalloc(al, &m.y1, 3 * (size_t)std::max(m.n1, 1), bytes));
   TRY(dalloc(al, &m.y1f, 3 * (size_t)std::max(m.n1, 1), bytes));
@@ -214,7 +218,8 @@ int alloc_workspace(const MeshState& ms, DevMesh& m, std::vector<void*>& al, siz
     TRY(dalloc(al, &m.sh_r, N, bytes));
     TRY(dalloc(al, &m.sh_df, N, bytes));
   }
-  TRY(dalloc(al, &m.sb, 3 * Ns, bytes));
+  TRY(dalloc(al, &m.sb, 3 * Ns + 3, bytes));
+  CK(cudaMemset(m.sb + 3 * Ns, 0, sizeof(double) * 3));      // words of k_skin_check
   TRY(dalloc(al, &m.pair_grad, 12 * (size_t)m.cap_act, bytes));
   TRY(dalloc(al, &m.pair_hess, 144 * (size_t)m.cap_act, bytes));
   TRY(dalloc(al, &m.x2mark, (size_t)std::max(m.n2, 1), bytes));
@@ -293,9 +298,13 @@ int with_graph(const Exec& ex, DevMesh& m, int slot, const void* key, int key2, 
   return FSIM_OK;
 }
 
-// graph slots: 0-5 global step (by precision and reduced-system path), 6-9
-// evaluation (by position buffer and precision), 10-11 CCD (by proxy-position
-// buffer)
+// graph slots: global step (by precision and reduced-system path), evaluation
+// (by position buffer and precision), CCD and first trial (by proxy-position
+// buffer and precision), gradient (by force buffer and precisions)
+enum { kGraphStep = 0, kGraphEval = 6, kGraphTrial = 10, kGraphGrad = 14 };
+static_assert(kGraphGrad + 4 == DevMesh::kGraphs, "graph slots");
+// more than the doublings of kappa in a frame (up to kKappaMaxRatio)
+constexpr int kKappaGens = 16;
 int graph_slot(const DevMesh& m, int first, int count, const void* key, int key2) {
   for (int k = first; k < first + count; ++k)
     if (m.graphs[k].exec && m.graphs[k].key == key && m.graphs[k].key2 == key2) return k;
@@ -315,15 +324,11 @@ int graph_slot(const DevMesh& m, int first, int count, const void* key, int key2
 int evaluate(const Exec& ex, const MeshState& ms, const DevMesh& m, const double* xb, double* sb,
              double* tetf, double* proj, int prec, double kappa) {
   cudaStream_t s = ex.stream;
-  CK(cudaMemsetAsync(m.counters, 0, sizeof(int) * 3, s));       // |C|, candidates, overflow
-  CK(cudaMemsetAsync(m.counters + 5, 0, sizeof(int), s));       // touching pair
-  CK(cudaMemsetAsync(m.counters + 8, 0, sizeof(int), s));       // near-pair list
-  CK(cudaMemsetAsync(m.scal, 0, sizeof(double) * 1, s));
   if (tetf) {
     launch_elastic(s, m, xb, tetf, proj, m.partials, prec);
     launch_sum_partials(s, m.partials, elastic_blocks(m.T), m.scal + 2);
   }
-  launch_proxy(s, m, xb, sb);
+  launch_proxy(s, m, xb, sb, RESET_EVAL);
   launch_detect(s, m, sb, ms.p.dhat, kappa);
   CK(cudaGetLastError());
   return FSIM_OK;
@@ -331,34 +336,51 @@ int evaluate(const Exec& ex, const MeshState& ms, const DevMesh& m, const double
 
 // Gradient g-hat (elastic from tetf, zero if NULL, + barrier over the pairs in
 // m.pairs at sb) into gout, the contact-affected set, B-check and ||g||^2.
-// Requires counters[0] (|C|) already on the host in npairs.
+// The pairs are those of the last evaluation (counters[0]).
 // bprec is the precision of the pairs' PSD eigen-solves (prec unless the
-// frame switched its contact Hessian to float64).
-int gradient_and_hessian(const Exec& ex, const MeshState& ms, DevMesh& m, const double* sb,
-                         const double* tetf, double* gout, int64_t npairs, int prec, int* nc_out,
-                         double* gn2_out, double kappa, int bprec = -1) {
+// frame switched its contact Hessian to float64).  graph: replay the launches
+// as a graph (a solve's own buffers; kgen numbers its values of kappa).
+int gradient_launches(const Exec& ex, const MeshState& ms, DevMesh& m, const double* sb,
+                      const double* tetf, double* gout, int prec, double kappa, int bprec,
+                      int cap_now) {
   cudaStream_t s = ex.stream;
   if (tetf) launch_gather_forces(s, m, tetf, gout, prec);
   else CK(cudaMemsetAsync(gout, 0, sizeof(double) * 3 * (size_t)m.n, s));
   CK(cudaMemsetAsync(m.x2mark, 0, sizeof(int) * std::max(m.n2, 1), s));
-  launch_barrier_pairs(s, m, npairs, sb, ms.p.dhat, kappa, bprec < 0 ? prec : bprec);
+  launch_barrier_pairs(s, m, sb, ms.p.dhat, kappa, bprec);
   if (m.n2 > 0) launch_mark_scan(s, m);
   else CK(cudaMemsetAsync(m.counters + 3, 0, sizeof(int), s));
-  // n_c stays on the device until the one read-back below: B-check is zeroed
-  // and assembled in place when it fits the current reduced buffers
-  const int cap_now = m.Bc != nullptr ? m.nc_cap : 0;
+  // n_c stays on the device until the one read-back after this: B-check is
+  // zeroed and assembled in place when it fits the current reduced buffers
   launch_zero_reduced(s, m, cap_now);
-  launch_barrier_scatter(s, m, npairs, cap_now, 3, gout);
+  launch_barrier_scatter(s, m, cap_now, 3, gout);
   const int nb = gnorm_blocks(m.n);
   launch_gnorm2(s, m, gout, m.partials, nb);
   launch_sum_partials(s, m.partials, nb, m.scal + 3);
+  CK(cudaGetLastError());
+  return FSIM_OK;
+}
+
+int gradient_and_hessian(const Exec& ex, const MeshState& ms, DevMesh& m, const double* sb,
+                         const double* tetf, double* gout, int prec, int* nc_out, double* gn2_out,
+                         double kappa, int bprec, bool graph = false, int kgen = 0) {
+  cudaStream_t s = ex.stream;
+  const int cap_now = m.Bc != nullptr ? m.nc_cap : 0;
+  auto body = [&] { return gradient_launches(ex, ms, m, sb, tetf, gout, prec, kappa, bprec, cap_now); };
+  if (graph) {
+    const int key2 = 2 * prec + bprec;
+    TRY(with_graph(ex, m, graph_slot(m, kGraphGrad, 4, tetf, key2), tetf, key2,
+                   kgen + kKappaGens * m.red_gen, body));
+  } else {
+    TRY(body());
+  }
   TRY(sync_read(ex, m));
   const int nc = ex.h_counters[3];
   TRY(ensure_reduced(ex, m, std::max(nc, 1)));
   if (nc > cap_now) {       // the buffers grew: assemble B-check again
     CK(cudaMemsetAsync(m.Bc, 0, sizeof(double) * 9 * (size_t)nc * nc, s));
     CK(cudaMemsetAsync(m.bocc, 0, sizeof(int) * (size_t)nc * nc, s));
-    launch_barrier_scatter(s, m, npairs, m.nc_cap, 2, gout);
+    launch_barrier_scatter(s, m, m.nc_cap, 2, gout);
   }
   *nc_out = nc;
   *gn2_out = ex.h_scal[3];
@@ -400,7 +422,7 @@ int solve_frame_impl(const Exec& ex, const MeshState& ms, DevMesh& m, const doub
     d_prev = d_min;
   };
   auto eval_at = [&](double* xb, double* sb, double* tetf) -> int {
-    const int slot = graph_slot(m, 6, 4, xb, prec);
+    const int slot = graph_slot(m, kGraphEval, 4, xb, prec);
     return with_graph(ex, m, slot, xb, prec, kgen,
                       [&] { return evaluate(ex, ms, m, xb, sb, tetf, nullptr, prec, kappa); });
   };
@@ -418,7 +440,7 @@ int solve_frame_impl(const Exec& ex, const MeshState& ms, DevMesh& m, const doub
   int nc = 0;
   if (rc == FSIM_OK) {
     double gn2;
-    TRY(gradient_and_hessian(ex, ms, m, m.s, m.tetf, m.g, npairs, prec, &nc, &gn2, kappa));
+    TRY(gradient_and_hessian(ex, ms, m, m.s, m.tetf, m.g, prec, &nc, &gn2, kappa, prec, true, kgen));
     gn = std::sqrt(gn2);
     st.grad_norm0 = gn;
     tol = std::max(p.tol_abs, p.tol_rel * gn);
@@ -451,7 +473,7 @@ int solve_frame_impl(const Exec& ex, const MeshState& ms, DevMesh& m, const doub
       const int gkey = 8 * gprec + (schur ? 4 : gprec == FSIM_FP64 && nc == 0
                                                     ? 5
                                                     : reduced_path(nc, gprec, m.one_cta_max));
-      TRY(with_graph(ex, m, graph_slot(m, 0, 6, m.g, gkey), m.g, gkey, m.red_gen, [&]() -> int {
+      TRY(with_graph(ex, m, graph_slot(m, kGraphStep, 6, m.g, gkey), m.g, gkey, m.red_gen, [&]() -> int {
         CK(cudaMemsetAsync(m.counters + 6, 0, sizeof(int) * 2, s));
         CK(global_step(s, m, m.g, m.dx, gprec, m.counters + 6, ex.coop_ctas, ex.alone, schur, nc));
         return FSIM_OK;
@@ -460,22 +482,29 @@ int solve_frame_impl(const Exec& ex, const MeshState& ms, DevMesh& m, const doub
     }
     st.sum_nc3 += (double)nc * nc * nc;
     if (p.solver == FSIM_SOLVER_WOODBURY) st.reduced_steps[reduced_path(nc, gprec, m.one_cta_max)]++;
-    // CCD step bound; the ACCD kernel reads the candidate count on the device,
-    // and the overflow / factorisation flags are checked at the next read-back
-    TRY(with_graph(ex, m, graph_slot(m, 10, 2, m.s, 0), m.s, 0, 0, [&]() -> int {
-      launch_proxy(s, m, m.dx, m.ds);
-      launch_ccd_reset(s, m);
+    // CCD step bound and the first trial (scale 1), evaluated, as one sequence;
+    // the ACCD kernel reads the candidate count on the device, and the overflow
+    // / factorisation flags are checked at the next read-back
+    auto ccd_bound = [&]() -> int {
+      launch_proxy(s, m, m.dx, m.ds, RESET_CCD);
       launch_ccd(s, m, m.s, m.ds, p.dhat, p.ccd_s, p.accd_max_iters);
       CK(cudaGetLastError());
       return FSIM_OK;
+    };
+    TRY(with_graph(ex, m, graph_slot(m, kGraphTrial, 4, m.s, prec), m.s, prec, kgen, [&]() -> int {
+      TRY(ccd_bound());
+      launch_axpy_positions(s, 3 * m.n, m.x, m.dx, m.scal + 1, 1.0, m.xt);
+      return evaluate(ex, ms, m, m.xt, m.st, m.tetf_t, nullptr, prec, kappa);
     }));
     // backtracking line search from alpha_m on E-hat = E + B
     bool accepted = false, redone = false;
     double scale = 1.0, Et = 0.0;
     int64_t np_t = 0;
     for (int k = 0; k <= p.max_ls; ++k) {
-      launch_axpy_positions(s, 3 * m.n, m.x, m.dx, m.scal + 1, scale, m.xt);
-      TRY(eval_at(m.xt, m.st, m.tetf_t));
+      if (k > 0 || redone) {
+        launch_axpy_positions(s, 3 * m.n, m.x, m.dx, m.scal + 1, scale, m.xt);
+        TRY(eval_at(m.xt, m.st, m.tetf_t));
+      }
       TRY(sync_read(ex, m));
       if (k == 0 && ex.h_counters[6] && gprec != FSIM_FP64 && p.solver != FSIM_SOLVER_PCG &&
           !redone) {
@@ -495,16 +524,13 @@ int solve_frame_impl(const Exec& ex, const MeshState& ms, DevMesh& m, const doub
         TRY(sync_read(ex, m));
         {
           double gn2r;
-          TRY(gradient_and_hessian(ex, ms, m, m.s, m.tetf, m.g, npairs, prec, &nc, &gn2r, kappa,
-                                   gprec));
+          TRY(gradient_and_hessian(ex, ms, m, m.s, m.tetf, m.g, prec, &nc, &gn2r, kappa, gprec, true,
+                                   kgen));
         }
         CK(cudaMemsetAsync(m.counters + 6, 0, sizeof(int) * 2, s));
         CK(global_step(s, m, m.g, m.dx, FSIM_FP64, m.counters + 6, ex.coop_ctas, ex.alone,
                        p.solver == FSIM_SOLVER_SCHUR, nc));
-        launch_proxy(s, m, m.dx, m.ds);
-        launch_ccd_reset(s, m);
-        launch_ccd(s, m, m.s, m.ds, p.dhat, p.ccd_s, p.accd_max_iters);
-        CK(cudaGetLastError());
+        TRY(ccd_bound());
         scale = 1.0;
         k = -1;
         continue;
@@ -535,7 +561,7 @@ int solve_frame_impl(const Exec& ex, const MeshState& ms, DevMesh& m, const doub
     npairs = np_t;
     st.iterations++;
     double gn2;
-    TRY(gradient_and_hessian(ex, ms, m, m.s, m.tetf, m.g, npairs, prec, &nc, &gn2, kappa, gprec));
+    TRY(gradient_and_hessian(ex, ms, m, m.s, m.tetf, m.g, prec, &nc, &gn2, kappa, gprec, true, kgen));
     gn = std::sqrt(gn2);
     if (!std::isfinite(gn)) rc = FSIM_ENONFINITE;
   }
@@ -616,12 +642,12 @@ fsim_status fsim_create(fsim_ctx_t* out, int device) {
     delete c;
     return FSIM_ECUDA;
   }
-  if (cudaHostAlloc((void**)&c->h_counters, sizeof(int) * kCounters, cudaHostAllocDefault) != cudaSuccess ||
-      cudaHostAlloc((void**)&c->h_scal, sizeof(double) * kScal, cudaHostAllocDefault) != cudaSuccess) {
+  if (cudaHostAlloc((void**)&c->h_scal, kStatusBytes, cudaHostAllocDefault) != cudaSuccess) {
     cudaStreamDestroy(c->stream);
     delete c;
     return FSIM_ENOMEM;
   }
+  c->h_counters = reinterpret_cast<int*>(c->h_scal + kScal);
   set_solver_smem_limits(200 * 1024);
   set_reduced_smem_limits();
   set_schur_smem_limits();
@@ -635,7 +661,6 @@ fsim_status fsim_destroy(fsim_ctx_t ctx) {
   cudaStreamSynchronize(ctx->stream);
   for (auto& m : ctx->meshes)
     if (m) free_mesh(*m);
-  cudaFreeHost(ctx->h_counters);
   cudaFreeHost(ctx->h_scal);
   cudaStreamDestroy(ctx->stream);
   delete ctx;
@@ -1116,7 +1141,7 @@ fsim_status fsim_eval_proxy(fsim_ctx_t ctx, int mesh_id, const double* x, double
   cudaSetDevice(ctx->device);
   DevMesh& m = ms->d;
   TRY(stage_x(ctx, *ms, x));
-  launch_proxy(ctx->stream, m, m.xt, m.st);
+  launch_proxy(ctx->stream, m, m.xt, m.st, RESET_NONE);
   CK(cudaMemcpyAsync(s_out, m.st, sizeof(double) * 3 * (size_t)m.Ns, cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
   return FSIM_OK;
@@ -1151,11 +1176,10 @@ fsim_status fsim_eval_barrier(fsim_ctx_t ctx, int mesh_id, const double* x, doub
   TRY(evaluate(ex, *ms, m, m.xt, m.st, nullptr, nullptr, 0, ms->kappa));
   TRY(sync_read(ex, m));
   if (ctx->h_counters[2]) return FSIM_ECONTACT_OVERFLOW;
-  const int64_t np = ctx->h_counters[0];
   // barrier gradient only: no elastic forces
   int nc = 0;
   double gn2 = 0.0;
-  TRY(gradient_and_hessian(ex, *ms, m, m.st, nullptr, ms->gtmp, np, 0, &nc, &gn2, ms->kappa));
+  TRY(gradient_and_hessian(ex, *ms, m, m.st, nullptr, ms->gtmp, 0, &nc, &gn2, ms->kappa, 0));
   if (n_c) *n_c = nc;
   if (grad_out)
     CK(cudaMemcpy(grad_out, ms->gtmp, sizeof(double) * 3 * (size_t)m.n, cudaMemcpyDeviceToHost));
@@ -1241,10 +1265,9 @@ fsim_status fsim_eval_global_step(fsim_ctx_t ctx, int mesh_id, const double* x, 
   TRY(evaluate(ex, *ms, m, m.xt, m.st, m.tetf_t, nullptr, precision, ms->kappa));
   TRY(sync_read(ex, m));
   if (ctx->h_counters[2]) return FSIM_ECONTACT_OVERFLOW;
-  const int64_t np = ctx->h_counters[0];
   int nc = 0;
   double gn2 = 0.0;
-  TRY(gradient_and_hessian(ex, *ms, m, m.st, m.tetf_t, ms->gtmp, np, precision, &nc, &gn2, ms->kappa));
+  TRY(gradient_and_hessian(ex, *ms, m, m.st, m.tetf_t, ms->gtmp, precision, &nc, &gn2, ms->kappa, precision));
   CK(cudaMemsetAsync(m.counters + 6, 0, sizeof(int) * 2, s));
   if (ms->p.solver == FSIM_SOLVER_PCG) {
     int cg_it = 0;
@@ -1274,9 +1297,8 @@ fsim_status fsim_eval_ccd(fsim_ctx_t ctx, int mesh_id, const double* x, const do
   cudaStream_t s = ctx->stream;
   TRY(stage_x(ctx, *ms, x));
   CK(cudaMemcpyAsync(ms->dxtmp, dx, sizeof(double) * 3 * (size_t)m.n, cudaMemcpyHostToDevice, s));
-  launch_proxy(s, m, m.xt, m.st);
-  launch_proxy(s, m, ms->dxtmp, m.ds);
-  launch_ccd_reset(s, m);
+  launch_proxy(s, m, m.xt, m.st, RESET_NONE);
+  launch_proxy(s, m, ms->dxtmp, m.ds, RESET_CCD);
   launch_ccd(s, m, m.st, m.ds, ms->p.dhat, ms->p.ccd_s, ms->p.accd_max_iters);
   TRY(sync_read(ctx_exec(ctx, *ms), m));
   if (ctx->h_counters[9]) return FSIM_ECONTACT_OVERFLOW;
@@ -1297,10 +1319,9 @@ fsim_status fsim_eval_energy(fsim_ctx_t ctx, int mesh_id, const double* x, int p
   TRY(sync_read(ex, m));
   if (ctx->h_counters[2]) return FSIM_ECONTACT_OVERFLOW;
   const double E = ctx->h_scal[2] + ctx->h_scal[0];
-  const int64_t np = ctx->h_counters[0];
   int nc = 0;
   double gn2 = 0.0;
-  TRY(gradient_and_hessian(ex, *ms, m, m.st, m.tetf_t, ms->gtmp, np, 0, &nc, &gn2, ms->kappa));
+  TRY(gradient_and_hessian(ex, *ms, m, m.st, m.tetf_t, ms->gtmp, 0, &nc, &gn2, ms->kappa, 0));
   if (energy_out) *energy_out = E;
   if (grad_norm_out) *grad_norm_out = std::sqrt(gn2);
   return FSIM_OK;

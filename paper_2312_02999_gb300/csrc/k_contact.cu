@@ -40,10 +40,44 @@ __device__ __forceinline__ void k_proxy_body(int Ns, const int64_t* __restrict__
   }
   s[3 * (size_t)r] = a; s[3 * (size_t)r + 1] = b; s[3 * (size_t)r + 2] = c;
 }
+// The counters and scalars that the kernels after this one add to start from
+// here: RESET_EVAL: [0] |C|, [1] candidates, [2] overflow, [5] touching, [8] near
+// list, scal[0] (barrier energy); RESET_CCD: [1] candidates, [9] overflow,
+// scal[1] (step bound) = 1.  (A memset or a kernel of its own costs a launch.)
+__device__ __forceinline__ void reset_counters(int reset, int* counters, double* scal) {
+  if (reset == RESET_NONE || blockIdx.x != 0 || threadIdx.x != 0) return;
+  counters[1] = 0;
+  if (reset == RESET_EVAL) {
+    counters[0] = 0; counters[2] = 0; counters[5] = 0; counters[8] = 0;
+    scal[0] = 0.0;
+  } else {
+    counters[9] = 0;
+    scal[1] = 1.0;
+  }
+}
 __global__ void k_proxy(int Ns, const int64_t* __restrict__ Wptr, const int* __restrict__ Wcol,
                         const double* __restrict__ Wval, const double* __restrict__ x,
-                        double* __restrict__ s) {
+                        double* __restrict__ s, int reset, int* counters, double* scal) {
+  reset_counters(reset, counters, scal);
   k_proxy_body(Ns, Wptr, Wcol, Wval, x, s);
+}
+
+// How the pairs of a list (length n, read on the device) are spread over the
+// warps of a launch: each warp takes as few lanes' worth as the list allows.
+// A pair is a chain of some hundred float64 instructions that costs its warp
+// the same for one lane as for 32, and more where the lanes take different
+// branches, so a short list finishes sooner on many sparse warps than on a
+// few full ones.
+struct PairSpread {
+  int64_t first, stride;     // first pair of this lane (past the end: none), and its step
+};
+__device__ __forceinline__ PairSpread spread_pairs(int64_t n) {
+  const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
+  const int64_t w = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  int64_t per = (n + nw - 1) / nw;
+  per = per < 1 ? 1 : per > 32 ? 32 : per;
+  return {lane < per ? w * per + lane : n, nw * per};
 }
 
 // float64 box of a primitive (1 vertex, a triangle or an edge) over s and,
@@ -751,7 +785,7 @@ __global__ void k_mark_scan(int n2, int* __restrict__ x2mark, int* __restrict__ 
 // gradient into g.  n_c is read on the device; B-check is written only when
 // it fits the reduced buffers (n_c <= nc_cap), else the host grows them and
 // scatters the Hessian blocks again.  mode: 1 gradient, 2 B-check, 3 both.
-__device__ __forceinline__ void k_barrier_scatter_body(int64_t np, const unsigned long long* __restrict__ pairs,
+__device__ __forceinline__ void k_barrier_scatter_body(const int* __restrict__ count, int64_t cap, const unsigned long long* __restrict__ pairs,
                                   const int* __restrict__ tris, const int* __restrict__ edges,
                                   const int64_t* __restrict__ Wptr, const int* __restrict__ Wcol,
                                   const double* __restrict__ Wval, const int* __restrict__ x2of,
@@ -759,44 +793,47 @@ __device__ __forceinline__ void k_barrier_scatter_body(int64_t np, const unsigne
                                   const double* __restrict__ phess, const int* __restrict__ ncp,
                                   int nc_cap, int mode, double* __restrict__ g,
                                   double* __restrict__ Bc, int* __restrict__ bocc) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int64_t p = t >> 4;
-  if (p >= np) return;
-  const int a = (int)((t >> 2) & 3), b = (int)(t & 3);
+  int64_t np = *count;
+  np = np < cap ? np : cap;
   const int nc = *ncp;
-  const bool grad = (mode & 1) && b == 0;
-  const bool hess = (mode & 2) && nc <= nc_cap;
-  if (!grad && !hess) return;
-  int type, i, j;
-  unpack_key(pairs[p], type, i, j);
-  int V[4];
-  load_pair(type, i, j, tris, edges, V);
-  const int ld = 3 * nc;
-  for (int64_t ea = Wptr[V[a]]; ea < Wptr[V[a] + 1]; ++ea) {
-    const int va = Wcol[ea];
-    const int qa = x2of[va];
-    if (qa < 0) continue;                         // pinned: no DOF
-    const double wa = Wval[ea];
-    if (grad)
-      for (int d = 0; d < 3; ++d) atomicAdd(g + 3 * (size_t)va + d, wa * pgrad[p * 12 + 3 * a + d]);
-    if (!hess) continue;
-    const int ca = x2mark[qa] - 1;
-    if (ca < 0 || ca >= nc) continue;
-    for (int64_t eb = Wptr[V[b]]; eb < Wptr[V[b] + 1]; ++eb) {
-      const int qb = x2of[Wcol[eb]];
-      if (qb < 0) continue;
-      const int cb = x2mark[qb] - 1;
-      if (cb < 0 || cb >= nc) continue;
-      const double ww = wa * Wval[eb];
-      const double* h = phess + p * 144 + (a * 4 + b) * 9;
-      double* dst = Bc + (size_t)(3 * ca) * ld + 3 * cb;
-      for (int r = 0; r < 3; ++r)
-        for (int c = 0; c < 3; ++c) atomicAdd(dst + (size_t)r * ld + c, ww * h[3 * r + c]);
-      bocc[(size_t)ca * nc + cb] = 1;
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < 16 * np;
+       t += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t p = t >> 4;
+    const int a = (int)((t >> 2) & 3), b = (int)(t & 3);
+    const bool grad = (mode & 1) && b == 0;
+    const bool hess = (mode & 2) && nc <= nc_cap;
+    if (!grad && !hess) continue;
+    int type, i, j;
+    unpack_key(pairs[p], type, i, j);
+    int V[4];
+    load_pair(type, i, j, tris, edges, V);
+    const int ld = 3 * nc;
+    for (int64_t ea = Wptr[V[a]]; ea < Wptr[V[a] + 1]; ++ea) {
+      const int va = Wcol[ea];
+      const int qa = x2of[va];
+      if (qa < 0) continue;                         // pinned: no DOF
+      const double wa = Wval[ea];
+      if (grad)
+        for (int d = 0; d < 3; ++d) atomicAdd(g + 3 * (size_t)va + d, wa * pgrad[p * 12 + 3 * a + d]);
+      if (!hess) continue;
+      const int ca = x2mark[qa] - 1;
+      if (ca < 0 || ca >= nc) continue;
+      for (int64_t eb = Wptr[V[b]]; eb < Wptr[V[b] + 1]; ++eb) {
+        const int qb = x2of[Wcol[eb]];
+        if (qb < 0) continue;
+        const int cb = x2mark[qb] - 1;
+        if (cb < 0 || cb >= nc) continue;
+        const double ww = wa * Wval[eb];
+        const double* h = phess + p * 144 + (a * 4 + b) * 9;
+        double* dst = Bc + (size_t)(3 * ca) * ld + 3 * cb;
+        for (int r = 0; r < 3; ++r)
+          for (int c = 0; c < 3; ++c) atomicAdd(dst + (size_t)r * ld + c, ww * h[3 * r + c]);
+        bocc[(size_t)ca * nc + cb] = 1;
+      }
     }
   }
 }
-__global__ void k_barrier_scatter(int64_t np, const unsigned long long* __restrict__ pairs,
+__global__ void k_barrier_scatter(const int* __restrict__ count, int64_t cap, const unsigned long long* __restrict__ pairs,
                                   const int* __restrict__ tris, const int* __restrict__ edges,
                                   const int64_t* __restrict__ Wptr, const int* __restrict__ Wcol,
                                   const double* __restrict__ Wval, const int* __restrict__ x2of,
@@ -804,7 +841,7 @@ __global__ void k_barrier_scatter(int64_t np, const unsigned long long* __restri
                                   const double* __restrict__ phess, const int* __restrict__ ncp,
                                   int nc_cap, int mode, double* __restrict__ g,
                                   double* __restrict__ Bc, int* __restrict__ bocc) {
-  k_barrier_scatter_body(np, pairs, tris, edges, Wptr, Wcol, Wval, x2of, x2mark, pgrad, phess, ncp, nc_cap, mode, g, Bc, bocc);
+  k_barrier_scatter_body(count, cap, pairs, tris, edges, Wptr, Wcol, Wval, x2of, x2mark, pgrad, phess, ncp, nc_cap, mode, g, Bc, bocc);
 }
 
 // Zero the first (3 n_c)^2 entries of B-check and n_c^2 of its block
@@ -1150,8 +1187,8 @@ __device__ __forceinline__ void k_near_pairs_body(const int* __restrict__ near_c
   int64_t n = *near_count;
   n = n < cap ? n : cap;
   double esum = 0.0;
-  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n;
-       p += (int64_t)gridDim.x * blockDim.x) {
+  const PairSpread sp = spread_pairs(n);
+  for (int64_t p = sp.first; p < n; p += sp.stride) {
     int type, i, j;
     unpack_key(nearl[p], type, i, j);
     int V[4];
@@ -1196,8 +1233,8 @@ __device__ __forceinline__ void k_accd_list_body(const int* __restrict__ cand_co
                             double s_ratio, int max_iters, float slack, double* __restrict__ alpha) {
   int64_t n = *cand_count;
   n = n < cap ? n : cap;
-  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n;
-       p += (int64_t)gridDim.x * blockDim.x) {
+  const PairSpread sp = spread_pairs(n);
+  for (int64_t p = sp.first; p < n; p += sp.stride) {
     int type, i, j;
     unpack_key(cand[p], type, i, j);
     int V[4];
@@ -1248,28 +1285,42 @@ __global__ void k_accd_list(const int* __restrict__ cand_count, int64_t cap,
 // counters: [10] list length, [11] rebuild now, [12] list valid,
 // [13] CCD needs the full sweep, [14] list overflow.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ double block_max_d(double v) {
-  __shared__ double red[32];
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+// Maximum over the block of the bits of non-negative doubles (they order like
+// the values); valid in thread 0.  Integer instructions: a float64 maximum is a
+// compare and a select on the float64 pipe.
+__device__ __forceinline__ unsigned long long block_max_bits(unsigned long long v) {
+  __shared__ unsigned long long red[32];
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long w = __shfl_xor_sync(0xffffffffu, v, o);
+    v = w > v ? w : v;
+  }
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  __syncthreads();
   if (lane == 0) red[wid] = v;
   __syncthreads();
-  v = (threadIdx.x < (blockDim.x >> 5)) ? red[threadIdx.x] : 0.0;
-  if (wid == 0)
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;   // valid in thread 0
+  if (threadIdx.x == 0)
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) v = red[w] > v ? red[w] : v;
+  return v;
 }
 
-// one CTA: decide whether the skin list must be rebuilt (detection) or the
-// CCD step needs the full sweep (ds != nullptr); a rebuild records sb = s
+// Decide whether the skin list must be rebuilt (detection) or the CCD step
+// needs the full sweep (ds != nullptr); a rebuild records sb = s.  One vertex per
+// thread; the last CTA to finish (ticket) decides from the maxima of all.  (One
+// CTA for everything took 9 to 12 us on 1,444 vertices: its float64 work had
+// one SM.)  words: three 64-bit words after sb: the maxima of the squared lengths
+// and the ticket, zero between launches.
+constexpr int kSkinThreads = 128;
 __device__ __forceinline__ void k_skin_check_body(int Ns, const double* __restrict__ s, double* __restrict__ sb,
                              const double* __restrict__ ds, double skin, double margin,
                              int* counters, double* scal) {
-  if (ds == nullptr && threadIdx.x == 0) scal[4] = __longlong_as_double(0x7ff0000000000000LL);  // d_min = inf
-  // maxima of the squared lengths; one square root each at the end
-  // (sqrt is monotone and correctly rounded, so this is max |.| exactly)
-  double dmax = 0.0, smax = 0.0;
-  for (int v = threadIdx.x; v < Ns; v += blockDim.x) {
+  auto* words = reinterpret_cast<unsigned long long*>(sb + 3 * (size_t)Ns);
+  if (ds == nullptr && blockIdx.x == 0 && threadIdx.x == 0)
+    scal[4] = __longlong_as_double(0x7ff0000000000000LL);  // d_min = inf
+  // squared lengths; one square root each at the end (sqrt is monotone and
+  // correctly rounded, so this is max |.| exactly); NaN counts as 0
+  const int v = blockIdx.x * kSkinThreads + threadIdx.x;
+  unsigned long long dm = 0, sm = 0;
+  if (v < Ns) {
     double d2 = 0.0, q2 = 0.0;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
@@ -1277,29 +1328,40 @@ __device__ __forceinline__ void k_skin_check_body(int Ns, const double* __restri
       d2 += e * e;
       if (ds) q2 += ds[3 * v + d] * ds[3 * v + d];
     }
-    dmax = fmax(dmax, d2);
-    smax = fmax(smax, q2);
+    dm = (unsigned long long)__double_as_longlong(d2);
+    sm = (unsigned long long)__double_as_longlong(q2);
+    if (dm > 0x7ff0000000000000ULL) dm = 0;
+    if (sm > 0x7ff0000000000000ULL) sm = 0;
   }
-  dmax = sqrt(block_max_d(dmax));
-  __syncthreads();
-  smax = sqrt(block_max_d(smax));
-  __shared__ int rebuild;
+  dm = block_max_bits(dm);
+  if (ds) sm = block_max_bits(sm);
+  __shared__ int last, rebuild;
   if (threadIdx.x == 0) {
-    const bool valid = counters[12] == 1 && counters[14] == 0;
-    if (ds) {
-      counters[13] = (valid && 2.0 * (dmax + smax) <= 0.4 * skin) ? 0 : 1;
-      rebuild = 0;
-    } else {
-      rebuild = (valid && 2.0 * dmax <= skin - margin) ? 0 : 1;
-      counters[11] = rebuild;
-      if (rebuild) { counters[10] = 0; counters[12] = 1; counters[14] = 0; }
+    atomicMax(words, dm);
+    if (ds) atomicMax(words + 1, sm);
+    __threadfence();
+    last = atomicAdd(words + 2, 1ULL) == (unsigned long long)gridDim.x - 1 ? 1 : 0;
+    rebuild = 0;
+    if (last) {
+      __threadfence();
+      const double dmax = sqrt(__longlong_as_double((long long)atomicExch(words, 0ULL)));
+      const double smax = sqrt(__longlong_as_double((long long)atomicExch(words + 1, 0ULL)));
+      atomicExch(words + 2, 0ULL);
+      const bool valid = counters[12] == 1 && counters[14] == 0;
+      if (ds) {
+        counters[13] = (valid && 2.0 * (dmax + smax) <= 0.4 * skin) ? 0 : 1;
+      } else {
+        rebuild = (valid && 2.0 * dmax <= skin - margin) ? 0 : 1;
+        counters[11] = rebuild;
+        if (rebuild) { counters[10] = 0; counters[12] = 1; counters[14] = 0; }
+      }
     }
   }
   __syncthreads();
-  if (rebuild)
-    for (int e = threadIdx.x; e < 3 * Ns; e += blockDim.x) sb[e] = s[e];
+  if (rebuild)      // every other CTA has read sb
+    for (int e = threadIdx.x; e < 3 * Ns; e += kSkinThreads) sb[e] = s[e];
 }
-__global__ void k_skin_check(int Ns, const double* __restrict__ s, double* __restrict__ sb,
+__global__ void __launch_bounds__(kSkinThreads) k_skin_check(int Ns, const double* __restrict__ s, double* __restrict__ sb,
                              const double* __restrict__ ds, double skin, double margin,
                              int* counters, double* scal) {
   k_skin_check_body(Ns, s, sb, ds, skin, margin, counters, scal);
@@ -1355,13 +1417,15 @@ __global__ void k_skin_cand(int* counters, int64_t cap, const unsigned long long
 }
 
 // ---------------------------------------------------------------------------
-void launch_proxy(cudaStream_t st, const DevMesh& m, const double* x, double* sp) {
-  k_proxy<<<(m.Ns + 255) / 256, 256, 0, st>>>(m.Ns, m.Wptr, m.Wcol, m.Wval, x, sp);
+void launch_proxy(cudaStream_t st, const DevMesh& m, const double* x, double* sp, int reset) {
+  k_proxy<<<(m.Ns + 255) / 256, 256, 0, st>>>(m.Ns, m.Wptr, m.Wcol, m.Wval, x, sp, reset, m.counters,
+                                              m.scal);
   count_launch();
 }
 
 namespace {
 int nprim(const DevMesh& m) { return m.Ns + m.Nt + m.Ne; }
+int skin_ctas(const DevMesh& m) { return std::max(1, (m.Ns + kSkinThreads - 1) / kSkinThreads); }
 // float32 rounding allowance of the skin tests (as for the CCD early-out)
 double skin_margin(const DevMesh& m, double dhat) { return fmax(0.01 * dhat, 1e-5 * m.coord_scale); }
 
@@ -1396,7 +1460,7 @@ void launch_detect(cudaStream_t st, const DevMesh& m, const double* sp, double d
   const float margin = (float)skin_margin(m, dhat);
   k_prim_prep<<<(np + 255) / 256, 256, 0, st>>>(m.Ns, m.Nt, m.Ne, sp, nullptr, m.tris, m.edges, pad,
                                                 m.pbox, m.pkey, m.sf, nullptr);
-  k_skin_check<<<1, 512, 0, st>>>(m.Ns, sp, m.sb, nullptr, m.skin, margin, m.counters, m.scal);
+  k_skin_check<<<skin_ctas(m), kSkinThreads, 0, st>>>(m.Ns, sp, m.sb, nullptr, m.skin, margin, m.counters, m.scal);
   launch_sweeps(st, m, 0, m.vlist, m.counters + 10, m.counters + 14, (float)pad + margin,
                 m.counters + 11);
   k_skin_near<<<2 * 152, 128, 0, st>>>(m.counters, m.cap, m.vlist, m.sf, m.tris, m.edges,
@@ -1418,7 +1482,7 @@ void launch_ccd(cudaStream_t st, const DevMesh& m, const double* sp, const doubl
                                                 m.pbox, m.pkey, m.sf, m.dsf);
   // candidates from the skin list when it still covers the step, else the
   // full sweep
-  k_skin_check<<<1, 512, 0, st>>>(m.Ns, sp, m.sb, dsp, m.skin, 0.0, m.counters, m.scal);
+  k_skin_check<<<skin_ctas(m), kSkinThreads, 0, st>>>(m.Ns, sp, m.sb, dsp, m.skin, 0.0, m.counters, m.scal);
   k_skin_cand<<<2 * 152, 128, 0, st>>>(m.counters, m.cap, m.vlist, m.pkey, m.Ns, m.Nt, m.cand);
   launch_sweeps(st, m, 1, m.cand, m.counters + 1, m.counters + 9, 0.0f, m.counters + 13);
   count_launch(2);
@@ -1431,23 +1495,19 @@ void launch_ccd(cudaStream_t st, const DevMesh& m, const double* sp, const doubl
   count_launch(2);
 }
 
-void launch_barrier_pairs(cudaStream_t st, const DevMesh& m, int64_t np, const double* sp,
-                          double dhat, double kappa, int precision) {
-  np = np < m.cap_act ? np : m.cap_act;
-  if (np <= 0) return;
+// The kernels read |C| on the device and stride over it: fixed grids, so that
+// the sequence can be replayed as a graph.
+void launch_barrier_pairs(cudaStream_t st, const DevMesh& m, const double* sp, double dhat,
+                          double kappa, int precision) {
   ProfScope ps(PROF_BARRIER, st);
-  const int64_t want = (np + kPairWarps - 1) / kPairWarps;      // one warp per pair
-  const unsigned grid = (unsigned)(want < 8 * 152 ? want : 8 * 152);
-  const unsigned mgrid = grid;
+  const unsigned grid = (unsigned)std::min<int64_t>(m.cap_act, 8 * 152);
   if (m.barrier_lanes) {                                          // one lane per pair
-    const int64_t lw = (np + kPairLanes - 1) / kPairLanes;
-    const unsigned lgrid = (unsigned)(lw < 8 * 152 ? lw : 8 * 152);
     if (precision == 0)
-      k_barrier_pairs_lanes<double><<<lgrid, kPairLanes, 0, st>>>(
+      k_barrier_pairs_lanes<double><<<grid, kPairLanes, 0, st>>>(
           m.counters, m.cap_act, m.pairs, sp, m.tris, m.edges, m.Wptr, m.Wcol, m.x2of, dhat, kappa,
           m.pair_grad, m.pair_hess, m.x2mark);
     else
-      k_barrier_pairs_lanes<float><<<lgrid, kPairLanes, 0, st>>>(
+      k_barrier_pairs_lanes<float><<<grid, kPairLanes, 0, st>>>(
           m.counters, m.cap_act, m.pairs, sp, m.tris, m.edges, m.Wptr, m.Wcol, m.x2of, dhat, kappa,
           m.pair_grad, m.pair_hess, m.x2mark);
   } else if (precision == 0)
@@ -1460,7 +1520,7 @@ void launch_barrier_pairs(cudaStream_t st, const DevMesh& m, int64_t np, const d
         m.pair_grad, m.pair_hess, m.x2mark);
   count_launch();
   if (m.ee_moll) {
-    k_mollify_ee<<<mgrid, 32, 0, st>>>(m.counters, m.cap_act, m.pairs, sp, m.edges, m.elen2, dhat,
+    k_mollify_ee<<<grid, 32, 0, st>>>(m.counters, m.cap_act, m.pairs, sp, m.edges, m.elen2, dhat,
                                       kappa, m.pair_grad, m.pair_hess);
     count_launch();
   }
@@ -1471,28 +1531,10 @@ void launch_mark_scan(cudaStream_t st, const DevMesh& m) {
   count_launch();
 }
 
-__device__ __forceinline__ void k_ccd_reset_body(int* counters, double* scal) {
-  counters[1] = 0;
-  counters[9] = 0;
-  scal[1] = 1.0;
-}
-__global__ void k_ccd_reset(int* counters, double* scal) {
-  k_ccd_reset_body(counters, scal);
-}
-
-void launch_ccd_reset(cudaStream_t st, const DevMesh& m) {
-  k_ccd_reset<<<1, 1, 0, st>>>(m.counters, m.scal);
-  count_launch();
-}
-
-void launch_barrier_scatter(cudaStream_t st, const DevMesh& m, int64_t np, int nc_cap, int mode,
-                            double* g) {
-  np = np < m.cap_act ? np : m.cap_act;
-  if (np <= 0) return;
-  const int64_t threads = 16 * np;
-  k_barrier_scatter<<<(unsigned)((threads + 127) / 128), 128, 0, st>>>(
-      np, m.pairs, m.tris, m.edges, m.Wptr, m.Wcol, m.Wval, m.x2of, m.x2mark, m.pair_grad,
-      m.pair_hess, m.counters + 3, nc_cap, mode, g, m.Bc, m.bocc);
+void launch_barrier_scatter(cudaStream_t st, const DevMesh& m, int nc_cap, int mode, double* g) {
+  k_barrier_scatter<<<2 * 152, 128, 0, st>>>(
+      m.counters, m.cap_act, m.pairs, m.tris, m.edges, m.Wptr, m.Wcol, m.Wval, m.x2of, m.x2mark,
+      m.pair_grad, m.pair_hess, m.counters + 3, nc_cap, mode, g, m.Bc, m.bocc);
   count_launch();
 }
 
@@ -1517,23 +1559,14 @@ __device__ __forceinline__ const DevMesh* bframe_c(const DevMesh* __restrict__ t
 }
 }  // namespace
 
-// counters [0] |C|, [1] candidates, [2] overflow, [5] touching, [8] near
-// list and scal[0] (barrier energy) of every active frame to zero
-__global__ void k_eval_reset_b(const DevMesh* __restrict__ tab) {
-  const DevMesh* m = bframe_c(tab, blockIdx.y);
-  if (!m || threadIdx.x != 0) return;
-  m->counters[0] = 0; m->counters[1] = 0; m->counters[2] = 0;
-  m->counters[5] = 0; m->counters[8] = 0;
-  m->scal[0] = 0.0;
-}
-
-// AT 0: s = W x, 1: st = W xt, 2: ds = W dx
+// AT 0: s = W x, 1: st = W xt (an evaluation starts), 2: ds = W dx (the CCD step starts)
 template <int AT>
 __global__ void k_proxy_b(const DevMesh* __restrict__ tab) {
   const DevMesh* m = bframe_c(tab, blockIdx.y);
   if (!m) return;
   const double* x = AT == 0 ? m->x : (AT == 1 ? m->xt : m->dx);
   double* sp = AT == 0 ? m->s : (AT == 1 ? m->st : m->ds);
+  reset_counters(AT == 2 ? RESET_CCD : RESET_EVAL, m->counters, m->scal);
   k_proxy_body(m->Ns, m->Wptr, m->Wcol, m->Wval, x, sp);
 }
 
@@ -1547,7 +1580,7 @@ __global__ void k_prim_prep_b(const DevMesh* __restrict__ tab, double pad) {
 }
 
 template <int AT, int CCD>
-__global__ void k_skin_check_b(const DevMesh* __restrict__ tab, double margin) {
+__global__ void __launch_bounds__(kSkinThreads) k_skin_check_b(const DevMesh* __restrict__ tab, double margin) {
   const DevMesh* m = bframe_c(tab, blockIdx.y);
   if (!m) return;
   k_skin_check_body(m->Ns, AT ? m->st : m->s, m->sb, CCD ? m->ds : nullptr, m->skin, margin,
@@ -1639,17 +1672,9 @@ __global__ void k_zero_reduced_b(const DevMesh* __restrict__ tab) {
 __global__ void k_barrier_scatter_b(const DevMesh* __restrict__ tab, int mode) {
   const DevMesh* m = bframe_c(tab, blockIdx.y);
   if (!m) return;
-  int64_t np = m->counters[0];
-  np = np < m->cap_act ? np : m->cap_act;
-  k_barrier_scatter_body(np, m->pairs, m->tris, m->edges, m->Wptr, m->Wcol, m->Wval, m->x2of,
+  k_barrier_scatter_body(m->counters, m->cap_act, m->pairs, m->tris, m->edges, m->Wptr, m->Wcol, m->Wval, m->x2of,
                          m->x2mark, m->pair_grad, m->pair_hess, m->counters + 3,
                          m->Bc != nullptr ? m->nc_cap : 0, mode, m->g, m->Bc, m->bocc);
-}
-
-__global__ void k_ccd_reset_b(const DevMesh* __restrict__ tab) {
-  const DevMesh* m = bframe_c(tab, blockIdx.y);
-  if (!m || threadIdx.x != 0) return;
-  k_ccd_reset_body(m->counters, m->scal);
 }
 
 __global__ void k_skin_cand_b(const DevMesh* __restrict__ tab) {
@@ -1684,10 +1709,13 @@ void launch_sweeps_b(cudaStream_t st, const DevMesh* tab, int nb, const DevMesh&
 }
 }  // namespace
 
-void launch_eval_reset_b(cudaStream_t st, const DevMesh* tab, int nb) {
-  k_eval_reset_b<<<dim3(1, nb), 32, 0, st>>>(tab);
-  count_launch();
-}
+// CTAs per frame of the kernels over lists whose length only the device knows:
+// eight CTAs per SM over all frames, and a few for each frame of a large batch
+// (CTAs without work still cost their launch: 304 of them per frame took 10 us
+// of a 32-frame launch)
+namespace {
+int list_ctas(int nb) { return std::max(16, (8 * 152 + nb - 1) / nb); }
+}  // namespace
 
 void launch_proxy_b(cudaStream_t st, const DevMesh* tab, int nb, const DevMesh& m0, int at) {
   const dim3 g((m0.Ns + 255) / 256, nb);
@@ -1707,16 +1735,16 @@ void launch_detect_b(cudaStream_t st, const DevMesh* tab, int nb, const DevMesh&
   const dim3 gp((np + 255) / 256, nb);
   if (at) {
     k_prim_prep_b<1, 0><<<gp, 256, 0, st>>>(tab, pad);
-    k_skin_check_b<1, 0><<<dim3(1, nb), 512, 0, st>>>(tab, margin);
+    k_skin_check_b<1, 0><<<dim3(skin_ctas(m0), nb), kSkinThreads, 0, st>>>(tab, margin);
   } else {
     k_prim_prep_b<0, 0><<<gp, 256, 0, st>>>(tab, pad);
-    k_skin_check_b<0, 0><<<dim3(1, nb), 512, 0, st>>>(tab, margin);
+    k_skin_check_b<0, 0><<<dim3(skin_ctas(m0), nb), kSkinThreads, 0, st>>>(tab, margin);
   }
   count_launch(2);
   launch_sweeps_b(st, tab, nb, m0, 0, (float)pad + margin);
-  k_skin_near_b<<<dim3(2 * 152, nb), 128, 0, st>>>(tab, 2.0f * (float)dhat);
-  if (at) k_near_pairs_b<1><<<dim3(2 * 152, nb), 128, 0, st>>>(tab, dhat);
-  else k_near_pairs_b<0><<<dim3(2 * 152, nb), 128, 0, st>>>(tab, dhat);
+  k_skin_near_b<<<dim3(list_ctas(nb), nb), 128, 0, st>>>(tab, 2.0f * (float)dhat);
+  if (at) k_near_pairs_b<1><<<dim3(list_ctas(nb), nb), 128, 0, st>>>(tab, dhat);
+  else k_near_pairs_b<0><<<dim3(list_ctas(nb), nb), 128, 0, st>>>(tab, dhat);
   count_launch(2);
 }
 
@@ -1738,11 +1766,10 @@ void launch_barrier_b(cudaStream_t st, const DevMesh* tab, int nb, const DevMesh
     }
   }
   k_mark_scan_b<<<dim3(1, nb), 1024, 0, st>>>(tab);
-  k_zero_reduced_b<<<dim3(2 * 152, nb), 256, 0, st>>>(tab);
+  k_zero_reduced_b<<<dim3(list_ctas(nb), nb), 256, 0, st>>>(tab);
   count_launch(2);
   if (np_max > 0) {
-    const int64_t threads = 16 * np_max;
-    k_barrier_scatter_b<<<dim3((unsigned)((threads + 127) / 128), nb), 128, 0, st>>>(tab, 3);
+    k_barrier_scatter_b<<<dim3(list_ctas(nb), nb), 128, 0, st>>>(tab, 3);
     count_launch();
   }
 }
@@ -1750,18 +1777,16 @@ void launch_barrier_b(cudaStream_t st, const DevMesh* tab, int nb, const DevMesh
 void launch_ccd_b(cudaStream_t st, const DevMesh* tab, int nb, const DevMesh& m0, double dhat,
                   double ccd_s, int accd_max_iters) {
   launch_proxy_b(st, tab, nb, m0, 2);
-  k_ccd_reset_b<<<dim3(1, nb), 32, 0, st>>>(tab);
-  count_launch();
   ProfScope ps(PROF_CCD, st);
   const int np = nprim(m0);
   if (np == 0) return;
   k_prim_prep_b<0, 1><<<dim3((np + 255) / 256, nb), 256, 0, st>>>(tab, dhat);
-  k_skin_check_b<0, 1><<<dim3(1, nb), 512, 0, st>>>(tab, 0.0);
-  k_skin_cand_b<<<dim3(2 * 152, nb), 128, 0, st>>>(tab);
+  k_skin_check_b<0, 1><<<dim3(skin_ctas(m0), nb), kSkinThreads, 0, st>>>(tab, 0.0);
+  k_skin_cand_b<<<dim3(list_ctas(nb), nb), 128, 0, st>>>(tab);
   count_launch(3);
   launch_sweeps_b(st, tab, nb, m0, 1, 0.0f);
   const double slack = fmax(0.01 * dhat, 1e-5 * m0.coord_scale);
-  k_accd_list_b<<<dim3(4 * 152, nb), 128, 0, st>>>(tab, ccd_s, accd_max_iters, (float)slack);
+  k_accd_list_b<<<dim3(list_ctas(nb), nb), 128, 0, st>>>(tab, ccd_s, accd_max_iters, (float)slack);
   count_launch();
 }
 

@@ -52,7 +52,8 @@ struct DevMesh {
   double* cg_q = nullptr;
   double* cg_tmp = nullptr;
   double* cg_red = nullptr;
-  double* sb = nullptr;       // 3 Ns proxy positions of the last skin-list build
+  double* sb = nullptr;       // 3 Ns proxy positions of the last skin-list build, then three
+                              // words of k_skin_check
   double* elen2 = nullptr;    // Ne squared rest lengths of the proxy edges (EE mollifier)
   int ee_moll = 0;            // 1: edge-edge terms carry IPC's mollifier
   double skin = 0.0;          // skin width of the list (length)
@@ -130,7 +131,7 @@ struct DevMesh {
     int64_t kernels = 0;        // kernel nodes (counted as launches per replay)
     bool failed = false;        // capture unsupported: launch directly
   };
-  static constexpr int kGraphs = 12;
+  static constexpr int kGraphs = 18;
   Graph graphs[kGraphs];
   // side stream and fork / join events of this workspace: the part of the
   // reduced system that does not need the right-hand side runs there while
@@ -181,28 +182,27 @@ void launch_gather_forces(cudaStream_t s, const DevMesh& m, const double* tetf, 
 void launch_sum_partials(cudaStream_t s, const double* partials, int n, double* out);
 
 // ---- contact (k_contact.cu) -----------------------------------------------
-void launch_proxy(cudaStream_t s, const DevMesh& m, const double* x, double* sp);
+// reset: the counters and scalars that the launches after it add to
+enum { RESET_NONE = 0, RESET_EVAL = 1, RESET_CCD = 2 };
+void launch_proxy(cudaStream_t s, const DevMesh& m, const double* x, double* sp, int reset);
 // Constraint set at proxy positions sp; appends keys to m.pairs and adds the
 // barrier energy to m.scal[0].
 void launch_detect(cudaStream_t s, const DevMesh& m, const double* sp, double dhat, double kappa);
 // Candidate pairs of the swept boxes sp -> sp + dsp (inflated by dhat) and
-// the ACCD time of impact (min into m.scal[1] as ordered bits); the caller
-// zeroes counters [1] and [9] and sets scal[1] = 1.
+// the ACCD time of impact (min into m.scal[1] as ordered bits); after a
+// launch_proxy with RESET_CCD.
 void launch_ccd(cudaStream_t s, const DevMesh& m, const double* sp, const double* dsp,
                 double dhat, double ccd_s, int accd_max_iters);
 // Per-pair barrier gradient and PSD Hessian blocks (pass A) and x2 marks.
-void launch_barrier_pairs(cudaStream_t s, const DevMesh& m, int64_t npairs, const double* sp,
-                          double dhat, double kappa, int precision);
+void launch_barrier_pairs(cudaStream_t s, const DevMesh& m, const double* sp, double dhat,
+                          double kappa, int precision);
 void launch_mark_scan(cudaStream_t s, const DevMesh& m);
 // Scatter pair gradients into g and Hessian blocks into the dense B-check (3nc)^2.
 // B-check and g from the per-pair blocks; n_c is read on the device and
 // B-check is written only when n_c <= nc_cap (mode: 1 gradient, 2 B-check, 3 both)
-void launch_barrier_scatter(cudaStream_t s, const DevMesh& m, int64_t npairs, int nc_cap, int mode,
-                            double* g);
+void launch_barrier_scatter(cudaStream_t s, const DevMesh& m, int nc_cap, int mode, double* g);
 // zero B-check and its block occupancy for the n_c on the device (when n_c <= nc_cap)
 void launch_zero_reduced(cudaStream_t s, const DevMesh& m, int nc_cap);
-// Reset the CCD outputs: counters[1] = counters[9] = 0 and scal[1] = 1.
-void launch_ccd_reset(cudaStream_t s, const DevMesh& m);
 
 // ---- global step (k_solve.cu) ----------------------------------------------
 // dx (by vertex) solving (H + B) dx = -g, with B-check already assembled for
@@ -264,7 +264,6 @@ constexpr int kBwdRowSplit = 256;
 // `tab` is a device array of nb DevMesh copies (frames of one mesh); m0 is a
 // host copy of any of them (mesh-wide sizes and constants).  Every launch
 // serves the frames whose `active` flag is set; `at` 0 evaluates at x, 1 at xt.
-void launch_eval_reset_b(cudaStream_t s, const DevMesh* tab, int nb);
 void launch_local_b(cudaStream_t s, const DevMesh* tab, int nb, const DevMesh& m0, int at);
 void launch_proxy_b(cudaStream_t s, const DevMesh* tab, int nb, const DevMesh& m0, int at);
 void launch_detect_b(cudaStream_t s, const DevMesh* tab, int nb, const DevMesh& m0, int at, double dhat);

@@ -15,6 +15,8 @@ namespace fsim {
 
 constexpr int kCounters = 16;   // device counter words of a workspace
 constexpr int kScal = 8;        // device float64 scalars of a workspace
+// a workspace's scalars followed by its counters
+constexpr size_t kStatusBytes = sizeof(double) * kScal + sizeof(int) * kCounters;
 
 // One uploaded mesh: constant device data (topology, factor, Sigma^-1) plus
 // its default workspace, all reachable through d.
@@ -45,7 +47,7 @@ struct MeshState {
 // of cooperative launches, and the list that owns buffers it grows.
 struct Exec {
   cudaStream_t stream = nullptr;
-  int* h_counters = nullptr;     // kCounters pinned ints
+  int* h_counters = nullptr;     // kCounters pinned ints, right after the scalars
   double* h_scal = nullptr;      // kScal pinned doubles
   int coop_ctas = 1;
   bool alone = true;             // no other solve shares the GPU

@@ -450,18 +450,16 @@ fsim_status fsim_server_create(fsim_ctx_t ctx, const fsim_server_config* cfg, fs
   cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi);
   for (auto& w : sv->workers) {
     if (cudaStreamCreateWithPriority(&w.stream, cudaStreamNonBlocking, prio_hi) != cudaSuccess ||
-        cudaHostAlloc((void**)&w.h_counters, sizeof(int) * kCounters, cudaHostAllocDefault) !=
-            cudaSuccess ||
-        cudaHostAlloc((void**)&w.h_scal, sizeof(double) * kScal, cudaHostAllocDefault) != cudaSuccess) {
+        cudaHostAlloc((void**)&w.h_scal, kStatusBytes, cudaHostAllocDefault) != cudaSuccess) {
       cudaGetLastError();
       for (auto& x : sv->workers) {
         if (x.stream) cudaStreamDestroy(x.stream);
-        if (x.h_counters) cudaFreeHost(x.h_counters);
         if (x.h_scal) cudaFreeHost(x.h_scal);
       }
       delete sv;
       return FSIM_ENOMEM;
     }
+    w.h_counters = reinterpret_cast<int*>(w.h_scal + kScal);
   }
   for (int i = 0; i < cfg->workers; ++i)
     sv->workers[i].th = std::thread(sv->batch_frames >= 2 ? batch_worker_main : worker_main, sv, i);
@@ -566,7 +564,6 @@ fsim_status fsim_server_destroy(fsim_server_t sv) {
   for (auto& w : sv->workers) {
     cudaStreamSynchronize(w.stream);
     cudaStreamDestroy(w.stream);
-    cudaFreeHost(w.h_counters);
     cudaFreeHost(w.h_scal);
   }
   for (auto& s : sv->slots) free_slot(*s);
