@@ -80,6 +80,8 @@ void free_mesh(MeshState& ms) {
   delete[] ms.d.h_fwd_ptr;
   delete[] ms.d.h_bwd_ptr;
   delete[] ms.d.h_bwd32_ptr;
+  delete[] ms.d.h_fwd32_ptr;
+  ms.d.h_fwd32_ptr = nullptr;
   ms.d.h_bwd32_ptr = nullptr;
   ms.d.h_level_ptr = nullptr;
   ms.d.h_level_maxns = nullptr;
@@ -862,22 +864,44 @@ fsim_status fsim_prefactor(fsim_ctx_t ctx, int mesh_id, const fsim_params* p) {
   m.h_fwd_ptr = new int[f.n_levels + 1];
   m.h_bwd_ptr = new int[f.n_levels + 1];
   m.h_bwd32_ptr = new int[f.n_levels + 1];
-  // work items: forward = 32-row chunks of Z_J, backward = 8-column chunks
-  // (32-column chunks for the multi-right-hand-side backward solve)
-  std::vector<int4> fwd, bwd, bwd32;
+  m.h_fwd32_ptr = new int[f.n_levels + 1];
+  // work items of the single-frame solves (rows of Z_J forward, columns
+  // backward; see k_fwd_chunk for the widths) and of the batched ones (32-row
+  // and 32-column chunks)
+  std::vector<int4> fwd, bwd, fwd32, bwd32;
   m.h_fwd_ptr[0] = 0;
   m.h_bwd_ptr[0] = 0;
+  m.h_fwd32_ptr[0] = 0;
   m.h_bwd32_ptr[0] = 0;
   for (int l = 0; l <= f.n_levels; ++l) m.h_level_ptr[l] = f.level_ptr[l];
   for (int l = 0; l < f.n_levels; ++l) {
     int mx = 1, mxld = 1;
+    auto width = [&](int widest, int least, auto length) {
+      for (; widest > least; widest /= 2) {
+        int count = 0;
+        for (int k = f.level_ptr[l]; k < f.level_ptr[l + 1]; ++k)
+          count += (length(f.level_sn[k]) + widest - 1) / widest;
+        if (count >= ctx->num_sms) break;
+      }
+      return widest;
+    };
+    // (short chains gain nothing, a lane's share is a few terms either way, and pay
+    // for the extra CTAs: small slabs 48.0 ms a frame so, 49.4 ms without the limits)
+    int long_ns = 0, long_ld = 0;
+    for (int k = f.level_ptr[l]; k < f.level_ptr[l + 1]; ++k) {
+      long_ns = std::max(long_ns, ns[f.level_sn[k]]);
+      long_ld = std::max(long_ld, ns[f.level_sn[k]] + nr1[f.level_sn[k]]);
+    }
+    const int wf = long_ns < 96 ? 32 : width(32, 8, [&](int J) { return ns[J] + nr1[J]; });
+    const int wb = long_ld < 256 ? 8 : width(8, 2, [&](int J) { return ns[J]; });
     for (int k = f.level_ptr[l]; k < f.level_ptr[l + 1]; ++k) {
       const int J = f.level_sn[k];
       const int ldj = ns[J] + nr1[J];
       mx = std::max(mx, ns[J]);
       mxld = std::max(mxld, ldj);
-      for (int r0 = 0; r0 < ldj; r0 += 32) fwd.push_back(make_int4(J, r0, std::min(32, ldj - r0), 0));
-      for (int k0 = 0; k0 < ns[J]; k0 += 8) bwd.push_back(make_int4(J, k0, std::min(8, ns[J] - k0), 0));
+      for (int r0 = 0; r0 < ldj; r0 += wf) fwd.push_back(make_int4(J, r0, std::min(wf, ldj - r0), wf));
+      for (int k0 = 0; k0 < ns[J]; k0 += wb) bwd.push_back(make_int4(J, k0, std::min(wb, ns[J] - k0), wb));
+      for (int r0 = 0; r0 < ldj; r0 += 32) fwd32.push_back(make_int4(J, r0, std::min(32, ldj - r0), 0));
       // 32 columns and up to kBwdRowSplit rows each: the long row ranges of
       // the top supernodes spread over many CTAs (partial sums added atomically)
       for (int k0 = 0; k0 < ns[J]; k0 += 32)
@@ -887,10 +911,12 @@ fsim_status fsim_prefactor(fsim_ctx_t ctx, int mesh_id, const fsim_params* p) {
     m.h_level_maxns[l] = mx;
     m.h_level_maxld[l] = mxld;
     m.h_fwd_ptr[l + 1] = (int)fwd.size();
+    m.h_fwd32_ptr[l + 1] = (int)fwd32.size();
     m.h_bwd_ptr[l + 1] = (int)bwd.size();
     m.h_bwd32_ptr[l + 1] = (int)bwd32.size();
   }
   TRY(upload(ms, s, &m.fwd_items, fwd.data(), fwd.size()));
+  TRY(upload(ms, s, &m.fwd_items32, fwd32.data(), fwd32.size()));
   TRY(upload(ms, s, &m.bwd_items, bwd.data(), bwd.size()));
   TRY(upload(ms, s, &m.bwd_items32, bwd32.data(), bwd32.size()));
   TRY(upload(ms, s, &m.Sinv, f.sigma_inv.data(), f.sigma_inv.size()));

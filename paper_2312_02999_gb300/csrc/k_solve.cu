@@ -63,17 +63,22 @@ __global__ void k_convert(int n, const S* __restrict__ a, T* __restrict__ b) {
 // ---------------------------------------------------------------------------
 // supernodal triangular solves with Z_J = [L_JJ^-1 ; L_RJ L_JJ^-1]
 // ---------------------------------------------------------------------------
-// Chunked forms: a level is a list of work items (J, first row/column, count)
-// so that one large supernode spreads over many CTAs.  A level's work is a
-// handful of dependent GEMV chunks, so the serial chain per lane sets its
+// Chunked forms: a level is a list of work items (J, first row/column, count,
+// width) so that one large supernode spreads over many CTAs.  A level's work is
+// a handful of dependent GEMV chunks, so the serial chain per lane sets its
 // time: a solve that has the GPU to itself uses 32 warps per item (NT =
 // 1024); solves that share the GPU with others, and the float64 form (bound
 // by the float64 pipe), use 8 warps per item (NT = 256) so that more items fit
-// on an SM.
-constexpr int kBwdCols = 8;                       // columns per backward item
+// on an SM.  The width is the widest of 32, 16, 8 rows (forward) or 8, 4, 2
+// columns (backward) that gives every SM an item of the level: the top levels
+// have one to eight supernodes, and 32 rows of 475 columns hold one SM's float64
+// pipes for 11 us while the other SMs idle.
+// One frame, 32 rows and 8 columns throughout -> this rule: 30k face float64 75.3 ->
+// 73.2 ms, 5k face mixed 29.4 -> 28.3 ms.
 
-// Forward item: rows [r0, r0+32) of Z_J times b_J; lanes own rows (coalesced
-// column-major reads), the 32 warps split the inner index and reduce through
+// Forward item: rows [r0, r0 + rn) of Z_J times b_J; a lane owns a row and every
+// (32 / width)-th of its warp's columns (coalesced column-major reads), the
+// warps split the inner index, the parts are added by shuffles and through
 // shared memory.
 template <typename T, int NT>
 __global__ void __launch_bounds__(NT)
@@ -86,22 +91,22 @@ k_fwd_chunk(const int4* __restrict__ items, const int* __restrict__ c0a, const i
   T* bj = reinterpret_cast<T*>(smem_raw);
   __shared__ T part[kSolveWarps][32][3];
   const int4 it = items[blockIdx.x];
-  const int J = it.x, r0 = it.y, rn = it.z;
+  const int J = it.x, r0 = it.y, rn = it.z, w = it.w;
   const int c0 = c0a[J], ns = nsa[J], nr = nra[J], ld = ns + nr;
   const T* Zj = Z + zoff[J];
   for (int k = threadIdx.x; k < 3 * ns; k += blockDim.x) bj[k] = b[3 * (size_t)c0 + k];
   __syncthreads();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int r = r0 + lane;
+  const int rl = lane & (w - 1), r = r0 + rl, split = 32 / w, step = kSolveWarps * split;
   T a0 = 0, a1 = 0, a2 = 0;
-  if (lane < rn) {
+  if (rl < rn) {
     const int kmax = r < ns ? r + 1 : ns;
     // two independent loads and accumulators in flight per lane
     T q0 = 0, q1 = 0, q2 = 0;
-    int k = wid;
-    for (; k + kSolveWarps < kmax; k += 2 * kSolveWarps) {
-      const T z0 = Zj[(size_t)k * ld + r], z1 = Zj[(size_t)(k + kSolveWarps) * ld + r];
-      const int k1 = k + kSolveWarps;
+    int k = wid * split + lane / w;
+    for (; k + step < kmax; k += 2 * step) {
+      const int k1 = k + step;
+      const T z0 = Zj[(size_t)k * ld + r], z1 = Zj[(size_t)k1 * ld + r];
       a0 += z0 * bj[3 * k]; a1 += z0 * bj[3 * k + 1]; a2 += z0 * bj[3 * k + 2];
       q0 += z1 * bj[3 * k1]; q1 += z1 * bj[3 * k1 + 1]; q2 += z1 * bj[3 * k1 + 2];
     }
@@ -111,22 +116,25 @@ k_fwd_chunk(const int4* __restrict__ items, const int* __restrict__ c0a, const i
     }
     a0 += q0; a1 += q1; a2 += q2;
   }
-  part[wid][lane][0] = a0; part[wid][lane][1] = a1; part[wid][lane][2] = a2;
+  for (int o = w; o < 32; o <<= 1) {
+    a0 += __shfl_xor_sync(0xffffffffu, a0, o);
+    a1 += __shfl_xor_sync(0xffffffffu, a1, o);
+    a2 += __shfl_xor_sync(0xffffffffu, a2, o);
+  }
+  if (lane < w) { part[wid][rl][0] = a0; part[wid][rl][1] = a1; part[wid][rl][2] = a2; }
   __syncthreads();
-  if (threadIdx.x < 96) {
-    const int rl = threadIdx.x / 3, d = threadIdx.x % 3;
-    if (rl < rn) {
-      T acc = 0;
+  if (threadIdx.x < 3 * rn) {
+    const int rr0 = threadIdx.x / 3, d = threadIdx.x % 3;
+    T acc = 0;
 #pragma unroll 8
-      for (int w = 0; w < kSolveWarps; ++w) acc += part[w][rl][d];
-      const int rr = r0 + rl;
-      if (rr < ns) y[3 * (size_t)(c0 + rr) + d] = acc;
-      else atomicAdd(b + 3 * (size_t)rows[roff[J] + rr - ns] + d, -acc);
-    }
+    for (int q = 0; q < kSolveWarps; ++q) acc += part[q][rr0][d];
+    const int rr = r0 + rr0;
+    if (rr < ns) y[3 * (size_t)(c0 + rr) + d] = acc;
+    else atomicAdd(b + 3 * (size_t)rows[roff[J] + rr - ns] + d, -acc);
   }
 }
 
-// Backward item: columns [k0, k0+kn) (kn <= 8) of Z_J^T [y_J ; -x_R]; NT/256
+// Backward item: columns [k0, k0 + kn) of Z_J^T [y_J ; -x_R]; NT / 32 / width
 // warps per column split its rows.  Reads y (forward result) and the
 // ancestors' x, writes x_J (x may alias b).
 template <typename T, int NT>
@@ -136,11 +144,10 @@ k_bwd_chunk(const int4* __restrict__ items, const int* __restrict__ c0a, const i
             const int64_t* __restrict__ zoff, const int* __restrict__ rows,
             const T* __restrict__ Z, const T* __restrict__ y, T* __restrict__ x) {
   extern __shared__ unsigned char smem_raw[];
-  constexpr int kBwdWarpsPerCol = NT / 32 / kBwdCols;
   T* wv = reinterpret_cast<T*>(smem_raw);
-  __shared__ T part[kBwdCols][kBwdWarpsPerCol][3];
+  __shared__ T part[NT / 32][3];
   const int4 it = items[blockIdx.x];
-  const int J = it.x, k0 = it.y, kn = it.z;
+  const int J = it.x, k0 = it.y, kn = it.z, per = NT / 32 / it.w;
   const int c0 = c0a[J], ns = nsa[J], nr = nra[J], ld = ns + nr;
   const T* Zj = Z + zoff[J];
   const int* Rj = rows + roff[J];
@@ -150,17 +157,16 @@ k_bwd_chunk(const int4* __restrict__ items, const int* __restrict__ c0a, const i
     wv[3 * ns + k] = -x[3 * (size_t)Rj[k / 3] + (k % 3)];
   __syncthreads();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int c = wid / kBwdWarpsPerCol, qw = wid % kBwdWarpsPerCol;
-  constexpr int kStride = 32 * kBwdWarpsPerCol;
+  const int c = wid / per, qw = wid % per, step = 32 * per;
   T a0 = 0, a1 = 0, a2 = 0;
   if (c < kn) {
     const int k = k0 + c;
     const T* zc = Zj + (size_t)k * ld;
     T q0 = 0, q1 = 0, q2 = 0;
     int r = k + qw * 32 + lane;
-    for (; r + kStride < ld; r += 2 * kStride) {
-      const T z0 = zc[r], z1 = zc[r + kStride];
-      const int s1 = r + kStride;
+    for (; r + step < ld; r += 2 * step) {
+      const int s1 = r + step;
+      const T z0 = zc[r], z1 = zc[s1];
       a0 += z0 * wv[3 * r]; a1 += z0 * wv[3 * r + 1]; a2 += z0 * wv[3 * r + 2];
       q0 += z1 * wv[3 * s1]; q1 += z1 * wv[3 * s1 + 1]; q2 += z1 * wv[3 * s1 + 2];
     }
@@ -171,16 +177,13 @@ k_bwd_chunk(const int4* __restrict__ items, const int* __restrict__ c0a, const i
     a0 += q0; a1 += q1; a2 += q2;
   }
   a0 = warp_sum_t(a0); a1 = warp_sum_t(a1); a2 = warp_sum_t(a2);
-  if (lane == 0) { part[c][qw][0] = a0; part[c][qw][1] = a1; part[c][qw][2] = a2; }
+  if (lane == 0) { part[wid][0] = a0; part[wid][1] = a1; part[wid][2] = a2; }
   __syncthreads();
-  if (threadIdx.x < 3 * kBwdCols) {
+  if (threadIdx.x < 3 * kn) {
     const int cc = threadIdx.x / 3, d = threadIdx.x % 3;
-    if (cc < kn) {
-      T acc = 0;
-#pragma unroll
-      for (int w = 0; w < kBwdWarpsPerCol; ++w) acc += part[cc][w][d];
-      x[3 * (size_t)(c0 + k0 + cc) + d] = acc;
-    }
+    T acc = 0;
+    for (int q = 0; q < per; ++q) acc += part[cc * per + q][d];
+    x[3 * (size_t)(c0 + k0 + cc) + d] = acc;
   }
 }
 
@@ -701,11 +704,11 @@ cudaError_t global_step_b(const BatchStep& bs) {
   if (e != cudaSuccess) return e;
   if (cudaEventRecord(bs.ev[1], s2) != cudaSuccess) return cudaGetLastError();
   for (int l = 0; l < m.n_levels && n1 > 0; ++l) {
-    const int a = m.h_fwd_ptr[l], z = m.h_fwd_ptr[l + 1];
+    const int a = m.h_fwd32_ptr[l], z = m.h_fwd32_ptr[l + 1];
     if (z <= a) continue;
     ProfScope ps(PROF_TRSV_FWD, s);
     const size_t sm = sizeof(float) * kMrCols * (size_t)m.h_level_maxns[l];
-    k_fwd_mr<<<dim3(z - a, chunks), 256, sm, s>>>(m.fwd_items + a, m.sn_c0, m.sn_ns, m.sn_nr1,
+    k_fwd_mr<<<dim3(z - a, chunks), 256, sm, s>>>(m.fwd_items32 + a, m.sn_c0, m.sn_ns, m.sn_nr1,
                                                    m.sn_roff, m.sn_zoff, m.sn_rows, m.Zf, bs.rb,
                                                    bs.yb, nr, nf);
     count_launch();

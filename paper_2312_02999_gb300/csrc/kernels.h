@@ -73,8 +73,10 @@ struct DevMesh {
   int* h_level_ptr = nullptr; // HOST array (n_levels + 1)
   int* h_level_maxns = nullptr;  // HOST: largest ns per level
   int* h_level_maxld = nullptr;  // HOST: largest ns + nr1 per level
-  int4* fwd_items = nullptr;  // (J, first row, rows, 0) work items, grouped by level
-  int4* bwd_items = nullptr;  // (J, first column, columns, 0)
+  int4* fwd_items = nullptr;  // (J, first row, rows, width) work items, grouped by level
+  int4* bwd_items = nullptr;  // (J, first column, columns, width)
+  int4* fwd_items32 = nullptr;  // (J, first row, rows <= 32, 0) for the batched solve
+  int* h_fwd32_ptr = nullptr;   // HOST (n_levels + 1)
   int* h_fwd_ptr = nullptr;   // HOST (n_levels + 1)
   int* h_bwd_ptr = nullptr;   // HOST (n_levels + 1)
   int4* bwd_items32 = nullptr;  // (J, first column, columns <= 32, first row) for the batched
