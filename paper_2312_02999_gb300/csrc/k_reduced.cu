@@ -86,7 +86,7 @@ struct RedArgs {
   int one_cta_max;      // largest n_c of the one-CTA path (float32 factors); the
                         // 4-CTA cluster takes n_c up to kClusNc above it
   FT* spk;              // small forms: L_s packed, its diagonal blocks inverted
-  unsigned* bar;        // grid form: two counters of each of its two kernels
+  unsigned* bar;        // grid form: counters of its two kernels' barriers
 };
 
 // Offsets of the workspace for a given n_c (every kernel of the reduced solve
@@ -191,6 +191,154 @@ __global__ void __launch_bounds__(256) k_z2_update(RedArgs<float> a) {
 }
 
 // ---------------------------------------------------------------------------
+// Diagonal blocks and panels of the grid form.
+// ---------------------------------------------------------------------------
+constexpr int kBk = 32;                     // block edge
+
+// x 2^-e and the significand of x (x = m 2^e, 1 <= m < 2), x positive and normal
+__device__ __forceinline__ int exponent_of(float x) {
+  return ((__float_as_int(x) >> 23) & 255) - 127;
+}
+__device__ __forceinline__ float significand(float x) {
+  return __int_as_float((__float_as_int(x) & 0x007fffff) | 0x3f800000);
+}
+__device__ __forceinline__ float scale_down(float x, int e) {
+  return x * __int_as_float((127 - max(-126, min(126, e))) << 23);
+}
+__device__ __forceinline__ int exponent_of(double x) {
+  return ((__double2hiint(x) >> 20) & 2047) - 1023;
+}
+__device__ __forceinline__ double significand(double x) {
+  return __hiloint2double((__double2hiint(x) & 0x000fffff) | 0x3ff00000, __double2loint(x));
+}
+__device__ __forceinline__ double scale_down(double x, int e) {   // integer work only
+  const int h = __double2hiint(x), ne = ((h >> 20) & 2047) - e;
+  return ne > 0 && ne < 2047 && ((h >> 20) & 2047) != 0
+             ? __hiloint2double(h - (int)((unsigned)e << 20), __double2loint(x))
+             : 0.0;
+}
+__device__ __forceinline__ float rsqrt_ft(float v) {
+  float r = rsqrtf(v);
+  return r * (1.5f - 0.5f * v * r * r);
+}
+
+// element e of the lower triangle of a 32 x 32 block, columns from the last to
+// the first: the elements of the columns > j are then the first ones, so that
+// the work left after column j fills whole warps
+__device__ __forceinline__ void tri_element(int e, int& r, int& c) {
+  int m = (int)((sqrtf(8.f * e + 1.f) - 1.f) * 0.5f);      // column 31 - m holds m + 1 elements
+  while ((m + 1) * (m + 2) / 2 <= e) ++m;
+  while (m * (m + 1) / 2 > e) --m;
+  c = kBk - 1 - m;
+  r = c + e - m * (m + 1) / 2;
+}
+
+// A panel's diagonal factor (Lt[q][r] = L[r][q], dv = 1 / diag) and the columns of
+// its elimination.
+struct ChSm {
+  float Lt[32][32];
+  float dv[32], rs[32];
+  float col[32][33];
+};
+constexpr int kDT = 256;                   // threads of diag_factor (the whole CTA)
+
+// Factor of the diagonal block with entries load(r, c) - P_r . P_c (r >= c; P the
+// panel before, transposed: P_r[l] = Pt[l ldp + r], none if Pt is null), into
+// sm.Lt / sm.dv and store(r, c, L[r][c]).  The elimination is free of divisions:
+// with pivot p = ph 2^e (1 <= ph < 2),
+//   D[r][c] <- D[r][c] ph - D[r][j] (D[c][j] 2^-e),
+// which is the Schur complement times ph, so that after column j every entry
+// carries the product of the ph so far (at most 2^31).  A column then costs two
+// dependent operations and one barrier; the square roots of all columns are
+// taken at once at the end.  Every thread owns two elements of the triangle (16
+// threads a third one, in column 0, which no step changes).
+template <typename Load, typename Store>
+__device__ __forceinline__ void diag_factor(ChSm& sm, const float* Pt, int ldp, int* info,
+                                            Load load, Store store) {
+  const int tid = threadIdx.x;
+  float v[3];
+  int er[3], ec[3];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const int e = tid + q * kDT;
+    er[q] = 0;
+    ec[q] = -1;
+    if (e >= 32 * 33 / 2) continue;
+    tri_element(e, er[q], ec[q]);
+    float x = load(er[q], ec[q]);
+    if (Pt) {
+      float a0 = 0.f, a1 = 0.f;
+#pragma unroll 8
+      for (int l = 0; l < 32; l += 2) {
+        a0 += Pt[l * ldp + er[q]] * Pt[l * ldp + ec[q]];
+        a1 += Pt[(l + 1) * ldp + er[q]] * Pt[(l + 1) * ldp + ec[q]];
+      }
+      x -= a0 + a1;
+    }
+    v[q] = x;
+    if (ec[q] == 0) sm.col[0][er[q]] = x;
+  }
+  for (int j = 0; j + 1 < 32; ++j) {
+    __syncthreads();
+    if (ec[0] <= j && ec[1] <= j) continue;
+    float p = sm.col[j][j];
+    if (!(p > 0.f)) p = 1.f;                         // reported below
+    const int e = exponent_of(p);
+    const float ph = significand(p);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      if (ec[q] <= j) continue;
+      const float w = scale_down(sm.col[j][ec[q]], e);
+      v[q] = v[q] * ph - sm.col[j][er[q]] * w;
+      if (ec[q] == j + 1) sm.col[j + 1][er[q]] = v[q];
+    }
+  }
+  __syncthreads();
+  if (tid < 32) {
+    float p = sm.col[tid][tid];
+    const bool bad = !(p > 0.f);
+    if (bad) { atomicOr(info, 1); p = 1.f; }
+    float pi = significand(p);
+#pragma unroll
+    for (int s = 1; s < 32; s <<= 1) {
+      const float x = __shfl_up_sync(0xffffffffu, pi, s);
+      if (tid >= s) pi *= x;
+    }
+    pi = __shfl_up_sync(0xffffffffu, pi, 1);
+    if (tid == 0) pi = 1.f;
+    const float rs = rsqrt_ft(p * pi);
+    sm.rs[tid] = rs;
+    sm.dv[tid] = pi * rs;
+    if (bad) sm.col[tid][tid] = 1.f;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    if (ec[q] < 0) continue;
+    const float x = sm.col[ec[q]][er[q]] * sm.rs[ec[q]];
+    sm.Lt[ec[q]][er[q]] = x;
+    store(er[q], ec[q], x);
+  }
+}
+
+// x L_kk^T = a for one row in registers (right-looking: the dependent chain is
+// one FMA per column; four entries of the factor per shared-memory read)
+__device__ __forceinline__ void panel_row(const ChSm& sm, float x[32]) {
+#pragma unroll
+  for (int q = 0; q < 32; ++q) {
+    x[q] *= sm.dv[q];
+#pragma unroll
+    for (int l4 = (q + 1) / 4; l4 < 8; ++l4) {
+      const float4 f = *reinterpret_cast<const float4*>(&sm.Lt[q][4 * l4]);
+      const float fv[4] = {f.x, f.y, f.z, f.w};
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (4 * l4 + u > q) x[4 * l4 + u] -= x[q] * fv[u];
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
 // Grid form: n_c of any size, float64 or float32 factors, the matrices in
 // global memory (L2) and G CTAs per system.
 //
@@ -212,7 +360,6 @@ __global__ void __launch_bounds__(256) k_z2_update(RedArgs<float> a) {
 // where they ran one after the other (60k face, 8 frames, two of them with
 // n_c > 128: 1,760 -> 375 us per iteration).
 // ---------------------------------------------------------------------------
-constexpr int kBk = 32;                     // block edge
 constexpr int kSpinLimit = 1 << 21;         // polls of a barrier before it gives up (about a second)
 
 // systems of a launch: grid = G n CTAs, CTA b works on system b / G
@@ -283,13 +430,24 @@ __device__ __forceinline__ void group_sync(GroupBar& b) {
     __syncthreads();
   }
 }
-__device__ __forceinline__ void group_leave(GroupBar& b) {
+// arrive without waiting (the CTA's stores before it are published)
+__device__ __forceinline__ void group_arrive(GroupBar& b) {
+  __syncthreads();
+  if (threadIdx.x == 0 && b.G > 1) {
+    b.target += b.G;
+    __threadfence();
+    atomicAdd(b.word, 1u);
+  }
+}
+// the last CTA to leave resets the counters (of `more` too)
+__device__ __forceinline__ void group_leave(GroupBar& b, unsigned* more) {
   __syncthreads();
   if (threadIdx.x == 0 && b.G > 1) {
     __threadfence();
     if (atomicAdd(b.word + 1, 1u) == (unsigned)b.G - 1u) {
       b.word[0] = 0;
       b.word[1] = 0;
+      if (more) more[0] = 0;
       __threadfence();
     }
   }
@@ -299,38 +457,14 @@ __device__ __forceinline__ void group_leave(GroupBar& b) {
 template <typename T>
 __device__ __forceinline__ T ldg2(const T* p) { return __ldcg(p); }
 
-// x 2^-e and the significand of x (x = m 2^e, 1 <= m < 2), x positive and normal
-__device__ __forceinline__ int exponent_of(float x) {
-  return ((__float_as_int(x) >> 23) & 255) - 127;
-}
-__device__ __forceinline__ float significand(float x) {
-  return __int_as_float((__float_as_int(x) & 0x007fffff) | 0x3f800000);
-}
-__device__ __forceinline__ float scale_down(float x, int e) {
-  return x * __int_as_float((127 - max(-126, min(126, e))) << 23);
-}
-__device__ __forceinline__ int exponent_of(double x) {
-  return ((__double2hiint(x) >> 20) & 2047) - 1023;
-}
-__device__ __forceinline__ double significand(double x) {
-  return __hiloint2double((__double2hiint(x) & 0x000fffff) | 0x3ff00000, __double2loint(x));
-}
-__device__ __forceinline__ double scale_down(double x, int e) {   // integer work only
-  const int h = __double2hiint(x), ne = ((h >> 20) & 2047) - e;
-  return ne > 0 && ne < 2047 && ((h >> 20) & 2047) != 0
-             ? __hiloint2double(h - (int)((unsigned)e << 20), __double2loint(x))
-             : 0.0;
-}
-__device__ __forceinline__ float rsqrt_ft(float v) {
-  float r = rsqrtf(v);
-  return r * (1.5f - 0.5f * v * r * r);
-}
-__device__ __forceinline__ double rsqrt_ft(double v) { return rsqrt(v); }
-
 template <typename FT>
 struct GridSmem {
   union {
-    struct {                       // diagonal block (CTA 0)
+    struct {                       // float32 diagonal blocks (CTA 0), block row's panel
+      ChSm ch;
+      float Pt[kBk][kBk + 1];      // [l][row]
+    } c;
+    struct {                       // float64 diagonal block (CTA 0)
       FT P[kBk][kBk + 1];
       FT col[kBk][kBk + 1];        // col[j][r]: column j before its scaling
       FT rs[kBk], dv[kBk];
@@ -357,40 +491,16 @@ struct GridSmem {
   };
 };
 
-// element e of the lower triangle of a 32 x 32 block, columns from the last to
-// the first: the elements of the columns > j are then the first ones, so that
-// the work left after column j fills whole warps
-__device__ __forceinline__ void tri_element(int e, int& r, int& c) {
-  int m = (int)((sqrtf(8.f * e + 1.f) - 1.f) * 0.5f);      // column 31 - m holds m + 1 elements
-  while ((m + 1) * (m + 2) / 2 <= e) ++m;
-  while (m * (m + 1) / 2 > e) --m;
-  c = kBk - 1 - m;
-  r = c + e - m * (m + 1) / 2;
-}
-
-// CTA 0: D = A(k, k) - P P^T (P the block row's panel of the step before; none
-// when kp < 0), its Cholesky factor into A, and the factor transposed with
-// 1 / diag into dg.
-//
-// The elimination is free of divisions: with pivot p = ph 2^e (1 <= ph < 2),
-//   D[r][c] <- D[r][c] ph - D[r][j] (D[c][j] 2^-e),
-// which is the Schur complement times ph, so that after column j every entry
-// carries the product of the ph so far (at most 2^31).  A column then costs two
-// dependent operations and a barrier; the reciprocal (float32: hardware
-// approximation; float64: half a dozen dependent float64 operations of about
-// 66 cycles) is off the chain, and the square roots of all columns are taken
-// at once at the end.  Every thread owns two elements of the triangle (16
-// threads a third one, in column 0, which no step changes).
-template <typename FT>
-__device__ void grid_diag(FT* A, int k, int ld, int kp, FT* dg, int* info, GridSmem<FT>& sm) {
+// float64, CTA 0: D = A(k, k) - P P^T (P the block row's panel of the step
+// before; none when kp < 0), its Cholesky factor into A, and the factor
+// transposed with 1 / diag into dg.  The elimination is diag_factor's; in
+// float64 the reciprocal it avoids would be half a dozen dependent operations
+// of about 66 cycles per column.  All global loads are issued together.
+__device__ void grid_diag(double* A, int k, int ld, int kp, double* dg, int* info,
+                          GridSmem<double>& sm) {
   const int tid = threadIdx.x;
   const size_t o = (size_t)kBk * k * ld + kBk * k;
-  __syncthreads();
-  if (kp >= 0)
-    for (int e = tid; e < kBk * kBk; e += kRT)
-      sm.d.P[e >> 5][e & 31] = ldg2(A + (size_t)(kBk * k + (e >> 5)) * ld + kBk * kp + (e & 31));
-  __syncthreads();
-  FT v[3];
+  double v[3], pre[4];
   int er[3], ec[3];
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
@@ -399,30 +509,44 @@ __device__ void grid_diag(FT* A, int k, int ld, int kp, FT* dg, int* info, GridS
     ec[q] = -1;
     if (e >= kBk * (kBk + 1) / 2) continue;
     tri_element(e, er[q], ec[q]);
-    FT x = ldg2(A + o + (size_t)er[q] * ld + ec[q]);
+    v[q] = ldg2(A + o + (size_t)er[q] * ld + ec[q]);
+  }
+  if (kp >= 0)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int e = tid + q * kRT;
+      pre[q] = ldg2(A + (size_t)(kBk * k + (e >> 5)) * ld + kBk * kp + (e & 31));
+    }
+  __syncthreads();
+  if (kp >= 0)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) sm.d.P[(tid + q * kRT) >> 5][tid & 31] = pre[q];
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    if (ec[q] < 0) continue;
     if (kp >= 0) {
-      FT a0 = 0, a1 = 0;
+      double a0 = 0.0, a1 = 0.0;
 #pragma unroll 8
       for (int l = 0; l < kBk; l += 2) {
         a0 += sm.d.P[er[q]][l] * sm.d.P[ec[q]][l];
         a1 += sm.d.P[er[q]][l + 1] * sm.d.P[ec[q]][l + 1];
       }
-      x -= a0 + a1;
+      v[q] -= a0 + a1;
     }
-    v[q] = x;
-    if (ec[q] == 0) sm.d.col[0][er[q]] = x;
+    if (ec[q] == 0) sm.d.col[0][er[q]] = v[q];
   }
   for (int j = 0; j + 1 < kBk; ++j) {
     __syncthreads();
     if (ec[0] <= j && ec[1] <= j) continue;          // (elements 0 and 1 exist for every thread)
-    FT p = sm.d.col[j][j];
-    if (!(p > FT(0))) p = FT(1);                     // reported below
+    double p = sm.d.col[j][j];
+    if (!(p > 0.0)) p = 1.0;                         // reported below
     const int e = exponent_of(p);
-    const FT ph = significand(p);
+    const double ph = significand(p);
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
       if (ec[q] <= j) continue;
-      const FT w = scale_down(sm.d.col[j][ec[q]], e);
+      const double w = scale_down(sm.d.col[j][ec[q]], e);
       v[q] = v[q] * ph - sm.d.col[j][er[q]] * w;
       if (ec[q] == j + 1) sm.d.col[j + 1][er[q]] = v[q];
     }
@@ -431,35 +555,82 @@ __device__ void grid_diag(FT* A, int k, int ld, int kp, FT* dg, int* info, GridS
   if (tid < kBk) {
     // pi = product of the significands before column tid; the true pivot is
     // col[j][j] / pi, so L[r][j] = col[j][r] / sqrt(col[j][j] pi)
-    FT p = sm.d.col[tid][tid];
-    const bool bad = !(p > FT(0));
-    if (bad) { atomicOr(info, 1); p = FT(1); }
-    FT pi = significand(p);
+    double p = sm.d.col[tid][tid];
+    const bool bad = !(p > 0.0);
+    if (bad) { atomicOr(info, 1); p = 1.0; }
+    double pi = significand(p);
 #pragma unroll
     for (int s = 1; s < 32; s <<= 1) {
-      const FT x = __shfl_up_sync(0xffffffffu, pi, s);
+      const double x = __shfl_up_sync(0xffffffffu, pi, s);
       if (tid >= s) pi *= x;
     }
     pi = __shfl_up_sync(0xffffffffu, pi, 1);
-    if (tid == 0) pi = FT(1);
-    const FT rs = rsqrt_ft(p * pi);
+    if (tid == 0) pi = 1.0;
+    const double rs = rsqrt(p * pi);
     sm.d.rs[tid] = rs;
     sm.d.dv[tid] = pi * rs;
     dg[kBk * kBk + tid] = pi * rs;
-    if (bad) sm.d.col[tid][tid] = FT(1);
+    if (bad) sm.d.col[tid][tid] = 1.0;
   }
   __syncthreads();
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
     if (ec[q] < 0) continue;
-    const FT x = sm.d.col[ec[q]][er[q]] * sm.d.rs[ec[q]];
+    const double x = sm.d.col[ec[q]][er[q]] * sm.d.rs[ec[q]];
     A[o + (size_t)er[q] * ld + ec[q]] = x;
     dg[ec[q] * kBk + er[q]] = x;
   }
 }
 
-// Panel k: every row below the diagonal block and every identity row so far,
-// x L_kk^T = a.  A row is one thread with its 32 values in registers (float32),
+// float32, CTA 0, which also solves the panel rows of the next block itself: it
+// has the factor of block k in shared memory, so block k + 1 waits neither for
+// the other CTAs' panel nor for theirs to reach it.  `step` is called when the
+// panel rows are stored.  (A mixed slabs frame, n_c > 128: 4 % less time than with
+// the block factored after the trailing update.)
+template <typename Step>
+__device__ void grid_next_diag(float* A, int k1, int ld, float* dg, int* info, GridSmem<float>& sm,
+                               Step step) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  const size_t o = (size_t)kBk * k1 * ld + kBk * k1;
+  float pre[3];                  // this thread's elements of the block, on their way
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    int r, c;
+    if (tid + q * kDT >= kBk * (kBk + 1) / 2) continue;
+    tri_element(tid + q * kDT, r, c);
+    pre[q] = ldg2(A + o + (size_t)r * ld + c);
+  }
+  if (k1 > 0 && tid < 32) {
+    float4* row = reinterpret_cast<float4*>(A + (size_t)(kBk * k1 + lane) * ld + kBk * (k1 - 1));
+    float x[32];
+#pragma unroll
+    for (int l = 0; l < 8; ++l) {
+      const float4 f = ldg2(row + l);
+      x[4 * l] = f.x; x[4 * l + 1] = f.y; x[4 * l + 2] = f.z; x[4 * l + 3] = f.w;
+    }
+    panel_row(sm.c.ch, x);
+#pragma unroll
+    for (int l = 0; l < 8; ++l)
+      row[l] = make_float4(x[4 * l], x[4 * l + 1], x[4 * l + 2], x[4 * l + 3]);
+#pragma unroll
+    for (int l = 0; l < 32; ++l) sm.c.Pt[l][lane] = x[l];
+  }
+  __syncthreads();
+  if (k1 > 0) step();
+  int nth = 0;                   // diag_factor asks for the elements in that order
+  diag_factor(
+      sm.c.ch, k1 > 0 ? &sm.c.Pt[0][0] : nullptr, kBk + 1, info, [&](int, int) { return pre[nth++]; },
+      [&](int r, int c, float x) {
+        A[o + (size_t)r * ld + c] = x;
+        dg[c * kBk + r] = x;
+      });
+  __syncthreads();
+  if (tid < kBk) dg[kBk * kBk + tid] = sm.c.ch.dv[tid];
+}
+
+// Panel k: every row below the diagonal block (float32: not those of block k + 1,
+// which CTA 0 solves) and every identity row so far, x L_kk^T = a.  A row is one
+// thread with its 32 values in registers (float32),
 // or one warp (float64: 32 x 2 dependent warp instructions per row where a
 // thread per row would need 528 per warp), four rows per CTA at a time so that
 // each SM sub-partition has one.
@@ -467,11 +638,11 @@ __device__ void grid_panel(float* A, float* U, int k, int nb, int ld, const floa
                            GridSmem<float>& sm) {
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   if (rank >= nb) return;
-  for (int e = tid; e < kBk * kBk / 4; e += kRT)
-    reinterpret_cast<float4*>(&sm.p.Lt[0][0])[e] = ldg2(reinterpret_cast<const float4*>(dg) + e);
-  if (tid < kBk) sm.p.dv[tid] = ldg2(dg + kBk * kBk + tid);
+  for (int e = tid; e < (kBk * kBk + kBk) / 4; e += kRT)      // Lt, dv
+    reinterpret_cast<float4*>(&sm.c.ch)[e] = ldg2(reinterpret_cast<const float4*>(dg) + e);
   __syncthreads();
   for (int b = rank + wid * G; b < nb; b += (kRT / 32) * G) {
+    if (b == k + 1) continue;
     float* row = (b > k ? A : U) + (size_t)(kBk * b + lane) * ld + kBk * k;
     float x[kBk];
     if (b == k) {
@@ -484,12 +655,7 @@ __device__ void grid_panel(float* A, float* U, int k, int nb, int ld, const floa
         x[4 * l] = f.x; x[4 * l + 1] = f.y; x[4 * l + 2] = f.z; x[4 * l + 3] = f.w;
       }
     }
-#pragma unroll
-    for (int q = 0; q < kBk; ++q) {
-      x[q] *= sm.p.dv[q];
-#pragma unroll
-      for (int l = q + 1; l < kBk; ++l) x[l] -= x[q] * sm.p.Lt[q][l];
-    }
+    panel_row(sm.c.ch, x);
 #pragma unroll
     for (int l = 0; l < kBk / 4; ++l)
       reinterpret_cast<float4*>(row)[l] = make_float4(x[4 * l], x[4 * l + 1], x[4 * l + 2], x[4 * l + 3]);
@@ -624,23 +790,59 @@ __device__ void grid_trail(double* A, double* U, int k, int nb, int ld, int slot
 }
 
 // A = L L^T (nb x nb blocks, lower; L in place) and U = L^-T (upper)
-template <typename FT>
-__device__ void grid_chol(FT* A, FT* U, int nb, int ld, FT* dg, GroupBar& bar, int rank,
-                          GridSmem<FT>& sm) {
+__device__ void grid_chol(double* A, double* U, int nb, int ld, double* dg, GroupBar& bar, int rank,
+                          GridSmem<double>& sm) {
   constexpr int kDg = kBk * kBk + kBk;
-  if (rank == 0) grid_diag<FT>(A, 0, ld, -1, dg, bar.info, sm);
+  if (rank == 0) grid_diag(A, 0, ld, -1, dg, bar.info, sm);
   group_sync(bar);
   for (int k = 0; k < nb; ++k) {
     grid_panel(A, U, k, nb, ld, dg + (k & 1) * kDg, rank, bar.G, sm);
     group_sync(bar);
     if (k + 1 < nb) {
       if (rank == 0) {
-        grid_diag<FT>(A, k + 1, ld, k, dg + ((k + 1) & 1) * kDg, bar.info, sm);
+        grid_diag(A, k + 1, ld, k, dg + ((k + 1) & 1) * kDg, bar.info, sm);
         __syncthreads();
       }
       if (bar.G == 1) grid_trail(A, U, k, nb, ld, 0, 1, sm);
       else if (rank > 0) grid_trail(A, U, k, nb, ld, rank - 1, bar.G - 1, sm);
       group_sync(bar);
+    }
+  }
+}
+// float32: CTA 0 only arrives at the first barrier of a panel (with its rows of
+// it stored) and makes the next diagonal factor; the others share the rest of
+// the panel and the trailing update.  `panel` counts the arrivals of the first
+// barrier apart from the second's, which CTA 0 may reach early.
+__device__ void grid_chol(float* A, float* U, int nb, int ld, float* dg, GroupBar& bar, GroupBar& panel,
+                          int rank, GridSmem<float>& sm) {
+  constexpr int kDg = kBk * kBk + kBk;
+  const bool lone = bar.G == 1;
+  if (rank == 0) grid_next_diag(A, 0, ld, dg, bar.info, sm, [] {});
+  group_sync(bar);
+  for (int k = 0; k < nb; ++k) {
+    if (rank == 0) {
+      if (k + 1 < nb)
+        grid_next_diag(A, k + 1, ld, dg + ((k + 1) & 1) * kDg, bar.info, sm, [&] { group_arrive(panel); });
+      else
+        group_arrive(panel);
+    }
+    if (rank > 0 || lone) {
+      if (lone) __syncthreads();
+      grid_panel(A, U, k, nb, ld, dg + (k & 1) * kDg, lone ? 0 : rank - 1, lone ? 1 : bar.G - 1, sm);
+      if (k + 1 < nb) {
+        if (lone) __syncthreads();
+        else group_sync(panel);
+        grid_trail(A, U, k, nb, ld, lone ? 0 : rank - 1, lone ? 1 : bar.G - 1, sm);
+      } else if (!lone) {
+        group_arrive(panel);
+      }
+    }
+    group_sync(bar);
+    if (lone && k + 1 < nb) {        // the factor of block k + 1 back into shared memory
+      for (int e = threadIdx.x; e < kDg / 4; e += kRT)
+        reinterpret_cast<float4*>(&sm.c.ch)[e] =
+            ldg2(reinterpret_cast<const float4*>(dg + ((k + 1) & 1) * kDg) + e);
+      __syncthreads();
     }
   }
 }
@@ -661,7 +863,11 @@ __device__ void grid_prepare(RedArgs<FT> a, int rank, int G, GridSmem<FT>& sm) {
   red_tail(a, nc);
   G = grid_ctas<FT>(g.nbn, G);
   if (rank >= G) return;
-  GroupBar bar{a.bar, 0u, G, a.info, false};
+  GroupBar bar{a.bar, 0u, G, a.info, false}, panel{a.bar + 4, 0u, G, a.info, false};
+  auto chol = [&](FT* M, FT* V, int nb, int ld) {
+    if constexpr (std::is_same<FT, double>::value) grid_chol(M, V, nb, ld, g.dg, bar, rank, sm);
+    else grid_chol(M, V, nb, ld, g.dg, bar, panel, rank, sm);
+  };
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, n3 = g.n3;
   const int gwarp = rank * (kRT / 32) + wid, nwarps = G * (kRT / 32);
   // 1. S (lower, padded by the identity) and the block-row lists
@@ -682,7 +888,7 @@ __device__ void grid_prepare(RedArgs<FT> a, int rank, int G, GridSmem<FT>& sm) {
   }
   group_sync(bar);
   // 2. L_s, U_s
-  grid_chol<FT>(g.S, g.Us, g.nbs, g.lds, g.dg, bar, rank, sm);
+  chol(g.S, g.Us, g.nbs, g.lds);
   // 3. X[(i,a),(k,b)] = sum_{j in row i, j >= k} B[(i,a),(j,b)] L_s[j][k]: a CTA
   // takes block row i and 256 columns k, the row's blocks of B staged (64 at a
   // time) in the factor's type; a thread keeps the nine values of one k
@@ -775,8 +981,8 @@ __device__ void grid_prepare(RedArgs<FT> a, int rank, int G, GridSmem<FT>& sm) {
   }
   group_sync(bar);
   // 5. L_N, U_N (over X)
-  grid_chol<FT>(g.N, g.U, g.nbn, g.ldn, g.dg, bar, rank, sm);
-  group_leave(bar);
+  chol(g.N, g.U, g.nbn, g.ldn);
+  group_leave(bar, a.bar + 4);
 }
 
 // out = (L_s (x) I_3)^T p (padded with zeros), one warp per entry
@@ -983,7 +1189,7 @@ __device__ void grid_solve(RedArgs<FT> a, int rank, int Gall, GridSmem<FT>& sm) 
   }
   // 8. z2 = u - (Sigma^-1[:, c] (x) I_3) v
   z2_update(a, nc, gwarp, nwarps);
-  group_leave(bar);
+  group_leave(bar, nullptr);
 }
 
 // A: per-system arguments on the device (batches), else `one`
@@ -1339,7 +1545,7 @@ __global__ void __launch_bounds__(256) k_small_n(RedArgs<float> a) {
 // term, the kRP parts (consecutive lanes) are summed by shuffles.  t is the
 // thread's index among nt threads taking part (nt a multiple of 32, the
 // same loop trip count in every lane).
-constexpr int kRP = 4;
+constexpr int kRP = 16;
 
 // w = S v with S = Sigma^-1[c, c] (x) I_3 (S64 gathered by k_small_s)
 __device__ void refine_sv(const RedArgs<float>& a, int nc, int t, int nt) {
@@ -1548,8 +1754,8 @@ __global__ void __launch_bounds__(kRT) k_small_u(RedArgs<float> a) {
 // cluster of kSolveCl CTAs: the vectors live in global memory and a cluster
 // barrier separates the products.  Warps and threads are numbered interleaved
 // over the CTAs, so that every SM gets its share of the float64 work.
-constexpr int kSolveCl = 8;
-constexpr int kSolveW = kRT / 32;           // warps per CTA
+constexpr int kSolveCl = 8, kSolveT = 512;
+constexpr int kSolveW = kSolveT / 32;       // warps per CTA
 __device__ __forceinline__ void k_small_solve_body(RedArgs<float> a) {
   namespace cgx = cooperative_groups;
   cgx::cluster_group cl = cgx::this_cluster();
@@ -1711,7 +1917,7 @@ __device__ __forceinline__ void k_small_solve_body(RedArgs<float> a) {
   }
   cl.sync();       // no CTA leaves while its shared memory may still be written
 }
-__global__ void __launch_bounds__(kRT) k_small_solve(RedArgs<float> a) {
+__global__ void __launch_bounds__(kSolveT) k_small_solve(RedArgs<float> a) {
   k_small_solve_body(a);
 }
 
@@ -2038,7 +2244,7 @@ template <typename K, typename A>
 cudaError_t launch_solve_clusters(cudaStream_t s, K kernel, int nsys, const A& arg) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(kSolveCl, nsys);
-  cfg.blockDim = dim3(kRT);
+  cfg.blockDim = dim3(kSolveT);
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
@@ -2180,7 +2386,7 @@ __global__ void __launch_bounds__(kRT) k_small_u_b(const RedArgs<float>* __restr
   const RedArgs<float> a = A[blockIdx.y];
   if (a.active) k_small_u_body(a, blockIdx.x);
 }
-__global__ void __launch_bounds__(kRT) k_small_solve_b(const RedArgs<float>* __restrict__ A) {
+__global__ void __launch_bounds__(kSolveT) k_small_solve_b(const RedArgs<float>* __restrict__ A) {
   const RedArgs<float> a = A[blockIdx.y];
   if (a.active) k_small_solve_body(a);       // uniform over a cluster
 }
