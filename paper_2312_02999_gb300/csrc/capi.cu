@@ -43,6 +43,21 @@ int dalloc(std::vector<void*>& allocs, T** p, size_t count, size_t* bytes = null
 template <typename T>
 int dalloc(MeshState& ms, T** p, size_t count) { return dalloc(ms.allocs, p, count); }
 
+// Where a workspace's buffers come from: allocations of their own (listed in
+// allocs, added to *bytes), or places in one arena.
+struct DeviceMem {
+  std::vector<void*>* allocs;
+  size_t* bytes;
+  Arena* arena;
+  template <typename T>
+  int take(T** p, size_t count) {
+    if (!arena) return dalloc(*allocs, p, count, bytes);
+    if (bytes) *bytes += sizeof(T) * std::max<size_t>(count, 1);
+    *p = static_cast<T*>(arena->take(sizeof(T) * std::max<size_t>(count, 1)));
+    return FSIM_OK;
+  }
+};
+
 #define TRY(x)                    \
   do {                            \
     int s_ = (x);                 \
@@ -117,6 +132,18 @@ size_t reduced_bytes(int cap) {
          (sizeof(double) + sizeof(float)) * (size_t)reduced_workspace_elems(cap);
 }
 
+// The reduced-system buffers of workspace m for cap contact vertices.
+int reduced_buffers(DeviceMem mem, DevMesh& m, int cap) {
+  const int64_t n3 = 3 * (int64_t)cap;
+  TRY(mem.take(&m.Bc, (size_t)(n3 * n3)));
+  TRY(mem.take(&m.bocc, (size_t)(2 * (int64_t)cap * cap + cap + 32)));
+  m.red_cap = reduced_workspace_elems(cap);
+  TRY(mem.take(&m.red, (size_t)m.red_cap));
+  TRY(mem.take(&m.redf, (size_t)m.red_cap));
+  m.nc_cap = cap;
+  return FSIM_OK;
+}
+
 int ensure_reduced(const Exec& ex, DevMesh& m, int nc) {
   if (nc <= m.nc_cap && m.Bc != nullptr) return FSIM_OK;
   int cap = std::max(nc, std::max(16, m.nc_cap * 3 / 2));
@@ -126,24 +153,19 @@ int ensure_reduced(const Exec& ex, DevMesh& m, int nc) {
   if (ex.grow && new_bytes > old_bytes && ex.grow(ex.grow_user, new_bytes - old_bytes) != 0)
     return FSIM_ENOMEM;
   CK(cudaStreamSynchronize(ex.stream));
-  auto release = [&](void* p) {
-    if (!p) return;
-    cudaFree(p);
+  auto release = [&](void* p) {      // (a buffer of a batch's one allocation stays in it)
     auto& v = *ex.allocs;
-    v.erase(std::remove(v.begin(), v.end(), p), v.end());
+    const auto it = std::find(v.begin(), v.end(), p);
+    if (it == v.end()) return;
+    cudaFree(p);
+    v.erase(it);
   };
   release(m.Bc); release(m.bocc); release(m.red); release(m.redf);
   m.Bc = nullptr; m.bocc = nullptr; m.red = nullptr; m.redf = nullptr;
   if (ex.bytes) *ex.bytes -= std::min(*ex.bytes, old_bytes);
-  const int64_t n3 = 3 * (int64_t)cap;
-  TRY(dalloc(*ex.allocs, &m.Bc, (size_t)(n3 * n3), ex.bytes));
-  TRY(dalloc(*ex.allocs, &m.bocc, (size_t)(2 * (int64_t)cap * cap + cap + 32), ex.bytes));
+  TRY(reduced_buffers(DeviceMem{ex.allocs, ex.bytes, nullptr}, m, cap));
   // the barrier counters after the lists start at zero (and are left at zero)
   CK(cudaMemsetAsync(m.bocc + 2 * (int64_t)cap * cap + cap, 0, sizeof(int) * 32, ex.stream));
-  m.red_cap = reduced_workspace_elems(cap);
-  TRY(dalloc(*ex.allocs, &m.red, (size_t)m.red_cap, ex.bytes));
-  TRY(dalloc(*ex.allocs, &m.redf, (size_t)m.red_cap, ex.bytes));
-  m.nc_cap = cap;
   m.red_gen++;
   return FSIM_OK;
 }
@@ -151,13 +173,84 @@ int ensure_reduced(const Exec& ex, DevMesh& m, int nc) {
 // Per-solve buffers of a workspace (everything a frame solve writes).  The
 // constant mesh data (factor, Sigma^-1, topology) stays shared.  Used for
 // the mesh's own workspace at prefactor and for the server's extra slots.
-int alloc_workspace(const MeshState& ms, DevMesh& m, std::vector<void*>& al, size_t* bytes) {
+// With an arena that has no memory yet, only adds up the bytes.
+int alloc_workspace(const MeshState& ms, DevMesh& m, DeviceMem mem) {
   // a copy must never replay (or destroy) another workspace's graphs, nor
   // use its side stream
   for (auto& g : m.graphs) g = DevMesh::Graph{};
   m.red_gen = 0;
   m.aux_stream = m.aux_stream2 = nullptr;
   m.ev_fork = m.ev_join = m.ev_fork2 = m.ev_join2 = nullptr;
+  const size_t n = m.n, T = m.T, Ns = m.Ns;
+  const size_t np = (size_t)m.Ns + m.Nt + m.Ne;
+  TRY(mem.take(&m.x, 3 * n));
+  TRY(mem.take(&m.xt, 3 * n));
+  TRY(mem.take(&m.dx, 3 * n));
+  TRY(mem.take(&m.g, 3 * n));
+  TRY(mem.take(&m.act, 6 * T));
+  TRY(mem.take(&m.act_df, 6 * T));
+  TRY(mem.take(&m.udf, 3 * n));
+  TRY(mem.take(&m.tetf, 12 * T));
+  TRY(mem.take(&m.tetf_t, 12 * T));
+  TRY(mem.take(&m.s, 3 * Ns));
+  TRY(mem.take(&m.st, 3 * Ns));
+  TRY(mem.take(&m.ds, 3 * Ns));
+  TRY(mem.take(&m.pbox, 12 * np));
+  TRY(mem.take(&m.pkey, 12 * np));
+  TRY(mem.take(&m.sf, 3 * Ns));
+  TRY(mem.take(&m.dsf, 3 * Ns));
+  char* zero = nullptr;
+  {   // scalars, then counters (read back by one copy); the skin list starts invalid
+    char* status = nullptr;
+    TRY(mem.take(&status, kStatusBytes));
+    zero = status;
+    m.scal = reinterpret_cast<double*>(status);
+    m.counters = reinterpret_cast<int*>(status + sizeof(double) * kScal);
+  }
+  TRY(mem.take(&m.partials, (size_t)m.n_partials));
+  TRY(mem.take(&m.y1, 3 * (size_t)std::max(m.n1, 1)));
+  TRY(mem.take(&m.y1f, 3 * (size_t)std::max(m.n1, 1)));
+  TRY(mem.take(&m.r, 3 * (size_t)m.nf));
+  TRY(mem.take(&m.u, 3 * (size_t)std::max(m.n2, 1)));
+  TRY(mem.take(&m.rf, 3 * (size_t)m.nf + 8));
+  TRY(mem.take(&m.bx, 3 * (size_t)m.nf + 8));
+  TRY(mem.take(&m.uf, 3 * (size_t)std::max(m.n2, 1)));
+  TRY(mem.take(&m.pairs, (size_t)m.cap_act));
+  TRY(mem.take(&m.cand, (size_t)m.cap));
+  TRY(mem.take(&m.nearl, (size_t)m.cap));
+  TRY(mem.take(&m.vlist, (size_t)m.cap));
+  if (ms.p.solver == FSIM_SOLVER_PCG) {
+    TRY(mem.take(&m.cg_r, 3 * n));
+    TRY(mem.take(&m.cg_z, 3 * n));
+    TRY(mem.take(&m.cg_p, 3 * n));
+    TRY(mem.take(&m.cg_q, 3 * n));
+    TRY(mem.take(&m.cg_tmp, 3 * n));
+    TRY(mem.take(&m.cg_red, 2));
+  }
+  if (ms.p.solver == FSIM_SOLVER_SCHUR && m.n2 > 0) {
+    const size_t N = 3 * (size_t)m.n2;
+    TRY(mem.take(&m.sh_A, N * N));
+    TRY(mem.take(&m.sh_Af, N * N));
+    TRY(mem.take(&m.sh_y, N));
+    TRY(mem.take(&m.sh_r, N));
+    TRY(mem.take(&m.sh_df, N));
+  }
+  TRY(mem.take(&m.sb, 3 * Ns + 3));
+  TRY(mem.take(&m.pair_grad, 12 * (size_t)m.cap_act));
+  TRY(mem.take(&m.pair_hess, 144 * (size_t)m.cap_act));
+  TRY(mem.take(&m.x2mark, (size_t)std::max(m.n2, 1)));
+  TRY(mem.take(&m.clist, (size_t)std::max(m.n2, 1)));
+  m.Bc = nullptr; m.bocc = nullptr; m.red = nullptr; m.redf = nullptr;
+  m.red_cap = 0; m.nc_cap = 0;
+  if (mem.arena && !mem.arena->base) return FSIM_OK;
+  CK(cudaMemset(zero, 0, kStatusBytes));
+  CK(cudaMemset(m.sb + 3 * Ns, 0, sizeof(double) * 3));      // words of k_skin_check
+  return FSIM_OK;
+}
+
+// The workspace's side streams and their events (once).
+int workspace_streams(DevMesh& m) {
+  if (m.aux_stream) return FSIM_OK;
   if (cudaStreamCreateWithFlags(&m.aux_stream, cudaStreamNonBlocking) != cudaSuccess ||
       cudaStreamCreateWithFlags(&m.aux_stream2, cudaStreamNonBlocking) != cudaSuccess ||
       cudaEventCreateWithFlags(&m.ev_fork, cudaEventDisableTiming) != cudaSuccess ||
@@ -167,68 +260,6 @@ int alloc_workspace(const MeshState& ms, DevMesh& m, std::vector<void*>& al, siz
     cudaGetLastError();
     return FSIM_ECUDA;
   }
-  const size_t n = m.n, T = m.T, Ns = m.Ns;
-  const size_t np = (size_t)m.Ns + m.Nt + m.Ne;
-  TRY(dalloc(al, &m.x, 3 * n, bytes));
-  TRY(dalloc(al, &m.xt, 3 * n, bytes));
-  TRY(dalloc(al, &m.dx, 3 * n, bytes));
-  TRY(dalloc(al, &m.g, 3 * n, bytes));
-  TRY(dalloc(al, &m.act, 6 * T, bytes));
-  TRY(dalloc(al, &m.act_df, 6 * T, bytes));
-  TRY(dalloc(al, &m.udf, 3 * n, bytes));
-  TRY(dalloc(al, &m.tetf, 12 * T, bytes));
-  TRY(dalloc(al, &m.tetf_t, 12 * T, bytes));
-  TRY(dalloc(al, &m.s, 3 * Ns, bytes));
-  TRY(dalloc(al, &m.st, 3 * Ns, bytes));
-  TRY(dalloc(al, &m.ds, 3 * Ns, bytes));
-  TRY(dalloc(al, &m.pbox, 12 * np, bytes));
-  TRY(dalloc(al, &m.pkey, 12 * np, bytes));
-  TRY(dalloc(al, &m.sf, 3 * Ns, bytes));
-  TRY(dalloc(al, &m.dsf, 3 * Ns, bytes));
-  {   // scalars, then counters (read back by one copy)
-    char* status = nullptr;
-    TRY(dalloc(al, &status, kStatusBytes, bytes));
-    CK(cudaMemset(status, 0, kStatusBytes));                 // skin list starts invalid
-    m.scal = reinterpret_cast<double*>(status);
-    m.counters = reinterpret_cast<int*>(status + sizeof(double) * kScal);
-  }
-  TRY(dalloc(al, &m.partials, (size_t)m.n_partials, bytes));
-  TRY(dalloc(al, &m.y1, 3 * (size_t)std::max(m.n1, 1), bytes));
-  TRY(dalloc(al, &m.y1f, 3 * (size_t)std::max(m.n1, 1), bytes));
-  TRY(dalloc(al, &m.r, 3 * (size_t)m.nf, bytes));
-  TRY(dalloc(al, &m.u, 3 * (size_t)std::max(m.n2, 1), bytes));
-  TRY(dalloc(al, &m.rf, 3 * (size_t)m.nf + 8, bytes));
-  TRY(dalloc(al, &m.bx, 3 * (size_t)m.nf + 8, bytes));
-  TRY(dalloc(al, &m.uf, 3 * (size_t)std::max(m.n2, 1), bytes));
-  TRY(dalloc(al, &m.pairs, (size_t)m.cap_act, bytes));
-  TRY(dalloc(al, &m.cand, (size_t)m.cap, bytes));
-  TRY(dalloc(al, &m.nearl, (size_t)m.cap, bytes));
-  TRY(dalloc(al, &m.vlist, (size_t)m.cap, bytes));
-  if (ms.p.solver == FSIM_SOLVER_PCG) {
-    TRY(dalloc(al, &m.cg_r, 3 * n, bytes));
-    TRY(dalloc(al, &m.cg_z, 3 * n, bytes));
-    TRY(dalloc(al, &m.cg_p, 3 * n, bytes));
-    TRY(dalloc(al, &m.cg_q, 3 * n, bytes));
-    TRY(dalloc(al, &m.cg_tmp, 3 * n, bytes));
-    TRY(dalloc(al, &m.cg_red, 2, bytes));
-  }
-  if (ms.p.solver == FSIM_SOLVER_SCHUR && m.n2 > 0) {
-    const size_t N = 3 * (size_t)m.n2;
-    TRY(dalloc(al, &m.sh_A, N * N, bytes));
-    TRY(dalloc(al, &m.sh_Af, N * N, bytes));
-    TRY(dalloc(al, &m.sh_y, N, bytes));
-    TRY(dalloc(al, &m.sh_r, N, bytes));
-    TRY(dalloc(al, &m.sh_df, N, bytes));
-  }
-  TRY(dalloc(al, &m.sb, 3 * Ns + 3, bytes));
-  CK(cudaMemset(m.sb + 3 * Ns, 0, sizeof(double) * 3));      // words of k_skin_check
-  TRY(dalloc(al, &m.pair_grad, 12 * (size_t)m.cap_act, bytes));
-  TRY(dalloc(al, &m.pair_hess, 144 * (size_t)m.cap_act, bytes));
-  TRY(dalloc(al, &m.x2mark, (size_t)std::max(m.n2, 1), bytes));
-  TRY(dalloc(al, &m.clist, (size_t)std::max(m.n2, 1), bytes));
-  m.Bc = nullptr; m.bocc = nullptr; m.red = nullptr; m.redf = nullptr;
-  m.red_cap = 0; m.nc_cap = 0;
-  (void)ms;
   return FSIM_OK;
 }
 
@@ -579,8 +610,17 @@ int solve_frame_impl(const Exec& ex, const MeshState& ms, DevMesh& m, const doub
 
 namespace fsim {
 int rt_alloc_workspace(const MeshState& ms, DevMesh& m, std::vector<void*>& allocs, size_t* bytes) {
-  return alloc_workspace(ms, m, allocs, bytes);
+  TRY(alloc_workspace(ms, m, DeviceMem{&allocs, bytes, nullptr}));
+  return workspace_streams(m);
 }
+int rt_place_workspace(const MeshState& ms, DevMesh& m, Arena& arena, int nc_cap, size_t* bytes) {
+  TRY(alloc_workspace(ms, m, DeviceMem{nullptr, bytes, &arena}));
+  TRY(reduced_buffers(DeviceMem{nullptr, nullptr, &arena}, m, nc_cap));
+  if (arena.base)
+    CK(cudaMemset(m.bocc + 2 * (int64_t)nc_cap * nc_cap + nc_cap, 0, sizeof(int) * 32));
+  return FSIM_OK;
+}
+int rt_workspace_streams(DevMesh& m) { return workspace_streams(m); }
 int rt_ensure_reduced(const Exec& ex, DevMesh& m, int nc) { return ensure_reduced(ex, m, nc); }
 size_t rt_reduced_bytes(int nc_cap) { return reduced_bytes(nc_cap); }
 int rt_solve_frame(const Exec& ex, const MeshState& ms, DevMesh& m, const double* x_init,
@@ -972,7 +1012,7 @@ fsim_status fsim_prefactor(fsim_ctx_t ctx, int mesh_id, const fsim_params* p) {
   TRY(dalloc(ms, &ms.gtmp, 3 * (size_t)m.n));
   TRY(dalloc(ms, &ms.dxtmp, 3 * (size_t)m.n));
   ms.ws_bytes = 0;
-  TRY(alloc_workspace(ms, m, ms.allocs, &ms.ws_bytes));
+  TRY(rt_alloc_workspace(ms, m, ms.allocs, &ms.ws_bytes));
   if (m.n1 > 0 && m.n2 > 0) {   // Phi = K11^-1 K12 Sigma^-1 for the mixed global step
     TRY(dalloc(ms, &m.Phi_t, (size_t)m.n1 * m.n2));
     CK(compute_phi(s, m, m.Phi_t));

@@ -485,6 +485,7 @@ k_gemm_mr(int n2, const float* __restrict__ A, const float* __restrict__ yv, flo
 __global__ void k_gather_rhs_mr(const DevMesh* __restrict__ tab, float* __restrict__ rb, int nr) {
   const DevMesh& m = tab[blockIdx.y];
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p == 0 && m.active) { m.counters[6] = 0; m.counters[7] = 0; }   // flags of this step
   if (p >= m.nf) return;
   float* dst = rb + (size_t)p * nr + 3 * m.col;
   if (!m.active) { dst[0] = 0.f; dst[1] = 0.f; dst[2] = 0.f; return; }
