@@ -117,10 +117,17 @@ Exec ctx_exec(fsim_ctx_t ctx, MeshState& ms) {
 
 // The scalars and the counters lie one after the other on the device and in the
 // pinned words (kStatusBytes): one copy reads both back.
-int sync_read(const Exec& ex, const DevMesh& m) {
+int copy_status(const Exec& ex, const DevMesh& m) {
   CK(cudaMemcpyAsync(ex.h_scal, m.scal, kStatusBytes, cudaMemcpyDeviceToHost, ex.stream));
+  return FSIM_OK;
+}
+int sync(const Exec& ex) {
   CK(cudaStreamSynchronize(ex.stream));
   return FSIM_OK;
+}
+int sync_read(const Exec& ex, const DevMesh& m) {
+  TRY(copy_status(ex, m));
+  return sync(ex);
 }
 
 // Make the reduced-system buffers of workspace m large enough for nc
@@ -214,7 +221,6 @@ int alloc_workspace(const MeshState& ms, DevMesh& m, DeviceMem mem) {
   TRY(mem.take(&m.u, 3 * (size_t)std::max(m.n2, 1)));
   TRY(mem.take(&m.rf, 3 * (size_t)m.nf + 8));
   TRY(mem.take(&m.bx, 3 * (size_t)m.nf + 8));
-  TRY(mem.take(&m.uf, 3 * (size_t)std::max(m.n2, 1)));
   TRY(mem.take(&m.pairs, (size_t)m.cap_act));
   TRY(mem.take(&m.cand, (size_t)m.cap));
   TRY(mem.take(&m.nearl, (size_t)m.cap));
@@ -288,7 +294,7 @@ int with_graph(const Exec& ex, DevMesh& m, int slot, const void* key, int key2, 
   DevMesh::Graph& g = m.graphs[slot];
   if (g.failed || prof_active()) return body();
   if (g.exec && (g.key != key || g.key2 != key2 || g.gen != gen || g.coop != ex.coop_ctas ||
-                 g.alone != ex.alone)) {
+                 g.alone != ex.alone || g.host != ex.h_scal)) {
     cudaGraphExecDestroy((cudaGraphExec_t)g.exec);
     g.exec = nullptr;
   }
@@ -324,6 +330,7 @@ int with_graph(const Exec& ex, DevMesh& m, int slot, const void* key, int key2, 
       return body();      // nothing ran during the capture: launch directly
     }
     g.exec = exec; g.key = key; g.key2 = key2; g.gen = gen; g.coop = ex.coop_ctas; g.alone = ex.alone;
+    g.host = ex.h_scal;
     g.kernels = kernels;
   }
   CK(cudaGraphLaunch((cudaGraphExec_t)g.exec, ex.stream));
@@ -355,10 +362,10 @@ int graph_slot(const DevMesh& m, int first, int count, const void* key, int key2
 // local step is left out (a caller that only wants the contacts).
 // ---------------------------------------------------------------------------
 int evaluate(const Exec& ex, const MeshState& ms, const DevMesh& m, const double* xb, double* sb,
-             double* tetf, double* proj, int prec, double kappa) {
+             double* tetf, double* proj, int prec, double kappa, bool disp_ready = false) {
   cudaStream_t s = ex.stream;
   if (tetf) {
-    launch_elastic(s, m, xb, tetf, proj, m.partials, prec);
+    launch_elastic(s, m, xb, tetf, proj, m.partials, prec, disp_ready);
     launch_sum_partials(s, m.partials, elastic_blocks(m.T), m.scal + 2);
   }
   launch_proxy(s, m, xb, sb, RESET_EVAL);
@@ -377,9 +384,12 @@ int gradient_launches(const Exec& ex, const MeshState& ms, DevMesh& m, const dou
                       const double* tetf, double* gout, int prec, double kappa, int bprec,
                       int cap_now) {
   cudaStream_t s = ex.stream;
-  if (tetf) launch_gather_forces(s, m, tetf, gout, prec);
-  else CK(cudaMemsetAsync(gout, 0, sizeof(double) * 3 * (size_t)m.n, s));
-  CK(cudaMemsetAsync(m.x2mark, 0, sizeof(int) * std::max(m.n2, 1), s));
+  if (tetf) {
+    launch_gather_forces(s, m, tetf, gout, prec, true);
+  } else {
+    CK(cudaMemsetAsync(gout, 0, sizeof(double) * 3 * (size_t)m.n, s));
+    CK(cudaMemsetAsync(m.x2mark, 0, sizeof(int) * std::max(m.n2, 1), s));
+  }
   launch_barrier_pairs(s, m, sb, ms.p.dhat, kappa, bprec);
   if (m.n2 > 0) launch_mark_scan(s, m);
   else CK(cudaMemsetAsync(m.counters + 3, 0, sizeof(int), s));
@@ -391,7 +401,7 @@ int gradient_launches(const Exec& ex, const MeshState& ms, DevMesh& m, const dou
   launch_gnorm2(s, m, gout, m.partials, nb);
   launch_sum_partials(s, m.partials, nb, m.scal + 3);
   CK(cudaGetLastError());
-  return FSIM_OK;
+  return copy_status(ex, m);
 }
 
 int gradient_and_hessian(const Exec& ex, const MeshState& ms, DevMesh& m, const double* sb,
@@ -407,7 +417,7 @@ int gradient_and_hessian(const Exec& ex, const MeshState& ms, DevMesh& m, const 
   } else {
     TRY(body());
   }
-  TRY(sync_read(ex, m));
+  TRY(sync(ex));
   const int nc = ex.h_counters[3];
   TRY(ensure_reduced(ex, m, std::max(nc, 1)));
   if (nc > cap_now) {       // the buffers grew: assemble B-check again
@@ -526,8 +536,10 @@ int solve_frame_impl(const Exec& ex, const MeshState& ms, DevMesh& m, const doub
     };
     TRY(with_graph(ex, m, graph_slot(m, kGraphTrial, 4, m.s, prec), m.s, prec, kgen, [&]() -> int {
       TRY(ccd_bound());
-      launch_axpy_positions(s, 3 * m.n, m.x, m.dx, m.scal + 1, 1.0, m.xt);
-      return evaluate(ex, ms, m, m.xt, m.st, m.tetf_t, nullptr, prec, kappa);
+      launch_axpy_positions(s, 3 * m.n, m.x, m.dx, m.scal + 1, 1.0, m.xt, m.rest,
+                            prec == FSIM_MIXED ? m.udf : nullptr);
+      TRY(evaluate(ex, ms, m, m.xt, m.st, m.tetf_t, nullptr, prec, kappa, true));
+      return copy_status(ex, m);
     }));
     // backtracking line search from alpha_m on E-hat = E + B
     bool accepted = false, redone = false;
@@ -535,10 +547,11 @@ int solve_frame_impl(const Exec& ex, const MeshState& ms, DevMesh& m, const doub
     int64_t np_t = 0;
     for (int k = 0; k <= p.max_ls; ++k) {
       if (k > 0 || redone) {
-        launch_axpy_positions(s, 3 * m.n, m.x, m.dx, m.scal + 1, scale, m.xt);
+        launch_axpy_positions(s, 3 * m.n, m.x, m.dx, m.scal + 1, scale, m.xt, m.rest, nullptr);
         TRY(eval_at(m.xt, m.st, m.tetf_t));
+        TRY(copy_status(ex, m));
       }
-      TRY(sync_read(ex, m));
+      TRY(sync(ex));
       if (k == 0 && ex.h_counters[6] && gprec != FSIM_FP64 && p.solver != FSIM_SOLVER_PCG &&
           !redone) {
         // the float32 factor of the reduced (or Schur) system lost positive

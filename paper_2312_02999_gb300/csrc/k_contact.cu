@@ -1646,13 +1646,6 @@ __global__ void __launch_bounds__(32) k_mollify_ee_b(const DevMesh* __restrict__
                     m->pair_grad, m->pair_hess);
 }
 
-__global__ void k_zero_x2mark_b(const DevMesh* __restrict__ tab) {
-  const DevMesh* m = bframe_c(tab, blockIdx.y);
-  if (!m) return;
-  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < m->n2; q += gridDim.x * blockDim.x)
-    m->x2mark[q] = 0;
-}
-
 __global__ void k_mark_scan_b(const DevMesh* __restrict__ tab) {
   const DevMesh* m = bframe_c(tab, blockIdx.y);
   if (!m) return;
@@ -1750,8 +1743,6 @@ void launch_detect_b(cudaStream_t st, const DevMesh* tab, int nb, const DevMesh&
 
 void launch_barrier_b(cudaStream_t st, const DevMesh* tab, int nb, const DevMesh& m0,
                       int64_t np_max, double dhat) {
-  k_zero_x2mark_b<<<dim3((std::max(m0.n2, 1) + 255) / 256, nb), 256, 0, st>>>(tab);
-  count_launch();
   np_max = np_max < m0.cap_act ? np_max : m0.cap_act;
   if (np_max > 0) {
     ProfScope ps(PROF_BARRIER, st);

@@ -625,16 +625,23 @@ __device__ __forceinline__ void gather_forces_df_body(int n, int T, const int* _
   g[3 * (size_t)v + 1] = df_to_double(s1);
   g[3 * (size_t)v + 2] = df_to_double(s2);
 }
+// x2mark: n2 <= n contact marks, cleared here for the barrier kernels that
+// follow (a memset of their own is a launch)
 __global__ void k_gather_forces_df(int n, int T, const int* __restrict__ vptr,
                                    const int* __restrict__ vslot, const float2* __restrict__ tetf,
-                                   const uint8_t* __restrict__ pinned, double* __restrict__ g) {
+                                   const uint8_t* __restrict__ pinned, double* __restrict__ g,
+                                   int n2, int* __restrict__ x2mark) {
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (x2mark && q < n2) x2mark[q] = 0;
   gather_forces_df_body(n, T, vptr, vslot, tetf, pinned, g);
 }
 
 __global__ void k_gather_forces(int n, int T, const int* __restrict__ vptr,
                                 const int* __restrict__ vslot, const double* __restrict__ tetf,
-                                const uint8_t* __restrict__ pinned, double* __restrict__ g) {
+                                const uint8_t* __restrict__ pinned, double* __restrict__ g,
+                                int n2, int* __restrict__ x2mark) {
   const int v = blockIdx.x * blockDim.x + threadIdx.x;
+  if (x2mark && v < n2) x2mark[v] = 0;
   if (v >= n) return;
   double s0 = 0.0, s1 = 0.0, s2 = 0.0;
   if (!pinned[v]) {
@@ -664,12 +671,25 @@ __global__ void k_sum_partials(const double* __restrict__ p, int n, double* __re
   sum_partials_body(p, n, out);
 }
 
-__global__ void k_axpy(int n3, const double* __restrict__ x, const double* __restrict__ dx,
-                       const double* __restrict__ alpha, double scale, double* __restrict__ out) {
+// out = x + alpha scale dx and, for the mixed local step at out, its displacement
+// from rest as float pairs (udf; NULL: not wanted)
+__device__ __forceinline__ void axpy_body(int n3, const double* __restrict__ x,
+                                          const double* __restrict__ dx, double a,
+                                          double* __restrict__ out, const double* __restrict__ rest,
+                                          float2* __restrict__ udf) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n3) return;
-  const double a = alpha[0] * scale;
-  out[i] = x[i] + a * dx[i];
+  const double o = x[i] + a * dx[i];
+  out[i] = o;
+  if (udf) {
+    const df u = df_from_double(__dsub_rn(o, rest[i]));
+    udf[i] = make_float2(u.hi, u.lo);
+  }
+}
+__global__ void k_axpy(int n3, const double* __restrict__ x, const double* __restrict__ dx,
+                       const double* __restrict__ alpha, double scale, double* __restrict__ out,
+                       const double* __restrict__ rest, float2* __restrict__ udf) {
+  axpy_body(n3, x, dx, alpha[0] * scale, out, rest, udf);
 }
 
 __device__ __forceinline__ void gnorm2_body(int n, const double* __restrict__ g,
@@ -698,11 +718,10 @@ __device__ __forceinline__ const DevMesh* bframe(const DevMesh* __restrict__ tab
   return m->active ? m : nullptr;
 }
 
-template <int AT>
 __global__ void k_disp_df_b(const DevMesh* __restrict__ tab) {
   const DevMesh* m = bframe(tab);
   if (!m) return;
-  disp_df_body(3 * m->n, AT ? m->xt : m->x, m->rest, m->udf);
+  disp_df_body(3 * m->n, m->x, m->rest, m->udf);
 }
 
 template <int AT>
@@ -723,18 +742,17 @@ __global__ void k_sum_partials_b(const DevMesh* __restrict__ tab, int nparts, in
 __global__ void k_gather_forces_df_b(const DevMesh* __restrict__ tab) {
   const DevMesh* m = bframe(tab);
   if (!m) return;
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q < m->n2) m->x2mark[q] = 0;
   gather_forces_df_body(m->n, m->T, m->vinc_ptr, m->vinc_slot,
                         reinterpret_cast<const float2*>(m->tetf), m->pinned, m->g);
 }
 
-// xt = x + (alpha_m * ls_scale) dx per frame
+// xt = x + (alpha_m * ls_scale) dx per frame, with xt's displacement
 __global__ void k_axpy_b(const DevMesh* __restrict__ tab) {
   const DevMesh* m = bframe(tab);
   if (!m) return;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= 3 * m->n) return;
-  const double a = m->scal[1] * m->ls_scale;
-  m->xt[i] = m->x[i] + a * m->dx[i];
+  axpy_body(3 * m->n, m->x, m->dx, m->scal[1] * m->ls_scale, m->xt, m->rest, m->udf);
 }
 
 __global__ void k_gnorm2_b(const DevMesh* __restrict__ tab) {
@@ -767,29 +785,33 @@ void launch_actuation(cudaStream_t s, int T, const double* fiber, const double* 
 int elastic_blocks(int T) { return (T + kElasticThreads - 1) / kElasticThreads; }
 
 void launch_elastic(cudaStream_t s, const DevMesh& m, const double* x, double* tetf,
-                    double* proj, double* partials, int precision) {
+                    double* proj, double* partials, int precision, bool disp_ready) {
   const int nb = elastic_blocks(m.T);
   ProfScope ps(PROF_ELASTIC, s);
   if (precision == 0) {
     k_elastic<<<nb, kElasticThreads, 0, s>>>(m.T, m.tets, m.dminv, m.w, m.act, x, tetf, proj, partials);
     count_launch();
   } else {
-    k_disp_df<<<(3 * m.n + 255) / 256, 256, 0, s>>>(3 * m.n, x, m.rest, m.udf);
+    if (!disp_ready) {
+      k_disp_df<<<(3 * m.n + 255) / 256, 256, 0, s>>>(3 * m.n, x, m.rest, m.udf);
+      count_launch();
+    }
     k_elastic_df<<<nb, kElasticThreads, 0, s>>>(m.T, m.tets, m.dminv_df, m.w_df, m.act_df, m.udf,
                                                reinterpret_cast<float2*>(tetf), proj, partials);
-    count_launch(2);
+    count_launch();
   }
 }
 
 void launch_gather_forces(cudaStream_t s, const DevMesh& m, const double* tetf, double* g,
-                          int precision) {
+                          int precision, bool clear_marks) {
+  int* marks = clear_marks ? m.x2mark : nullptr;
   if (precision != 0)
     k_gather_forces_df<<<(m.n + 255) / 256, 256, 0, s>>>(m.n, m.T, m.vinc_ptr, m.vinc_slot,
                                                          reinterpret_cast<const float2*>(tetf),
-                                                         m.pinned, g);
+                                                         m.pinned, g, m.n2, marks);
   else
     k_gather_forces<<<(m.n + 255) / 256, 256, 0, s>>>(m.n, m.T, m.vinc_ptr, m.vinc_slot, tetf,
-                                                      m.pinned, g);
+                                                      m.pinned, g, m.n2, marks);
   count_launch();
 }
 
@@ -799,8 +821,9 @@ void launch_sum_partials(cudaStream_t s, const double* partials, int n, double* 
 }
 
 void launch_axpy_positions(cudaStream_t s, int n3, const double* x, const double* dx,
-                           const double* alpha_dev, double alpha_scale, double* out) {
-  k_axpy<<<(n3 + 255) / 256, 256, 0, s>>>(n3, x, dx, alpha_dev, alpha_scale, out);
+                           const double* alpha_dev, double alpha_scale, double* out,
+                           const double* rest, float2* udf) {
+  k_axpy<<<(n3 + 255) / 256, 256, 0, s>>>(n3, x, dx, alpha_dev, alpha_scale, out, rest, udf);
   count_launch();
 }
 
@@ -809,15 +832,15 @@ int gnorm_blocks(int n) { return (n + 255) / 256; }
 void launch_local_b(cudaStream_t s, const DevMesh* tab, int nb, const DevMesh& m0, int at) {
   ProfScope ps(PROF_ELASTIC, s);
   const dim3 gv((3 * m0.n + 255) / 256, nb), gt(elastic_blocks(m0.T), nb);
-  if (at) {
-    k_disp_df_b<1><<<gv, 256, 0, s>>>(tab);
+  if (at) {          // the displacement comes with the trial point (launch_axpy_b)
     k_elastic_df_b<1><<<gt, kElasticThreads, 0, s>>>(tab);
   } else {
-    k_disp_df_b<0><<<gv, 256, 0, s>>>(tab);
+    k_disp_df_b<<<gv, 256, 0, s>>>(tab);
+    count_launch();
     k_elastic_df_b<0><<<gt, kElasticThreads, 0, s>>>(tab);
   }
   k_sum_partials_b<<<dim3(1, nb), 1024, 0, s>>>(tab, elastic_blocks(m0.T), 2);
-  count_launch(3);
+  count_launch(2);
 }
 
 void launch_gather_forces_b(cudaStream_t s, const DevMesh* tab, int nb, const DevMesh& m0) {

@@ -45,13 +45,14 @@ __global__ void k_gather_rhs(int nf, const int* __restrict__ perm, const double*
   for (int d = 0; d < 3; ++d) r[3 * (size_t)p + d] = (T)(-g[3 * (size_t)v + d]);
 }
 
-__global__ void k_scatter_dx(int nf, const int* __restrict__ perm, const double* __restrict__ z,
+// (zero on pinned vertices)
+__global__ void k_scatter_dx(int n, const int* __restrict__ pos, const double* __restrict__ z,
                              double* __restrict__ dx) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= nf) return;
-  const int v = perm[p];
+  const int v = blockIdx.x * blockDim.x + threadIdx.x;
+  if (v >= n) return;
+  const int p = pos[v];
 #pragma unroll
-  for (int d = 0; d < 3; ++d) dx[3 * (size_t)v + d] = z[3 * (size_t)p + d];
+  for (int d = 0; d < 3; ++d) dx[3 * (size_t)v + d] = p >= 0 ? z[3 * (size_t)p + d] : 0.0;
 }
 
 template <typename S, typename T>
@@ -187,9 +188,11 @@ k_bwd_chunk(const int4* __restrict__ items, const int* __restrict__ c0a, const i
   }
 }
 
-// u = Sinv y (n2 x n2 dense, 3 right-hand sides), one warp per row
+// u = Sinv y (n2 x n2 dense, 3 right-hand sides) in float64 and, with ub, as it
+// was summed (the x2 rows of the contact-free backward solve), one warp per row
 template <typename T>
-__global__ void k_gemv3(int n2, const T* __restrict__ A, const T* __restrict__ y, T* __restrict__ u) {
+__global__ void k_gemv3(int n2, const T* __restrict__ A, const T* __restrict__ y,
+                        double* __restrict__ u, T* __restrict__ ub) {
   const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (row >= n2) return;
@@ -200,7 +203,11 @@ __global__ void k_gemv3(int n2, const T* __restrict__ A, const T* __restrict__ y
     a0 += s * y[3 * j]; a1 += s * y[3 * j + 1]; a2 += s * y[3 * j + 2];
   }
   a0 = warp_sum_t(a0); a1 = warp_sum_t(a1); a2 = warp_sum_t(a2);
-  if (lane == 0) { u[3 * row] = a0; u[3 * row + 1] = a1; u[3 * row + 2] = a2; }
+  if (lane < 3) {
+    const T v = lane == 0 ? a0 : lane == 1 ? a1 : a2;
+    u[3 * row + lane] = (double)v;
+    if (ub) ub[3 * row + lane] = v;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -623,15 +630,13 @@ cudaError_t global_step_t(cudaStream_t s, const DevMesh& m, const double* g, dou
     if (phi) {
       {
         ProfScope psg(PROF_GEMV, s);
-        k_gemv3<float><<<nblk(n2, 8), 256, 0, s>>>(n2, m.Sinvf, (const float*)y2, m.uf);
-        k_convert<float, double><<<nblk(3 * (int64_t)n2, 256), 256, 0, s>>>(3 * n2, m.uf, u);
-        count_launch(2);
+        k_gemv3<float><<<nblk(n2, 8), 256, 0, s>>>(n2, m.Sinvf, (const float*)y2, u,
+                                                   m.bx + 3 * (size_t)n1);
+        count_launch();
       }
       cudaStream_t s2 = m.aux_stream2;
       if (cudaEventRecord(m.ev_fork2, s) != cudaSuccess || cudaStreamWaitEvent(s2, m.ev_fork2, 0) != cudaSuccess)
         return cudaGetLastError();
-      k_convert<float, float><<<nblk(3 * (int64_t)n2, 256), 256, 0, s2>>>(3 * n2, m.uf, m.bx + 3 * (size_t)n1);
-      count_launch();
       trisolve_bwd<float>(s2, m, m.Zf, m.y1f, m.bx, false);
       if (cudaEventRecord(m.ev_join2, s2) != cudaSuccess) return cudaGetLastError();
       {
@@ -642,8 +647,7 @@ cudaError_t global_step_t(cudaStream_t s, const DevMesh& m, const double* g, dou
       if (cudaStreamWaitEvent(s, m.ev_join2, 0) != cudaSuccess) return cudaGetLastError();
       const cudaError_t e = phi_apply(s, m, u, y2, z2, info, m.bx, r);
       if (e != cudaSuccess) return e;
-      cudaMemsetAsync(dx, 0, sizeof(double) * 3 * (size_t)m.n, s);
-      k_scatter_dx<<<nblk(nf, 256), 256, 0, s>>>(nf, m.perm, r, dx);
+      k_scatter_dx<<<nblk(m.n, 256), 256, 0, s>>>(m.n, m.pos, r, dx);
       count_launch();
       return cudaGetLastError();
     }
@@ -655,14 +659,11 @@ cudaError_t global_step_t(cudaStream_t s, const DevMesh& m, const double* g, dou
       {
         ProfScope psg(PROF_GEMV, s);
         if (f64) {
-          k_gemv3<double><<<nblk(n2, 8), 256, 0, s>>>(n2, m.Sinv, (const double*)y2, u);
-          count_launch();
+          k_gemv3<double><<<nblk(n2, 8), 256, 0, s>>>(n2, m.Sinv, (const double*)y2, u, nullptr);
         } else {
-          float* uf = m.uf;
-          k_gemv3<float><<<nblk(n2, 8), 256, 0, s>>>(n2, m.Sinvf, (const float*)y2, uf);
-          k_convert<float, double><<<nblk(3 * (int64_t)n2, 256), 256, 0, s>>>(3 * n2, uf, u);
-          count_launch(2);
+          k_gemv3<float><<<nblk(n2, 8), 256, 0, s>>>(n2, m.Sinvf, (const float*)y2, u, nullptr);
         }
+        count_launch();
       }
       // The reduced system carries the barrier stiffness (cond ~ kappa b''):
       // float64 factors, or float32 factors refined with float64 residuals.
@@ -681,8 +682,7 @@ cudaError_t global_step_t(cudaStream_t s, const DevMesh& m, const double* g, dou
     k_convert<T, double><<<nblk(3 * (int64_t)n1, 256), 256, 0, s>>>(3 * n1, b, r);
     count_launch();
   }
-  cudaMemsetAsync(dx, 0, sizeof(double) * 3 * (size_t)m.n, s);
-  k_scatter_dx<<<nblk(nf, 256), 256, 0, s>>>(nf, m.perm, r, dx);
+  k_scatter_dx<<<nblk(m.n, 256), 256, 0, s>>>(m.n, m.pos, r, dx);
   count_launch();
   return cudaGetLastError();
 }

@@ -98,7 +98,6 @@ struct DevMesh {
   // global-step work (solver positions, AoS 3)
   double* r = nullptr;        // nf*3
   double* u = nullptr;        // n2*3
-  float* uf = nullptr;        // n2*3 (mixed)
   float* rf = nullptr;        // nf*3 (mixed)
   // contact work
   int64_t cap = 0;            // capacity of the near-pair and CCD candidate lists
@@ -130,6 +129,7 @@ struct DevMesh {
     const void* key = nullptr;  // buffer the sequence was captured on
     int key2 = 0, gen = -1, coop = 0;
     bool alone = true;
+    const void* host = nullptr; // pinned words its read-back goes to
     int64_t kernels = 0;        // kernel nodes (counted as launches per replay)
     bool failed = false;        // capture unsupported: launch directly
   };
@@ -175,12 +175,14 @@ void launch_actuation(cudaStream_t s, int T, const double* fiber, const double* 
                       float2* act_df);
 // precision 0: float64 SVD; 1: float32 SVD refined to float64 accuracy in
 // double-float arithmetic (k_elastic_df; tetf then holds float pairs).
+// disp_ready: m.udf already holds x's displacement.
 void launch_elastic(cudaStream_t s, const DevMesh& m, const double* x, double* tetf,
-                    double* proj, double* partials, int precision);
+                    double* proj, double* partials, int precision, bool disp_ready = false);
 int elastic_blocks(int T);
 // g = per-vertex sums of tetf, written by launch_elastic with the same precision
+// (clear_marks: clears m.x2mark too, for the barrier kernels after it)
 void launch_gather_forces(cudaStream_t s, const DevMesh& m, const double* tetf, double* g,
-                          int precision);
+                          int precision, bool clear_marks = false);
 void launch_sum_partials(cudaStream_t s, const double* partials, int n, double* out);
 
 // ---- contact (k_contact.cu) -----------------------------------------------
@@ -252,8 +254,10 @@ void set_solver_smem_limits(int max_bytes);
 void set_reduced_smem_limits();
 
 // ---- misc ------------------------------------------------------------------
+// out = x + alpha dx; with udf also out - rest as float pairs (launch_elastic's)
 void launch_axpy_positions(cudaStream_t s, int n3, const double* x, const double* dx,
-                           const double* alpha_dev, double alpha_scale, double* out);
+                           const double* alpha_dev, double alpha_scale, double* out,
+                           const double* rest, float2* udf);
 void launch_gnorm2(cudaStream_t s, const DevMesh& m, const double* g, double* partials, int nblk);
 int gnorm_blocks(int n);
 void launch_reset_pinned(cudaStream_t s, const DevMesh& m, double* x);
