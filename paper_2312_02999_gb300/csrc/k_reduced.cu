@@ -1233,6 +1233,7 @@ constexpr int kST = 512;                   // threads of the one-CTA kernels
 constexpr int kSW = kST / 32;
 
 constexpr int kPtLd = kSmallN3;            // panel scratch: 32 x kPtLd floats
+constexpr int kPanelsDone = 16;            // word of RedArgs::bar: panels of N factored
 
 // Outer-product elimination of the unscaled 32 x 32 diagonal block Ds: after
 // step j, Ds[i][c] (c > j) holds the Schur complement; Ds[.][j] (j < i) stays
@@ -1264,13 +1265,13 @@ __device__ __forceinline__ void eliminate_diag(float (*Ds)[33], int kb) {
 // barrier per column), every row below solves its own panel segment by
 // substitution (one thread per row) while the last warp inverts the
 // diagonal block, and the trailing update A -= P P^T runs with 4 x 4
-// register tiles from a transposed copy Pt of the panel.  With inv_diag
-// the diagonal blocks are left holding L_kk^-1 (for the solves below);
-// Lout (row-major, leading dimension ldo), if given, receives the plain
-// diagonal blocks.  Loops stay rolled: straight-line code this size would
-// run out of the instruction cache.
-__device__ void cta_chol_packed(float* A, int n, float* Pt, int* info, bool inv_diag, float* Lout,
-                                int ldo, float* DIout) {
+// register tiles from a transposed copy Pt of the panel.
+// With `out`, every panel goes to the packed matrix out in global memory as
+// soon as it is solved, its diagonal block inverted, and *done then counts it.
+// DIout, if given, receives the inverted diagonal blocks.  Loops stay rolled:
+// straight-line code this size would run out of the instruction cache.
+__device__ void cta_chol_packed(float* A, int n, float* Pt, int* info, float* out, unsigned* done,
+                                float* DIout) {
   __shared__ float Ds[32][33];
   __shared__ float Li[32][33];
   __shared__ float dv[32];
@@ -1305,12 +1306,6 @@ __device__ void cta_chol_packed(float* A, int n, float* Pt, int* info, bool inv_
     __syncthreads();
     if (tid < kb) Ds[tid][tid] = Ds[tid][tid] * dv[tid];    // sqrt(d)
     __syncthreads();
-    if (Lout) {
-      for (int e = tid; e < kb * 32; e += kST) {
-        const int i = e >> 5, j = e & 31;
-        if (j <= i) Lout[(size_t)(k0 + i) * ldo + k0 + j] = Ds[i][j];
-      }
-    }
     if (tid < m) {
       // row k1 + tid: x L_kk^T = a in registers (right-looking, so the
       // dependent chain is one FMA per column), then its transposed copy
@@ -1329,6 +1324,12 @@ __device__ void cta_chol_packed(float* A, int n, float* Pt, int* info, bool inv_
         row[l] = x[l];
         Pt[l * kPtLd + tid] = x[l];
       }
+      if (out) {
+        float4* o = reinterpret_cast<float4*>(out + prow(k1 + tid) + k0);
+#pragma unroll
+        for (int l = 0; l < 8; ++l)
+          o[l] = make_float4(x[4 * l], x[4 * l + 1], x[4 * l + 2], x[4 * l + 3]);
+      }
     } else if (wid == kSW - 1) {
       // Li = L_kk^-1, column `lane` in registers (right-looking)
       float x[32];
@@ -1342,8 +1343,17 @@ __device__ void cta_chol_packed(float* A, int n, float* Pt, int* info, bool inv_
       }
 #pragma unroll
       for (int i = 0; i < 32; ++i) Li[i][lane] = (i >= lane) ? x[i] : 0.f;
+      if (out)
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+          if (lane <= i && i < kb) out[prow(k0 + i) + k0 + lane] = x[i];
     }
     __syncthreads();
+    if (out && tid == kST - 1) {     // (a thread of the last, least loaded warp)
+      __threadfence();
+      asm volatile("st.release.gpu.u32 [%0], %1;" ::"l"(done), "r"((unsigned)(k0 >> 5) + 1u)
+                   : "memory");
+    }
     if (m > 0) {
       // trailing update A -= P P^T, 4 x 4 tiles of the lower triangle
       const int mb = (m + 3) >> 2, nt = mb * (mb + 1) / 2;
@@ -1379,10 +1389,10 @@ __device__ void cta_chol_packed(float* A, int n, float* Pt, int* info, bool inv_
         }
       }
     }
-    // the diagonal block: plain factor, or its inverse for the solves
+    // the diagonal block
     for (int e = tid; e < kb * 32; e += kST) {
       const int i = e >> 5, j = e & 31;
-      if (j <= i) A[prow(k0 + i) + k0 + j] = inv_diag ? Li[i][j] : Ds[i][j];
+      if (j <= i) A[prow(k0 + i) + k0 + j] = Ds[i][j];
       if (DIout) DIout[(size_t)(k0 >> 5) * 1024 + e] = (j <= i) ? Li[i][j] : 0.f;
     }
     __syncthreads();
@@ -1400,7 +1410,7 @@ __device__ __forceinline__ void k_small_s_body(RedArgs<float> a) {
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   float* P = smem_f;                      // prow(kClusNc) floats
   float* Pt = P + prow(kClusNc);          // 32 x kPtLd
-  if (tid == 0) a.nrm[2] = 0.0;
+  if (tid == 0) { a.nrm[2] = 0.0; a.bar[kPanelsDone] = 0; }
   for (int i = wid; i < nc; i += kSW) {
     if (!FSIM_CHECK_IDX(a.clist[i], a.n2, CHECK_CLIST)) continue;
     const double* srow = a.Sinv + (size_t)a.clist[i] * a.n2;
@@ -1431,7 +1441,7 @@ __device__ __forceinline__ void k_small_s_body(RedArgs<float> a) {
   __syncthreads();
   // L_s: row-major into a.S (for the grid products), packed plain into
   // a.spk followed by its inverted diagonal blocks (for the one-CTA solves)
-  cta_chol_packed(P, nc, Pt, a.info, false, nullptr, 0, a.spk + prow(nc));
+  cta_chol_packed(P, nc, Pt, a.info, nullptr, nullptr, a.spk + prow(nc));
   for (int e = tid; e < nc * nc; e += kST) {
     const int i = e / nc, j = e % nc;
     a.S[e] = (j <= i) ? P[prow(i) + j] : 0.f;
@@ -1622,130 +1632,182 @@ __device__ double refine_rho(const RedArgs<float>& a, int nc, int t, int nt) {
   return r2;
 }
 
-// k_small_v (1 CTA): L_N in shared memory, back to the packed N with inverted
-// diagonal blocks
+// Block column j of V = L^-1 (n x n, row-major) from the packed factor P:
+// V_jj = L_jj^-1, then down the column V_kj = -L_kk^-1 sum_{i = j .. k-1} L_ki V_ij.
+// The sums are formed as the blocks V_kj become known: a group of 64 threads owns
+// the block rows 1 + group and 9 + group and keeps their sums in registers (4 x 4
+// values per thread: rows ti + 8 p, columns tj + 8 q), so a step is one product per
+// row and the product with the inverted diagonal block.  The diagonal blocks of P
+// are inverted ones, unless DI holds those.  `done`, if given, counts the panels
+// of P that are there, and step k waits for panel k.
+constexpr int kULd = 36;
+constexpr size_t kInvSmem = sizeof(float) * (size_t)(3 + 16) * 32 * kULd;
+__device__ __forceinline__ void inverse_column(const float* P, const float* DI, float* V, int n, int j,
+                                               const unsigned* done, int* info, float* sm) {
+  const int nb = (n + 31) / 32;
+  const int tid = threadIdx.x, gr = tid >> 6, tq = tid & 63, ti = tq >> 3, tj = tq & 7;
+  const int lane = tid & 31, wid = tid >> 5;
+  float(*VT)[kULd] = reinterpret_cast<float(*)[kULd]>(sm);     // V_kj [column][row]
+  float(*St)[kULd] = VT + 32;                                  // the sum of row k [column][row]
+  float(*Di)[kULd] = St + 32;                                  // L_kk^-1
+  float(*Lk)[kULd] = Di + 32 + gr * 64;                        // L_ik of the group's rows
+  float acc[2][4][4];
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[h][p][q] = 0.f;
+  for (int k = j; k < nb; ++k) {
+    if (done && tid == 0) {
+      int polls = 0;
+      unsigned v;
+      do {
+        asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(v) : "l"(done) : "memory");
+      } while (v <= (unsigned)k && ++polls <= kSpinLimit);
+      if (v <= (unsigned)k) {      // (gave up: the step fails, later panels are not waited for)
+        atomicOr(info, 4);
+        done = nullptr;
+      }
+      __threadfence();
+    }
+    __syncthreads();               // and the tiles of the step before are read
+    // (past L1: a line read for an earlier panel may hold the start of this one)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int i = 1 + gr + 8 * h;
+      if (i <= k || i >= nb) continue;
+      float4 f[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int e = tq + 64 * u, r = 32 * i + (e >> 3);
+        f[u] = r < n ? __ldcg(reinterpret_cast<const float4*>(P + prow(r) + 32 * k) + (e & 7))
+                     : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int e = tq + 64 * u;
+        *reinterpret_cast<float4*>(&Lk[32 * h + (e >> 3)][4 * (e & 7)]) = f[u];
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int e = tid + kST * h, r = e >> 5, c = e & 31;
+      float v = 0.f;               // zero above the diagonal and past n
+      if (c <= r && 32 * k + r < n)
+        v = DI ? __ldcg(DI + 1024 * k + e) : __ldcg(P + prow(32 * k + r) + 32 * k + c);
+      Di[r][c] = v;
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int i = 1 + gr + 8 * h;
+      if (i == k) {
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) St[tj + 8 * q][ti + 8 * p] = acc[h][p][q];
+      }
+    }
+    __syncthreads();
+    // row `lane`, columns wid and wid + 16 of V_kj
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int c = wid + 16 * h;
+      float o = 0.f;
+      if (k == j) {
+        o = Di[lane][c];
+      } else {
+#pragma unroll
+        for (int l = 0; l < 32; l += 4) {
+          const float4 dv = *reinterpret_cast<const float4*>(&Di[lane][l]);
+          const float4 sv = *reinterpret_cast<const float4*>(&St[c][l]);
+          o -= dv.x * sv.x + dv.y * sv.y + dv.z * sv.z + dv.w * sv.w;
+        }
+      }
+      VT[c][lane] = o;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int r = wid + 16 * h;
+      if (32 * k + r < n && 32 * j + lane < n)
+        V[(size_t)(32 * k + r) * n + 32 * j + lane] = VT[lane][r];
+      const int i = 1 + gr + 8 * h;
+      if (i <= k || i >= nb) continue;
+#pragma unroll 2
+      for (int l = 0; l < 32; l += 4) {
+        float4 x[4], y[4];
+#pragma unroll
+        for (int p = 0; p < 4; ++p) x[p] = *reinterpret_cast<const float4*>(&Lk[32 * h + ti + 8 * p][l]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) y[q] = *reinterpret_cast<const float4*>(&VT[tj + 8 * q][l]);
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            acc[h][p][q] += x[p].x * y[q].x + x[p].y * y[q].y + x[p].z * y[q].z + x[p].w * y[q].w;
+      }
+    }
+  }
+  __syncthreads();                 // (the next column reuses the tiles)
+}
+
+// k_small_v: a cluster of kVCl CTAs.  CTA 0 factors N in its shared memory and
+// publishes every panel; the others form the inverses beside it, V_s = L_s^-1
+// and then the columns of V = L_N^-1, each step as soon as its panel is there,
+// so that all but the last step of every column is done when the factor is.
+// (They wait for CTA 0 only; the CTAs of a cluster run together.)  As a kernel of
+// its own after the factor, V took 62 us of a 536 us iteration (30k face, n_c =
+// 92, under a tracer); beside it a frame takes 36.3 -> 35.4 ms (5k: 27.1 -> 26.4).
+constexpr int kVCl = 8;
 __device__ __forceinline__ void k_small_v_body(RedArgs<float> a) {
-  extern __shared__ float smem_f[];
+  extern __shared__ __align__(16) float smem_f[];
   const int nc = *a.nc_dev;
   if (nc == 0 || nc > a.one_cta_max) return;
   red_layout(a, nc);
-  const int n3 = 3 * nc;
-  const int tid = threadIdx.x;
-  float* A = smem_f;                      // prow(kSmallN3) floats
-  float* Pt = A + prow(kSmallN3);         // 32 x kPtLd
-  // packed N (padding included: prow(n3) is a multiple of 4)
-  float4* gN = reinterpret_cast<float4*>(a.N);
-  float4* sN = reinterpret_cast<float4*>(A);
+  const int n3 = 3 * nc, cta = blockIdx.x % kVCl;
+  if (cta == 0) {
+    float* A = smem_f;                      // prow(kSmallN3) floats
+    float* Pt = A + prow(kSmallN3);         // 32 x kPtLd
+    // packed N (padding included: prow(n3) is a multiple of 4)
+    const float4* gN = reinterpret_cast<const float4*>(a.N);
+    float4* sN = reinterpret_cast<float4*>(A);
 #pragma unroll 4
-  for (int e = tid; e < prow(n3) / 4; e += kST) sN[e] = gN[e];
-  __syncthreads();
-  cta_chol_packed(A, n3, Pt, a.info, true, nullptr, 0, nullptr);
-#pragma unroll 4
-  for (int e = tid; e < prow(n3) / 4; e += kST) gN[e] = sN[e];
+    for (int e = threadIdx.x; e < prow(n3) / 4; e += kST) sN[e] = gN[e];
+    __syncthreads();
+    cta_chol_packed(A, n3, Pt, a.info, a.N, a.bar + kPanelsDone, nullptr);
+    return;
+  }
+  const int w = cta - 1, nw = kVCl - 1;
+  // one column of V_s for the CTAs with the shorter columns of V
+  for (int j = nw - 1 - w; 32 * j < nc; j += nw)
+    inverse_column(a.spk, a.spk + prow(nc), a.Vs, nc, j, nullptr, a.info, smem_f);
+  for (int b = 0; 32 * b * nw < n3; ++b) {      // columns forth and back over the CTAs
+    const int j = b * nw + (b & 1 ? nw - 1 - w : w);
+    if (32 * j < n3)
+      inverse_column(a.N, nullptr, a.X, n3, j, a.bar + kPanelsDone, a.info, smem_f);
+  }
 }
 __global__ void __launch_bounds__(kST) k_small_v(RedArgs<float> a) {
   k_small_v_body(a);
 }
 
-// k_small_u: a CTA per block column j of V = L^-1 (the first kUN CTAs V of L_N,
-// the others V_s of L_s): V_jj = L_jj^-1, then down the column
-//   V_ij = -L_ii^-1 sum_{k = j .. i-1} L_ik V_kj.
-// The column's blocks stay in shared memory, transposed, so that both operands
-// of the products are read along l; four groups of 64 threads take every
-// fourth k (4 x 4 values per thread: rows ti + 8 p, columns tj + 8 q) and their
-// partial sums are added before the product with the inverted diagonal block.
+// k_small_u: the inverses after the factor of the cluster form, a CTA per block
+// column (the first kUN CTAs V of L_N, the others V_s of L_s)
 constexpr int kUN = kClusN3 / 32, kUCtas = kUN + kClusNc / 32;
-constexpr int kULd = 36;
-constexpr size_t kSmallSmemU = sizeof(float) * (size_t)(kUN + 4 + 1) * 32 * kULd;
 __device__ __forceinline__ void k_small_u_body(RedArgs<float> a, int cta) {
   extern __shared__ __align__(16) float smem_f[];
   const int nc = *a.nc_dev;
-  if (nc == 0 || nc > a.small_lim) return;
+  if (nc <= a.one_cta_max || nc > a.small_lim) return;
   red_layout(a, nc);
-  const bool is_n = cta < kUN;
-  const int n = is_n ? 3 * nc : nc, j = is_n ? cta : cta - kUN, nb = (n + 31) / 32;
-  if (j >= nb) return;
-  const float* P = is_n ? a.N : a.spk;                  // packed factor
-  const float* DI = is_n ? nullptr : a.spk + prow(nc);  // inverted diagonal blocks, else in P
-  float* V = is_n ? a.X : a.Vs;
-  const int tid = threadIdx.x, gr = tid >> 6, tq = tid & 63, ti = tq >> 3, tj = tq & 7;
-  float(*VT)[kULd] = reinterpret_cast<float(*)[kULd]>(smem_f);            // [32 block + column][row]
-  float(*Lk)[kULd] = VT + kUN * 32 + gr * 32;                              // this group's L_ik
-  float(*part)[kULd] = VT + kUN * 32;                                      // 4 x 32 rows
-  float(*Di)[kULd] = VT + (kUN + 4) * 32;
-  auto load_diag = [&](int i) {          // L_ii^-1, zero above the diagonal and past n
-    for (int e = tid; e < 32 * 32; e += kRT) {
-      const int r = e >> 5, c = e & 31;
-      float v = 0.f;
-      if (c <= r && 32 * i + r < n) v = DI ? DI[1024 * i + e] : P[prow(32 * i + r) + 32 * i + c];
-      Di[r][c] = v;
-    }
-  };
-  auto store = [&](int i, int r, int c, float v) {
-    VT[32 * i + c][r] = v;
-    if (32 * i + r < n && 32 * j + c < n) V[(size_t)(32 * i + r) * n + 32 * j + c] = v;
-  };
-  load_diag(j);
-  __syncthreads();
-  for (int e = tid; e < 32 * 32; e += kRT) store(j, e >> 5, e & 31, Di[e >> 5][e & 31]);
-  for (int i = j + 1; i < nb; ++i) {
-    __syncthreads();
-    load_diag(i);
-    float acc[4][4];
-#pragma unroll
-    for (int p = 0; p < 4; ++p)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) acc[p][q] = 0.f;
-    for (int k = j + gr; k < i; k += 4) {
-      float4 f[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int e = tq + 64 * u, r = 32 * i + (e >> 3);
-        f[u] = r < n ? *(reinterpret_cast<const float4*>(P + prow(r) + 32 * k) + (e & 7))
-                     : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-      asm volatile("bar.sync %0, 64;" ::"r"(gr + 1) : "memory");   // the tile before is read
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int e = tq + 64 * u;
-        *reinterpret_cast<float4*>(&Lk[e >> 3][4 * (e & 7)]) = f[u];
-      }
-      asm volatile("bar.sync %0, 64;" ::"r"(gr + 1) : "memory");
-#pragma unroll 2
-      for (int l = 0; l < 32; l += 4) {
-        float4 x[4], y[4];
-#pragma unroll
-        for (int p = 0; p < 4; ++p) x[p] = *reinterpret_cast<const float4*>(&Lk[ti + 8 * p][l]);
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-          y[q] = *reinterpret_cast<const float4*>(&VT[32 * k + tj + 8 * q][l]);
-#pragma unroll
-        for (int p = 0; p < 4; ++p)
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            acc[p][q] += x[p].x * y[q].x + x[p].y * y[q].y + x[p].z * y[q].z + x[p].w * y[q].w;
-      }
-    }
-    __syncthreads();                     // all tiles are read: part overlays them
-#pragma unroll
-    for (int p = 0; p < 4; ++p)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) part[32 * gr + tj + 8 * q][ti + 8 * p] = acc[p][q];   // [column][row]
-    __syncthreads();
-    // column c, rows r0 .. r0 + 3 of -L_ii^-1 (sum of the parts)
-    const int c = tid >> 3, r0 = 4 * (tid & 7);
-    float o[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
-    for (int l = 0; l < 32; ++l) {
-      const float s = part[c][l] + part[32 + c][l] + part[64 + c][l] + part[96 + c][l];
-#pragma unroll
-      for (int p = 0; p < 4; ++p) o[p] -= Di[r0 + p][l] * s;
-    }
-#pragma unroll
-    for (int p = 0; p < 4; ++p) store(i, r0 + p, c, o[p]);
+  const int n3 = 3 * nc, j = cta < kUN ? cta : cta - kUN;
+  if (cta < kUN) {
+    if (32 * j < n3) inverse_column(a.N, nullptr, a.X, n3, j, nullptr, a.info, smem_f);
+  } else if (32 * j < nc) {
+    inverse_column(a.spk, a.spk + prow(nc), a.Vs, nc, j, nullptr, a.info, smem_f);
   }
 }
-__global__ void __launch_bounds__(kRT) k_small_u(RedArgs<float> a) {
+__global__ void __launch_bounds__(kST) k_small_u(RedArgs<float> a) {
   k_small_u_body(a, blockIdx.x);
 }
 
@@ -1754,7 +1816,8 @@ __global__ void __launch_bounds__(kRT) k_small_u(RedArgs<float> a) {
 // cluster of kSolveCl CTAs: the vectors live in global memory and a cluster
 // barrier separates the products.  Warps and threads are numbered interleaved
 // over the CTAs, so that every SM gets its share of the float64 work.
-constexpr int kSolveCl = 8, kSolveT = 512;
+// (512 threads a CTA: 2.4 % more time for a 5k face's frame, 0.3 % for 60k faces.)
+constexpr int kSolveCl = 8, kSolveT = 256;
 constexpr int kSolveW = kSolveT / 32;       // warps per CTA
 __device__ __forceinline__ void k_small_solve_body(RedArgs<float> a) {
   namespace cgx = cooperative_groups;
@@ -2185,6 +2248,7 @@ __global__ void __maxnreg__(128) k_clus_v(RedArgs<float> a) {
 
 constexpr size_t kSmallSmemS = sizeof(float) * ((size_t)prow(kClusNc) + 32 * kPtLd);
 constexpr size_t kSmallSmemV = sizeof(float) * ((size_t)prow(kSmallN3) + 32 * kPtLd);
+static_assert(kInvSmem <= kSmallSmemV, "the CTAs beside the factor use its shared memory");
 
 template <typename FT>
 RedArgs<FT> make_args(const DevMesh& m, const double* u, const FT* y2, double* z2, int* info,
@@ -2204,21 +2268,23 @@ RedArgs<FT> make_args(const DevMesh& m, const double* u, const FT* y2, double* z
   return a;
 }
 
-// Launch one of the cluster kernels (kCl CTAs per cluster).
-cudaError_t launch_clus_v(cudaStream_t s, const RedArgs<float>& a) {
+// Launch one of the cluster kernels: a cluster of `ctas` CTAs per system.
+template <typename K, typename A>
+cudaError_t launch_clusters(cudaStream_t s, K kernel, int ctas, int threads, size_t smem, int nsys,
+                            const A& arg) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(kCl);
-  cfg.blockDim = dim3(kST);
-  cfg.dynamicSmemBytes = kClusSmem;
+  cfg.gridDim = dim3(ctas, nsys);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = kCl;
+  at[0].val.clusterDim.x = ctas;
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_clus_v, a);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, arg);
   count_launch();
   return e;
 }
@@ -2239,27 +2305,9 @@ cudaError_t launch_grid(cudaStream_t s, RedArgs<FT> a, int ctas, bool prepare) {
   return e;
 }
 
-// Launch k_small_solve(_b): one cluster of kSolveCl CTAs per system.
-template <typename K, typename A>
-cudaError_t launch_solve_clusters(cudaStream_t s, K kernel, int nsys, const A& arg) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(kSolveCl, nsys);
-  cfg.blockDim = dim3(kSolveT);
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = kSolveCl;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, arg);
-  count_launch();
-  return e;
-}
-
 // float32 factors, n_c <= kClusNc, on the side stream: one-CTA factor up to
-// one_cta_max, the 4-CTA cluster above it, then the inverses of both factors.
+// one_cta_max, beside the inverses of both factors; the 4-CTA cluster above it,
+// then the inverses.
 // No cooperative launch (whose grid must find all of its SMs free at once when
 // other solves share the GPU).
 cudaError_t launch_small_prepare(cudaStream_t s2, const RedArgs<float>& a, int num_sms, int nc) {
@@ -2267,14 +2315,12 @@ cudaError_t launch_small_prepare(cudaStream_t s2, const RedArgs<float>& a, int n
   k_small_s<<<1, kST, kSmallSmemS, s2>>>(a);
   k_small_x<<<2 * std::max(1, num_sms), 256, 0, s2>>>(a);
   k_small_n<<<kNTiles, 256, 0, s2>>>(a);
-  if (nc <= a.one_cta_max) {
-    k_small_v<<<1, kST, kSmallSmemV, s2>>>(a);
-  } else {
-    const cudaError_t e = launch_clus_v(s2, a);
-    if (e != cudaSuccess) return e;
-  }
-  k_small_u<<<kUCtas, kRT, kSmallSmemU, s2>>>(a);
-  count_launch(nc <= a.one_cta_max ? 5 : 4);
+  count_launch(3);
+  if (nc <= a.one_cta_max) return launch_clusters(s2, k_small_v, kVCl, kST, kSmallSmemV, 1, a);
+  const cudaError_t e = launch_clusters(s2, k_clus_v, kCl, kST, kClusSmem, 1, a);
+  if (e != cudaSuccess) return e;
+  k_small_u<<<kUCtas, kST, kInvSmem, s2>>>(a);
+  count_launch();
   return cudaGetLastError();
 }
 // the solve, and the z2 update as a plain launch
@@ -2283,7 +2329,7 @@ cudaError_t launch_small(cudaStream_t s, const DevMesh& m, const RedArgs<float>&
   ProfScope ps(PROF_CHOL, s);
   const int zgrid = std::max(1, std::min(2 * std::max(1, num_sms), (m.n2 + 7) / 8));
   if (nc > 0) {
-    const cudaError_t e = launch_solve_clusters(s, k_small_solve, 1, a);
+    const cudaError_t e = launch_clusters(s, k_small_solve, kSolveCl, kSolveT, 0, 1, a);
     if (e != cudaSuccess) return e;
   }
   k_z2_update<<<zgrid, 256, 0, s>>>(a);
@@ -2382,7 +2428,7 @@ __global__ void __launch_bounds__(256) k_small_x_b(const RedArgs<float>* __restr
   const RedArgs<float> a = A[blockIdx.y];
   if (a.active) k_small_x_body(a);
 }
-__global__ void __launch_bounds__(kRT) k_small_u_b(const RedArgs<float>* __restrict__ A) {
+__global__ void __launch_bounds__(kST) k_small_u_b(const RedArgs<float>* __restrict__ A) {
   const RedArgs<float> a = A[blockIdx.y];
   if (a.active) k_small_u_body(a, blockIdx.x);
 }
@@ -2522,28 +2568,15 @@ cudaError_t reduced_prepare_b(cudaStream_t s2, const void* args_dev, const void*
     k_small_n_b<<<dim3(kNTiles, nb), 256, 0, s2>>>(A);
     count_launch(3);
     if (any_small) {
-      k_small_v_b<<<dim3(1, nb), kST, kSmallSmemV, s2>>>(A);
-      count_launch();
-    }
-    if (any_clus) {
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3(kCl, nb);
-      cfg.blockDim = dim3(kST);
-      cfg.dynamicSmemBytes = kClusSmem;
-      cfg.stream = s2;
-      cudaLaunchAttribute at[1];
-      at[0].id = cudaLaunchAttributeClusterDimension;
-      at[0].val.clusterDim.x = kCl;
-      at[0].val.clusterDim.y = 1;
-      at[0].val.clusterDim.z = 1;
-      cfg.attrs = at;
-      cfg.numAttrs = 1;
-      e = cudaLaunchKernelEx(&cfg, k_clus_v_b, A);
-      count_launch();
+      e = launch_clusters(s2, k_small_v_b, kVCl, kST, kSmallSmemV, nb, A);
       if (e != cudaSuccess) return e;
     }
-    k_small_u_b<<<dim3(kUCtas, nb), kRT, kSmallSmemU, s2>>>(A);
-    count_launch();
+    if (any_clus) {
+      e = launch_clusters(s2, k_clus_v_b, kCl, kST, kClusSmem, nb, A);
+      if (e != cudaSuccess) return e;
+      k_small_u_b<<<dim3(kUCtas, nb), kST, kInvSmem, s2>>>(A);
+      count_launch();
+    }
   }
   // n_c beyond the cluster path: the grid form, all such frames side by side
   e = launch_grid_b(s2, A, H, nb, nc_host, coop_ctas, true);
@@ -2558,7 +2591,7 @@ cudaError_t reduced_solve_b(cudaStream_t s, const void* args_dev, const void* ar
   for (int f = 0; f < nb; ++f) any |= H[f].active && nc_host[f] > 0 && nc_host[f] <= kClusNc;
   ProfScope ps(PROF_CHOL, s);
   if (any) {
-    const cudaError_t e = launch_solve_clusters(s, k_small_solve_b, nb, A);
+    const cudaError_t e = launch_clusters(s, k_small_solve_b, kSolveCl, kSolveT, 0, nb, A);
     if (e != cudaSuccess) return e;
   }
   const cudaError_t eg = launch_grid_b(s, A, H, nb, nc_host, coop_ctas, false);
@@ -2618,8 +2651,8 @@ void set_reduced_smem_limits() {
   cudaFuncSetAttribute(k_small_s_b, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallSmemS);
   cudaFuncSetAttribute(k_small_v_b, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallSmemV);
   cudaFuncSetAttribute(k_clus_v_b, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClusSmem);
-  cudaFuncSetAttribute(k_small_u, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallSmemU);
-  cudaFuncSetAttribute(k_small_u_b, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallSmemU);
+  cudaFuncSetAttribute(k_small_u, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kInvSmem);
+  cudaFuncSetAttribute(k_small_u_b, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kInvSmem);
 }
 FSIM_CHECK_READER(check_word_reduced)
 
