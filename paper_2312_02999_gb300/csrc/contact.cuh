@@ -38,7 +38,7 @@ struct PairGeom {
 };
 
 __device__ __forceinline__ double dot3(const double* a, const double* b) {
-  return a[0] * b[0] + a[1] * b[1] + a[2] * b[2];
+  return fma(a[2], b[2], fma(a[1], b[1], a[0] * b[0]));
 }
 
 // Closest point of segment [A, B] to P: clamped parameter and squared distance.
@@ -55,7 +55,7 @@ __device__ __forceinline__ void seg_closest(const double* P, const double* A, co
 __device__ __forceinline__ void geom_finish(PairGeom& g, const double X[4][3]) {
 #pragma unroll
   for (int d = 0; d < 3; ++d)
-    g.v[d] = g.c[0] * X[0][d] + g.c[1] * X[1][d] + g.c[2] * X[2][d] + g.c[3] * X[3][d];
+    g.v[d] = fma(g.c[3], X[3][d], fma(g.c[2], X[2][d], fma(g.c[1], X[1][d], g.c[0] * X[0][d])));
   g.d2 = dot3(g.v, g.v);
 }
 
@@ -70,9 +70,10 @@ __device__ void pt_geometry(const double X[4][3], PairGeom& g) {
   double r[3] = {p[0] - a[0], p[1] - a[1], p[2] - a[2]};
   double a11 = dot3(e1, e1), a12 = dot3(e1, e2), a22 = dot3(e2, e2);
   double r1 = dot3(e1, r), r2 = dot3(e2, r);
-  double det = a11 * a22 - a12 * a12;
-  double u = (a22 * r1 - a12 * r2) / det;
-  double w = (a11 * r2 - a12 * r1) / det;
+  // (products and sums fused explicitly: pair_features_warp rounds alike)
+  double det = fma(a11, a22, -(a12 * a12));
+  double u = fma(a22, r1, -(a12 * r2)) / det;
+  double w = fma(a11, r2, -(a12 * r1)) / det;
 #pragma unroll
   for (int i = 0; i < 4; ++i) { g.c[i] = 0.0; g.cp[0][i] = 0.0; g.cp[1][i] = 0.0; }
   if (u >= 0.0 && w >= 0.0 && u + w <= 1.0) {
@@ -112,13 +113,13 @@ __device__ void ee_geometry(const double X[4][3], PairGeom& g) {
   double v[3] = {b1[0] - b0[0], b1[1] - b0[1], b1[2] - b0[2]};
   double w0[3] = {a0[0] - b0[0], a0[1] - b0[1], a0[2] - b0[2]};
   double A = dot3(u, u), B = dot3(u, v), C = dot3(v, v), D = dot3(u, w0), E = dot3(v, w0);
-  double den = A * C - B * B;
+  double den = fma(A, C, -(B * B));
 #pragma unroll
   for (int i = 0; i < 4; ++i) { g.c[i] = 0.0; g.cp[0][i] = 0.0; g.cp[1][i] = 0.0; }
   bool interior = false;
   if (den > FSIM_PARALLEL_EPS * A * C) {
-    double s = (B * E - C * D) / den;
-    double t = (A * E - B * D) / den;
+    double s = fma(B, E, -(C * D)) / den;
+    double t = fma(A, E, -(B * D)) / den;
     if (s > 0.0 && s < 1.0 && t > 0.0 && t < 1.0) {
       interior = true;
       g.k = 2;
@@ -370,6 +371,202 @@ __device__ void pair_reduced(int type, const double X[4][3], double dhat, double
       r.A[i][j] = h;
       r.A[j][i] = h;
     }
+}
+
+// Workspace of the one-warp forms, where the lanes share a pair's float64 work.
+struct PairWarp {
+  double X[4][3];       // the pair's vertices
+  double D[3][3];       // edge vectors, vertex difference
+  double C[3][4];       // c, c'_1, c'_2
+  double W[3][4];       // v, E_1, E_2 (last entry 0)
+  double Q[3][4];       // c^, q_1, q_2
+  double F[5][2], T[5][2];
+  double vh[3];
+};
+
+// Closest features of the pair at w.X (visible to the warp): its number of free
+// parameters; C = c, c'_1, c'_2.  One lane per difference component, dot product,
+// quotient and segment: about 25 float64 instructions where one lane needs 70
+// (interior features), 65 where it needs 180.
+__device__ __forceinline__ int pair_features_warp(int type, int lane, PairWarp& w) {
+  constexpr unsigned full = 0xffffffffu;
+  int k;
+  if (lane < 9) {       // PT: b - a, c - a, p - a;  EE: a1 - a0, b1 - b0, a0 - b0
+    const int q = lane / 3, dd = lane % 3;
+    const int hi = type == 0 ? (q == 0 ? 2 : q == 1 ? 3 : 0) : (q == 0 ? 1 : q == 1 ? 3 : 0);
+    const int lo = type == 0 ? 1 : (q == 0 ? 0 : 2);
+    w.D[q][dd] = w.X[hi][dd] - w.X[lo][dd];
+  }
+  __syncwarp();
+  double m = 0.0;
+  if (lane < 5) {       // 0.0, 0.1, 1.1, 0.2, 1.2
+    const int a = lane == 2 || lane == 4, b = lane == 0 ? 0 : lane < 3 ? 1 : 2;
+    m = dot3(w.D[a], w.D[b]);
+  }
+  const double m0 = __shfl_sync(full, m, 0), m1 = __shfl_sync(full, m, 1),
+               m2 = __shfl_sync(full, m, 2), m3 = __shfl_sync(full, m, 3),
+               m4 = __shfl_sync(full, m, 4);
+  const double det = fma(m0, m2, -(m1 * m1));
+  const bool odd = lane & 1, ee = type != 0;
+  // even lanes (a22 r1 - a12 r2) / det or (B E - C D) / det, odd (m0 m4 - m1 m3) / det
+  const double par = fma(odd ? m0 : ee ? m1 : m2, odd || ee ? m4 : m3,
+                         -((ee && !odd ? m2 : m1) * (odd || ee ? m3 : m4))) / det;
+  const double pu = __shfl_sync(full, par, 0), pt = __shfl_sync(full, par, 1);
+  bool inside;
+  if (type == 0) {
+    inside = pu >= 0.0 && pt >= 0.0 && pu + pt <= 1.0;
+  } else {
+    inside = det > FSIM_PARALLEL_EPS * m0 * m2 && pu > 0.0 && pu < 1.0 && pt > 0.0 && pt < 1.0;
+  }
+  double c = 0.0, c1 = 0.0, c2 = 0.0;             // this lane's vertex (lanes 0 .. 3)
+  const int i4 = lane & 3;
+  if (inside) {
+    k = 2;
+    if (type == 0) {
+      c = i4 == 0 ? 1.0 : i4 == 1 ? -(1.0 - pu - pt) : i4 == 2 ? -pu : -pt;
+      c1 = i4 == 1 ? 1.0 : i4 == 2 ? -1.0 : 0.0;
+      c2 = i4 == 1 ? 1.0 : i4 == 3 ? -1.0 : 0.0;
+    } else {
+      const double f = i4 < 2 ? pu : pt;
+      c = (odd ? f : 1.0 - f) * (i4 < 2 ? 1.0 : -1.0);
+      c1 = i4 == 0 ? -1.0 : i4 == 1 ? 1.0 : 0.0;
+      c2 = i4 == 2 ? 1.0 : i4 == 3 ? -1.0 : 0.0;
+    }
+  } else {
+    // lane l: feature l, a point against a segment (PT: three, EE: four)
+    const int nseg = type == 0 ? 3 : 4;
+    auto feature = [&](int l, int& P, int& A, int& B) {
+      if (type == 0) { P = 0; A = 1 + l; B = l == 2 ? 1 : 2 + l; }
+      else { P = l; A = l < 2 ? 2 : 0; B = A + 1; }
+    };
+    int P, A, B;
+    feature(i4 < nseg ? i4 : nseg - 1, P, A, B);
+    double ts, ds;
+    seg_closest(w.X[P], w.X[A], w.X[B], ts, ds);
+    int best = 0;
+    double dm = __shfl_sync(full, ds, 0);
+    for (int l = 1; l < nseg; ++l) {
+      const double dl = __shfl_sync(full, ds, l);
+      if (dl < dm) { best = l; dm = dl; }
+    }
+    const double t = __shfl_sync(full, ts, best);
+    feature(best, P, A, B);
+    const double sg = type == 1 && best >= 2 ? -1.0 : 1.0;
+    const bool mid = t > 0.0 && t < 1.0;
+    k = mid ? 1 : 0;
+    const double tb = mid ? t : t <= 0.0 ? 0.0 : 1.0;
+    c = i4 == P ? sg : i4 == A ? -sg * (1.0 - tb) : i4 == B ? -sg * tb : 0.0;
+    if (mid) c1 = i4 == A ? sg : i4 == B ? -sg : 0.0;
+  }
+  if (lane < 4) { w.C[0][lane] = c; w.C[1][lane] = c1; w.C[2][lane] = c2; }
+  __syncwarp();
+  return k;
+}
+
+// pair_reduced by the lanes of one warp.  The chain of one pair is float64
+// instructions (66 cycles each, however many lanes are active), about 500 of them
+// when every lane runs pair_reduced; here the entries of each small vector or
+// matrix sit in different lanes and one instruction forms them all: about 140
+// (interior features) to 180.  Divisions and square roots are taken in one go
+// each: with the Gram matrix M of the c'_k off c, scaled by |c|^2 (M_ij = |c|^2
+// c'_i.c'_j - (c.c'_i)(c.c'_j), D = det M),
+//   q_1 = (|c|^2 c'_1 - (c.c'_1) c) r2,                        r2 = (|c|^2 M_11)^-1/2,
+//   q_2 = (|c|^2 c'_2 - (c.c'_2) c - |c|^2 (q_1.c'_2) q_1) M_11 r3,
+//                                                             r3 = (|c|^2 M_11 D)^-1/2,
+//   q_1.c'_1 = M_11 r2,  q_1.c'_2 = M_12 r2,  q_2.c'_2 = D r3,
+// so that four reciprocal square roots (those of |v|^2 and |c|^2 too) need nothing
+// but dot products, and 2 log(d / dhat) = log(|v|^2 / dhat^2).
+// The workspace afterwards holds what the lift needs (C[0] = c, Q = c^, q_1, q_2
+// and vh); lane l < 15 returns the entry (i, j), i <= j, of the reduced Hessian.
+__device__ __forceinline__ double pair_reduced_warp(int type, const double* __restrict__ s,
+                                                    const int V[4], double dhat, double kappa,
+                                                    int lane, PairWarp& w, int& k, double& gfac,
+                                                    int& ri, int& rj) {
+  constexpr unsigned full = 0xffffffffu;
+  if (lane < 12) {
+    const int v = lane < 3 ? V[0] : lane < 6 ? V[1] : lane < 9 ? V[2] : V[3];
+    w.X[lane / 3][lane % 3] = s[3 * (size_t)v + lane % 3];
+  }
+  __syncwarp();
+  k = pair_features_warp(type, lane, w);
+  const bool odd = lane & 1;
+  const int i4 = lane & 3;
+  if (lane < 9) {
+    const double* cr = w.C[lane / 3];
+    const int dd = lane % 3;
+    w.W[lane / 3][dd] =
+        fma(cr[3], w.X[3][dd], fma(cr[2], w.X[2][dd], fma(cr[1], w.X[1][dd], cr[0] * w.X[0][dd])));
+  } else if (lane < 12) {
+    w.W[lane - 9][3] = 0.0;
+  }
+  __syncwarp();
+  double g = 0.0;
+  if (lane < 10) {      // v.v, E1.E1, E1.E2, E2.E2;  c.c, c.c1, c.c2, c1.c1, c1.c2, c2.c2
+    const int a = lane < 4 ? (0x2110 >> (4 * lane)) & 3 : (0x211000 >> (4 * (lane - 4))) & 3;
+    const int b = lane < 4 ? (0x2210 >> (4 * lane)) & 3 : (0x221210 >> (4 * (lane - 4))) & 3;
+    const double(*base)[4] = lane < 4 ? w.W : w.C;
+    g = dot4(base[a], base[b]);
+  }
+  const double d2 = __shfl_sync(full, g, 0), cn2 = __shfl_sync(full, g, 4),
+               a1 = __shfl_sync(full, g, 5), a2 = __shfl_sync(full, g, 6);
+  const double e00 = k > 0 ? __shfl_sync(full, g, 1) : 1.0;
+  const double e01 = k > 1 ? __shfl_sync(full, g, 2) : 0.0;
+  const double e11 = k > 1 ? __shfl_sync(full, g, 3) : 1.0;
+  // M: entries 1.1, 1.2, 2.2 in lanes 7, 8, 9
+  const double mm = fma(-(lane == 9 ? a2 : a1), lane == 7 ? a1 : a2, cn2 * g);
+  const double M00 = k > 0 ? __shfl_sync(full, mm, 7) : 1.0;
+  const double M01 = k > 1 ? __shfl_sync(full, mm, 8) : 0.0;
+  const double M11 = k > 1 ? __shfl_sync(full, mm, 9) : 1.0;
+  const double DD = fma(M00, M11, -(M01 * M01));
+  const double cM = cn2 * M00;
+  // 1 / det(E^T E) and |v|^2 / dhat^2; the reciprocal square roots
+  const double qt = (odd ? d2 : 1.0) / (odd ? dhat * dhat : fma(e00, e11, -(e01 * e01)));
+  const double id = __shfl_sync(full, qt, 0), L2 = log(__shfl_sync(full, qt, 1));
+  const double rr = rsqrt(i4 == 0 ? d2 : i4 == 1 ? cn2 : i4 == 2 ? cM : cM * DD);
+  const double inv_d = __shfl_sync(full, rr, 0), icn = __shfl_sync(full, rr, 1),
+               r2 = __shfl_sync(full, rr, 2), r3 = __shfl_sync(full, rr, 3);
+  double d = d2 * inv_d;
+  d = fma(fma(-d, d, d2), 0.5 * inv_d, d);
+  const double u = d - dhat, q = u * inv_d;
+  gfac = kappa * (-u * (L2 + q));
+  const double K1 = gfac * inv_d, K2 = kappa * fma(q, q, -fma(4.0, q, L2)) * cn2;
+  const double q01 = M01 * r2;                                   // (0 unless k = 2)
+  // c^; lanes 0 .. 3 q_1, lanes 4 .. 7 q_2
+  const double t = fma(cn2, w.C[lane & 4 ? 2 : 1][i4], -((lane & 4 ? a2 : a1) * w.C[0][i4]));
+  const double q1 = t * r2;
+  const double q1i = __shfl_sync(full, q1, i4);
+  const double q2 = fma(-cn2 * q01, q1i, t) * (M00 * r3);
+  if (lane < 4) {
+    w.Q[0][lane] = w.C[0][lane] * icn;
+    w.Q[1][lane] = k > 0 ? q1 : 0.0;
+  } else if (lane < 8) {
+    w.Q[2][i4] = k > 1 ? q2 : 0.0;
+  }
+  const int fa = lane >> 1;
+  double f = 0.0;
+  if (fa < 3) {
+    const double ch = (odd ? a2 : a1) * icn;
+    f = fma(ch, w.W[0][fa], cn2 * icn * w.W[1 + odd][fa]);
+  } else if (fa == 3) {
+    f = (odd ? q01 : M00 * r2) * d;
+  } else if (odd) {
+    f = DD * r3 * d;
+  }
+  f = (odd ? k > 1 : k > 0) ? f : 0.0;
+  if (lane < 10) w.F[fa][odd] = f;
+  else if (lane < 13) w.vh[lane - 10] = w.W[0][lane - 10] * inv_d;
+  // (E^T E)^-1 F'^T: the two entries of row fa sit in neighbouring lanes
+  const double fo = __shfl_xor_sync(full, f, 1);
+  if (lane < 10) w.T[fa][odd] = fma((odd ? e00 : e11) * id, f, -(e01 * id) * fo);
+  __syncwarp();
+  const int l15 = lane < 15 ? lane : 14;
+  ri = (int)(0x433222111100000ull >> (4 * l15)) & 7;
+  rj = (int)(0x443432432143210ull >> (4 * l15)) & 7;
+  const double vv = rj < 3 ? w.vh[ri] * w.vh[rj] : 0.0;
+  double h = -fma(w.F[ri][0], w.T[rj][0], w.F[ri][1] * w.T[rj][1]);
+  if (rj < 3) h = fma(cn2, (ri == rj ? 1.0 : 0.0) - vv, h);
+  h = fma(K1, h, K2 * vv);
+  return rj < 3 + k ? h : 0.0;
 }
 
 // Plane rotation (c, s, t = s / c) of a cyclic Jacobi step that annihilates

@@ -248,14 +248,107 @@ k_cand_ee(int Ns, int Ne, const double* __restrict__ s, const double* __restrict
   }
 }
 
+// Eigen-solve of a pair's n x n matrix (n <= 5) by one warp: lane 5 a + b holds
+// the entry x = A[a][b] and q = Q[a][b], on return the eigenvalues (diagonal of x)
+// and eigenvectors (columns of q; q is the start on entry, A = Q^T A0 Q).  Cyclic
+// Jacobi in rounds of two disjoint rotations, (r+1, r+4) and (r+2, r+3) mod 5 in
+// round r: a round rotates columns, then rows, every entry in its own lane: about
+// 20 float64 instructions of 65 cycles for two rotations.
+__device__ __forceinline__ int upper5(int a, int b) {     // lane < 15 of (a, b) in row-major upper order
+  const int i = min(a, b), j = max(a, b);
+  return i * 5 - i * (i - 1) / 2 + j - i;
+}
+// |x| as bits that order like it (float64: the upper word)
+__device__ __forceinline__ unsigned mag_bits(float x) { return __float_as_uint(x) & 0x7fffffffu; }
+__device__ __forceinline__ unsigned mag_bits(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
+__device__ __forceinline__ float bits_mag(unsigned b, float) { return __uint_as_float(b); }
+__device__ __forceinline__ double bits_mag(unsigned b, double) { return __hiloint2double((int)b, 0); }
+
+template <typename ET>
+__device__ __forceinline__ void jacobi_warp(ET& x, ET& q, int ea, int eb, int n) {
+  constexpr unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const ET tiny = sizeof(ET) == 8 ? ET(1e-300) : ET(1e-30);
+  const ET tol = sizeof(ET) == 8 ? ET(5e-16) : ET(1.5e-7);   // largest off-diagonal / diagonal
+  for (int sweep = 0; sweep < 12; ++sweep) {
+    const unsigned off = __reduce_max_sync(full, ea == eb ? 0u : mag_bits(x));
+    const unsigned dia = __reduce_max_sync(full, ea == eb ? mag_bits(x) : 0u);
+    if (!(bits_mag(off, ET(0)) > tol * bits_mag(dia, ET(0)))) break;
+    for (int r = 0; r < 5; ++r) {
+      // the rotation of this lane's pair (even lanes the first, odd the second)
+      const int u0 = (r + 1) % 5, u1 = (r + 4) % 5, u2 = (r + 2) % 5, u3 = (r + 3) % 5;
+      const int p0 = min(u0, u1), q0 = max(u0, u1), p1 = min(u2, u3), q1 = max(u2, u3);
+      const int pp = lane & 1 ? p1 : p0, qq = lane & 1 ? q1 : q0;
+      const ET app = __shfl_sync(full, x, 6 * pp), aqq = __shfl_sync(full, x, 6 * qq),
+               apq = __shfl_sync(full, x, 5 * pp + qq);
+      ET c = 1, sn = 0, t = 0;
+      if (qq < n && fabs(apq) > tiny) jacobi_rotation(app, aqq, apq, c, sn, t);
+      // columns, then rows: index i of pair h turns with its partner
+      auto pair_of = [&](int i) { return i == p0 || i == q0 ? 0 : 1; };
+      const int ha = pair_of(ea), hb = pair_of(eb);
+      const int pa = ea == r ? ea : ha ? p1 + q1 - ea : p0 + q0 - ea;
+      const int pb = eb == r ? eb : hb ? p1 + q1 - eb : p0 + q0 - eb;
+      const ET cb0 = __shfl_sync(full, c, hb), sb0 = __shfl_sync(full, sn, hb);
+      const ET ca0 = __shfl_sync(full, c, ha), sa0 = __shfl_sync(full, sn, ha);
+      const ET cb = eb == r ? ET(1) : cb0, sb = eb == r ? ET(0) : eb < pb ? -sb0 : sb0;
+      const ET ca = ea == r ? ET(1) : ca0, sa = ea == r ? ET(0) : ea < pa ? -sa0 : sa0;
+      const ET y = cb * x + sb * __shfl_sync(full, x, 5 * ea + pb);
+      ET z = ca * y + sa * __shfl_sync(full, y, 5 * pa + eb);
+      q = cb * q + sb * __shfl_sync(full, q, 5 * ea + pb);
+      if (sizeof(ET) == 4) {             // the rotated 2 x 2 block by the textbook formulas
+        const ET tb = __shfl_sync(full, t, hb), ab = __shfl_sync(full, apq, hb);
+        if (ea != r && (eb == ea || eb == pa)) z = eb != ea ? ET(0) : eb < pb ? x - tb * ab : x + tb * ab;
+      }
+      x = __shfl_sync(full, z, 5 * min(ea, eb) + max(ea, eb));   // (both triangles alike)
+    }
+  }
+}
+
+// A start for the float64 solve: float32 eigenvectors, made orthogonal in float64
+// (two Newton-Schulz steps, 1e-7 -> 1e-14 -> rounding), and the matrix in that
+// basis, nearly diagonal.  It leaves one or two float64 sweeps of five.
+__device__ __forceinline__ void jacobi_start(float&, float&, int, int, int) {}
+__device__ __forceinline__ void jacobi_start(double& x, double& q, int ea, int eb, int n) {
+  constexpr unsigned full = 0xffffffffu;
+  const unsigned big = __reduce_max_sync(full, mag_bits(x)) >> 20;      // biased exponent
+  if (big < 64 || big > 1982) return;                                   // (also 0, inf, NaN)
+  float xf = (float)(x * __hiloint2double((int)((2046 - big) << 20), 0)), qf = (float)q;
+  jacobi_warp(xf, qf, ea, eb, n);
+  double g = (double)qf;
+#pragma unroll
+  for (int it = 0; it < 2; ++it) {
+    double m = 0.0;                      // Q^T Q
+#pragma unroll
+    for (int l = 0; l < 5; ++l)
+      m = fma(__shfl_sync(full, g, 5 * l + ea), __shfl_sync(full, g, 5 * l + eb), m);
+    m = fma(-0.5, m, ea == eb ? 1.5 : 0.0);
+    double o = 0.0;
+#pragma unroll
+    for (int l = 0; l < 5; ++l)
+      o = fma(__shfl_sync(full, g, 5 * ea + l), __shfl_sync(full, m, 5 * l + eb), o);
+    g = o;
+  }
+  double y = 0.0, z = 0.0;               // Q^T (A Q)
+#pragma unroll
+  for (int l = 0; l < 5; ++l)
+    y = fma(__shfl_sync(full, x, 5 * ea + l), __shfl_sync(full, g, 5 * l + eb), y);
+#pragma unroll
+  for (int l = 0; l < 5; ++l)
+    z = fma(__shfl_sync(full, g, 5 * l + ea), __shfl_sync(full, y, 5 * l + eb), z);
+  x = __shfl_sync(full, z, 5 * min(ea, eb) + max(ea, eb));
+  q = g;
+}
+
 // Pass A, one warp per pair (single frames: few pairs, so the latency of
 // a pair's chain sets the time and the lanes share its Jacobi rotations and
 // lift).  Per-pair gradient and PSD Hessian blocks (PositiveDefinite of
 // Algorithm 1); marks the touched x2 vertices.  One warp per pair: the
-// reduced (n <= 5) Hessian is built redundantly by every lane, each cyclic
-// Jacobi rotation updates its rows, columns and eigenvectors lane-parallel,
-// and the 144 block entries of the lift are spread over the lanes.  ET is the
-// type of the small eigen-solve (float64, or float32 in the mixed form).
+// lanes share the reduced (n <= 5) Hessian's entries (pair_reduced_warp), each
+// cyclic Jacobi rotation updates its rows, columns and eigenvectors
+// lane-parallel, and the 144 block entries of the lift are spread over the lanes.
+// ET is the type of the small eigen-solve (float64, or float32 in the mixed form).
+// (Every lane forming the whole Hessian, one rotation at a time: 45 us mixed, 107
+// us float64 a launch, 30k face; so 18 and 32.)
 // One pair-warp per CTA: the float64 geometry of a pair is a long chain of
 // float64 instructions, and an SM's float64 pipe is narrow on this part, so
 // the pairs are spread over as many SMs as possible.
@@ -268,13 +361,10 @@ __device__ __forceinline__ void k_barrier_pairs_warp_body(const int* __restrict_
                 const int* __restrict__ Wcol, const int* __restrict__ x2of, double dhat,
                 double kappa, double* __restrict__ pgrad, double* __restrict__ phess,
                 int* __restrict__ x2mark) {
-  __shared__ ET As[kPairWarps][5][5];
-  __shared__ ET Qs[kPairWarps][5][5];
-  __shared__ double Qd[kPairWarps][5][5], Ld[kPairWarps][5];
   __shared__ double Hp[kPairWarps][5][5];
   __shared__ double hv[kPairWarps][4][3];
   __shared__ double sq[kPairWarps][4][4];
-  __shared__ double cs[kPairWarps][4], chs[kPairWarps][4], qs[kPairWarps][2][4], vs[kPairWarps][3];
+  __shared__ PairWarp pw[kPairWarps];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int64_t np = *count;
   np = np < cap ? np : cap;
@@ -284,124 +374,50 @@ __device__ __forceinline__ void k_barrier_pairs_warp_body(const int* __restrict_
     unpack_key(pairs[p], type, i, j);
     int V[4];
     load_pair(type, i, j, tris, edges, V);
-    double X[4][3];
-    gather_X(s, V, X);
-    int n, k;
+    int k, ri, rj;
     double gfac;
-    {   // every lane forms the pair's reduced Hessian; lane 0 stores it for the
-        // lane-parallel parts, which index it by lane
-      PairReduced r;
-      pair_reduced(type, X, dhat, kappa, r);
-      n = r.n; k = r.k; gfac = r.gfac;
-      if (lane == 0) {
-#pragma unroll
-        for (int a = 0; a < 5; ++a)
-#pragma unroll
-          for (int b = a; b < 5; ++b) {
-            const ET v = (ET)r.A[a][b];
-            As[w][a][b] = v;
-            As[w][b][a] = v;
-          }
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-          cs[w][a] = r.c[a]; chs[w][a] = r.ch[a];
-          qs[w][0][a] = r.q[0][a]; qs[w][1][a] = r.q[1][a];
-        }
-#pragma unroll
-        for (int a = 0; a < 3; ++a) vs[w][a] = r.vh[a];
-      }
-    }
-    if (lane < 25) Qs[w][lane / 5][lane % 5] = lane / 5 == lane % 5 ? ET(1) : ET(0);
-    __syncwarp();
-    const ET tiny = sizeof(ET) == 8 ? ET(1e-300) : ET(1e-30);
-    const ET tol = sizeof(ET) == 8 ? ET(1e-30) : ET(1e-13);
-    for (int sweep = 0; sweep < 12; ++sweep) {
-      ET off = 0, dia = 0;
-      for (int a = 0; a < n; ++a) {
-        dia += As[w][a][a] * As[w][a][a];
-        for (int b = a + 1; b < n; ++b) off += As[w][a][b] * As[w][a][b];
-      }
-      if (!(off > tol * dia)) break;
-      for (int pp = 0; pp < n - 1; ++pp)
-        for (int qq = pp + 1; qq < n; ++qq) {
-          const ET apq = As[w][pp][qq];
-          if (!(fabs(apq) > tiny)) continue;
-          const ET app = As[w][pp][pp], aqq = As[w][qq][qq];
-          ET c, sn, t;
-          jacobi_rotation(app, aqq, apq, c, sn, t);
-          // lanes 0..4: rows of A (columns pp, qq), lanes 8..12: rows of Q,
-          // lanes 16..18: the 2 x 2 block itself
-          ET x0 = 0, x1 = 0;
-          const bool rowl = lane < n && lane != pp && lane != qq;
-          const bool qlan = lane >= 8 && lane < 8 + n;
-          if (rowl) { x0 = As[w][lane][pp]; x1 = As[w][lane][qq]; }
-          if (qlan) { x0 = Qs[w][lane - 8][pp]; x1 = Qs[w][lane - 8][qq]; }
-          const ET np_ = c * x0 - sn * x1, nq = sn * x0 + c * x1;
-          ET blk = 0;
-          if (sizeof(ET) == 8) {
-            const ET cc = c * c, ss = sn * sn, sc = c * sn;
-            const ET k0 = lane == 16 ? cc : lane == 17 ? ss : sc;
-            const ET k1 = lane == 16 ? -2 * sc : lane == 17 ? 2 * sc : cc - ss;
-            const ET k2 = lane == 16 ? ss : lane == 17 ? cc : -sc;
-            blk = k0 * app + k1 * apq + k2 * aqq;
-          } else {
-            blk = lane == 16 ? app - t * apq : lane == 17 ? aqq + t * apq : ET(0);
-          }
-          __syncwarp();
-          if (rowl) {
-            As[w][lane][pp] = np_; As[w][pp][lane] = np_;
-            As[w][lane][qq] = nq; As[w][qq][lane] = nq;
-          }
-          if (qlan) {
-            Qs[w][lane - 8][pp] = np_;
-            Qs[w][lane - 8][qq] = nq;
-          }
-          if (lane == 16) As[w][pp][pp] = blk;
-          if (lane == 17) As[w][qq][qq] = blk;
-          if (lane == 18) { As[w][pp][qq] = blk; As[w][qq][pp] = blk; }
-          __syncwarp();
-        }
-    }
+    const ET h = (ET)pair_reduced_warp(type, s, V, dhat, kappa, lane, pw[w], k, gfac, ri, rj);
+    const int n = 3 + k;
+    const double *cs = pw[w].C[0], *chs = pw[w].Q[0], *vs = pw[w].vh;
+    const double(*qs)[4] = &pw[w].Q[1];
+    // lane 5 a + b holds the entries (a, b) of the Hessian and of its eigenvectors
+    const int ea = min(lane, 24) / 5, eb = min(lane, 24) % 5;
+    ET x = __shfl_sync(0xffffffffu, h, upper5(ea, eb)), q = ea == eb ? ET(1) : ET(0);
+    jacobi_start(x, q, ea, eb, n);
+    jacobi_warp(x, q, ea, eb, n);
     // projection: keep eigenvalues above a relative floor (zero in float64;
     // float32 rounding noise of the largest one in the mixed form)
     ET lmax = 0;
-    for (int a = 0; a < n; ++a) lmax = fmax(lmax, As[w][a][a]);
-    const ET floor_ = sizeof(ET) == 8 ? ET(0) : ET(1e-6) * lmax;
-    if (lane < 25) {
-      const int a = lane / 5, b = lane % 5;
-      Qd[w][a][b] = a < n && b < n ? (double)Qs[w][a][b] : 0.0;
-    } else if (lane < 30) {
-      const int l = lane - 25;
-      const ET lam = l < n ? As[w][l][l] : ET(0);
-      Ld[w][l] = lam > floor_ ? (double)lam : 0.0;
-    }
-    __syncwarp();
-    if (lane < 25) {
-      const int a = lane / 5, b = lane % 5;
-      double acc = 0.0;
 #pragma unroll
-      for (int l = 0; l < 5; ++l) acc = fma(Qd[w][a][l] * Ld[w][l], Qd[w][b][l], acc);
-      Hp[w][a][b] = acc;
-    }
+    for (int l = 0; l < 5; ++l) lmax = fmax(lmax, __shfl_sync(0xffffffffu, x, 6 * l));
+    const ET floor_ = sizeof(ET) == 8 ? ET(0) : ET(1e-6) * lmax;
+    const ET lam = __shfl_sync(0xffffffffu, x, 6 * eb);
+    const double qd = (double)q, ql = eb < n && lam > floor_ ? qd * (double)lam : 0.0;
+    double acc = 0.0;
+#pragma unroll
+    for (int l = 0; l < 5; ++l)
+      acc = fma(__shfl_sync(0xffffffffu, ql, 5 * ea + l), __shfl_sync(0xffffffffu, qd, 5 * eb + l),
+                acc);
+    if (lane < 25) Hp[w][ea][eb] = ea < n && eb < n ? acc : 0.0;
     __syncwarp();
     if (lane < 12) {                  // hv[i][a] = sum_m q_m[i] Hp[a][3+m]
       const int ii = lane / 3, a = lane % 3;
-      hv[w][ii][a] = fma(qs[w][1][ii], Hp[w][a][4], qs[w][0][ii] * Hp[w][a][3]);
+      hv[w][ii][a] = fma(qs[1][ii], Hp[w][a][4], qs[0][ii] * Hp[w][a][3]);
     } else if (lane < 28) {           // sq[i][j] = sum q_m[i] q_l[j] Hp[3+m][3+l]
       const int ii = (lane - 12) / 4, jj = (lane - 12) % 4;
-      const double t0 = fma(Hp[w][3][4], qs[w][1][jj], Hp[w][3][3] * qs[w][0][jj]);
-      const double t1 = fma(Hp[w][4][4], qs[w][1][jj], Hp[w][4][3] * qs[w][0][jj]);
-      sq[w][ii][jj] = fma(qs[w][1][ii], t1, qs[w][0][ii] * t0);
+      const double t0 = fma(Hp[w][3][4], qs[1][jj], Hp[w][3][3] * qs[0][jj]);
+      const double t1 = fma(Hp[w][4][4], qs[1][jj], Hp[w][4][3] * qs[0][jj]);
+      sq[w][ii][jj] = fma(qs[1][ii], t1, qs[0][ii] * t0);
     }
     __syncwarp();
-    if (lane < 12) pgrad[p * 12 + lane] = gfac * cs[w][lane / 3] * vs[w][lane % 3];
+    if (lane < 12) pgrad[p * 12 + lane] = gfac * cs[lane / 3] * vs[lane % 3];
     // block (i, j) entry (a, b), factored as in the lane-per-pair form
     for (int e = lane; e < 144; e += 32) {
       const int ab = e / 9, rc = e % 9;
       const int ii = ab / 4, jj = ab % 4, a = rc / 3, b = rc % 3;
-      const double t1 = fma(hv[w][jj][a], vs[w][b], chs[w][jj] * Hp[w][a][b]);
-      const double t2 = fma(sq[w][ii][jj], vs[w][b], chs[w][jj] * hv[w][ii][b]);
-      phess[p * 144 + e] = fma(chs[w][ii], t1, vs[w][a] * t2);
+      const double t1 = fma(hv[w][jj][a], vs[b], chs[jj] * Hp[w][a][b]);
+      const double t2 = fma(sq[w][ii][jj], vs[b], chs[jj] * hv[w][ii][b]);
+      phess[p * 144 + e] = fma(chs[ii], t1, vs[a] * t2);
     }
     if (lane < 4)
       for (int64_t e = Wptr[V[lane]]; e < Wptr[V[lane] + 1]; ++e) {
@@ -1652,6 +1668,21 @@ __global__ void __launch_bounds__(kPairLanes) k_barrier_pairs_b(const DevMesh* _
                                 m->pair_hess, m->x2mark);
 }
 
+// a warp per pair
+__global__ void __launch_bounds__(32 * kPairWarps) k_barrier_pairs_warp_b(
+    const DevMesh* __restrict__ tab, double dhat) {
+  const DevMesh* m = bframe_c(tab, blockIdx.y);
+  if (!m) return;
+  if (m->bar64)
+    k_barrier_pairs_warp_body<double>(m->counters, m->cap_act, m->pairs, m->s, m->tris, m->edges,
+                                      m->Wptr, m->Wcol, m->x2of, dhat, m->kappa_f, m->pair_grad,
+                                      m->pair_hess, m->x2mark);
+  else
+    k_barrier_pairs_warp_body<float>(m->counters, m->cap_act, m->pairs, m->s, m->tris, m->edges,
+                                     m->Wptr, m->Wcol, m->x2of, dhat, m->kappa_f, m->pair_grad,
+                                     m->pair_hess, m->x2mark);
+}
+
 __global__ void __launch_bounds__(32) k_mollify_ee_b(const DevMesh* __restrict__ tab, double dhat) {
   const DevMesh* m = bframe_c(tab, blockIdx.y);
   if (!m) return;
@@ -1754,15 +1785,27 @@ void launch_detect_b(cudaStream_t st, const DevMesh* tab, int nb, const DevMesh&
   count_launch(2);
 }
 
+// Most pairs (frames x longest list) of a batch that take a warp each: a warp's
+// chain is about 180 float64 instructions for one pair, a lane's 700 for 32 of
+// them, so the first form ends sooner until several warps share each SM
+// sub-partition.  16 5k faces: 67 us a launch with lanes, 21 with warps; three
+// batches of 32 30k faces in flight: 427 ms with lanes, 430 with warps for up to 4096
+// pairs, 422 to 425 so.
+constexpr int64_t kPairWarpMax = 1536;
+
 void launch_barrier_b(cudaStream_t st, const DevMesh* tab, int nb, const DevMesh& m0,
                       int64_t np_max, double dhat) {
   np_max = np_max < m0.cap_act ? np_max : m0.cap_act;
   if (np_max > 0) {
     ProfScope ps(PROF_BARRIER, st);
-    const int64_t want = (np_max + kPairLanes - 1) / kPairLanes;    // one lane per pair
-    const unsigned grid = (unsigned)(want < 8 * 152 ? want : 8 * 152);
     const unsigned mgrid = (unsigned)(np_max < 8 * 152 ? np_max : 8 * 152);
-    k_barrier_pairs_b<<<dim3(grid, nb), kPairLanes, 0, st>>>(tab, dhat);
+    if (np_max * nb <= kPairWarpMax) {
+      k_barrier_pairs_warp_b<<<dim3(mgrid, nb), 32 * kPairWarps, 0, st>>>(tab, dhat);
+    } else {
+      const int64_t want = (np_max + kPairLanes - 1) / kPairLanes;
+      const unsigned grid = (unsigned)(want < 8 * 152 ? want : 8 * 152);
+      k_barrier_pairs_b<<<dim3(grid, nb), kPairLanes, 0, st>>>(tab, dhat);
+    }
     count_launch();
     if (m0.ee_moll) {
       k_mollify_ee_b<<<dim3(mgrid, nb), 32, 0, st>>>(tab, dhat);
