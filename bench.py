@@ -746,7 +746,7 @@ def batch_rooflines(bprof, info):
         if cls == "local_step":
             flop = LOCAL_FLOP_PER_TET * T * nb
             ach = flop / (avg * 1e-3) / 1e12
-            e.update({"bound": "alu", "kernel": "k_elastic_df_b (+ k_disp_df_b, partial sums)",
+            e.update({"bound": "alu", "kernel": "k_elastic_df_b (+ partial sums)",
                       "achieved": ach, "peak": FP32_TFLOPS_PEAK, "unit": "TFLOP/s",
                       "frac": ach / FP32_TFLOPS_PEAK,
                       "work": f"{LOCAL_FLOP_PER_TET:.0f} float32 flop per tet x T x frames",

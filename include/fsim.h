@@ -166,8 +166,9 @@ enum {
                                    the mixed form for n_c > 128)                   */
   FSIM_REDUCED_NONE = 1,        /* mixed form, n_c = 0: dx2 = Sigma^-1 y2          */
   FSIM_REDUCED_ONE_CTA = 2,     /* mixed form, 0 < n_c <= reduced_one_cta_max
-                                   (96 by default): one CTA                       */
-  FSIM_REDUCED_CLUSTER = 3      /* mixed form, above that up to 128: 4-CTA cluster */
+                                   (96 by default): the factor in one CTA         */
+  FSIM_REDUCED_CLUSTER = 3      /* mixed form, above that up to 128: the factor on
+                                   a 4-CTA cluster                                 */
 };
 
 /* Fill *p with the defaults: weight_scale 1e3, kappa auto, tol_abs 1e-8,

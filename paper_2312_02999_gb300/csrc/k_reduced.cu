@@ -27,7 +27,7 @@
 // Steps 1-5 need only B-check and Sigma^-1, so they run on a side stream while
 // the forward solve makes u.  Two forms: the grid form (float64, and float32
 // with n_c > 128), and for float32 n_c <= 128 the one-CTA and cluster kernels
-// k_small_s/x/n/v and k_clus_v.
+// k_small_s/x/n/v, k_clus_v, k_small_u and k_small_solve.
 #include <cooperative_groups.h>
 
 #include <algorithm>
