@@ -251,6 +251,9 @@ int alloc_workspace(const MeshState& ms, DevMesh& m, DeviceMem mem) {
   if (mem.arena && !mem.arena->base) return FSIM_OK;
   CK(cudaMemset(zero, 0, kStatusBytes));
   CK(cudaMemset(m.sb + 3 * Ns, 0, sizeof(double) * 3));      // words of k_skin_check
+  // a memset may return before it has run, and the workspace's own stream does
+  // not wait for the legacy one
+  CK(cudaStreamSynchronize(cudaStreamLegacy));
   return FSIM_OK;
 }
 
