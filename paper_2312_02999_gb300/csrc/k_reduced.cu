@@ -34,6 +34,7 @@
 #include <cmath>
 #include <cstring>
 #include <type_traits>
+#include <utility>
 #include <vector>
 
 #include "kernels.h"
@@ -1827,6 +1828,9 @@ __device__ __forceinline__ void k_small_solve_body(RedArgs<float> a) {
   __shared__ double nrm_parts[2][kSolveCl];
   const int nc = *a.nc_dev;
   if (nc == 0 || nc > a.small_lim) return;          // uniform over the cluster
+  // every CTA of the cluster has to have started before another one stores into
+  // its shared memory: arrive here, wait just before the first such store
+  auto started = cl.barrier_arrive();
   red_layout(a, nc);
   const int n3 = 3 * nc, rank = (int)cl.block_rank();
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -1965,6 +1969,7 @@ __device__ __forceinline__ void k_small_solve_body(RedArgs<float> a) {
   }
   double ys = 0.0;
   for (int e = gt; e < 3 * a.n2; e += nt) ys += (double)a.y2[e] * (double)a.y2[e];
+  cl.barrier_wait(std::move(started));
   ys = cluster_sum(ys, 0);
   apply(a.y, false);
   double prev = -1.0;
