@@ -152,10 +152,13 @@ typedef struct {
   int32_t reduced_steps[4]; /* global steps of the frame by the path that solved
                                the reduced system (index = FSIM_REDUCED_*)    */
   int32_t fp64_steps;       /* FSIM_MIXED: global steps taken with the float64
-                               factors because a float32 factor of the reduced
-                               (or Schur) system lost positive definiteness:
-                               the failed step is redone in float64 and every
-                               later global step of the frame stays there   */
+                               factors because a float32 factor failed.  Where a
+                               factor of the reduced (or Schur) system lost
+                               positive definiteness, the step is redone in
+                               float64 and every later global step of the frame
+                               stays there; where the refinement of a reduced
+                               system's solve left more than 1e-5 of its
+                               right-hand side, that step alone is redone     */
 } fsim_frame_stats;
 
 /* Path that solves the reduced contact system of Eq. 11 in one global step
@@ -314,7 +317,10 @@ fsim_status fsim_eval_sigma_inv_mr(fsim_ctx_t ctx, int mesh_id, const double* y,
 /* Global step (Eq. 4 through Eq. 8-11): dx_out [3n] solves
  * (H + PositiveDefinite(B)) dx = -g-hat at x (zero on pinned vertices).
  * path_out (may be NULL) receives the FSIM_REDUCED_* path that solved the
- * reduced system. */
+ * reduced system.  As in a frame, a FSIM_MIXED step whose float32 factor lost
+ * positive definiteness, or whose float32 solve could not be refined to 1e-5 of
+ * its right-hand side, is taken with float64 factors (path
+ * FSIM_REDUCED_COOPERATIVE). */
 fsim_status fsim_eval_global_step(fsim_ctx_t ctx, int mesh_id, const double* x,
                                   int precision, double* dx_out, int32_t* path_out);
 

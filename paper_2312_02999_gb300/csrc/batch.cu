@@ -433,8 +433,8 @@ class Batch {
   }
 
   // The single-frame float64 global step (Eq. 8-11) and CCD bound of frame f
-  // on its own workspace, on the batch's stream.  With `hessian` (the frame's
-  // first float64 step) the frame's contact Hessian is first assembled again
+  // on its own workspace, on the batch's stream.  With `hessian` (the first step of
+  // a frame that stays in float64) the frame's contact Hessian is first assembled again
   // at x with float64 pair eigen-solves, as it is for the rest of the frame;
   // x is evaluated again because the trial evaluation replaced its pair list.
   int redo_fp64(int f, bool hessian) {
@@ -550,16 +550,18 @@ class Batch {
         if (!srch[f]) continue;
         Frame& fr = frames_[f];
         if (fr.trial == 0 && cnt(f)[6] && !fr.redone) {
-          // the float32 factor of the frame's reduced system lost positive
-          // definiteness: its step again in float64 (the single-frame global
-          // step on its own workspace), then its CCD bound; its line search
-          // starts over at the next trial
+          // the float32 factor of the frame's reduced system failed: its step again
+          // in float64 (the single-frame global step on its own workspace), then
+          // its CCD bound; its line search starts over at the next trial.  Where
+          // the factor lost positive definiteness the frame stays in float64; a
+          // refinement that only stalled costs this step
+          const bool stays = cnt(f)[6] != kInfoStalled;
           fr.redone = true;
-          fr.fp64 = true;
+          fr.fp64 = stays;
           fr.st.fp64_steps++;
           fr.st.reduced_steps[reduced_path(fr.nc, FSIM_MIXED, tab_[f].one_cta_max)]--;
           fr.st.reduced_steps[reduced_path(fr.nc, FSIM_FP64, tab_[f].one_cta_max)]++;
-          BTRY(redo_fp64(f, true));
+          BTRY(redo_fp64(f, stays));
           fr.scale = 1.0;
           continue;
         }

@@ -494,7 +494,8 @@ int solve_frame_impl(const Exec& ex, const MeshState& ms, DevMesh& m, const doub
   }
   // precision of the contact Hessian and the global step: the frame's own,
   // until a float32 factor of the reduced (or Schur) system loses positive
-  // definiteness; from then on the frame's pair eigen-solves and global steps
+  // definiteness (one whose refinement stalls costs that step only); from then
+  // on the frame's pair eigen-solves and global steps
   // run in float64 (a frame that got that stiff stays stiff while its pairs
   // stay close, and the float32 eigen-solve's relative floor drops the soft
   // directions of such pairs)
@@ -557,21 +558,22 @@ int solve_frame_impl(const Exec& ex, const MeshState& ms, DevMesh& m, const doub
       TRY(sync(ex));
       if (k == 0 && ex.h_counters[6] && gprec != FSIM_FP64 && p.solver != FSIM_SOLVER_PCG &&
           !redone) {
-        // the float32 factor of the reduced (or Schur) system lost positive
-        // definiteness (cond ~ 1 / u32 at very stiff pairs): the contact
+        // the float32 factor of the reduced (or Schur) system failed (cond ~ 1 / u32
+        // at very stiff pairs): this global step in float64, its CCD bound and a
+        // fresh line search.  Where it lost positive definiteness, first the contact
         // Hessian at x again with float64 eigen-solves (the trial evaluation
-        // replaced the pair list, so x is evaluated again first), this global
-        // step in float64, its CCD bound and a fresh line search
+        // replaced the pair list, so x is evaluated again), and the frame stays
+        // there; a refinement that only stalled keeps Hessian and precision
         redone = true;
-        gprec = FSIM_FP64;
         st.fp64_steps++;
         if (p.solver == FSIM_SOLVER_WOODBURY) {
           st.reduced_steps[reduced_path(nc, prec, m.one_cta_max)]--;
           st.reduced_steps[reduced_path(nc, FSIM_FP64, m.one_cta_max)]++;
         }
-        TRY(eval_at(m.x, m.s, m.tetf));
-        TRY(sync_read(ex, m));
-        {
+        if (ex.h_counters[6] != kInfoStalled) {
+          gprec = FSIM_FP64;
+          TRY(eval_at(m.x, m.s, m.tetf));
+          TRY(sync_read(ex, m));
           double gn2r;
           TRY(gradient_and_hessian(ex, ms, m, m.s, m.tetf, m.g, prec, &nc, &gn2r, kappa, gprec, true,
                                    kgen));
@@ -1361,10 +1363,24 @@ fsim_status fsim_eval_global_step(fsim_ctx_t ctx, int mesh_id, const double* x, 
                    ms->p.solver == FSIM_SOLVER_SCHUR, nc));
   }
   TRY(sync_read(ex, m));
+  int form = precision;            // of the reduced system's solve
+  const int failed = ctx->h_counters[6];
+  if (precision != FSIM_FP64 && ms->p.solver == FSIM_SOLVER_WOODBURY && failed &&
+      !(failed & kInfoTimeout)) {
+    // as in a frame: the step again with float64 factors, and after a lost pivot
+    // with the pairs' eigen-solves in float64 too
+    form = FSIM_FP64;
+    if (failed & kInfoPivot)
+      TRY(gradient_and_hessian(ex, *ms, m, m.st, m.tetf_t, ms->gtmp, precision, &nc, &gn2, ms->kappa,
+                               FSIM_FP64));
+    CK(cudaMemsetAsync(m.counters + 6, 0, sizeof(int) * 2, s));
+    CK(global_step(s, m, ms->gtmp, ms->dxtmp, form, m.counters + 6, ex.coop_ctas, ex.alone, false, nc));
+    TRY(sync_read(ex, m));
+  }
   if (ctx->h_counters[6]) return FSIM_ENOT_SPD;
   CK(cudaMemcpy(dx_out, ms->dxtmp, sizeof(double) * 3 * (size_t)m.n, cudaMemcpyDeviceToHost));
   if (path_out)
-    *path_out = ms->p.solver == FSIM_SOLVER_WOODBURY ? reduced_path(nc, precision, m.one_cta_max)
+    *path_out = ms->p.solver == FSIM_SOLVER_WOODBURY ? reduced_path(nc, form, m.one_cta_max)
                                                      : FSIM_REDUCED_UNUSED;
   return FSIM_OK;
 }

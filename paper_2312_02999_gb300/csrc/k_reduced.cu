@@ -23,6 +23,10 @@
 //     ~1e-3 d0 with every vertex of the reduced set in contact) a float32
 //     factor gains only 4-10x per step, and 4 steps left |rho| near
 //     1e-3 |y2|; the stopping rule ends well-conditioned solves after 1-2.
+//     Beyond cond(N) of a few 1e6 a step may gain nothing or lose (a pair at 5.7e-4
+//     d0: |rho| 2 to 40 |y2|, with every pivot positive), so the v of the smaller
+//     residual is kept and, if that is above kAcceptRho |y2|, the solve is
+//     reported (kInfoStalled): the caller solves it again with float64 factors.
 //   8 z2 = u - (Sigma^-1[:, c] (x) I_3) v
 // Steps 1-5 need only B-check and Sigma^-1, so they run on a side stream while
 // the forward solve makes u.  Two forms: the grid form (float64, and float32
@@ -46,6 +50,10 @@ namespace fsim {
 namespace {
 
 constexpr int kRT = 256;   // threads per CTA
+// Largest |rho| / |y2| a refined float32 solve may leave: rho reaches the step as
+// (Sigma + B)^-1 rho.  Solves with cond(N) below 1e6 end at 1e-7 or less, those that
+// stop gaining end at 1e-3 to 40, so the line may lie anywhere between.
+constexpr double kAcceptRho = 1e-5;
 
 // Padded packed lower storage: row i holds columns 0..i, padded to a
 // multiple of 4 floats, so 32-column segments of a row are 16-byte aligned.
@@ -79,6 +87,7 @@ struct RedArgs {
   double* v;            // n3
   double* rho;          // n3
   double* w;            // n3
+  double* vp;           // n3: v before the last refinement step
   double* nrm;          // 3: |rho|^2 of a refinement step (two slots), |y2|^2
   double* S64;          // small forms: Sigma^-1[c, c] in float64 (n_c x n_c)
   int* info;
@@ -98,8 +107,8 @@ template <typename FT>
 __device__ __forceinline__ void red_tail(RedArgs<FT>& a, int nc) {
   const int n3 = 3 * nc;
   a.nc = nc;
-  a.y = a.dtail_end - 4 * (size_t)n3 - 8;
-  a.v = a.y + n3; a.rho = a.v + n3; a.w = a.rho + n3; a.nrm = a.w + n3;
+  a.y = a.dtail_end - 5 * (size_t)n3 - 8;
+  a.v = a.y + n3; a.rho = a.v + n3; a.w = a.rho + n3; a.vp = a.w + n3; a.nrm = a.vp + n3;
   a.S64 = a.y - (size_t)nc * nc;
   a.list = a.ibase;
   a.cnt = a.list + (size_t)nc * nc;
@@ -298,7 +307,7 @@ __device__ __forceinline__ void diag_factor(ChSm& sm, const float* Pt, int ldp, 
   if (tid < 32) {
     float p = sm.col[tid][tid];
     const bool bad = !(p > 0.f);
-    if (bad) { atomicOr(info, 1); p = 1.f; }
+    if (bad) { atomicOr(info, kInfoPivot); p = 1.f; }
     float pi = significand(p);
 #pragma unroll
     for (int s = 1; s < 32; s <<= 1) {
@@ -422,7 +431,7 @@ __device__ __forceinline__ void group_sync(GroupBar& b) {
         asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(v) : "l"(b.word) : "memory");
         if ((int)(v - b.target) >= 0) break;
         if (++polls > kSpinLimit) {
-          atomicOr(b.info, 4);
+          atomicOr(b.info, kInfoTimeout);
           b.dead = true;
         }
       }
@@ -558,7 +567,7 @@ __device__ void grid_diag(double* A, int k, int ld, int kp, double* dg, int* inf
     // col[j][j] / pi, so L[r][j] = col[j][r] / sqrt(col[j][j] pi)
     double p = sm.d.col[tid][tid];
     const bool bad = !(p > 0.0);
-    if (bad) { atomicOr(info, 1); p = 1.0; }
+    if (bad) { atomicOr(info, kInfoPivot); p = 1.0; }
     double pi = significand(p);
 #pragma unroll
     for (int s = 1; s < 32; s <<= 1) {
@@ -1040,6 +1049,20 @@ __device__ __forceinline__ void grid_u(const GridLay<FT>& g, const FT* x, FT* ou
   }
 }
 
+// Refinement of a float32 factor's solve by |rho|^2 (tot; of the step before:
+// prev, negative before the first) and |y2|^2 (ys).  refined: no further step;
+// step_lost: the last one is taken back; accepted: what is left is small enough.
+// A NaN ends the steps, is taken back where that helps and is not accepted.
+__device__ __forceinline__ bool refined(double tot, double prev, double ys, int it, int steps) {
+  return !(tot > 1e-14 * ys) || (prev >= 0.0 && !(tot < 0.25 * prev)) || it >= steps;
+}
+__device__ __forceinline__ bool step_lost(double tot, double prev) {
+  return prev >= 0.0 && !(tot <= prev);
+}
+__device__ __forceinline__ bool accepted(double tot, double prev, double ys) {
+  return (step_lost(tot, prev) ? prev : tot) <= kAcceptRho * kAcceptRho * ys;
+}
+
 template <typename FT>
 __device__ void grid_solve(RedArgs<FT> a, int rank, int Gall, GridSmem<FT>& sm) {
   const int nc = *a.nc_dev;
@@ -1107,7 +1130,9 @@ __device__ void grid_solve(RedArgs<FT> a, int rank, int Gall, GridSmem<FT>& sm) 
       }
       if (lane < 3) {
         const double d = (double)(lane == 0 ? s0 : lane == 1 ? s1 : s2);
-        a.v[3 * i + lane] = (add ? ldg2(a.v + 3 * i + lane) : 0.0) + d;
+        const double v0 = add ? ldg2(a.v + 3 * i + lane) : 0.0;
+        if (add) a.vp[3 * i + lane] = v0;
+        a.v[3 * i + lane] = v0 + d;
       }
     }
     group_sync(bar);
@@ -1115,11 +1140,11 @@ __device__ void grid_solve(RedArgs<FT> a, int rank, int Gall, GridSmem<FT>& sm) 
   apply(a.y, false);
   // 7. refinement with float64 residuals: a.refine steps with float64 factors;
   //    with float32 factors until |rho| <= 1e-7 |y2|, until a step fails to
-  //    halve |rho|, or after a.refine steps.  |rho|^2 alternates between two
-  //    accumulators
+  //    halve |rho|, or after a.refine steps, and the v of the smaller |rho|
+  //    stays.  |rho|^2 alternates between two accumulators
   constexpr bool f64 = std::is_same<FT, double>::value;
   double prev = -1.0;
-  for (int it = 0; it < a.refine; ++it) {
+  for (int it = 0; !f64 || it < a.refine; ++it) {
     // w = S v with S = Sigma^-1[c, c] (x) I_3 in float64, a warp per row
     for (int i = gwarp; i < nc; i += nwarps) {
       const double* srow = a.Sinv + (size_t)a.clist[i] * a.n2;
@@ -1182,8 +1207,14 @@ __device__ void grid_solve(RedArgs<FT> a, int rank, int Gall, GridSmem<FT>& sm) 
     if (!f64) {
       // the same values for every thread of the system: a uniform decision
       const double tot = ldg2(a.nrm + (it & 1)), ys = ldg2(a.nrm + 2);
-      if (!(tot > 1e-14 * ys)) break;
-      if (prev >= 0.0 && !(tot < 0.25 * prev)) break;
+      if (refined(tot, prev, ys, it, a.refine)) {
+        if (step_lost(tot, prev)) {
+          for (int e = gtid; e < n3; e += gsz) a.v[e] = ldg2(a.vp + e);
+          group_sync(bar);
+        }
+        if (gtid == 0 && !accepted(tot, prev, ys)) atomicOr(a.info, kInfoStalled);
+        break;
+      }
       prev = tot;
     }
     apply(a.rho, true);
@@ -1289,7 +1320,7 @@ __device__ void cta_chol_packed(float* A, int n, float* Pt, int* info, float* ou
     if (tid < kb) {
       float d = Ds[tid][tid];
       if (!(d > 0.f)) {
-        atomicOr(info, 1);
+        atomicOr(info, kInfoPivot);
         d = 1.f;
         Ds[tid][tid] = 1.f;
       }
@@ -1667,7 +1698,7 @@ __device__ __forceinline__ void inverse_column(const float* P, const float* DI, 
         asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(v) : "l"(done) : "memory");
       } while (v <= (unsigned)k && ++polls <= kSpinLimit);
       if (v <= (unsigned)k) {      // (gave up: the step fails, later panels are not waited for)
-        atomicOr(info, 4);
+        atomicOr(info, kInfoTimeout);
         done = nullptr;
       }
       __threadfence();
@@ -1928,7 +1959,9 @@ __device__ __forceinline__ void k_small_solve_body(RedArgs<float> a) {
         float s = 0.f;
 #pragma unroll
         for (int w = 0; w < kSolveW; ++w) s += part[wid][w][lane];
-        a.v[3 * i + wid] = (add ? a.v[3 * i + wid] : 0.0) + (double)s;
+        const double v0 = add ? a.v[3 * i + wid] : 0.0;
+        if (add) a.vp[3 * i + wid] = v0;
+        a.v[3 * i + wid] = v0 + (double)s;
       }
     }
     cl.sync();
@@ -1973,13 +2006,17 @@ __device__ __forceinline__ void k_small_solve_body(RedArgs<float> a) {
   ys = cluster_sum(ys, 0);
   apply(a.y, false);
   double prev = -1.0;
-  for (int it = 0; it < a.refine; ++it) {
+  for (int it = 0;; ++it) {
     refine_sv(a, nc, gt, nt);
     cl.sync();
     // two slots in turn: a CTA may still read the one of the step before
     const double r2 = cluster_sum(refine_rho(a, nc, gt, nt), (it + 1) & 1);
-    if (!(r2 > 1e-14 * ys)) break;
-    if (prev >= 0.0 && !(r2 < 0.25 * prev)) break;
+    if (refined(r2, prev, ys, it, a.refine)) {
+      if (step_lost(r2, prev))
+        for (int e = gt; e < n3; e += nt) a.v[e] = a.vp[e];
+      if (gt == 0 && !accepted(r2, prev, ys)) atomicOr(a.info, kInfoStalled);
+      break;
+    }
     prev = r2;
     apply(a.rho, true);
   }
@@ -2092,7 +2129,7 @@ __device__ __forceinline__ void k_clus_v_body(RedArgs<float> a) {
       if (tid < kb) {
         float d = Ds[tid][tid];
         if (!(d > 0.f)) {
-          atomicOr(a.info, 1);
+          atomicOr(a.info, kInfoPivot);
           d = 1.f;
           Ds[tid][tid] = 1.f;
         }
@@ -2350,8 +2387,8 @@ int64_t reduced_workspace_elems(int nc) {
   // inverted diagonal blocks (each rounded up to 16 bytes)
   const int64_t small = 2 * (int64_t)nc * nc + n3 * n3 + n3 * (n3 + 4) / 2 + 8 + 2 * n3 +
                         (int64_t)nc * (nc + 4) / 2 + 8 + 1024 * (((int64_t)nc + 31) / 32) + 64;
-  // at the tail of the float64 buffer four float64 vectors, three norms and S64
-  return std::max(small, grid_front_elems(nc)) + 4 * n3 + (int64_t)nc * nc + 64;
+  // at the tail of the float64 buffer five float64 vectors, three norms and S64
+  return std::max(small, grid_front_elems(nc)) + 5 * n3 + (int64_t)nc * nc + 64;
 }
 
 // Most float64 refinement steps of a float32 reduced factor (see step 7).

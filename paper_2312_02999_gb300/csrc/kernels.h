@@ -217,6 +217,12 @@ void launch_zero_reduced(cudaStream_t s, const DevMesh& m, int nc_cap);
 // nc_host: n_c as read back by the host (selects the reduced-system path).
 cudaError_t global_step(cudaStream_t s, const DevMesh& m, const double* g, double* dx, int precision,
                         int* info_dev, int num_sms, bool alone, bool dense_schur, int nc_host);
+// Bits of a global step's info word.
+enum {
+  kInfoPivot = 1,      // a factor lost positive definiteness
+  kInfoStalled = 2,    // a float32 reduced factor's refinement left too large a residual
+  kInfoTimeout = 4     // a wait between CTAs ran out
+};
 // Reduced-system path a global step takes for this n_c and precision (graph key).
 int reduced_path(int nc_host, int precision, int one_cta_max);
 // Schur-only variant of the x2 block (k_schur.cu): z2 = Sigma-hat^-1 y2 with
