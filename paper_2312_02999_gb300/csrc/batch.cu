@@ -386,7 +386,7 @@ class Batch {
       Frame& fr = frames_[f];
       DevMesh& m = tab_[f];
       const int nc = cnt(f)[3];
-      const int cap_now = m.Bc != nullptr ? m.nc_cap : 0;
+      const int cap_now = m.nc_cap;
       BTRY(rt_ensure_reduced(ex, m, std::max(nc, 1)));
       if (nc > cap_now) {          // buffers grew: assemble B-check again (one frame)
         BCK(cudaMemsetAsync(m.Bc, 0, sizeof(double) * 9 * (size_t)nc * nc, s_));

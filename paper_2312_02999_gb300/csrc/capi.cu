@@ -130,50 +130,35 @@ int sync_read(const Exec& ex, const DevMesh& m) {
   return sync(ex);
 }
 
-// Make the reduced-system buffers of workspace m large enough for nc
-// contact vertices (grows by 1.5x, at most to n2).
 size_t reduced_bytes(int cap) {
-  if (cap <= 0) return 0;
-  const int64_t n3 = 3 * (int64_t)cap;
-  return sizeof(double) * (size_t)(n3 * n3) + sizeof(int) * (size_t)(2 * (int64_t)cap * cap + cap + 32) +
-         (sizeof(double) + sizeof(float)) * (size_t)reduced_workspace_elems(cap);
+  return cap <= 0 ? 0 : reduced_view_bytes(cap, reduced_workspace_elems(cap));
 }
 
-// The reduced-system buffers of workspace m for cap contact vertices.
-int reduced_buffers(DeviceMem mem, DevMesh& m, int cap) {
-  const int64_t n3 = 3 * (int64_t)cap;
-  TRY(mem.take(&m.Bc, (size_t)(n3 * n3)));
-  TRY(mem.take(&m.bocc, (size_t)(2 * (int64_t)cap * cap + cap + 32)));
-  m.red_cap = reduced_workspace_elems(cap);
-  TRY(mem.take(&m.red, (size_t)m.red_cap));
-  TRY(mem.take(&m.redf, (size_t)m.red_cap));
-  m.nc_cap = cap;
-  return FSIM_OK;
-}
-
+// Make the reduced-system buffers of workspace m large enough for nc contact
+// vertices.
 int ensure_reduced(const Exec& ex, DevMesh& m, int nc) {
-  if (nc <= m.nc_cap && m.Bc != nullptr) return FSIM_OK;
-  int cap = std::max(nc, std::max(16, m.nc_cap * 3 / 2));
-  cap = std::min(cap, std::max(m.n2, 1));
-  const size_t old_bytes = m.Bc != nullptr ? reduced_bytes(m.nc_cap) : 0;
-  const size_t new_bytes = reduced_bytes(cap);
+  if (reduced_fits(m, nc)) return FSIM_OK;
+  const int cap = grown_reduced_cap(nc, m.nc_cap, m.n2);
+  const size_t old_bytes = reduced_bytes(m.nc_cap), new_bytes = reduced_bytes(cap);
   if (ex.grow && new_bytes > old_bytes && ex.grow(ex.grow_user, new_bytes - old_bytes) != 0)
     return FSIM_ENOMEM;
   CK(cudaStreamSynchronize(ex.stream));
-  auto release = [&](void* p) {      // (a buffer of a batch's one allocation stays in it)
+  auto alloc = [&](size_t bytes) -> void* {
+    char* p = nullptr;
+    return dalloc(*ex.allocs, &p, bytes, ex.bytes) == FSIM_OK ? p : nullptr;
+  };
+  auto release = [&](void* p) {      // (a place in a batch's one allocation stays in it)
     auto& v = *ex.allocs;
     const auto it = std::find(v.begin(), v.end(), p);
-    if (it == v.end()) return;
-    cudaFree(p);
-    v.erase(it);
+    if (it != v.end()) {
+      cudaFree(p);
+      v.erase(it);
+    }
+    if (ex.bytes) *ex.bytes -= std::min(*ex.bytes, old_bytes);
   };
-  release(m.Bc); release(m.bocc); release(m.red); release(m.redf);
-  m.Bc = nullptr; m.bocc = nullptr; m.red = nullptr; m.redf = nullptr;
-  if (ex.bytes) *ex.bytes -= std::min(*ex.bytes, old_bytes);
-  TRY(reduced_buffers(DeviceMem{ex.allocs, ex.bytes, nullptr}, m, cap));
+  if (!grow_reduced(m, cap, reduced_workspace_elems(cap), alloc, release)) return FSIM_ENOMEM;
   // the barrier counters after the lists start at zero (and are left at zero)
   CK(cudaMemsetAsync(m.bocc + 2 * (int64_t)cap * cap + cap, 0, sizeof(int) * 32, ex.stream));
-  m.red_gen++;
   return FSIM_OK;
 }
 
@@ -246,8 +231,7 @@ int alloc_workspace(const MeshState& ms, DevMesh& m, DeviceMem mem) {
   TRY(mem.take(&m.pair_hess, 144 * (size_t)m.cap_act));
   TRY(mem.take(&m.x2mark, (size_t)std::max(m.n2, 1)));
   TRY(mem.take(&m.clist, (size_t)std::max(m.n2, 1)));
-  m.Bc = nullptr; m.bocc = nullptr; m.red = nullptr; m.redf = nullptr;
-  m.red_cap = 0; m.nc_cap = 0;
+  set_reduced(m, ReducedViews{}, 0, 0);
   if (mem.arena && !mem.arena->base) return FSIM_OK;
   CK(cudaMemset(zero, 0, kStatusBytes));
   CK(cudaMemset(m.sb + 3 * Ns, 0, sizeof(double) * 3));      // words of k_skin_check
@@ -411,7 +395,7 @@ int gradient_and_hessian(const Exec& ex, const MeshState& ms, DevMesh& m, const 
                          const double* tetf, double* gout, int prec, int* nc_out, double* gn2_out,
                          double kappa, int bprec, bool graph = false, int kgen = 0) {
   cudaStream_t s = ex.stream;
-  const int cap_now = m.Bc != nullptr ? m.nc_cap : 0;
+  const int cap_now = m.nc_cap;
   auto body = [&] { return gradient_launches(ex, ms, m, sb, tetf, gout, prec, kappa, bprec, cap_now); };
   if (graph) {
     const int key2 = 2 * prec + bprec;
@@ -633,7 +617,8 @@ int rt_alloc_workspace(const MeshState& ms, DevMesh& m, std::vector<void*>& allo
 }
 int rt_place_workspace(const MeshState& ms, DevMesh& m, Arena& arena, int nc_cap, size_t* bytes) {
   TRY(alloc_workspace(ms, m, DeviceMem{nullptr, bytes, &arena}));
-  TRY(reduced_buffers(DeviceMem{nullptr, nullptr, &arena}, m, nc_cap));
+  const int64_t elems = reduced_workspace_elems(nc_cap);
+  set_reduced(m, reduced_views(arena, nc_cap, elems), nc_cap, elems);
   if (arena.base)
     CK(cudaMemset(m.bocc + 2 * (int64_t)nc_cap * nc_cap + nc_cap, 0, sizeof(int) * 32));
   return FSIM_OK;

@@ -10,6 +10,7 @@
 
 #include "../../include/fsim.h"
 #include "kernels.h"
+#include "workspace.h"
 
 namespace fsim {
 
@@ -62,17 +63,6 @@ struct Exec {
 // Allocate the per-solve buffers of workspace m (a copy of a prefactored
 // mesh's DevMesh whose constant pointers stay shared).
 int rt_alloc_workspace(const MeshState& ms, DevMesh& m, std::vector<void*>& allocs, size_t* bytes);
-// One device allocation handed out in 512-byte steps; with base NULL it only
-// counts what it would hand out.
-struct Arena {
-  char* base = nullptr;
-  size_t used = 0;
-  void* take(size_t bytes) {
-    void* p = base ? base + used : nullptr;
-    used += (bytes + 511) / 512 * 512;
-    return p;
-  }
-};
 // A workspace (without side streams) and its reduced-system buffers for nc_cap
 // contact vertices in an arena; *bytes grows by the workspace's own bytes.
 int rt_place_workspace(const MeshState& ms, DevMesh& m, Arena& arena, int nc_cap, size_t* bytes);
