@@ -1404,7 +1404,8 @@ fsim_status fsim_eval_energy(fsim_ctx_t ctx, int mesh_id, const double* x, int p
   const double E = ctx->h_scal[2] + ctx->h_scal[0];
   int nc = 0;
   double gn2 = 0.0;
-  TRY(gradient_and_hessian(ex, *ms, m, m.st, m.tetf_t, ms->gtmp, 0, &nc, &gn2, ms->kappa, 0));
+  TRY(gradient_and_hessian(ex, *ms, m, m.st, m.tetf_t, ms->gtmp, precision, &nc, &gn2, ms->kappa,
+                           FSIM_FP64));
   if (energy_out) *energy_out = E;
   if (grad_norm_out) *grad_norm_out = std::sqrt(gn2);
   return FSIM_OK;
