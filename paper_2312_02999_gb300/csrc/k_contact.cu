@@ -877,6 +877,9 @@ __global__ void k_zero_reduced(const int* __restrict__ ncp, int nc_cap, double* 
   k_zero_reduced_body(ncp, nc_cap, Bc, bocc);
 }
 
+// 1 / l_p, finite: no advance of a touching pair becomes 0 * inf
+__device__ __forceinline__ double accd_reciprocal(double lp) { return fmin(1.0 / lp, 1e308); }
+
 // Additive CCD (Li, Kaufman & Jiang 2021) time of impact of one candidate, or 1
 // if that is not before *least, the smallest one any pair has found so far: only
 // the minimum over the pairs counts, and a march's t never decreases, so the march
@@ -886,6 +889,9 @@ __global__ void k_zero_reduced(const int* __restrict__ ncp, int nc_cap, double* 
 // step bound of 0.02: the twenty first, largest steps of a batch of 16 5k faces
 // took up to 8.6 ms here, 44 of a solve's 107 ms.  With the bound: that solve 108.8
 // -> 101.2 ms, one step and its bound of a pressed 12k face 1.98 -> 1.60 ms.
+// accd_toi_warp rounds every operation alike (fused where this is, quotients by l_p
+// as products with 1 / l_p), so the bound does not depend on which form a pair
+// meets, and repeats to the bit.
 __device__ double accd_toi(int type, double X[4][3], double dX[4][3], double s_ratio, int max_iters,
                            const double* least) {
   auto reached = [&](double t) { return t >= *reinterpret_cast<const volatile double*>(least); };
@@ -897,7 +903,7 @@ __device__ double accd_toi(int type, double X[4][3], double dX[4][3], double s_r
   for (int k = 0; k < 4; ++k) {
 #pragma unroll
     for (int d = 0; d < 3; ++d) dX[k][d] -= mean[d];
-    nrm[k] = sqrt((dX[k][0] * dX[k][0] + dX[k][1] * dX[k][1]) + dX[k][2] * dX[k][2]);
+    nrm[k] = sqrt(dot3(dX[k], dX[k]));
   }
   const double lp = type == 1 ? fmax(nrm[0], nrm[1]) + fmax(nrm[2], nrm[3])
                               : nrm[0] + fmax(fmax(nrm[1], nrm[2]), nrm[3]);
@@ -911,21 +917,21 @@ __device__ double accd_toi(int type, double X[4][3], double dX[4][3], double s_r
     const double df = (double)pair_distance_f(type, Xf);
     if ((1.0 - s_ratio) * df * (1.0 - 1e-3) > lp * (1.0 + 1e-3)) return 1.0;
   }
-  const double d0 = pair_distance(type, X);
+  const double d0 = pair_distance(type, X), ilp = accd_reciprocal(lp);
   const double gap = s_ratio * d0;
   double t = 0.0;
-  double step = (1.0 - s_ratio) * d0 / lp;
+  double step = (1.0 - s_ratio) * d0 * ilp;
   if (reached(step)) return 1.0;
   for (int it = 0; it < max_iters; ++it) {
 #pragma unroll
     for (int k = 0; k < 4; ++k)
 #pragma unroll
-      for (int d = 0; d < 3; ++d) X[k][d] += step * dX[k][d];
+      for (int d = 0; d < 3; ++d) X[k][d] = fma(step, dX[k][d], X[k][d]);
     const double d = pair_distance(type, X);
     if (t > 0.0 && d < gap) return t;
     t += step;
     if (t > 1.0 || reached(t)) return 1.0;
-    step = 0.9 * d / lp;
+    step = 0.9 * d * ilp;
   }
   return fmin(t, 1.0);
 }
@@ -1252,7 +1258,7 @@ __global__ void k_near_pairs(const int* __restrict__ near_count, int64_t cap, in
 
 // accd_toi by the lanes of one warp, for a pair at w.X (one coordinate per lane, as
 // loaded) with the step dx (lane 3 k + d < 12): about 75 float64 instructions an
-// iteration where one lane needs 250.  Quotients by l_p are products with 1 / l_p.
+// iteration where one lane needs 250, each rounded as there.
 __device__ double accd_toi_warp(int type, double dx, double s_ratio, int max_iters,
                                 const double* least, int lane, PairWarp& w) {
   constexpr unsigned full = 0xffffffffu;
@@ -1277,7 +1283,7 @@ __device__ double accd_toi_warp(int type, double dx, double s_ratio, int max_ite
                  v2 = __shfl_sync(full, v, 2);
     return sqrt(fma(v2, v2, fma(v1, v1, v0 * v0)));
   };
-  const double d0 = distance(), ilp = 1.0 / lp;
+  const double d0 = distance(), ilp = accd_reciprocal(lp);
   const double gap = s_ratio * d0;
   double t = 0.0, step = (1.0 - s_ratio) * d0 * ilp;
   // (one lane's view of *least for all: the lanes leave together)
