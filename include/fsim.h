@@ -191,6 +191,10 @@ fsim_status fsim_destroy(fsim_ctx_t ctx);
 /* Number of kernel launches this context issued so far (instrumentation). */
 fsim_status fsim_launch_count(fsim_ctx_t ctx, int64_t* count);
 
+/* Number of launch sequences captured as CUDA graphs so far (instrumentation):
+ * a workspace captures the sequences of its first frames and replays them. */
+fsim_status fsim_capture_count(fsim_ctx_t ctx, int64_t* count);
+
 /*
  * Upload one simulation mesh and its collision proxy (Sec. 2.1, Sec. 3.1).
  *   rest_xyz   [3n]    rest positions (also the initial state)

@@ -5,6 +5,7 @@
 // that steer the loop (gradient norm, n_c, candidate count, trial energy);
 // every arithmetic step of an iteration runs in the CUDA kernels.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -271,6 +272,8 @@ void destroy_graphs(DevMesh& m) {
   m.aux_stream = m.aux_stream2 = nullptr;
 }
 
+std::atomic<int64_t> g_captures{0};      // launch sequences captured so far
+
 // Run a fixed launch sequence through a CUDA graph captured on first use
 // (one host launch instead of one per kernel).  The graph is recaptured
 // when its key buffer, precision, reduced-buffer generation or cooperative
@@ -318,6 +321,7 @@ int with_graph(const Exec& ex, DevMesh& m, int slot, const void* key, int key2, 
     }
     g.exec = exec; g.key = key; g.key2 = key2; g.gen = gen; g.coop = ex.coop_ctas; g.alone = ex.alone;
     g.host = ex.h_scal;
+    g_captures.fetch_add(1);
     g.kernels = kernels;
   }
   CK(cudaGraphLaunch((cudaGraphExec_t)g.exec, ex.stream));
@@ -715,6 +719,12 @@ fsim_status fsim_destroy(fsim_ctx_t ctx) {
 fsim_status fsim_launch_count(fsim_ctx_t ctx, int64_t* count) {
   if (!ctx || !count) return FSIM_EINVAL;
   *count = launch_counter();
+  return FSIM_OK;
+}
+
+fsim_status fsim_capture_count(fsim_ctx_t ctx, int64_t* count) {
+  if (!ctx || !count) return FSIM_EINVAL;
+  *count = g_captures.load();
   return FSIM_OK;
 }
 

@@ -1,9 +1,9 @@
 // Request server: continuous batching of frame solves (Algorithm 1) over
 // the meshes of one context.
 //
-// Each worker is one host thread with its own CUDA stream and pinned
-// read-back words.  A request runs on a workspace slot (a private copy of
-// the per-solve buffers of its mesh, sharing the mesh's factor, Sigma^-1 and
+// Each worker is one host thread with its own CUDA stream.  A request runs on
+// a workspace slot (a private copy of the per-solve buffers of its mesh with its
+// own pinned read-back words, sharing the mesh's factor, Sigma^-1 and
 // topology), so solves of different meshes, or several frames of the same
 // mesh, run concurrently and their kernels overlap on the GPU.  A worker that
 // finishes a request immediately takes the next admissible one from the
@@ -68,15 +68,17 @@ struct Slot {
   size_t bytes = 0;
   bool busy = false;
   int64_t last_used = 0;
-  double* h_x = nullptr;      // pinned staging: 3n positions
+  // pinned status words: the captured graphs of d copy into them, so they belong to
+  // the slot, whichever worker runs it
+  int* h_counters = nullptr;
+  double* h_scal = nullptr;
+  double* h_x = nullptr;      // pinned staging: 3n positions (same allocation, after them)
   double* h_act = nullptr;    // pinned staging: 3T fiber + T stretch
 };
 
 struct Worker {
   std::thread th;
   cudaStream_t stream = nullptr;
-  int* h_counters = nullptr;
-  double* h_scal = nullptr;
 };
 
 }  // namespace
@@ -108,10 +110,10 @@ namespace {
 void free_slot(Slot& s) {
   rt_destroy_graphs(s.d);
   rt_free_list(s.allocs);
-  if (s.h_x) cudaFreeHost(s.h_x);
+  if (s.h_scal) cudaFreeHost(s.h_scal);
   if (s.h_act) cudaFreeHost(s.h_act);
-  s.h_x = nullptr;
-  s.h_act = nullptr;
+  s.h_scal = s.h_x = s.h_act = nullptr;
+  s.h_counters = nullptr;
 }
 
 size_t slot_need(const MeshState& ms) { return rt_slot_bytes(ms); }
@@ -121,13 +123,15 @@ int make_slot(fsim_server_s* sv, const MeshState& ms, int mesh_id, Slot& s) {
   s.d = ms.d;   // constant pointers shared, per-solve ones replaced below
   int rc = rt_alloc_workspace(ms, s.d, s.allocs, &s.bytes);
   if (rc != FSIM_OK) return rc;
-  if (cudaHostAlloc((void**)&s.h_x, sizeof(double) * 3 * (size_t)ms.d.n, cudaHostAllocDefault) !=
-          cudaSuccess ||
+  if (cudaHostAlloc((void**)&s.h_scal, kStatusBytes + sizeof(double) * 3 * (size_t)ms.d.n,
+                    cudaHostAllocDefault) != cudaSuccess ||
       cudaHostAlloc((void**)&s.h_act, sizeof(double) * 4 * (size_t)ms.d.T, cudaHostAllocDefault) !=
           cudaSuccess) {
     cudaGetLastError();
     return FSIM_ENOMEM;
   }
+  s.h_counters = reinterpret_cast<int*>(s.h_scal + kScal);
+  s.h_x = s.h_scal + kStatusBytes / sizeof(double);
   (void)sv;
   return FSIM_OK;
 }
@@ -156,8 +160,8 @@ int run_job(fsim_server_s* sv, Worker& w, Slot& s, Job& J, Growth* growth) {
   const size_t n = (size_t)m.n, T = (size_t)m.T;
   Exec ex;
   ex.stream = st;
-  ex.h_counters = w.h_counters;
-  ex.h_scal = w.h_scal;
+  ex.h_counters = s.h_counters;
+  ex.h_scal = s.h_scal;
   ex.coop_ctas = sv->coop_ctas;
   ex.alone = sv->n_workers == 1;
   ex.allocs = &s.allocs;
@@ -449,17 +453,13 @@ fsim_status fsim_server_create(fsim_ctx_t ctx, const fsim_server_config* cfg, fs
   int prio_lo = 0, prio_hi = 0;     // worker streams above the side streams
   cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi);
   for (auto& w : sv->workers) {
-    if (cudaStreamCreateWithPriority(&w.stream, cudaStreamNonBlocking, prio_hi) != cudaSuccess ||
-        cudaHostAlloc((void**)&w.h_scal, kStatusBytes, cudaHostAllocDefault) != cudaSuccess) {
+    if (cudaStreamCreateWithPriority(&w.stream, cudaStreamNonBlocking, prio_hi) != cudaSuccess) {
       cudaGetLastError();
-      for (auto& x : sv->workers) {
+      for (auto& x : sv->workers)
         if (x.stream) cudaStreamDestroy(x.stream);
-        if (x.h_scal) cudaFreeHost(x.h_scal);
-      }
       delete sv;
       return FSIM_ENOMEM;
     }
-    w.h_counters = reinterpret_cast<int*>(w.h_scal + kScal);
   }
   for (int i = 0; i < cfg->workers; ++i)
     sv->workers[i].th = std::thread(sv->batch_frames >= 2 ? batch_worker_main : worker_main, sv, i);
@@ -564,7 +564,6 @@ fsim_status fsim_server_destroy(fsim_server_t sv) {
   for (auto& w : sv->workers) {
     cudaStreamSynchronize(w.stream);
     cudaStreamDestroy(w.stream);
-    cudaFreeHost(w.h_scal);
   }
   for (auto& s : sv->slots) free_slot(*s);
   delete sv;

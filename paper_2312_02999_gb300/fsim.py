@@ -115,6 +115,7 @@ _SIGS = {
     "fsim_create": [C.POINTER(_P), C.c_int],
     "fsim_destroy": [_P],
     "fsim_launch_count": [_P, _I64],
+    "fsim_capture_count": [_P, _I64],
     "fsim_mesh_upload": [_P, C.POINTER(C.c_int), _D, C.c_int64, _I32, C.c_int64, _U8, _I32,
                          C.c_int64, _I64, _I32, _D, C.c_int64, _U8],
     "fsim_prefactor": [_P, C.c_int, C.POINTER(Params)],
@@ -245,6 +246,11 @@ class Context:
     def launch_count(self) -> int:
         v = C.c_int64()
         _chk(self.lib.fsim_launch_count(self.h, C.byref(v)), "fsim_launch_count")
+        return int(v.value)
+
+    def capture_count(self) -> int:
+        v = C.c_int64()
+        _chk(self.lib.fsim_capture_count(self.h, C.byref(v)), "fsim_capture_count")
         return int(v.value)
 
     def stream_ptr(self) -> int:
