@@ -151,10 +151,9 @@ int ensure_reduced(const Exec& ex, DevMesh& m, int nc) {
   auto release = [&](void* p) {      // (a place in a batch's one allocation stays in it)
     auto& v = *ex.allocs;
     const auto it = std::find(v.begin(), v.end(), p);
-    if (it != v.end()) {
-      cudaFree(p);
-      v.erase(it);
-    }
+    if (it == v.end()) return;
+    cudaFree(p);
+    v.erase(it);
     if (ex.bytes) *ex.bytes -= std::min(*ex.bytes, old_bytes);
   };
   if (!grow_reduced(m, cap, reduced_workspace_elems(cap), alloc, release)) return FSIM_ENOMEM;

@@ -406,6 +406,10 @@ void batch_worker_main(fsim_server_s* sv, int wi) {
     const int rc = batch_run(b, pull, done);
     lk.lock();
     sv->running--;
+    // what its frames' reduced buffers grew by
+    const size_t b_now = batch_bytes(b);
+    sv->used += b_now - b_bytes;
+    b_bytes = b_now;
     if (rc == FSIM_ECUDA) {      // a failed batch is not reused
       lk.unlock();
       batch_destroy(b);
