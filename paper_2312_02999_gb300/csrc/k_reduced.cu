@@ -41,6 +41,7 @@
 #include <utility>
 #include <vector>
 
+#include "df64.cuh"
 #include "kernels.h"
 
 namespace cg = cooperative_groups;
@@ -2419,49 +2420,79 @@ namespace {
 // (coalesced reads of the rows of Phi_t) with kPhiSplit warps, each summing
 // a strided share of the n_c columns; v (as float) and the c list are staged
 // in shared memory.  The work is bound by load latency, hence the split.
+// PAIRS: v and the sums as float pairs.  The forces v of a pair nearly cancel in
+// x1; with float32 sums the worst entry's error is 0.73 u32 of the contact-free step
+// at n_c = 162 (median of 40 states), with pairs 0.48, which is Phi's own rounding.
+// Taken for n_c > 128, where x1 would otherwise be a backward solve from z2 on the
+// solve's own stream (40 to 60k faces: 11 to 14 % more time a frame); float32 sums
+// there made the whole step's median error 1.15 to 1.6 times that of the solve.
+// Below, pairs would cost 0.5 to 0.9 % of a frame.
 constexpr int kPhiSplit = 8;
+template <bool PAIRS>
 __global__ void __launch_bounds__(32 * kPhiSplit) k_phi_apply(RedArgs<float> a, int n1,
                                                              const float* __restrict__ phi_t,
                                                              const float* __restrict__ bx1,
                                                              double* __restrict__ x1) {
-  __shared__ float vs[3 * kClusNc];
+  constexpr int kParts = PAIRS ? 2 : 1;            // high parts, then low parts
+  __shared__ float vs[kParts][3 * kClusNc];
   __shared__ int cs[kClusNc];
-  __shared__ float part[kPhiSplit][3][32];
+  __shared__ float part[kParts][kPhiSplit][3][32];
   const int nc = *a.nc_dev;
   if (nc > 0) red_tail(a, nc);
   const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
   const int p = blockIdx.x * 32 + lane;
-  float c0 = 0.f, c1 = 0.f, c2 = 0.f;
+  float c[3] = {0.f, 0.f, 0.f}, e[3] = {0.f, 0.f, 0.f};
+  auto add = [&](int d, float h, float l) {        // c + e += h + l
+    const df s = df_two_sum(c[d], h);
+    c[d] = s.hi;
+    e[d] += s.lo + l;
+  };
   for (int k0 = 0; k0 < nc; k0 += kClusNc) {       // n_c in chunks of the staging size
     const int kn = min(kClusNc, nc - k0);
     __syncthreads();
     for (int k = threadIdx.x; k < kn; k += blockDim.x) {
       const bool okc = FSIM_CHECK_IDX(a.clist[k0 + k], a.n2, CHECK_CLIST);
       cs[k] = okc ? a.clist[k0 + k] : 0;
-      vs[3 * k] = okc ? (float)a.v[3 * (k0 + k)] : 0.f;
-      vs[3 * k + 1] = okc ? (float)a.v[3 * (k0 + k) + 1] : 0.f;
-      vs[3 * k + 2] = okc ? (float)a.v[3 * (k0 + k) + 2] : 0.f;
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        const double v = okc ? a.v[3 * (k0 + k) + d] : 0.0;
+        vs[0][3 * k + d] = (float)v;
+        if (PAIRS) vs[kParts - 1][3 * k + d] = df_from_double(v).lo;
+      }
     }
     __syncthreads();
     if (p < n1) {
 #pragma unroll 4
       for (int k = wq; k < kn; k += kPhiSplit) {
         const float f = phi_t[(size_t)cs[k] * n1 + p];
-        c0 += f * vs[3 * k];
-        c1 += f * vs[3 * k + 1];
-        c2 += f * vs[3 * k + 2];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          if (PAIRS) {
+            const df t = df_two_prod(f, vs[0][3 * k + d]);
+            add(d, t.hi, __fmaf_rn(f, vs[kParts - 1][3 * k + d], t.lo));
+          } else {
+            c[d] += f * vs[0][3 * k + d];
+          }
+        }
       }
     }
   }
-  part[wq][0][lane] = c0;
-  part[wq][1][lane] = c1;
-  part[wq][2][lane] = c2;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    part[0][wq][d][lane] = c[d];
+    if (PAIRS) part[kParts - 1][wq][d][lane] = e[d];
+  }
   __syncthreads();
   if (wq < 3 && p < n1) {
-    float t = 0.f;
+    const float b = bx1[3 * (size_t)p + wq];
+    c[0] = PAIRS ? b : 0.f;
+    e[0] = 0.f;
 #pragma unroll
-    for (int q = 0; q < kPhiSplit; ++q) t += part[q][wq][lane];
-    x1[3 * (size_t)p + wq] = (double)bx1[3 * (size_t)p + wq] + (double)t;
+    for (int q = 0; q < kPhiSplit; ++q) {
+      if (PAIRS) add(0, part[0][q][wq][lane], part[kParts - 1][q][wq][lane]);
+      else c[0] += part[0][q][wq][lane];
+    }
+    x1[3 * (size_t)p + wq] = (double)c[0] + (double)(PAIRS ? e[0] : b);
   }
 }
 
@@ -2657,9 +2688,10 @@ cudaError_t phi_apply_b(cudaStream_t s, const void* args_dev, const int* cols_de
 }
 
 cudaError_t phi_apply(cudaStream_t s, const DevMesh& m, const double* u, const void* y2, double* z2,
-                      int* info, const float* bx1, double* x1) {
+                      int* info, const float* bx1, double* x1, int nc_host) {
   const RedArgs<float> a = make_args<float>(m, u, (const float*)y2, z2, info, kMixedRefineSteps);
-  k_phi_apply<<<(m.n1 + 31) / 32, 32 * kPhiSplit, 0, s>>>(a, m.n1, m.Phi_t, bx1, x1);
+  const auto kernel = nc_host > kClusNc ? k_phi_apply<true> : k_phi_apply<false>;
+  kernel<<<(m.n1 + 31) / 32, 32 * kPhiSplit, 0, s>>>(a, m.n1, m.Phi_t, bx1, x1);
   count_launch();
   return cudaGetLastError();
 }

@@ -645,7 +645,7 @@ cudaError_t global_step_t(cudaStream_t s, const DevMesh& m, const double* g, dou
         if (e != cudaSuccess) return e;
       }
       if (cudaStreamWaitEvent(s, m.ev_join2, 0) != cudaSuccess) return cudaGetLastError();
-      const cudaError_t e = phi_apply(s, m, u, y2, z2, info, m.bx, r);
+      const cudaError_t e = phi_apply(s, m, u, y2, z2, info, m.bx, r, nc_host);
       if (e != cudaSuccess) return e;
       k_scatter_dx<<<nblk(m.n, 256), 256, 0, s>>>(m.n, m.pos, r, dx);
       count_launch();

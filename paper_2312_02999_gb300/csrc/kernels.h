@@ -252,7 +252,7 @@ cudaError_t reduced_prepare(cudaStream_t s, const DevMesh& m, const double* u, c
 // x1 = bx1 + Phi[:, c] v (float64 out, solver order, 3 per position) after a
 // prepared reduced solve (k_reduced.cu); reads n_c on the device.
 cudaError_t phi_apply(cudaStream_t s, const DevMesh& m, const double* u, const void* y2, double* z2,
-                      int* info, const float* bx1, double* x1);
+                      int* info, const float* bx1, double* x1, int nc_host);
 // Phi_t at prefactor time (k_solve.cu), from the float64 factor and Sigma^-1,
 // using the mesh workspace's float64 solve vectors as scratch.
 cudaError_t compute_phi(cudaStream_t s, const DevMesh& m, float* phi_t);
