@@ -2,8 +2,9 @@
 
 Each translation unit is compiled by nvcc in parallel and the objects are
 linked into a shared library next to this file.  The contact kernels are
-compiled without FMA contraction so that their float64 distance and
-box arithmetic rounds every operation like the CPU reference does.
+compiled without FMA contraction: their float64 boxes round every operation like
+the CPU reference does, and where their distances, closest points and marches fuse,
+they say so, so that the forms of a kernel (a lane or a warp per pair) round alike.
 """
 from __future__ import annotations
 
